@@ -301,65 +301,151 @@ NNS_DEV void group_sync(int bar) {
   else asm volatile("bar.sync %0, %1;" ::"r"(bar), "r"(TG_THREADS) : "memory");
 }
 
-// One 256-thread group: for the consumers cons[c0 .. c0+nc) (positions in the
-// active consumer list, or c0.. directly when cons is null) and the suppliers
-// at positions [p0, p1), the lowest (key32 bits << 32 | position).  Each
-// thread owns 4 consumers x 4 suppliers of a tile; the key of every pair is
-// accumulated over k = 0..d-1 in order (fma from +0, which equals the
-// definition's first product), so it is bit-identical to key32.  Returns, in
-// the threads with tx == 0, the keys of their 4 consumers (others: ~0).
-template <bool L1>
-NNS_DEV void group_nns_tile(const float* __restrict__ x, const int* __restrict__ ia, int p0, int p1,
-                            const float* __restrict__ y, const int* __restrict__ ja, const int* __restrict__ cons,
-                            int c0, int nc, int d, TileSmem& T, int gt, int bar, unsigned long long out[4]) {
+// One 256-thread group: the FP32 keys of the consumers cons[c0 .. c0+nc)
+// (positions in the list ja, or c0.. directly when cons is null; positions
+// are row numbers where ja is null) against the suppliers at positions
+// [p0, p1) (likewise through ia), TG_N suppliers at a time.  A thread owns 4
+// consumers x 4 suppliers of a tile, the consumers packed two per FP32x2
+// register; every pair's key is accumulated over k = 0..d-1 in order (fma
+// from +0, which equals the definition's first product), so it is
+// bit-identical to key32.  emit(pt, acc) takes each finished tile of
+// suppliers pt..: acc[i][j] holds consumers 2i, 2i+1 of this thread against
+// its supplier j (suppliers past p1 are NaN, consumers past nc arbitrary).
+//
+// Bound by the FP32 pipe (2 packed instructions per 2 pairs and coordinate)
+// as long as the tiles arrive: rows of whole 16-byte vectors are read 16
+// bytes per lane, 4 lanes to a 64-byte piece of one row (a warp touches 8
+// rows per load; one row per lane with 4-byte loads cost 32 L1 lookups a load
+// and kept the pipe at 0.30: the 16,384-point FP32 solve at d = 64 went from
+// 6.87 to 3.55 ms, the 300 x 700 pair at d = 128 from 580 to 430 us).  PRE fetches the next 32 coordinates into registers
+// while the current ones are used (for kernels with registers to spare).
+template <bool L1, bool PRE, class Emit>
+NNS_DEV void group_tiles(const float* __restrict__ x, const int* ia, int p0, int p1, const float* __restrict__ y,
+                         const int* ja, const int* cons, int c0, int nc, int d, TileSmem& T, int gt, int bar,
+                         Emit emit) {
   const int tx = gt & 15, ty = gt >> 4;
+  const bool vec = (d & 3) == 0 && ((reinterpret_cast<uintptr_t>(x) | reinterpret_cast<uintptr_t>(y)) & 15) == 0;
+  // loader: row lr of the tile, coordinates lk..lk+3 and lk+16..lk+19 of a chunk
+  const int lr = gt >> 2, lk = (gt & 3) * 4;
+  const float* yrow = nullptr;
+  if (lr < nc) {
+    const int q = cons ? cons[c0 + lr] : c0 + lr;
+    yrow = y + (size_t)(ja ? ja[q] : q) * d;
+  }
+  const int nch = (d + TG_K - 1) / TG_K;
+  const int steps = (p1 - p0 + TG_N - 1) / TG_N * nch;
+  float4 rx[2], ry[2];
+  auto fetch = [&](const float* row, int k, float pad) -> float4 {
+    float4 v = make_float4(pad, pad, pad, pad);
+    if (row) {
+      if (vec) {
+        v = k < d ? *reinterpret_cast<const float4*>(row + k) : make_float4(0.f, 0.f, 0.f, 0.f);
+      } else {
+        v.x = k < d ? row[k] : 0.f;
+        v.y = k + 1 < d ? row[k + 1] : 0.f;
+        v.z = k + 2 < d ? row[k + 2] : 0.f;
+        v.w = k + 3 < d ? row[k + 3] : 0.f;
+      }
+    }
+    return v;
+  };
+  int lt = p0, lc = 0;  // supplier tile and chunk of the next fetch
+  const float* xrow = nullptr;
+  auto load = [&]() {
+    if (lc == 0) {
+      const int sp = lt + lr;
+      xrow = sp < p1 ? x + (size_t)(ia ? ia[sp] : sp) * d : nullptr;
+    }
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      const int k = lc * TG_K + lk + 16 * h;
+      rx[h] = fetch(xrow, k, CUDART_NAN_F);
+      ry[h] = fetch(yrow, k, 0.f);
+    }
+    if (++lc == nch) {
+      lc = 0;
+      lt += TG_N;
+    }
+  };
+  unsigned long long acc[2][4];
+#pragma unroll
+  for (int i = 0; i < 2; ++i)
+#pragma unroll
+    for (int j = 0; j < 4; ++j) acc[i][j] = 0ULL;
+  int pt = p0, ch = 0;
+  if (PRE && steps > 0) load();
+  for (int s = 0; s < steps; ++s) {
+    if (!PRE) load();
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      const int k = lk + 16 * h;
+      T.Xs[k][lr] = rx[h].x;
+      T.Xs[k + 1][lr] = rx[h].y;
+      T.Xs[k + 2][lr] = rx[h].z;
+      T.Xs[k + 3][lr] = rx[h].w;
+      T.Ys[k][lr] = ry[h].x;
+      T.Ys[k + 1][lr] = ry[h].y;
+      T.Ys[k + 2][lr] = ry[h].z;
+      T.Ys[k + 3][lr] = ry[h].w;
+    }
+    group_sync(bar);
+    if (PRE && s + 1 < steps) load();
+    const int kn = min(TG_K, (d - ch * TG_K + 7) & ~7);  // coordinates past d are 0 - 0 on both sides
+#pragma unroll 1
+    for (int kb = 0; kb < kn; kb += 8)
+#pragma unroll
+      for (int ku = 0; ku < 8; ++ku) {
+        const int k = kb + ku;
+        const float4 xv = *reinterpret_cast<const float4*>(&T.Xs[k][tx * 4]);
+        const ulonglong2 yv = *reinterpret_cast<const ulonglong2*>(&T.Ys[k][ty * 4]);
+        const float xa[4] = {xv.x, xv.y, xv.z, xv.w};
+        const unsigned long long ya[2] = {yv.x, yv.y};
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+          const unsigned long long xx = f2_pack(xa[j], xa[j]);
+#pragma unroll
+          for (int i = 0; i < 2; ++i) {
+            const unsigned long long t = f2_sub(xx, ya[i]);
+            acc[i][j] = L1 ? f2_add(acc[i][j], t & 0x7fffffff7fffffffULL) : f2_fma(t, t, acc[i][j]);
+          }
+        }
+      }
+    group_sync(bar);
+    if (++ch == nch) {
+      ch = 0;
+      emit(pt, acc);
+      pt += TG_N;
+#pragma unroll
+      for (int i = 0; i < 2; ++i)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) acc[i][j] = 0ULL;
+    }
+  }
+}
+
+// The lowest (key32 bits << 32 | position) over the suppliers [p0, p1) of
+// each consumer of group_tiles; returned, in the threads with tx == 0, for
+// their 4 consumers (others: ~0).
+template <bool L1, bool PRE = false>
+NNS_DEV void group_nns_tile(const float* __restrict__ x, const int* ia, int p0, int p1, const float* __restrict__ y,
+                            const int* ja, const int* cons, int c0, int nc, int d, TileSmem& T, int gt, int bar,
+                            unsigned long long out[4]) {
+  const int tx = gt & 15;
   float best[4];
   int bpos[4];
 #pragma unroll
   for (int i = 0; i < 4; ++i) { best[i] = CUDART_INF_F; bpos[i] = -1; }
-  // loader mapping: row r of the tile, 8 consecutive coordinates
-  const int lr = gt & 63, lk = (gt >> 6) * 8;
-  const int cq = c0 + lr;
-  const float* yrow = nullptr;
-  if (lr < nc) yrow = y + (size_t)ja[cons ? cons[cq] : cq] * d;
-  for (int pt = p0; pt < p1; pt += TG_N) {
-    float acc[4][4];
+  group_tiles<L1, PRE>(x, ia, p0, p1, y, ja, cons, c0, nc, d, T, gt, bar,
+                       [&](int pt, const unsigned long long (&acc)[2][4]) {
 #pragma unroll
-    for (int i = 0; i < 4; ++i)
+                         for (int j = 0; j < 4; ++j)
 #pragma unroll
-      for (int j = 0; j < 4; ++j) acc[i][j] = 0.f;
-    const int sp = pt + lr;
-    const float* xrow = sp < p1 ? x + (size_t)ia[sp] * d : nullptr;
-    for (int k0 = 0; k0 < d; k0 += TG_K) {
-#pragma unroll
-      for (int e = 0; e < 8; ++e) {
-        const int k = k0 + lk + e;
-        T.Ys[lk + e][lr] = (yrow && k < d) ? yrow[k] : 0.f;
-        T.Xs[lk + e][lr] = xrow ? (k < d ? xrow[k] : 0.f) : CUDART_NAN_F;
-      }
-      group_sync(bar);
-#pragma unroll 8
-      for (int k = 0; k < TG_K; ++k) {
-        const float4 xv = *reinterpret_cast<const float4*>(&T.Xs[k][tx * 4]);
-        const float4 yv = *reinterpret_cast<const float4*>(&T.Ys[k][ty * 4]);
-        const float xa[4] = {xv.x, xv.y, xv.z, xv.w};
-        const float ya[4] = {yv.x, yv.y, yv.z, yv.w};
-#pragma unroll
-        for (int i = 0; i < 4; ++i)
-#pragma unroll
-          for (int j = 0; j < 4; ++j) {
-            const float t = __fsub_rn(xa[j], ya[i]);
-            acc[i][j] = L1 ? __fadd_rn(acc[i][j], fabsf(t)) : __fmaf_rn(t, t, acc[i][j]);
-          }
-      }
-      group_sync(bar);
-    }
-#pragma unroll
-    for (int i = 0; i < 4; ++i)
-#pragma unroll
-      for (int j = 0; j < 4; ++j)
-        if (acc[i][j] < best[i]) { best[i] = acc[i][j]; bpos[i] = pt + tx * 4 + j; }
-  }
+                           for (int i = 0; i < 2; ++i) {
+                             const float lo = f2_lo(acc[i][j]), hi = f2_hi(acc[i][j]);
+                             if (lo < best[2 * i]) { best[2 * i] = lo; bpos[2 * i] = pt + tx * 4 + j; }
+                             if (hi < best[2 * i + 1]) { best[2 * i + 1] = hi; bpos[2 * i + 1] = pt + tx * 4 + j; }
+                           }
+                       });
   // reduce over the 16 threads sharing each consumer (adjacent lanes)
 #pragma unroll
   for (int i = 0; i < 4; ++i) {

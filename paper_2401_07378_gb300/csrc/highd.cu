@@ -22,7 +22,7 @@
 namespace nnsemd {
 
 template <bool L1>
-__global__ void __launch_bounds__(TG_THREADS)
+__global__ void __launch_bounds__(TG_THREADS, 3)
     k_nns_f32_tiled(const float* __restrict__ x, const int* __restrict__ ia, int mt, int chunk,
                     const float* __restrict__ y, const int* __restrict__ ja, const int* __restrict__ cons,
                     const int* __restrict__ ncons_dev, int ncons, int d, unsigned long long* __restrict__ nnkey) {
@@ -34,7 +34,7 @@ __global__ void __launch_bounds__(TG_THREADS)
   const int p1 = min(p0 + chunk, mt);
   if (p0 >= p1) return;
   unsigned long long out[4];
-  group_nns_tile<L1>(x, ia, p0, p1, y, ja, cons, c0, min(TG_M, nc_all - c0), d, T, threadIdx.x, 0, out);
+  group_nns_tile<L1, true>(x, ia, p0, p1, y, ja, cons, c0, min(TG_M, nc_all - c0), d, T, threadIdx.x, 0, out);
   const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
   if (tx == 0) {
 #pragma unroll

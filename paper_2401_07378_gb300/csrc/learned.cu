@@ -208,7 +208,7 @@ void adam_update(nnsemd_proposal* P, const float* grad, float lr, cudaStream_t s
 // --------------------------------------------------------------------------
 
 template <bool L1>
-__global__ void __launch_bounds__(TG_THREADS)
+__global__ void __launch_bounds__(TG_THREADS, 3)
     k_nearest(const float* __restrict__ x, const int* __restrict__ iota, int m, int chunk,
               const float* __restrict__ y, int n, int d, unsigned long long* __restrict__ keys) {
   __shared__ TileSmem T;
@@ -217,7 +217,7 @@ __global__ void __launch_bounds__(TG_THREADS)
   const int p1 = min(p0 + chunk, m);
   if (c0 >= n || p0 >= p1) return;
   unsigned long long out[4];
-  group_nns_tile<L1>(x, iota, p0, p1, y, iota, nullptr, c0, min(TG_M, n - c0), d, T, threadIdx.x, 0, out);
+  group_nns_tile<L1, true>(x, iota, p0, p1, y, iota, nullptr, c0, min(TG_M, n - c0), d, T, threadIdx.x, 0, out);
   const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
   if (tx == 0)
 #pragma unroll
