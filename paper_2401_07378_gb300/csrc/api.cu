@@ -724,6 +724,7 @@ static int solve_batched_impl(nnsemd_ctx* ctx, int32_t num_pairs, const float* x
   auto y_len = [&](int p) -> int64_t { return y_off ? y_off[p + 1] - y_off[p] : n_shared; };
   std::vector<int> small, large;
   int64_t small_max = 0, small_mn = 0;
+  int64_t km_tiny = 0, km_big = 0;  // largest key matrices (floats) of the 256- and the 1,024-thread FP32 solvers
   for (int p = 0; p < num_pairs; ++p) {
     const int64_t m = x_off[p + 1] - x_off[p], n = y_len(p);
     if (m < 1 || n < 1) return fail(ctx, NNSEMD_ERR_INVALID_ARG, "pair %d has an empty side", p);
@@ -733,6 +734,8 @@ static int solve_batched_impl(nnsemd_ctx* ctx, int32_t num_pairs, const float* x
     if (fits) {
       small_max = std::max(small_max, std::max(m, n));
       small_mn = std::max(small_mn, m * n);
+      int64_t& km = m <= HD_SMALL_CAP && n <= HD_SMALL_CAP ? km_tiny : km_big;
+      km = std::max<int64_t>(km, m * kmat_ld(n));
     }
   }
   // FP32, d > 8: pairs of at most HD_SMALL_CAP points per side go to the
@@ -769,46 +772,62 @@ static int solve_batched_impl(nnsemd_ctx* ctx, int32_t num_pairs, const float* x
   };
   if (tc && (double)slot_of(kc_cap) * grid > KC_BUDGET_BYTES) kc_cap = 0;
   const size_t slot = tc ? slot_of(kc_cap) : 0;
-  // workspace: offsets, pair list, queue/error/counters, per-pair counters,
-  // tensor-core scratch slots, then the buffers of the large pairs
-  Carve C(nullptr);
-  C.take<int64_t>(num_pairs + 1);
-  C.take<int64_t>(num_pairs + 1);
-  C.take<int>(small.size() + 1);
-  C.take<unsigned long long>(6);
-  C.take<long long>(num_pairs);
-  C.take<long long>(num_pairs);
-  C.take<uint8_t>(tc ? slot * grid : 0);
   // flow records of the d > 8 solvers, one slice per CTA (the tensor-core
   // kernel's grid; the 1,024- and the 256-thread FP32 kernels' grids)
   const long long fl_big = tc ? 2LL * cap : 2LL * FIN_MAX_HD, fl_small = 2LL * HD_SMALL_CAP;
   const size_t fl_n = d <= 8 || small.empty() ? 0 : (size_t)(nsm * fl_big + (tc ? 0 : nsm * 4 * fl_small));
-  C.take<int32_t>(fl_n);
-  C.take<int32_t>(fl_n);
-  C.take<double>(fl_n);
-  const size_t head = (C.off + 511) & ~(size_t)255;  // keeps the solve buffers 256-byte aligned
-  size_t bytes = head;
+  // key matrices of the d > 8 FP32 solvers, one slot per CTA; a solver whose
+  // slots exceed the budget, or any if the memory is not there, computes the
+  // keys again in every round instead
+  const int nbig_pairs = (int)small.size() - ntiny;
+  const int gbig = std::min(nbig_pairs, nsm), gtiny = std::min(ntiny, nsm * 4);
+  auto km_slot = [&](int64_t km, int g) -> long long {
+    return tc || d <= 8 || (double)km * g * sizeof(float) > KC_BUDGET_BYTES ? 0 : (km + 63) & ~63LL;
+  };
+  long long kc_big = km_slot(km_big, gbig), kc_tiny = km_slot(km_tiny, gtiny);
+  // workspace: offsets, pair list, queue/error/counters, per-pair counters,
+  // tensor-core scratch slots, flow records, key matrices, then the buffers
+  // of the large pairs
+  int64_t *xo_d, *yo_d;
+  int* ids_d;
+  // [0]: queue | err << 32, [1] certified, [2] fallbacks, [3] the 256-thread
+  // kernel's queue, [4] near-ties
+  unsigned long long* ctr_d;
+  long long *rounds_d, *pe_d;
+  uint8_t* scratch;
+  int32_t *fl_i, *fl_j;
+  double* fl_f;
+  float* kmat;
+  auto layout_head = [&](void* base) -> size_t {
+    Carve C(base);
+    xo_d = C.take<int64_t>(num_pairs + 1);
+    yo_d = C.take<int64_t>(num_pairs + 1);
+    ids_d = C.take<int>(small.size() + 1);
+    ctr_d = C.take<unsigned long long>(6);
+    rounds_d = C.take<long long>(num_pairs);
+    pe_d = C.take<long long>(num_pairs);
+    scratch = C.take<uint8_t>(tc ? slot * grid : 0);
+    fl_i = C.take<int32_t>(fl_n);
+    fl_j = C.take<int32_t>(fl_n);
+    fl_f = C.take<double>(fl_n);
+    kmat = C.take<float>((size_t)(kc_big * gbig + kc_tiny * gtiny));
+    return (C.off + 511) & ~(size_t)255;  // keeps the solve buffers 256-byte aligned
+  };
   int64_t maxm = 0, maxn = 0;
   for (int p : large) {
     maxm = std::max(maxm, x_off[p + 1] - x_off[p]);
     maxn = std::max(maxn, y_len(p));
   }
   SolveBufs B{};
-  if (!large.empty()) bytes += layout_solve(nullptr, maxm, maxn, d, B, precision);
-  if ((rc = ensure_ws(ctx, bytes))) return rc;
-  Carve W(ctx->ws);
-  int64_t* xo_d = W.take<int64_t>(num_pairs + 1);
-  int64_t* yo_d = W.take<int64_t>(num_pairs + 1);
-  int* ids_d = W.take<int>(small.size() + 1);
-  // [0]: queue | err << 32, [1] certified, [2] fallbacks, [3] the 256-thread
-  // kernel's queue, [4] near-ties
-  unsigned long long* ctr_d = W.take<unsigned long long>(6);
-  long long* rounds_d = W.take<long long>(num_pairs);
-  long long* pe_d = W.take<long long>(num_pairs);
-  uint8_t* scratch = W.take<uint8_t>(tc ? slot * grid : 0);
-  int32_t* fl_i = W.take<int32_t>(fl_n);
-  int32_t* fl_j = W.take<int32_t>(fl_n);
-  double* fl_f = W.take<double>(fl_n);
+  const size_t large_bytes = large.empty() ? 0 : layout_solve(nullptr, maxm, maxn, d, B, precision);
+  rc = ensure_ws(ctx, layout_head(nullptr) + large_bytes);
+  if (rc == NNSEMD_ERR_OOM && (kc_big || kc_tiny)) {
+    kc_big = kc_tiny = 0;
+    ctx->err.clear();
+    rc = ensure_ws(ctx, layout_head(nullptr) + large_bytes);
+  }
+  if (rc) return rc;
+  const size_t head = layout_head(ctx->ws);
   unsigned* q_d = reinterpret_cast<unsigned*>(ctr_d);
   unsigned* q2_d = reinterpret_cast<unsigned*>(ctr_d + 3);  // queue of the 256-thread kernel
   CK(cudaMemcpyAsync(xo_d, x_off, (num_pairs + 1) * sizeof(int64_t), cudaMemcpyHostToDevice, st));
@@ -840,7 +859,9 @@ static int solve_batched_impl(nnsemd_ctx* ctx, int32_t num_pairs, const float* x
       BatchArgs Ab = A;
       Ab.pair_ids = ids_d + ntiny;
       Ab.num = nbig;
-      r |= launch_batched_hd(Ab, std::min(nbig, nsm), s);
+      Ab.kmat = kc_big ? kmat : nullptr;
+      Ab.kcap = kc_big;
+      r |= launch_batched_hd(Ab, gbig, s);
     }
     if (ntiny > 0) {
       BatchArgs At = A;
@@ -852,7 +873,9 @@ static int solve_batched_impl(nnsemd_ctx* ctx, int32_t num_pairs, const float* x
         At.fl_f = fl_f + nsm * fl_big;
         At.fl_cap = fl_small;
       }
-      r |= launch_batched_hd_small(At, std::min(ntiny, nsm * 4), s);
+      At.kmat = kc_tiny ? kmat + kc_big * gbig : nullptr;
+      At.kcap = kc_tiny;
+      r |= launch_batched_hd_small(At, gtiny, s);
     }
     return r;
   };
@@ -897,6 +920,7 @@ static int solve_batched_impl(nnsemd_ctx* ctx, int32_t num_pairs, const float* x
                                           (uintptr_t)num_pairs, (uintptr_t)small.size(), (uintptr_t)d,
                                           (uintptr_t)metric, (uintptr_t)precision, (uintptr_t)cap, (uintptr_t)bn,
                                           (uintptr_t)nstage, (uintptr_t)ntiny, (uintptr_t)kc_cap,
+                                          (uintptr_t)kc_big, (uintptr_t)kc_tiny,
                                           (uintptr_t)(opt ? opt->protocol : 0), (uintptr_t)(opt ? opt->seed : 0),
                                           (uintptr_t)(opt ? opt->rerank_k : 0),
                                           (uintptr_t)(y_off ? 0 : n_shared)};

@@ -466,6 +466,13 @@ struct GeoGlobal {
   const float* x;  // [m][d] original coordinates (global)
   const float* y;  // [n][d]
   int d;
+  // The pair's key matrix (nullable): the FP32 key of every original
+  // supplier (row, kld floats apart) and consumer, computed once in the first
+  // round's NNS step; every round is then a minimum over rows of active
+  // suppliers instead of m_t n_t d operations (1 x 4,096 documents, d = 300:
+  // 11.7 -> 3.09 ms).
+  float* kmat;
+  int kld, km, kn, kready;
   TileSmem tiles[NT / TG_THREADS];
   struct PX {};
   NNS_DEV void load_x(int, PX&) const {}
@@ -476,8 +483,87 @@ struct GeoGlobal {
   NNS_DEV double dist64(const CtaCore<C>& S, int p, int q, int metric) const {
     return cost_dist64(x + (size_t)S.iidx[p] * d, y + (size_t)S.jidx[q] * d, d, metric);
   }
+  // Set up a pair (thread 0; the caller's barrier follows): kcap floats at
+  // km_ for its key matrix, used where the pair's fits.
+  NNS_DEV void begin(const float* x_, const float* y_, int m, int n, int d_, float* km_, long long kcap) {
+    x = x_;
+    y = y_;
+    d = d_;
+    kld = (int)kmat_ld(n);
+    km = m;
+    kn = n;
+    kmat = km_ && (long long)m * kld <= kcap ? km_ : nullptr;
+    kready = 0;
+  }
+  // The whole key matrix, one 64 x 64 tile per group at a time.
+  NNS_DEV void fill() {
+    const int g = threadIdx.x / TG_THREADS, gt = threadIdx.x % TG_THREADS;
+    const int tx = gt & 15, ty = gt >> 4;
+    const int ct = (kn + TG_M - 1) / TG_M, items = ct * ((km + TG_N - 1) / TG_N);
+    for (int it = g; it < items; it += NT / TG_THREADS) {
+      const int c0 = (it % ct) * TG_M, p0 = (it / ct) * TG_N;
+      group_tiles<L1, false>(x, nullptr, p0, min(p0 + TG_N, km), y, nullptr, nullptr, c0, min(TG_M, kn - c0), d,
+                             tiles[g], gt, 1 + g, [&](int pt, const unsigned long long (&acc)[2][4]) {
+                               const int q = c0 + ty * 4;  // four consecutive consumers: one 16-byte store
+                               if (q >= kn) return;
+#pragma unroll
+                               for (int j = 0; j < 4; ++j) {
+                                 const int p = pt + tx * 4 + j;
+                                 if (p < km)
+                                   *reinterpret_cast<ulonglong2*>(kmat + (size_t)p * kld + q) =
+                                       make_ulonglong2(acc[0][j], acc[1][j]);
+                               }
+                             });
+    }
+  }
+  // The NNS step on the key matrix: a warp takes 32 consumers (one per lane)
+  // and a contiguous chunk of the active suppliers, eight rows in flight;
+  // keys order like their bit patterns (no key is negative or NaN), each
+  // lane keeps its first minimum, and chunks merge by atomicMin.
+  template <int C>
+  NNS_DEV void scan(CtaCore<C>& S, int mt, int nt) const {
+    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    constexpr int NW = NT / 32;
+    const int cg = (nt + 31) >> 5, chunks = max(1, NW / cg);
+    if (chunks > 1) {
+      for (int q = threadIdx.x; q < nt; q += NT) S.nnk[q] = ~0ULL;
+      __syncthreads();
+    }
+    for (int u = w; u < cg * chunks; u += NW) {
+      const int q = 32 * (u % cg) + lane, ch = u / cg;
+      const int s0 = (int)((unsigned)(mt * ch) / (unsigned)chunks);
+      const int s1 = (int)((unsigned)(mt * (ch + 1)) / (unsigned)chunks);
+      const float* col = kmat + S.jidx[q < nt ? q : 0];
+      unsigned best = 0xffffffffu;
+      int bp = 0;
+      for (int p = s0; p < s1; p += 8) {
+        unsigned v[8];
+#pragma unroll
+        for (int e = 0; e < 8; ++e)
+          v[e] = p + e < s1 ? __float_as_uint(col[(size_t)S.iidx[p + e] * kld]) : 0xffffffffu;
+#pragma unroll
+        for (int e = 0; e < 8; ++e)
+          if (v[e] < best) { best = v[e]; bp = p + e; }
+      }
+      const unsigned long long key = ((unsigned long long)best << 32) | (unsigned)bp;
+      if (q < nt && s0 < s1) {
+        if (chunks > 1) atomicMin(&S.nnk[q], key);
+        else S.nnk[q] = key;
+      }
+    }
+    __syncthreads();
+  }
   template <int C>
   NNS_DEV const unsigned long long* nns(CtaCore<C>& S, int mt, int nt, long long = 0) {
+    if (kmat) {
+      if (!kready) {
+        fill();
+        __syncthreads();
+        if (threadIdx.x == 0) kready = 1;  // (read again after this step's barriers)
+      }
+      scan(S, mt, nt);
+      return S.nnk;
+    }
     const int g = threadIdx.x / TG_THREADS, gt = threadIdx.x % TG_THREADS;
     const int ngroups = blockDim.x / TG_THREADS;
     for (int c0 = g * TG_M; c0 < nt; c0 += ngroups * TG_M) {

@@ -86,9 +86,7 @@ __global__ void __launch_bounds__(FIN_THREADS, 1) k_finish_hd(SolveBufs B, long 
     return;
   }
   if (tid == 0) {
-    H.G.x = B.x;
-    H.G.y = B.y;
-    H.G.d = B.d;
+    H.G.begin(B.x, B.y, (int)B.m, (int)B.n, B.d, nullptr, 0);
     S.mt = mt;
     S.nt = nt;
   }
@@ -143,11 +141,8 @@ __global__ void __launch_bounds__(FIN_THREADS, 1) k_batched_hd(BatchArgs A) {
     const int pr = A.pair_ids[item];
     const int64_t xo = A.x_off[pr], yo = A.n_shared ? 0 : A.y_off[pr];
     const int m = (int)(A.x_off[pr + 1] - xo), n = A.n_shared ? A.n_shared : (int)(A.y_off[pr + 1] - yo);
-    if (tid == 0) {
-      H.G.x = A.x + xo * A.d;
-      H.G.y = A.y + yo * A.d;
-      H.G.d = A.d;
-    }
+    if (tid == 0)
+      H.G.begin(A.x + xo * A.d, A.y + yo * A.d, m, n, A.d, A.kmat ? A.kmat + blockIdx.x * A.kcap : nullptr, A.kcap);
     __syncthreads();
     double cost = 0.0;
     long long rounds = 0, pe = 0;
@@ -207,11 +202,8 @@ __global__ void __launch_bounds__(HD_SMALL_THREADS, 4) k_batched_hd_small(BatchA
       if (tid == 0) atomicOr(A.err, EF_INTERNAL);
       break;
     }
-    if (tid == 0) {
-      H.G.x = A.x + xo * A.d;
-      H.G.y = A.y + yo * A.d;
-      H.G.d = A.d;
-    }
+    if (tid == 0)
+      H.G.begin(A.x + xo * A.d, A.y + yo * A.d, m, n, A.d, A.kmat ? A.kmat + blockIdx.x * A.kcap : nullptr, A.kcap);
     __syncthreads();
     double cost = 0.0;
     long long rounds = 0, pe = 0;

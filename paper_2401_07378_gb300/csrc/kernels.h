@@ -29,6 +29,9 @@ constexpr int FIN_MAX_HD = 2048;
 constexpr int FIN_CL_MAX = 2048;
 __host__ __device__ constexpr int fin_cl_cap(int dp) { return dp <= 4 ? FIN_CL_MAX : 1024; }
 
+// Row length of a key matrix over n consumers (rows start on 16 bytes).
+__host__ __device__ inline long long kmat_ld(long long n) { return (n + 3) & ~3LL; }
+
 __host__ __device__ inline int padded_dim(int d) { return d <= 2 ? 2 : (d <= 4 ? 4 : 8); }
 __host__ __device__ inline int64_t pad_points(int64_t n) { return (n + PAD_POINTS - 1) / PAD_POINTS * PAD_POINTS; }
 
@@ -142,6 +145,10 @@ struct BatchArgs {
   int32_t* fl_j;
   double* fl_f;
   long long fl_cap;
+  // key matrices (nullable; d > 8, FP32): kcap floats per CTA, a multiple of
+  // 4, used by the pairs whose matrix (m rows of kmat_ld(n) floats) fits
+  float* kmat;
+  long long kcap;
 };
 int launch_batched_lowd(const BatchArgs& A, int grid, cudaStream_t st);
 
