@@ -562,6 +562,7 @@ int nnsemd_destroy(nnsemd_ctx* ctx) {
   cudaSetDevice(ctx->device);
   cudaStreamSynchronize(ctx->stream);
   if (ctx->ws) cudaFree(ctx->ws);
+  if (ctx->cws) cudaFree(ctx->cws);
   if (ctx->hstate) cudaFreeHost(ctx->hstate);
   if (ctx->hmap) cudaFreeHost((void*)ctx->hmap);
   for (cudaEvent_t e : ctx->ev)
