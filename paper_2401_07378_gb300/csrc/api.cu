@@ -328,7 +328,8 @@ int run_solve(nnsemd_ctx* ctx, SolveBufs& B, const double* a, const double* b, d
     // small pair: the whole solve in one launch, one host synchronisation
     CK(cudaMemsetAsync(B.st, 0, sizeof(DevState), st));
     if (timed) CK(cudaEventRecord(ctx->ev[2], st));
-    if (launch_solve_small(B, a, b, st)) return fail(ctx, NNSEMD_ERR_CUDA, "small-pair launch");
+    const bool cap = B.m <= LOWD_SMALL_CAP && B.n <= LOWD_SMALL_CAP;
+    if (cap ? launch_solve_small_cap(B, a, b, st) : launch_solve_small(B, a, b, st)) return fail(ctx, NNSEMD_ERR_CUDA, "small-pair launch");
     if (timed) CK(cudaEventRecord(ctx->ev[3], st));
     CK(cudaGetLastError());
     CK(cudaMemcpyAsync(ctx->hstate, B.st, sizeof(DevState), cudaMemcpyDeviceToHost, st));
@@ -739,15 +740,15 @@ static int solve_batched_impl(nnsemd_ctx* ctx, int32_t num_pairs, const float* x
       km = std::max<int64_t>(km, m * kmat_ld(n));
     }
   }
-  // FP32, d > 8: pairs of at most HD_SMALL_CAP points per side go to the
-  // 256-thread kernel (several pairs per SM); they come first in the list
+  // FP32: pairs of at most HD_SMALL_CAP (d <= 8: LOWD_SMALL_CAP) points per
+  // side go to the kernels with fewer threads (several pairs per SM); they
+  // come first in the list
   int ntiny = 0;
-  if (!tc && d > 8) {
-    std::stable_partition(small.begin(), small.end(), [&](int p) {
-      return x_off[p + 1] - x_off[p] <= HD_SMALL_CAP && y_len(p) <= HD_SMALL_CAP;
-    });
-    for (int p : small)
-      if (x_off[p + 1] - x_off[p] <= HD_SMALL_CAP && y_len(p) <= HD_SMALL_CAP) ++ntiny;
+  if (!tc) {
+    const int tcap = d <= 8 ? LOWD_SMALL_CAP : HD_SMALL_CAP;
+    auto tiny = [&](int p) { return x_off[p + 1] - x_off[p] <= tcap && y_len(p) <= tcap; };
+    std::stable_partition(small.begin(), small.end(), tiny);
+    for (int p : small) ntiny += tiny(p);
   }
   CK(cudaSetDevice(ctx->device));
   cudaStream_t st = ctx->stream;
@@ -781,7 +782,7 @@ static int solve_batched_impl(nnsemd_ctx* ctx, int32_t num_pairs, const float* x
   // slots exceed the budget, or any if the memory is not there, computes the
   // keys again in every round instead
   const int nbig_pairs = (int)small.size() - ntiny;
-  const int gbig = std::min(nbig_pairs, nsm), gtiny = std::min(ntiny, nsm * 4);
+  const int gbig = std::min(nbig_pairs, nsm), gtiny = std::min(ntiny, nsm * (d <= 8 ? LOWD_SMALL_PER_SM : 4));
   auto km_slot = [&](int64_t km, int g) -> long long {
     return tc || d <= 8 || (double)km * g * sizeof(float) > KC_BUDGET_BYTES ? 0 : (km + 63) & ~63LL;
   };
@@ -853,7 +854,6 @@ static int solve_batched_impl(nnsemd_ctx* ctx, int32_t num_pairs, const float* x
     if (tc)  // (grid <= one CTA per SM)
       return launch_batched_tc(A, precision, cap, kb, tbn, tns, scratch, slot, ctr_d + 1, ctr_d + 2, ctr_d + 4,
                                opt ? opt->rerank_k : 0, tkc, g, s);
-    if (d <= 8) return launch_batched_lowd(A, g, s);
     int r = 0;
     const int nbig = nsmall - ntiny;
     if (nbig > 0) {
@@ -862,7 +862,7 @@ static int solve_batched_impl(nnsemd_ctx* ctx, int32_t num_pairs, const float* x
       Ab.num = nbig;
       Ab.kmat = kc_big ? kmat : nullptr;
       Ab.kcap = kc_big;
-      r |= launch_batched_hd(Ab, gbig, s);
+      r |= d <= 8 ? launch_batched_lowd(Ab, gbig, s) : launch_batched_hd(Ab, gbig, s);
     }
     if (ntiny > 0) {
       BatchArgs At = A;
@@ -876,7 +876,7 @@ static int solve_batched_impl(nnsemd_ctx* ctx, int32_t num_pairs, const float* x
       }
       At.kmat = kc_tiny ? kmat + kc_big * gbig : nullptr;
       At.kcap = kc_tiny;
-      r |= launch_batched_hd_small(At, gtiny, s);
+      r |= d <= 8 ? launch_batched_lowd_small(At, gtiny, s) : launch_batched_hd_small(At, gtiny, s);
     }
     return r;
   };

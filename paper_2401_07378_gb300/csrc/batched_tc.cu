@@ -106,6 +106,7 @@ template <bool KIND8, int CAP>
 struct GeoTC {
   static constexpr int kDP = 0;
   static constexpr int kThreads = FIN_THREADS;
+  static constexpr bool kWarpRounds = false;
   struct PX {};
   const float* x;  // this pair's coordinates
   const float* y;

@@ -200,46 +200,24 @@ NNS_DEV void xs_add(unsigned long long* acc, double v) {
 }
 
 // The same add for the 32 lanes of a warp at once: every lane calls it (a
-// lane with nothing to add passes 0).  Lanes whose values start at the same
-// limb sum their digits by shuffles first (at most 32 digits below 2^32
-// each: no overflow), then one of them adds the sums, so values that share
-// an exponent cost three atomics per warp, not per lane.
+// lane with nothing to add passes 0).  Limb by limb over those the warp's
+// values touch (three for values of one exponent, a few more in general), the
+// lanes' 32-bit digits are summed as 16-bit halves by two warp reductions and
+// one lane adds the result.  (Summing the lanes of equal limbs by shuffles
+// took 192 of them whenever two exponents met.)
 static __device__ __noinline__ void xs_add_warp(unsigned long long* acc, double v) {  // one copy per file, not inlined at every site
   int L = -1;
   unsigned long long c0 = 0, c1 = 0, c2 = 0;
   if (v > 0.0) xs_digits(v, L, c0, c1, c2);
+  const int hi = __reduce_max_sync(0xffffffffu, L);
+  if (hi < 0) return;  // nothing to add
+  const int lo = (int)__reduce_min_sync(0xffffffffu, (unsigned)L);  // (-1 is the largest)
   const int lane = threadIdx.x & 31;
-  const unsigned grp = __match_any_sync(0xffffffffu, L);
-  if (grp == 0xffffffffu) {  // one limb for the whole warp (the same for every lane)
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      c0 += __shfl_xor_sync(0xffffffffu, c0, o);
-      c1 += __shfl_xor_sync(0xffffffffu, c1, o);
-      c2 += __shfl_xor_sync(0xffffffffu, c2, o);
-    }
-    if (L >= 0 && lane == 0) {
-      if (c0) atomicAdd(acc + L, c0);
-      if (c1) atomicAdd(acc + L + 1, c1);
-      if (c2) atomicAdd(acc + L + 2, c2);
-    }
-    return;
-  }
-  unsigned long long s0 = 0, s1 = 0, s2 = 0;
-#pragma unroll 4
-  for (int k = 0; k < 32; ++k) {
-    const unsigned long long a0 = __shfl_sync(0xffffffffu, c0, k);
-    const unsigned long long a1 = __shfl_sync(0xffffffffu, c1, k);
-    const unsigned long long a2 = __shfl_sync(0xffffffffu, c2, k);
-    if ((grp >> k) & 1u) {
-      s0 += a0;
-      s1 += a1;
-      s2 += a2;
-    }
-  }
-  if (L >= 0 && lane == __ffs(grp) - 1) {
-    if (s0) atomicAdd(acc + L, s0);
-    if (s1) atomicAdd(acc + L + 1, s1);
-    if (s2) atomicAdd(acc + L + 2, s2);
+  for (int l = lo; l <= hi + 2; ++l) {
+    const int k = l - L;
+    const unsigned dig = L < 0 ? 0u : (unsigned)(k == 0 ? c0 : (k == 1 ? c1 : (k == 2 ? c2 : 0ULL)));
+    const unsigned s0 = __reduce_add_sync(0xffffffffu, dig & 0xffffu), s1 = __reduce_add_sync(0xffffffffu, dig >> 16);
+    if (lane == 0 && (s0 | s1)) atomicAdd(acc + l, (unsigned long long)s0 + ((unsigned long long)s1 << 16));
   }
 }
 
@@ -255,18 +233,19 @@ NNS_DEV unsigned long long xs_bits64(const unsigned long long* a, int pos) {
   return r ? ((lo >> r) | (hi << (64 - r))) : lo;
 }
 
-// Correctly rounded value of the accumulator (single thread; a is modified).
-NNS_DEV double xs_round(unsigned long long* a) {
+// Correctly rounded value of the accumulator (single thread; a is modified),
+// whose limbs outside [lo, hi] are zero.
+NNS_DEV double xs_round_span(unsigned long long* a, int lo, int hi) {
   unsigned long long carry = 0;
-  for (int L = 0; L < XS_LIMBS; ++L) {
-    unsigned long long v = a[L] + carry;
-    a[L] = v & 0xffffffffULL;
+  int last = -1;  // the highest non-zero digit
+  for (int L = lo; L < XS_LIMBS && (L <= hi || carry); ++L) {
+    const unsigned long long v = a[L] + carry, dig = v & 0xffffffffULL;
+    a[L] = dig;
     carry = v >> 32;
+    if (dig) last = L;
   }
-  int top = -1;
-  for (int L = XS_LIMBS - 1; L >= 0; --L)
-    if (a[L]) { top = L * 32 + (63 - __clzll((long long)a[L])); break; }
-  if (top < 0) return 0.0;
+  if (last < 0) return 0.0;
+  const int top = last * 32 + (63 - __clzll((long long)a[last]));
   if (top <= 52) return __longlong_as_double((long long)xs_bits64(a, 0));
   int shift = top - 52;
   unsigned long long mant = xs_bits64(a, shift) & ((1ULL << 53) - 1);
@@ -274,7 +253,7 @@ NNS_DEV double xs_round(unsigned long long* a) {
   unsigned long long round = (xs_bits64(a, rpos) & 1ULL);
   bool sticky = false;
   int Lr = rpos >> 5;
-  for (int L = 0; L < Lr && !sticky; ++L) sticky = a[L] != 0;
+  for (int L = lo; L < Lr && !sticky; ++L) sticky = a[L] != 0;
   if (!sticky && (rpos & 31)) sticky = (a[Lr] & ((1ULL << (rpos & 31)) - 1)) != 0;
   if (round && (sticky || (mant & 1ULL))) {
     ++mant;
@@ -283,6 +262,27 @@ NNS_DEV double xs_round(unsigned long long* a) {
   int E = shift + 1;
   if (E >= 2047) return __longlong_as_double(0x7ff0000000000000LL);
   return __longlong_as_double((long long)(((unsigned long long)E << 52) | (mant & ((1ULL << 52) - 1))));
+}
+
+NNS_DEV double xs_round(unsigned long long* a) { return xs_round_span(a, 0, XS_LIMBS - 1); }
+
+// The same for a whole warp (every lane calls it; the value is lane 0's): the
+// lanes look for the limbs in use first, usually about six of the 68, so
+// that lane 0's dependent walk takes those alone (shared memory: about 1.2 us
+// less a sum; global memory: k_xs_round2 went from 7.5 to 3 us).
+NNS_DEV double xs_round_warp(unsigned long long* a) {
+  const int lane = threadIdx.x & 31;
+  const unsigned b0 = __ballot_sync(0xffffffffu, a[lane] != 0), b1 = __ballot_sync(0xffffffffu, a[32 + lane] != 0);
+  const unsigned b2 = __ballot_sync(0xffffffffu, lane < XS_LIMBS - 64 && a[64 + (lane & 3)] != 0);
+  static_assert(XS_LIMBS == 68, "three ballots cover the limbs");
+  double r = 0.0;
+  if (lane == 0 && (b0 | b1 | b2)) {
+    const int lo = b0 ? __ffs(b0) - 1 : (b1 ? 31 + __ffs(b1) : 63 + __ffs(b2));
+    const int hi = b2 ? 95 - __clz(b2) : (b1 ? 63 - __clz(b1) : 31 - __clz(b0));
+    r = xs_round_span(a, lo, hi);
+  }
+  __syncwarp();
+  return r;
 }
 
 // --------------------------------------------------------------------------

@@ -71,11 +71,11 @@ struct CtaCore {
   unsigned long long mem2[CAP];
   int cnt[CAP + 1];
   int off[CAP + 1];
-  unsigned long long acc[XS_LIMBS];
+  unsigned long long acc[2][XS_LIMBS];  // exact sums (acc[0]: R; both: the sides' totals)
   int wt[33];
   int mt, nt;
   unsigned nflow;
-  double total;
+  double total[2];
   // running totals handed back by the one-warp rounds (warp_rounds)
   unsigned long long w_nnz;
   long long w_rounds, w_pe;
@@ -117,11 +117,11 @@ struct CtaOut {
 // coordinate policies
 // --------------------------------------------------------------------------
 
-template <int D, int DP, bool L1, int CAP>
+template <int D, int DP, bool L1, int CAP, int NT = FIN_THREADS>
 struct GeoSmem {
   static constexpr int kDP = DP;
   static constexpr int kD = D;
-  static constexpr int kThreads = FIN_THREADS;  // threads of the CTA
+  static constexpr int kThreads = NT;  // threads of the CTA
   float xs[CAP * DP];
   float ys[CAP * DP];
   struct PX { float v[DP]; };
@@ -152,36 +152,104 @@ struct GeoSmem {
   NNS_DEV double dist64(const CtaCore<C>& S, int p, int q, int metric) const {
     return cost_dist64(xs + p * DP, ys + q * DP, D, metric);
   }
+  // keys of supplier p against two consumers: coordinates ya, yb, also
+  // packed in y2
+  NNS_DEV unsigned long long key_two(int p, const unsigned long long* y2, const float* ya, const float* yb) const {
+    float xv[D];
+#pragma unroll
+    for (int k = 0; k < D; ++k) xv[k] = xs[p * DP + k];
+    if (L1) return f2_pack(key_pair(xv, ya), key_pair(xv, yb));
+    unsigned long long t = f2_sub(f2_pack(xv[0], xv[0]), y2[0]);
+    unsigned long long acc = f2_mul(t, t);
+#pragma unroll
+    for (int k = 1; k < D; ++k) {
+      t = f2_sub(f2_pack(xv[k], xv[k]), y2[k]);
+      acc = f2_fma(t, t, acc);
+    }
+    return acc;
+  }
+  // This lane's consumers qa, qb (those below n; others read as 0) against
+  // the suppliers [s0, s1), s0 < s1: the packed (key, first position) of each.
+  // All lanes read the same supplier (a broadcast).  Four keys at a time go
+  // through minima, and the winning four are looked at once more for the
+  // position: the chain of a compare and two selects per supplier, with the
+  // load before it, took 60 cycles a supplier for one resident pair.
+  NNS_DEV void scan_chunk(int qa, int qb, int n, int s0, int s1, unsigned long long& ka, unsigned long long& kb) const {
+    float ya[D], yb[D];
+    unsigned long long y2[D];
+#pragma unroll
+    for (int k = 0; k < D; ++k) {
+      ya[k] = qa < n ? ys[qa * DP + k] : 0.f;
+      yb[k] = qb < n ? ys[qb * DP + k] : 0.f;
+      y2[k] = f2_pack(ya[k], yb[k]);
+    }
+    float ba = CUDART_INF_F, bb = CUDART_INF_F;
+    int pa = s0, pb = s0, p = s0;
+    for (; p + 4 <= s1; p += 4) {
+      unsigned long long v[4];
+#pragma unroll
+      for (int e = 0; e < 4; ++e) v[e] = key_two(p + e, y2, ya, yb);
+      const float ma = fmin3(fminf(f2_lo(v[0]), f2_lo(v[1])), f2_lo(v[2]), f2_lo(v[3]));
+      const float mb = fmin3(fminf(f2_hi(v[0]), f2_hi(v[1])), f2_hi(v[2]), f2_hi(v[3]));
+      if (ma < ba) { ba = ma; pa = p; }
+      if (mb < bb) { bb = mb; pb = p; }
+    }
+    for (; p < s1; ++p) {
+      const unsigned long long v = key_two(p, y2, ya, yb);
+      if (f2_lo(v) < ba) { ba = f2_lo(v); pa = p; }
+      if (f2_hi(v) < bb) { bb = f2_hi(v); pb = p; }
+    }
+    auto first = [&](int g, float best, const float* yv) {
+      int r = g;
+#pragma unroll
+      for (int e = 3; e >= 0; --e)
+        if (g + e < s1 && key_pair(xs + (g + e) * DP, yv) == best) r = g + e;
+      return r;
+    };
+    ka = pack_key(ba, (unsigned)first(pa, ba, ya));
+    kb = pack_key(bb, (unsigned)first(pb, bb, yb));
+  }
   // S.nnk[q] = (key32 bits << 32 | p) of the nearest active supplier;
-  // returns S.nnk (every NNS policy returns the array holding the keys)
+  // returns S.nnk (every NNS policy returns the array holding the keys).  A
+  // warp takes 64 consumers and a contiguous chunk of the suppliers; chunks
+  // merge by atomicMin on (key, position).
   template <int C>
   NNS_DEV const unsigned long long* nns(CtaCore<C>& S, int mt, int nt, long long = 0) const {
-    const int tid = threadIdx.x, T = blockDim.x;
-    int split = 1;
-    while (split < 32 && nt * split * 2 <= T) split <<= 1;
-    for (int base = 0; base < nt; base += T / split) {
-      const int q = base + tid / split, part = tid & (split - 1);
-      unsigned long long bk = ~0ULL;
-      if (q < nt) {
-        float yv[D];
-#pragma unroll
-        for (int k = 0; k < D; ++k) yv[k] = ys[q * DP + k];
-        float best = CUDART_INF_F;
-        int bp = -1;
-        for (int p = part; p < mt; p += split) {
-          const float v = L1 ? key32<METRIC_L1>(xs + p * DP, yv, D) : key32<METRIC_SQL2>(xs + p * DP, yv, D);
-          if (bp < 0 || v < best) { best = v; bp = p; }
-        }
-        if (bp >= 0) bk = pack_key(best, (unsigned)bp);
+    constexpr int NW = NT / 32;
+    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int cg = (nt + 63) >> 6, chunks = max(1, NW / cg);
+    if (chunks > 1) {
+      for (int q = threadIdx.x; q < nt; q += NT) S.nnk[q] = ~0ULL;
+      __syncthreads();
+    }
+    for (int u = w; u < cg * chunks; u += NW) {
+      const int qa = 64 * (u % cg) + lane, qb = qa + 32, ch = u / cg;
+      const int s0 = (int)((unsigned)(mt * ch) / (unsigned)chunks);
+      const int s1 = (int)((unsigned)(mt * (ch + 1)) / (unsigned)chunks);
+      if (s0 >= s1) continue;
+      unsigned long long ka, kb;
+      scan_chunk(qa, qb, nt, s0, s1, ka, kb);
+      if (chunks > 1) {
+        if (qa < nt) atomicMin(&S.nnk[qa], ka);
+        if (qb < nt) atomicMin(&S.nnk[qb], kb);
+      } else {
+        if (qa < nt) S.nnk[qa] = ka;
+        if (qb < nt) S.nnk[qb] = kb;
       }
-      for (int o = 1; o < split; o <<= 1) {
-        const unsigned long long other = __shfl_xor_sync(0xffffffffu, bk, o);
-        bk = other < bk ? other : bk;
-      }
-      if (q < nt && part == 0) S.nnk[q] = bk;
     }
     __syncthreads();
     return S.nnk;
+  }
+  // the same for at most 64 consumers, by one warp
+  static constexpr bool kWarpRounds = true;
+  NNS_DEV bool warp_ready() const { return true; }
+  template <int C>
+  NNS_DEV void warp_nns(CtaCore<C>& S, int mt, int nt) const {
+    const int qa = threadIdx.x & 31, qb = qa + 32;
+    unsigned long long ka, kb;
+    scan_chunk(qa, qb, nt, 0, mt, ka, kb);
+    if (qa < nt) S.nnk[qa] = ka;
+    if (qb < nt) S.nnk[qb] = kb;
   }
 };
 
@@ -209,25 +277,6 @@ struct GeoSmemCluster : GeoSmem<D, DP, L1, CAP> {
   unsigned long long xk[2][CAP];          // receive buffers (round parity)
   unsigned long long red[kSlice];         // the slice's keys merged over chunks; all ones between rounds
 
-  NNS_DEV float key_one(const float* xv, const float* yv) const {
-    return L1 ? key32<METRIC_L1>(xv, yv, D) : key32<METRIC_SQL2>(xv, yv, D);
-  }
-  // keys of supplier p against the two consumers packed in y2
-  NNS_DEV unsigned long long key_two(int p, const unsigned long long* y2, const float* ya, const float* yb) const {
-    float xv[D];
-#pragma unroll
-    for (int k = 0; k < D; ++k) xv[k] = this->xs[p * DP + k];
-    if (L1) return f2_pack(key_one(xv, ya), key_one(xv, yb));
-    unsigned long long t = f2_sub(f2_pack(xv[0], xv[0]), y2[0]);
-    unsigned long long acc = f2_mul(t, t);
-#pragma unroll
-    for (int k = 1; k < D; ++k) {
-      t = f2_sub(f2_pack(xv[k], xv[k]), y2[k]);
-      acc = f2_fma(t, t, acc);
-    }
-    return acc;
-  }
-
   // Set red to all ones (before the first round; each round restores it).
   NNS_DEV void init() {
     for (int i = threadIdx.x; i < kSlice; i += blockDim.x) red[i] = ~0ULL;
@@ -246,28 +295,13 @@ struct GeoSmemCluster : GeoSmem<D, DP, L1, CAP> {
     if (cgroups > 0 && w < nw / cgroups * cgroups) {
       const int chunks = nw / cgroups, ch = w / cgroups;
       const int qa = 64 * (w % cgroups) + lane, qb = qa + 32;  // slice positions
-      float ya[D], yb[D];
-      unsigned long long y2[D];
-#pragma unroll
-      for (int k = 0; k < D; ++k) {
-        ya[k] = qa < ns ? this->ys[(q0 + qa) * DP + k] : 0.f;
-        yb[k] = qb < ns ? this->ys[(q0 + qb) * DP + k] : 0.f;
-        y2[k] = f2_pack(ya[k], yb[k]);
-      }
       const int s0 = (int)((unsigned)(mt * ch) / (unsigned)chunks);
       const int s1 = (int)((unsigned)(mt * (ch + 1)) / (unsigned)chunks);
       if (s0 < s1) {
-        unsigned long long kk = key_two(s0, y2, ya, yb);
-        float ba = f2_lo(kk), bb = f2_hi(kk);
-        int pa = s0, pb = s0;
-        for (int p = s0 + 1; p < s1; ++p) {
-          kk = key_two(p, y2, ya, yb);
-          const float ka = f2_lo(kk), kb = f2_hi(kk);
-          if (ka < ba) { ba = ka; pa = p; }
-          if (kb < bb) { bb = kb; pb = p; }
-        }
-        if (qa < ns) atomicMin(&red[qa], pack_key(ba, (unsigned)pa));
-        if (qb < ns) atomicMin(&red[qb], pack_key(bb, (unsigned)pb));
+        unsigned long long ka, kb;
+        this->scan_chunk(q0 + qa, q0 + qb, q1, s0, s1, ka, kb);
+        if (qa < ns) atomicMin(&red[qa], ka);
+        if (qb < ns) atomicMin(&red[qb], kb);
       }
     }
     __syncthreads();
@@ -553,6 +587,33 @@ struct GeoGlobal {
     }
     __syncthreads();
   }
+  // the same for at most 64 consumers, by one warp
+  static constexpr bool kWarpRounds = true;
+  NNS_DEV bool warp_ready() const { return kmat != nullptr && kready; }
+  template <int C>
+  NNS_DEV void warp_nns(CtaCore<C>& S, int mt, int nt) const {
+    const int qa = threadIdx.x & 31, qb = qa + 32;
+    const float* ca = kmat + S.jidx[qa < nt ? qa : 0];
+    const float* cb = kmat + S.jidx[qb < nt ? qb : 0];
+    unsigned ba = 0xffffffffu, bb = 0xffffffffu;
+    int pa = 0, pb = 0;
+    for (int p = 0; p < mt; p += 8) {
+      unsigned va[8], vb[8];
+#pragma unroll
+      for (int e = 0; e < 8; ++e) {
+        const size_t row = (size_t)S.iidx[min(p + e, mt - 1)] * kld;
+        va[e] = __float_as_uint(ca[row]);
+        vb[e] = __float_as_uint(cb[row]);
+      }
+#pragma unroll
+      for (int e = 0; e < 8; ++e) {  // (repeats of the last supplier never win)
+        if (va[e] < ba) { ba = va[e]; pa = p + e; }
+        if (vb[e] < bb) { bb = vb[e]; pb = p + e; }
+      }
+    }
+    if (qa < nt) S.nnk[qa] = ((unsigned long long)ba << 32) | (unsigned)pa;
+    if (qb < nt) S.nnk[qb] = ((unsigned long long)bb << 32) | (unsigned)pb;
+  }
   template <int C>
   NNS_DEV const unsigned long long* nns(CtaCore<C>& S, int mt, int nt, long long = 0) {
     if (kmat) {
@@ -687,22 +748,20 @@ template <class Geo>
 NNS_DEV constexpr int warp_cap() { return 64; }
 
 // The remaining rounds of a pair whose active sets both hold at most
-// warp_cap<Geo>() points, run by the calling warp alone (shared-memory
-// coordinates, kDP > 0): with a few dozen points left, a round of the
+// warp_cap<Geo>() points, run by the calling warp alone (policies with
+// kWarpRounds): with a few dozen points left, a round of the
 // block-wide steps below is mostly barrier latency, and one warp needs none.
 // The same steps in the same arithmetic as cta_rounds, so every result is
 // identical:
-//   NNS     lane = consumer (q = lane, lane + 32, ...), a scan of every
-//           active supplier in ascending position, first minimum kept;
-//   order   every consumer's rank by (supplier position, serving key,
-//           position), counted against all consumers; the members of a
+//   NNS     the policy's warp_nns, consumers lane and lane + 32;
+//   order   every consumer's (supplier position, serving key, position) as
+//           one 64-bit word and its rank among all of them; the members of a
 //           group then lie in serving order, groups in supplier order;
 //   flow    lane = supplier, the FP64 residual chain over its group;
 //   compact ballots keep the points with residual left, in order.
 template <int CAP, class Geo>
 NNS_DEV void warp_rounds(CtaCore<CAP>& S, Geo& G, int metric, const CtaOut& O, unsigned long long& nnz,
                          long long& rounds, long long& pair_evals, long long round_limit) {
-  constexpr int D = Geo::kD;
   constexpr int WH = warp_cap<Geo>() / 32;  // points per lane
   const int lane = threadIdx.x & 31;
   const unsigned lt = (1u << lane) - 1u;
@@ -715,37 +774,15 @@ NNS_DEV void warp_rounds(CtaCore<CAP>& S, Geo& G, int metric, const CtaOut& O, u
       break;
     }
     if (lane == 0) S.nflow = 0;
-    // ---- NNS: one pass over the suppliers (each read once, a broadcast)
-    // for all WH consumers of the lane
-    {
-      float yv[WH][D], best[WH];
-      int bp[WH];
 #pragma unroll
-      for (int h = 0; h < WH; ++h) {
-        const int q = lane + 32 * h;
-#pragma unroll
-        for (int k = 0; k < D; ++k) yv[h][k] = q < nt ? G.ys[q * Geo::kDP + k] : 0.f;
-        best[h] = CUDART_INF_F;
-        bp[h] = -1;
-      }
-      for (int p = 0; p < mt; ++p) {
-        float xv[D];
-#pragma unroll
-        for (int k = 0; k < D; ++k) xv[k] = G.xs[p * Geo::kDP + k];
-#pragma unroll
-        for (int h = 0; h < WH; ++h) {
-          const float v = Geo::key_pair(xv, yv[h]);
-          if (bp[h] < 0 || v < best[h]) { best[h] = v; bp[h] = p; }
-        }
-      }
-#pragma unroll
-      for (int h = 0; h < WH; ++h) {
-        const int q = lane + 32 * h;
-        if (q < nt) S.nnk[q] = pack_key(best[h], (unsigned)bp[h]);
-      }
-    }
-    __syncwarp();
-    // ---- order: the serving key of every consumer, then its rank
+    for (int h = 0; h < WH; ++h)
+      if (lane + 32 * h < mt) S.cnt[lane + 32 * h] = 0;
+    // ---- NNS
+    G.warp_nns(S, mt, nt);
+    // ---- order: (supplier, serving key, consumer) of every consumer (each
+    // lane reads back its own keys), then its rank among all of them
+    static_assert(WH == 2, "two consumers per lane");
+    unsigned long long ma = ~0ULL, mb = ~0ULL;
 #pragma unroll
     for (int h = 0; h < WH; ++h) {
       const int q = lane + 32 * h;
@@ -753,36 +790,33 @@ NNS_DEV void warp_rounds(CtaCore<CAP>& S, Geo& G, int metric, const CtaOut& O, u
         const unsigned long long key = S.nnk[q];
         const unsigned ord = O.protocol == 1 ? rp_key32(O.seed, O.round_base + rounds, S.jidx[q])
                                              : (unsigned)(key >> 32);
-        S.mem[q] = ((key & 0xffffffffULL) << 32) | ord;
+        const unsigned long long mine = ((key & 0xffffULL) << 40) | ((unsigned long long)ord << 8) | (unsigned)q;
+        if (h == 0) ma = mine;
+        else mb = mine;
+        S.mem[q] = mine;
+      } else if (q < ((nt + 3) & ~3)) {
+        S.mem[q] = ~0ULL;
       }
     }
     __syncwarp();
-#pragma unroll
-    for (int h = 0; h < WH; ++h) {
-      const int q = lane + 32 * h;
-      if (q < nt) {
-        const unsigned long long mine = S.mem[q];
-        int rank = 0;
-        for (int u = 0; u < nt; ++u) {
-          const unsigned long long o = S.mem[u];
-          rank += (o < mine) | ((o == mine) & (u < q));
-        }
-        S.mem2[rank] = (unsigned long long)(unsigned)q;
-      }
+    int ra = 0, rb = 0;
+    for (int u = 0; u < nt; u += 4) {
+      const ulonglong2 o = *reinterpret_cast<const ulonglong2*>(&S.mem[u]);
+      const ulonglong2 v = *reinterpret_cast<const ulonglong2*>(&S.mem[u + 2]);
+      ra += (o.x < ma) + (o.y < ma) + (v.x < ma) + (v.y < ma);
+      rb += (o.x < mb) + (o.y < mb) + (v.x < mb) + (v.y < mb);
     }
-    // group bounds of every supplier: members of lower suppliers, its own
+    if (lane < nt) S.mem2[ra] = ma;
+    if (lane + 32 < nt) S.mem2[rb] = mb;
+    __syncwarp();
+    // group bounds: where the supplier changes along the order
 #pragma unroll
     for (int h = 0; h < WH; ++h) {
-      const int p = lane + 32 * h;
-      if (p < mt) {
-        int lo = 0, len = 0;
-        for (int u = 0; u < nt; ++u) {
-          const int pp = (int)(S.mem[u] >> 32);
-          lo += pp < p;
-          len += pp == p;
-        }
-        S.off[p] = lo;
-        S.cnt[p] = len;
+      const int r = lane + 32 * h;
+      if (r < nt) {
+        const int p = (int)(S.mem2[r] >> 40);
+        if (r == 0 || (int)(S.mem2[r - 1] >> 40) != p) S.off[p] = r;
+        if (r == nt - 1 || (int)(S.mem2[r + 1] >> 40) != p) S.cnt[p] = r + 1;  // the group's end
       }
     }
     __syncwarp();
@@ -791,11 +825,11 @@ NNS_DEV void warp_rounds(CtaCore<CAP>& S, Geo& G, int metric, const CtaOut& O, u
     for (int h = 0; h < WH; ++h) {
       const int p = lane + 32 * h;
       if (p < mt && S.cnt[p] > 0) {
-        const int b = S.off[p], en = b + S.cnt[p];
+        const int b = S.off[p], en = S.cnt[p];
         double s = S.sres[p];
         for (int r = b; r < en; ++r) {
           if (!residual_positive(s)) break;
-          const int q = (int)(S.mem2[r] & 0xffffffffULL);
+          const int q = (int)(S.mem2[r] & 0xffULL);
           double c = S.cres[q];
           const double f = greedy_step(s, c);
           S.cres[q] = c;
@@ -919,8 +953,8 @@ NNS_DEV void cta_rounds(CtaCore<CAP>& S, Geo& G, int metric, const CtaOut& O, un
       if (tid == 0) atomicOr(O.err, EF_ITER);
       break;
     }
-    if constexpr (Geo::kDP > 0) {
-      if (mt <= warp_cap<Geo>() && nt <= warp_cap<Geo>()) {
+    if constexpr (Geo::kWarpRounds) {
+      if (mt <= warp_cap<Geo>() && nt <= warp_cap<Geo>() && G.warp_ready()) {
         if (tid < 32) {
           warp_rounds(S, G, metric, O, nnz, rounds, pair_evals, round_limit);
           if (tid == 0) {
@@ -1065,60 +1099,84 @@ NNS_DEV void cta_rounds(CtaCore<CAP>& S, Geo& G, int metric, const CtaOut& O, un
   }
 }
 
-// Load one side of a pair (raw rows, weights) into the CTA state, check it,
-// and normalise its weights by their correctly rounded total.  With DP > 0
-// the coordinates are copied (zero-padded to DP) into dst.
+// Load both sides of a pair (raw rows, weights) into the CTA state, check
+// them, and normalise each side's weights by their correctly rounded total.
+// With DP > 0 the coordinates are copied (zero-padded to DP) into xs / ys.
+// The sides go through every step together (one after the other they took
+// twice the latency: 7 us of a 256-point solve).  Clears acc[0].
 template <int DP, int CAP>
-NNS_DEV bool cta_load_side(const float* pts, const double* w, int cnt, int d, float* dst, double* res, int* idx,
-                           CtaCore<CAP>& S, unsigned* err) {
+NNS_DEV bool cta_load_sides(const float* x, const double* a, int m, const float* y, const double* b, int n, int d,
+                            float* xs, float* ys, CtaCore<CAP>& S, unsigned* err) {
   const int tid = threadIdx.x;
-  for (int i = tid; i < XS_LIMBS; i += blockDim.x) S.acc[i] = 0ULL;
+  for (int i = tid; i < 2 * XS_LIMBS; i += blockDim.x) (&S.acc[0][0])[i] = 0ULL;
   __syncthreads();
-  bool nonfinite = false, negative = false;
-  for (int base = 0; base < cnt; base += blockDim.x) {  // whole warps (xs_add_warp)
+  unsigned bad = 0;  // bits 0, 1: a value of x / y not finite; bits 2, 3: a weight of a / b negative
+#pragma unroll 1
+  for (int base = 0; base < max(m, n); base += blockDim.x) {  // whole warps (xs_add_warp)
     const int p = base + tid;
-    double add = 0.0;
-    if (p < cnt) {
-    if (DP > 0) {
+    double add[2] = {0.0, 0.0};
 #pragma unroll
-      for (int k = 0; k < (DP > 0 ? DP : 1); ++k) {
-        const float v = k < d ? pts[(size_t)p * d + k] : 0.f;
-        if (!isfinite(v)) nonfinite = true;
-        dst[p * DP + k] = v;
+    for (int sd = 0; sd < 2; ++sd) {
+      if (p < (sd ? n : m)) {
+        const float* pts = sd ? y : x;
+        if (DP > 0) {
+#pragma unroll
+          for (int k = 0; k < (DP > 0 ? DP : 1); ++k) {
+            const float v = k < d ? pts[(size_t)p * d + k] : 0.f;
+            if (!isfinite(v)) bad |= 1u << sd;
+            (sd ? ys : xs)[p * DP + k] = v;
+          }
+        }
+        const double wv = (sd ? b : a)[p];
+        if (!isfinite(wv)) bad |= 1u << sd;
+        else if (wv < 0.0) bad |= 4u << sd;
+        (sd ? S.cres : S.sres)[p] = wv;
+        (sd ? S.jidx : S.iidx)[p] = p;
+        add[sd] = isfinite(wv) && wv > 0.0 ? wv : 0.0;
       }
-    } else {
-      for (int k = 0; k < d; ++k)
-        if (!isfinite(pts[(size_t)p * d + k])) nonfinite = true;
     }
-    const double wv = w[p];
-    if (!isfinite(wv)) nonfinite = true;
-    else if (wv < 0.0) negative = true;
-    res[p] = wv;
-    idx[p] = p;
-    add = isfinite(wv) && wv > 0.0 ? wv : 0.0;
-    }
-    xs_add_warp(S.acc, add);  // one call site for the whole warp
+    xs_add_warp(S.acc[0], add[0]);
+    xs_add_warp(S.acc[1], add[1]);
   }
-  nonfinite = __syncthreads_or(nonfinite);
-  negative = __syncthreads_or(negative);
-  if (tid == 0) S.total = xs_round(S.acc);
+  if (DP == 0) {
+    // rows checked by the whole CTA, consecutive lanes on consecutive values
+#pragma unroll 1
+    for (int sd = 0; sd < 2; ++sd) {
+      const float* pts = sd ? y : x;
+      const int64_t cnt = (int64_t)(sd ? n : m) * d;
+      for (int64_t i = tid; i < cnt; i += blockDim.x)
+        if (!isfinite(pts[i])) bad |= 1u << sd;
+    }
+  }
+  unsigned all = 0;
+#pragma unroll
+  for (int k = 0; k < 4; ++k) all |= __syncthreads_or((bad >> k) & 1u) ? 1u << k : 0u;
+  if (tid < 64) {
+    const double t = xs_round_warp(S.acc[tid >> 5]);
+    if ((tid & 31) == 0) S.total[tid >> 5] = t;
+  }
   __syncthreads();
-  const double total = S.total;
-  if (nonfinite || negative || !(total > 0.0)) {
-    if (tid == 0) atomicOr(err, nonfinite ? EF_NONFINITE : (negative ? EF_NEGATIVE : EF_ZERO_MASS));
+  const double ta = S.total[0], tb = S.total[1];
+  // the first side's error is reported before the second side's
+  const bool ex = (all & 5u) || !(ta > 0.0), ey = (all & 10u) || !(tb > 0.0);
+  if (ex || ey) {
+    const unsigned e = ex ? all : all >> 1;
+    if (tid == 0) atomicOr(err, (e & 1u) ? EF_NONFINITE : ((e & 4u) ? EF_NEGATIVE : EF_ZERO_MASS));
     __syncthreads();
     return false;
   }
-  for (int p = tid; p < cnt; p += blockDim.x) res[p] = __ddiv_rn(res[p], total);
+  for (int p = tid; p < m; p += blockDim.x) S.sres[p] = __ddiv_rn(S.sres[p], ta);
+  for (int p = tid; p < n; p += blockDim.x) S.cres[p] = __ddiv_rn(S.cres[p], tb);
+  for (int i = tid; i < XS_LIMBS; i += blockDim.x) S.acc[0][i] = 0ULL;
   __syncthreads();
   return true;
 }
 
 // Shared memory of a one-CTA solver for d <= 8 (coordinates included).
-template <int D, int DP, bool L1>
+template <int D, int DP, bool L1, int CAP = FIN_MAX, int NT = FIN_THREADS>
 struct LowdSmem {
-  CtaCore<FIN_MAX> S;
-  GeoSmem<D, DP, L1, FIN_MAX> G;
+  CtaCore<CAP> S;
+  GeoSmem<D, DP, L1, CAP, NT> G;
 };
 
 // Whole pair in one CTA: load both sides, drop zero weights, run all rounds,
@@ -1129,17 +1187,14 @@ NNS_DEV bool cta_solve_pair(CtaCore<CAP>& S, Geo& G, float* xs, float* ys, const
                             long long& rounds, long long& pe, int protocol = 0, unsigned long long seed = 0,
                             int32_t* fl_i = nullptr, int32_t* fl_j = nullptr, double* fl_f = nullptr,
                             long long fl_cap = 0) {
-  bool ok = cta_load_side<Geo::kDP, CAP>(x, a, m, d, xs, S.sres, S.iidx, S, err);
-  if (ok) ok = cta_load_side<Geo::kDP, CAP>(y, b, n, d, ys, S.cres, S.jidx, S, err);
-  if (!ok) return false;
+  if (!cta_load_sides<Geo::kDP, CAP>(x, a, m, y, b, n, d, xs, ys, S, err)) return false;
   if (threadIdx.x == 0) {
     S.mt = m;
     S.nt = n;
   }
-  for (int i = threadIdx.x; i < XS_LIMBS; i += blockDim.x) S.acc[i] = 0ULL;
   __syncthreads();
   cta_compact(S, G);  // drop zero weights
-  CtaOut O{S.acc, nullptr, nullptr, nullptr, 0, nullptr, nullptr, err};
+  CtaOut O{S.acc[0], nullptr, nullptr, nullptr, 0, nullptr, nullptr, err};
   O.protocol = protocol;
   O.seed = seed;
   if (fl_i) {
@@ -1159,7 +1214,7 @@ NNS_DEV bool cta_solve_pair(CtaCore<CAP>& S, Geo& G, float* xs, float* ys, const
   pe = 0;
   cta_rounds(S, G, metric, O, nnz, rounds, pe, (long long)m + n);
   __syncthreads();
-  if (threadIdx.x == 0) cost = xs_round(S.acc);
+  if (threadIdx.x < 32) cost = xs_round_warp(S.acc[0]);  // (thread 0 has it)
   return true;
 }
 

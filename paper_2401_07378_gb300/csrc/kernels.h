@@ -151,6 +151,18 @@ struct BatchArgs {
   long long kcap;
 };
 int launch_batched_lowd(const BatchArgs& A, int grid, cudaStream_t st);
+// The same two for pairs of at most LOWD_SMALL_CAP points per side
+// (lowd_pairs_small.cu): fewer threads per pair, several pairs per SM.  A
+// round of such a pair is barrier and memory latency, which more resident
+// pairs hide and more threads lengthen: 2,048 image pairs of 80..400 points
+// took 2.01 ms with one 1,024-thread CTA per SM, 881 us with two of 512
+// threads, 610 us with four of 256 and 607 us with six of 128; a single
+// 256-point pair 84 us at 1,024 threads, 58 at 512, 62 at 256 and at 128.
+constexpr int LOWD_SMALL_CAP = 512;
+constexpr int LOWD_SMALL_THREADS = 256;
+constexpr int LOWD_SMALL_PER_SM = 4;
+int launch_solve_small_cap(const SolveBufs& B, const double* a, const double* b, cudaStream_t st);
+int launch_batched_lowd_small(const BatchArgs& A, int grid, cudaStream_t st);
 
 // highd.cu (d > 8) ---------------------------------------------------------
 // FP32 NNS over all active suppliers for the first `ncons` active consumers,

@@ -158,8 +158,9 @@ __global__ void __launch_bounds__(XS_THREADS) k_final_sums(FinalArgs A) {
 
 // out0 / out1 = the correctly rounded values of acc0 / acc1.
 __global__ void k_xs_round2(unsigned long long* acc0, double* out0, unsigned long long* acc1, double* out1) {
-  if (blockIdx.x == 0 && threadIdx.x == 0) *out0 = xs_round(acc0);
-  if (blockIdx.x == 0 && threadIdx.x == 32 && acc1) *out1 = xs_round(acc1);
+  if (threadIdx.x >= 32 && !acc1) return;
+  const double v = xs_round_warp(threadIdx.x < 32 ? acc0 : acc1);
+  if ((threadIdx.x & 31) == 0) *(threadIdx.x < 32 ? out0 : out1) = v;
 }
 
 // Both sides' normalisation in one launch: blocks [0, ga) take (w0, n0, acc0),
@@ -175,11 +176,14 @@ __global__ void k_normalise2(const double* __restrict__ w0, int64_t n0, const un
   const int bid = second ? blockIdx.x - ga : blockIdx.x, nb = second ? gridDim.x - ga : ga;
   for (int i = threadIdx.x; i < XS_LIMBS; i += blockDim.x) a[i] = acc[i];
   __syncthreads();
-  if (threadIdx.x == 0) {
-    total = xs_round(a);
-    if (bid == 0) {
-      *(second ? total1 : total0) = total;
-      if (!(total > 0.0)) atomicOr(err, EF_ZERO_MASS);
+  if (threadIdx.x < 32) {
+    const double v = xs_round_warp(a);
+    if (threadIdx.x == 0) {
+      total = v;
+      if (bid == 0) {
+        *(second ? total1 : total0) = v;
+        if (!(v > 0.0)) atomicOr(err, EF_ZERO_MASS);
+      }
     }
   }
   __syncthreads();
