@@ -118,7 +118,9 @@ typedef struct {
                                    also caps larger values at 8; with 1..8 the nnsemd_solve scan keeps
                                    8 per chunk, half the list upkeep).  Fewer candidates make the scan
                                    and the re-rank cheaper and the certificate weaker (more FP32
-                                   rescans); results never change.  Outside the range: INVALID_ARG. */
+                                   rescans); results never change.  Batched pairs of at most 512 points
+                                   per side see the exact key of every supplier whatever the value.
+                                   Outside the range: INVALID_ARG. */
   int32_t flags;                /* NNSEMD_FLAG_* bits, 0 for none */
   const void *proposal;         /* learned candidate proposal, NULL = full scan */
   int32_t protocol;             /* nnsemd_protocol (0 = greedy) */
@@ -147,7 +149,8 @@ typedef struct {
   double tail_kernel_ms;        /* NNSEMD_FLAG_TIME_KERNELS: duration of the one-CTA tail kernel */
   int64_t near_ties;            /* reduced precision: consumer searches whose exact FP32 re-rank picked
                                    another supplier than the one the operand-precision distances ranked
-                                   first (ties at that precision).  0 on the FP32 paths: their decisions
+                                   first (ties at that precision); in a batch, of the searches that made
+                                   a candidate list.  0 on the FP32 paths: their decisions
                                    are the FP32 decisions themselves (the FP32 / FP64 near-ties of the
                                    method are the oracle's to count). */
   int64_t widened;              /* learned proposal: consumer searches certified by the second tier (the

@@ -724,42 +724,51 @@ static int solve_batched_impl(nnsemd_ctx* ctx, int32_t num_pairs, const float* x
   if (opt && opt->proposal) return fail(ctx, NNSEMD_ERR_UNSUPPORTED, "proposals serve nnsemd_solve only");
   auto y_begin = [&](int p) -> int64_t { return y_off ? y_off[p] : 0; };
   auto y_len = [&](int p) -> int64_t { return y_off ? y_off[p + 1] - y_off[p] : n_shared; };
+  // pairs that fit a CTA go to the one-CTA solvers, the smaller ones of them
+  // (`tiny`, first in the list) to those with fewer threads, several pairs
+  // per SM.  With d > 8 the tiny pairs take the FP32 key matrix whatever the
+  // precision: each of their searches sees the exact key of every supplier,
+  // which is what the reduced-precision candidates and their certificate
+  // lead to, and one FP32 matrix costs less than packing, contracting,
+  // ranking and re-ranking (us a pair at 64 / 256 / 512 points: d = 64: 0.39 /
+  // 1.04 / 2.9 against 1.06 / 3.1 / 5.0 on the tensor cores, d = 300: 0.68 /
+  // 3.1 / 9.5 against 2.0 / 8.0 / 16.6).
   std::vector<int> small, large;
-  int64_t small_max = 0, small_mn = 0;
-  int64_t km_tiny = 0, km_big = 0;  // largest key matrices (floats) of the 256- and the 1,024-thread FP32 solvers
+  int64_t small_max = 0, small_mn = 0;  // small_mn: values of the tensor-core kernel's distance cache
+  int64_t km_tiny = 0, km_big = 0;  // largest key matrices (floats) of the solvers with fewer and with 1,024 threads
+  const int tcap = d <= 8 ? LOWD_SMALL_CAP : HD_SMALL_CAP;
+  auto tiny = [&](int p) { return x_off[p + 1] - x_off[p] <= tcap && y_len(p) <= tcap; };
+  int ntiny = 0;
   for (int p = 0; p < num_pairs; ++p) {
     const int64_t m = x_off[p + 1] - x_off[p], n = y_len(p);
     if (m < 1 || n < 1) return fail(ctx, NNSEMD_ERR_INVALID_ARG, "pair %d has an empty side", p);
     const int cap = d <= 8 ? FIN_MAX : FIN_MAX_HD;
     const bool fits = m <= cap && n <= cap;
     (fits ? small : large).push_back(p);
-    if (fits) {
-      small_max = std::max(small_max, std::max(m, n));
-      small_mn = std::max(small_mn, m * n);
-      int64_t& km = m <= HD_SMALL_CAP && n <= HD_SMALL_CAP ? km_tiny : km_big;
-      km = std::max<int64_t>(km, m * kmat_ld(n));
+    if (!fits) continue;
+    small_max = std::max(small_max, std::max(m, n));
+    const int64_t km = m * kmat_ld(n);
+    if (tiny(p)) {
+      ++ntiny;
+      km_tiny = std::max(km_tiny, km);
+    } else {
+      km_big = std::max(km_big, km);
+      small_mn = std::max<int64_t>(small_mn, batched_tc_cache_values(m, n));
     }
   }
-  // FP32: pairs of at most HD_SMALL_CAP (d <= 8: LOWD_SMALL_CAP) points per
-  // side go to the kernels with fewer threads (several pairs per SM); they
-  // come first in the list
-  int ntiny = 0;
-  if (!tc) {
-    const int tcap = d <= 8 ? LOWD_SMALL_CAP : HD_SMALL_CAP;
-    auto tiny = [&](int p) { return x_off[p + 1] - x_off[p] <= tcap && y_len(p) <= tcap; };
-    std::stable_partition(small.begin(), small.end(), tiny);
-    for (int p : small) ntiny += tiny(p);
-  }
+  std::stable_partition(small.begin(), small.end(), tiny);
+  const int nbig = (int)small.size() - ntiny;  // 1,024-thread solvers
   CK(cudaSetDevice(ctx->device));
   cudaStream_t st = ctx->stream;
   const int nsm = num_sms();
-  const int grid = (int)std::min<size_t>(small.size(), (size_t)nsm);
-  // tensor-core kernel geometry: capacity class, bytes per packed row, tile
-  // rows and pipeline stages (autotuned or default)
-  const int cap = small_max <= 512 ? 512 : 2048;
+  const int gbig = std::min(nbig, nsm), gtiny = std::min(ntiny, nsm * (d <= 8 ? LOWD_SMALL_PER_SM : 4));
+  // tensor-core kernel geometry: bytes per packed row, tile rows and
+  // pipeline stages (autotuned or default).  A batch whose rows are too long
+  // for its largest pair's kernel is refused, tiny pairs too.
+  constexpr int cap = FIN_MAX_HD;
   const int kb = tc ? (int)tc_kb(d, precision) : 0;
   int bn = tc ? tc_bn(kb) : 0;
-  int nstage = tc ? batched_tc_max_stages(cap, kb, bn, precision) : 0;
+  int nstage = tc ? batched_tc_max_stages(small_max <= HD_SMALL_CAP ? HD_SMALL_CAP : cap, kb, bn, precision) : 0;
   if (tc && !small.empty() && nstage < 1) return fail(ctx, NNSEMD_ERR_UNSUPPORTED, "d = %d too large for the batched tensor-core kernel", d);
   const auto tkey = std::make_tuple(d, precision, cap);
   int kc_use = 1;
@@ -772,21 +781,19 @@ static int solve_batched_impl(nnsemd_ctx* ctx, int32_t num_pairs, const float* x
   auto slot_of = [&](long long kc) {
     return std::max(batched_tc_slot_bytes(cap, kb, 64, kc), batched_tc_slot_bytes(cap, kb, 128, kc));
   };
-  if (tc && (double)slot_of(kc_cap) * grid > KC_BUDGET_BYTES) kc_cap = 0;
-  const size_t slot = tc ? slot_of(kc_cap) : 0;
-  // flow records of the d > 8 solvers, one slice per CTA (the tensor-core
-  // kernel's grid; the 1,024- and the 256-thread FP32 kernels' grids)
-  const long long fl_big = tc ? 2LL * cap : 2LL * FIN_MAX_HD, fl_small = 2LL * HD_SMALL_CAP;
-  const size_t fl_n = d <= 8 || small.empty() ? 0 : (size_t)(nsm * fl_big + (tc ? 0 : nsm * 4 * fl_small));
+  if (tc && (double)slot_of(kc_cap) * gbig > KC_BUDGET_BYTES) kc_cap = 0;
+  const size_t slot = tc && nbig ? slot_of(kc_cap) : 0;
+  // flow records of the d > 8 solvers, one slice per CTA (the 1,024-thread
+  // kernels' grid, then the 256-thread kernel's)
+  const long long fl_big = 2LL * FIN_MAX_HD, fl_small = 2LL * HD_SMALL_CAP;
+  const size_t fl_n = d <= 8 || small.empty() ? 0 : (size_t)(nsm * fl_big + nsm * 4 * fl_small);
   // key matrices of the d > 8 FP32 solvers, one slot per CTA; a solver whose
   // slots exceed the budget, or any if the memory is not there, computes the
   // keys again in every round instead
-  const int nbig_pairs = (int)small.size() - ntiny;
-  const int gbig = std::min(nbig_pairs, nsm), gtiny = std::min(ntiny, nsm * (d <= 8 ? LOWD_SMALL_PER_SM : 4));
   auto km_slot = [&](int64_t km, int g) -> long long {
-    return tc || d <= 8 || (double)km * g * sizeof(float) > KC_BUDGET_BYTES ? 0 : (km + 63) & ~63LL;
+    return d <= 8 || (double)km * g * sizeof(float) > KC_BUDGET_BYTES ? 0 : (km + 63) & ~63LL;
   };
-  long long kc_big = km_slot(km_big, gbig), kc_tiny = km_slot(km_tiny, gtiny);
+  long long kc_big = tc ? 0 : km_slot(km_big, gbig), kc_tiny = km_slot(km_tiny, gtiny);
   // workspace: offsets, pair list, queue/error/counters, per-pair counters,
   // tensor-core scratch slots, flow records, key matrices, then the buffers
   // of the large pairs
@@ -808,7 +815,7 @@ static int solve_batched_impl(nnsemd_ctx* ctx, int32_t num_pairs, const float* x
     ctr_d = C.take<unsigned long long>(6);
     rounds_d = C.take<long long>(num_pairs);
     pe_d = C.take<long long>(num_pairs);
-    scratch = C.take<uint8_t>(tc ? slot * grid : 0);
+    scratch = C.take<uint8_t>(slot * gbig);
     fl_i = C.take<int32_t>(fl_n);
     fl_j = C.take<int32_t>(fl_n);
     fl_f = C.take<double>(fl_n);
@@ -838,11 +845,12 @@ static int solve_batched_impl(nnsemd_ctx* ctx, int32_t num_pairs, const float* x
     CK(cudaMemcpyAsync(ids_d, small.data(), small.size() * sizeof(int), cudaMemcpyHostToDevice, st));
   long long L = 0;
   // the device work of the small pairs: clear the counters, one persistent launch
-  auto issue = [&](cudaStream_t s, int nsmall, int g, int tbn, int tns, long long tkc) -> int {
+  // (nb of the 1,024-thread solvers' pairs on g CTAs, nt of the others)
+  auto issue = [&](cudaStream_t s, int nb, int g, int nt, int tbn, int tns, long long tkc) -> int {
     if (cudaMemsetAsync(ctr_d, 0, 6 * sizeof(unsigned long long), s) != cudaSuccess) return -1;
     if (cudaMemsetAsync(rounds_d, 0, num_pairs * sizeof(long long), s) != cudaSuccess) return -1;
     if (cudaMemsetAsync(pe_d, 0, num_pairs * sizeof(long long), s) != cudaSuccess) return -1;
-    BatchArgs A{x_packed, a_packed, xo_d, y_packed, b_packed, yo_d, ids_d, nsmall, d, metric,
+    BatchArgs A{x_packed, a_packed, xo_d, y_packed, b_packed, yo_d, ids_d, 0, d, metric,
                 costs_out, rounds_d, pe_d, q_d, q_d + 1, opt ? opt->protocol : 0, opt ? opt->seed : 0ULL,
                 y_off ? 0 : (int)n_shared};
     if (fl_n) {
@@ -851,22 +859,22 @@ static int solve_batched_impl(nnsemd_ctx* ctx, int32_t num_pairs, const float* x
       A.fl_f = fl_f;
       A.fl_cap = fl_big;
     }
-    if (tc)  // (grid <= one CTA per SM)
-      return launch_batched_tc(A, precision, cap, kb, tbn, tns, scratch, slot, ctr_d + 1, ctr_d + 2, ctr_d + 4,
-                               opt ? opt->rerank_k : 0, tkc, g, s);
     int r = 0;
-    const int nbig = nsmall - ntiny;
-    if (nbig > 0) {
+    if (nb > 0) {
       BatchArgs Ab = A;
       Ab.pair_ids = ids_d + ntiny;
-      Ab.num = nbig;
+      Ab.num = nb;
       Ab.kmat = kc_big ? kmat : nullptr;
       Ab.kcap = kc_big;
-      r |= d <= 8 ? launch_batched_lowd(Ab, gbig, s) : launch_batched_hd(Ab, gbig, s);
+      if (tc)  // (at most one CTA per SM)
+        r |= launch_batched_tc(Ab, precision, cap, kb, tbn, tns, scratch, slot, ctr_d + 1, ctr_d + 2, ctr_d + 4,
+                               opt ? opt->rerank_k : 0, tkc, g, s);
+      else
+        r |= d <= 8 ? launch_batched_lowd(Ab, g, s) : launch_batched_hd(Ab, g, s);
     }
-    if (ntiny > 0) {
+    if (nt > 0) {
       BatchArgs At = A;
-      At.num = ntiny;
+      At.num = nt;
       At.queue = q2_d;
       if (fl_n) {  // the slices after the 1,024-thread kernel's
         At.fl_i = fl_i + nsm * fl_big;
@@ -876,13 +884,14 @@ static int solve_batched_impl(nnsemd_ctx* ctx, int32_t num_pairs, const float* x
       }
       At.kmat = kc_tiny ? kmat + kc_big * gbig : nullptr;
       At.kcap = kc_tiny;
+      if (tc) At.searches = ctr_d + 1;  // settled with every supplier a candidate: certified
       r |= d <= 8 ? launch_batched_lowd_small(At, gtiny, s) : launch_batched_hd_small(At, gtiny, s);
     }
     return r;
   };
-  if (!small.empty() && tc && (flags & NNSEMD_FLAG_AUTOTUNE) && !ctx->tuned.count(tkey)) {
+  if (nbig > 0 && tc && (flags & NNSEMD_FLAG_AUTOTUNE) && !ctx->tuned.count(tkey)) {
     // time every feasible (tile rows, stages, cache on / off) on a sample of the batch
-    const int nsample = (int)std::min<size_t>(small.size(), 2 * (size_t)nsm);
+    const int nsample = std::min(nbig, 2 * nsm);
     const int gs = std::min(nsample, nsm);
     if (!ctx->ev[0])
       for (int k = 0; k < 4; ++k) CK(cudaEventCreate(&ctx->ev[k]));
@@ -893,10 +902,10 @@ static int solve_batched_impl(nnsemd_ctx* ctx, int32_t num_pairs, const float* x
         if (tbn == 128 && kb > 384) continue;
         const int maxs = batched_tc_max_stages(cap, kb, tbn, precision);
         for (int tns = 1; tns <= maxs; ++tns) {
-          if (issue(st, nsample, gs, tbn, tns, tkc ? kc_cap : 0))
+          if (issue(st, nsample, gs, 0, tbn, tns, tkc ? kc_cap : 0))
             return fail(ctx, NNSEMD_ERR_CUDA, "autotune launch");
           CK(cudaEventRecord(ctx->ev[0], st));
-          if (issue(st, nsample, gs, tbn, tns, tkc ? kc_cap : 0))
+          if (issue(st, nsample, gs, 0, tbn, tns, tkc ? kc_cap : 0))
             return fail(ctx, NNSEMD_ERR_CUDA, "autotune launch");
           CK(cudaEventRecord(ctx->ev[1], st));
           CK(cudaEventSynchronize(ctx->ev[1]));
@@ -932,7 +941,7 @@ static int solve_batched_impl(nnsemd_ctx* ctx, int32_t num_pairs, const float* x
         if (!ctx->capture_stream) CK(cudaStreamCreateWithFlags(&ctx->capture_stream, cudaStreamNonBlocking));
         cudaGraph_t graph = nullptr;
         CK(cudaStreamBeginCapture(ctx->capture_stream, cudaStreamCaptureModeThreadLocal));
-        brc = issue(ctx->capture_stream, (int)small.size(), grid, bn, nstage, kc_cap);
+        brc = issue(ctx->capture_stream, nbig, gbig, ntiny, bn, nstage, kc_cap);
         cudaError_t ce = cudaStreamEndCapture(ctx->capture_stream, &graph);
         if (brc || ce != cudaSuccess) {
           if (graph) cudaGraphDestroy(graph);
@@ -947,7 +956,7 @@ static int solve_batched_impl(nnsemd_ctx* ctx, int32_t num_pairs, const float* x
       }
       CK(cudaGraphLaunch(g->exec, st));
     } else {
-      brc = issue(st, (int)small.size(), grid, bn, nstage, kc_cap);
+      brc = issue(st, nbig, gbig, ntiny, bn, nstage, kc_cap);
     }
     if (brc) return fail(ctx, NNSEMD_ERR_CUDA, "batched launch (%d)", brc);
     CK(cudaGetLastError());

@@ -16,6 +16,9 @@
 //      cannot be certified are scanned again in FP32 (64 x 64 tiles);
 //   4. groups, serves, retires and compacts exactly as the other one-CTA
 //      solvers (cta.cuh).
+// A pair whose m * n values fit the CTA's distance cache runs 1 and 2 in its
+// first round alone and answers every round from candidate lists
+// (GeoTC::nns_lists).
 // The result equals the FP32 path's.  All waits are bounded (EF_TIMEOUT).
 #include <math_constants.h>
 
@@ -26,9 +29,11 @@
 
 namespace nnsemd {
 
-// Candidates per consumer in the batched kernel (its 1,024 threads have 64
-// registers each; the multi-CTA kernel keeps TC_K = 16).
+// Candidates per consumer in the batched kernel's pass without the distance
+// cache (its 1,024 threads have 64 registers each; the multi-CTA kernel keeps
+// TC_K = 16).
 constexpr int BTC_K = 8;
+constexpr int BTC_FILL_WARPS = 16;  // epilogue warps while the distance cache fills (from warp 4 on)
 
 // Per-CTA scratch in global memory.
 struct BtcScratch {
@@ -41,16 +46,32 @@ struct BtcScratch {
   float* scale_y;
   float* cand_v;    // [cap][BTC_K]
   int* cand_p;
-  // distance cache of a pair with m * n <= kc_cap (see GeoTC::nns_cached),
-  // indexed [original consumer][original supplier]
-  float* vcache;    // approximate ranking values v' of the tensor-core pass
-  float* kcache;    // exact FP32 keys, NaN until computed
-  float* ny_o;      // per original consumer: FP32 squared norm, scale, FP64 norms
+  // distance cache of a pair that fits kc_cap values (see GeoTC::nns_lists), by
+  // original consumer j and supplier i: approximate ranking values v' of the
+  // tensor-core pass, [j / 32][i / 4][j % 32][i % 4] (a warp of 32 consumers
+  // writes four columns as 512 contiguous bytes), and the minimum of each 16
+  // suppliers, [j / 32][i / 16][j % 32]
+  float* vcache;
+  float* vmin;
+  // candidate lists by original consumer: (exact key bits << 32 | original
+  // supplier) ascending, the next entry to look at | length << 8, and the
+  // value a key must stay below to be the nearest (certify_floor)
+  unsigned long long* list;
+  int* lnext;
+  double* lfloor;
+  float* ny_o;      // per original consumer: FP32 squared norm, scale, norms rounded up
   float* sy_o;
-  double* yl2_o;
-  double* yl1_o;
+  float* yl2_o;
+  float* yl1_o;
   double* e_o;      // per original consumer: E of the certificate (certify_E)
 };
+
+// Values of a pair's distance cache (rows padded to whole warps, columns to
+// whole vectors, at least 16).
+__host__ __device__ inline long long btc_cache_values(long long m, long long n) {
+  return (kmat_ld(m) < 16 ? 16 : kmat_ld(m)) * ((n + 31) & ~31LL);
+}
+long long batched_tc_cache_values(long long m, long long n) { return btc_cache_values(m, n); }
 
 __host__ __device__ inline size_t btc_slot_layout(uint8_t* base, int cap, int kb, int bn, BtcScratch* out,
                                                   long long kc_cap = 0) {
@@ -74,11 +95,14 @@ __host__ __device__ inline size_t btc_slot_layout(uint8_t* base, int cap, int kb
   s.cand_v = (float*)take((size_t)cap * BTC_K * sizeof(float));
   s.cand_p = (int*)take((size_t)cap * BTC_K * sizeof(int));
   s.vcache = (float*)take((size_t)kc_cap * sizeof(float));
-  s.kcache = (float*)take((size_t)kc_cap * sizeof(float));
+  s.vmin = (float*)take((size_t)(kc_cap / 8) * sizeof(float));  // (kc_ld / 16 rounded up is at most kc_ld / 8 from 16 columns on)
+  s.list = (unsigned long long*)take(kc_cap ? (size_t)cap * BTC_K * sizeof(unsigned long long) : 0);
+  s.lnext = (int*)take(kc_cap ? (size_t)cap * sizeof(int) : 0);
+  s.lfloor = (double*)take(kc_cap ? (size_t)cap * sizeof(double) : 0);
   s.ny_o = (float*)take(kc_cap ? (size_t)cap * sizeof(float) : 0);
   s.sy_o = (float*)take(kc_cap ? (size_t)cap * sizeof(float) : 0);
-  s.yl2_o = (double*)take(kc_cap ? (size_t)cap * sizeof(double) : 0);
-  s.yl1_o = (double*)take(kc_cap ? (size_t)cap * sizeof(double) : 0);
+  s.yl2_o = (float*)take(kc_cap ? (size_t)cap * sizeof(float) : 0);
+  s.yl1_o = (float*)take(kc_cap ? (size_t)cap * sizeof(float) : 0);
   s.e_o = (double*)take(kc_cap ? (size_t)cap * sizeof(double) : 0);
   if (out) *out = s;
   return (off + 255) & ~(size_t)255;
@@ -106,7 +130,10 @@ template <bool KIND8, int CAP>
 struct GeoTC {
   static constexpr int kDP = 0;
   static constexpr int kThreads = FIN_THREADS;
+  // (a list is a warp's work of 20 us and more: the last rounds of a pair make
+  // theirs in 32 warps rather than in warp_rounds' one)
   static constexpr bool kWarpRounds = false;
+  static constexpr int SEL_BUF = 128;  // words a warp's selection collects at most
   struct PX {};
   const float* x;  // this pair's coordinates
   const float* y;
@@ -119,25 +146,30 @@ struct GeoTC {
   uint64_t bar_empty[8];
   uint64_t bar_acc_full[2];
   uint64_t bar_acc_empty[2];
+  // the same for passes that fill the distance cache (BTC_FILL_WARPS
+  // epilogue warps, one arrival each)
+  uint64_t bar_accf_full[2];
+  uint64_t bar_accf_empty[2];
   uint64_t bar_a_full;
   uint64_t bar_a_empty;
   // pipeline counters: prod_* only by the producer thread, mma_* only by the
   // MMA thread; epi_acc is read by the epilogue threads at the start of a
   // phase and advanced by one thread after it
-  unsigned prod_a, prod_b, mma_a, mma_b, mma_acc, epi_acc;
+  unsigned prod_a, prod_b, mma_a, mma_b, mma_acc, epi_acc, mma_accf, epi_accf;
   unsigned stat_rx, stat_rx1, stat_sx;  // certificate maxima of this round (float bits)
-  int nfb;
+  int nfb, nscan;
   unsigned long long ncert, nfall, nnear;
   // distance cache of the current pair: on (m * n fits), filled (after the
   // pair's first round), the pair's supplier and consumer counts (the row
   // length and the number of rows)
-  int kc_on, kc_ready, kc_m, kc_n;
+  int kc_on, kc_ready, kc_m, kc_n, kc_ld;
   double kc_gam;  // gamma_d of the certificate
   int fb[CAP];
   // staging: tensor-core operand tiles or FP32 fallback tiles (never both at
   // once); the launch reserves max(sizeof(tiles), A + stages * B) bytes
   union __align__(128) Stage {
     TileSmem tiles[FIN_THREADS / TG_THREADS];
+    unsigned long long sel[FIN_THREADS / 32 * SEL_BUF];  // make_lists
     uint8_t bytes[16];
   } U;
 
@@ -151,156 +183,315 @@ struct GeoTC {
   }
 
   // The NNS step of a round from the pair's distance cache (the tensor-core
-  // pass of its first round filled every v'): one warp per active consumer.
-  //   1. the rk active suppliers with the smallest v' (each lane keeps the
-  //      best rk of its share of the suppliers, then rk warp-wide minima
-  //      merge the lists; ties by position);
-  //   2. their exact FP32 keys, from the key cache or computed (and cached)
-  //      by one lane each, in the definition's sequential order;
-  //   3. the certificate of the best of them against tau, the rk-th v'
-  //      (every other active supplier has v' >= tau; with no other active
-  //      supplier every one was a candidate and the best is the answer);
-  //   4. otherwise the exact key of every active supplier (cached or
-  //      computed), the smallest with its position.
-  // The per-supplier maxima of the certificate are those of the first
-  // round's active suppliers, a superset of every later round's, so the
-  // bound only gets more conservative.  Exact keys are written and read by
-  // the warp that owns the consumer in that round; a barrier separates
-  // rounds, so a key cached by one warp is seen by the next.
+  // pass of its first round filled every v').  Active suppliers only ever
+  // leave, so a consumer keeps a list of the rk active suppliers with the
+  // smallest v' at the time it was made, ordered by exact FP32 key, and walks
+  // it from round to round: its first entry that is still active is the
+  // nearest active supplier as long as its key is below the list's
+  // certificate bound (every supplier outside the list has v' >= tau, the
+  // list's largest).  A consumer whose list runs out, or whose next entry the
+  // bound does not certify, makes a new one from the suppliers active now
+  // (a warp makes four at a time):
+  //   1. the rk smallest v' (ties by position), their exact FP32 keys, one
+  //      per lane in the definition's sequential order, ordered by (key,
+  //      original index: positions keep that order);
+  //   2. the certificate of the first against tau, with the first round's
+  //      supplier maxima (a superset of every later round's); with no other
+  //      active supplier every entry is the answer in its turn;
+  //   3. not certified: the FP32 tiles over every active supplier, for all
+  //      such consumers of the round together.
+  // A consumer takes about two searches, so 8 entries serve it; 32 cost more
+  // in exact keys (each lane walks its own row) than they saved.  1,000
+  // retrieval pairs (256..2,048 points, d = 128, FP16): 43.5 ms with the
+  // candidates selected anew in every round, 16.3 ms so.
+  //
+  // S.off holds, by original index, the position of each active supplier
+  // (free until the round's grouping); a stale entry fails its check.
   template <int C>
-  NNS_DEV const unsigned long long* nns_cached(CtaCore<C>& S, int mt, int nt) {
-    const int tid = threadIdx.x, T = blockDim.x;
-    const int warp = tid >> 5, lane = tid & 31;
-    const int K = rk < mt ? rk : mt;
-    for (int q = warp; q < nt; q += T / 32) {
-      const int j = S.jidx[q];
-      const float* vrow = scr.vcache + (size_t)j * kc_m;
-      float* krow = scr.kcache + (size_t)j * kc_m;
-      const float* yrow = y + (size_t)j * d;
-      // 1. candidates: this lane's best BTC_K, then the warp's best K
-      float tv[BTC_K];
-      int tp[BTC_K];
-#pragma unroll
-      for (int k = 0; k < BTC_K; ++k) { tv[k] = CUDART_INF_F; tp[k] = -1; }
-      // four loads in flight per lane before the insertions that use them
-      for (int p0 = lane; p0 < mt; p0 += 128) {
-        float v[4];
-#pragma unroll
-        for (int u = 0; u < 4; ++u) {
-          const int p = p0 + 32 * u;
-          v[u] = p < mt ? vrow[S.iidx[p]] : CUDART_INF_F;
-        }
-#pragma unroll
-        for (int u = 0; u < 4; ++u)
-          if (p0 + 32 * u < mt) topk_insert(tv, tp, v[u], p0 + 32 * u);
+  NNS_DEV void map_positions(CtaCore<C>& S, int mt, int first, int step) const {
+    for (int p = first; p < mt; p += step) S.off[S.iidx[p]] = p;
+  }
+  // One consumer from its list: true and its packed key, or false.
+  template <int C>
+  NNS_DEV bool serve(const CtaCore<C>& S, int mt, int j, unsigned long long& key) const {
+    const int st = scr.lnext[j], end = st >> 8;
+    const unsigned long long* l = scr.list + (size_t)j * BTC_K;
+    for (int t = st & 0xff; t < end; ++t) {
+      const unsigned long long e = l[t];
+      const int i = (int)(unsigned)e, p = S.off[i];
+      if ((unsigned)p >= (unsigned)mt || S.iidx[p] != i) continue;  // retired
+      if (!((double)__uint_as_float((unsigned)(e >> 32)) < scr.lfloor[j])) return false;
+      scr.lnext[j] = (st & ~0xff) | t;
+      key = (e & 0xffffffff00000000ULL) | (unsigned)p;
+      return true;
+    }
+    return false;
+  }
+  NNS_DEV size_t v_at(int j, int i) const {
+    return ((((size_t)(j >> 5) * (kc_ld >> 2)) + (i >> 2)) * 32 + (j & 31)) * 4 + (i & 3);
+  }
+  // The 8 smallest of the warp's words v (four a lane, ~0 for none), in order
+  // in lanes 0..7 with their ids: eight minima over the warp, each by one
+  // reduction; equal words by lane.
+  NNS_DEV void extract8(unsigned (&v)[4], const int (&id)[4], unsigned& rv, int& rid) const {
+    const int lane = threadIdx.x & 31;
+    rv = 0xffffffffu;
+    rid = 0;
+#pragma unroll 1
+    for (int k = 0; k < 8; ++k) {
+      const unsigned mine = min(min(v[0], v[1]), min(v[2], v[3]));
+      const unsigned w = __reduce_min_sync(0xffffffffu, mine);
+      if (w == 0xffffffffu) break;
+      const int src = __ffs(__ballot_sync(0xffffffffu, mine == w)) - 1;
+      int my = id[3];
+      const int u = v[0] == w ? 0 : (v[1] == w ? 1 : (v[2] == w ? 2 : 3));
+      my = u == 0 ? id[0] : (u == 1 ? id[1] : (u == 2 ? id[2] : id[3]));
+      my = __shfl_sync(0xffffffffu, my, src);
+      if (lane == src) {
+        if (u == 0) v[0] = 0xffffffffu;
+        else if (u == 1) v[1] = 0xffffffffu;
+        else if (u == 2) v[2] = 0xffffffffu;
+        else v[3] = 0xffffffffu;
       }
-      unsigned long long sel = ~0ULL, first = ~0ULL, kth = ~0ULL;
-      for (int k = 0; k < K; ++k) {
-        const unsigned long long mine =
-            tp[0] >= 0 ? ((unsigned long long)ordered_bits(tv[0]) << 32) | (unsigned)tp[0] : ~0ULL;
-        unsigned long long w = mine;
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-          const unsigned long long other = __shfl_xor_sync(0xffffffffu, w, o);
-          w = other < w ? other : w;
-        }
-        if (mine == w && w != ~0ULL) {  // the winning lane drops its head
-#pragma unroll
-          for (int i = 0; i + 1 < BTC_K; ++i) {
-            tv[i] = tv[i + 1];
-            tp[i] = tp[i + 1];
-          }
-          tv[BTC_K - 1] = CUDART_INF_F;
-          tp[BTC_K - 1] = -1;
-        }
-        if (lane == k) sel = w;
-        if (k == 0) first = w;
-        kth = w;
-      }
-      // 2. exact keys of the candidates
-      unsigned long long best = ~0ULL;
-      if (lane < K && sel != ~0ULL) {
-        const int p = (int)(unsigned)sel;
-        const int i = S.iidx[p];
-        float key = krow[i];
-        if (key != key) {
-          key = key32<METRIC_SQL2>(x + (size_t)i * d, yrow, d);
-          krow[i] = key;
-        }
-        best = pack_key(key, (unsigned)p);
-      }
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) {
-        const unsigned long long other = __shfl_xor_sync(0xffffffffu, best, o);
-        best = other < best ? other : best;
-      }
-      // 3. the certificate (tau = +inf: no other active supplier)
-      bool cert = false;
-      if (lane == 0) {
-        const unsigned tb = (unsigned)(kth >> 32);
-        // (E of this consumer was computed once, when the cache was filled)
-        const float tau = mt > K ? __uint_as_float((tb & 0x80000000u) ? (tb & 0x7fffffffu) : ~tb) : CUDART_INF_F;
-        cert = best != ~0ULL &&
-               (mt <= K || (double)__uint_as_float((unsigned)(best >> 32)) <
-                               certify_floor_from_E(scr.ny_o[j], tau, scr.e_o[j], kc_gam));
-      }
-      cert = __shfl_sync(0xffffffffu, cert, 0);
-      if (cert) {
-        if (lane == 0) {
-          S.nnk[q] = best;
-          atomicAdd(&ncert, 1ULL);
-          if ((unsigned)best != (unsigned)first) atomicAdd(&nnear, 1ULL);
-        }
-        continue;
-      }
-      // 4. the exact scan
-      unsigned long long m2 = ~0ULL;
-      for (int p = lane; p < mt; p += 32) {
-        const int i = S.iidx[p];
-        float key = krow[i];
-        if (key != key) {
-          key = key32<METRIC_SQL2>(x + (size_t)i * d, yrow, d);
-          krow[i] = key;
-        }
-        const unsigned long long kk = pack_key(key, (unsigned)p);
-        m2 = kk < m2 ? kk : m2;
-      }
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) {
-        const unsigned long long other = __shfl_xor_sync(0xffffffffu, m2, o);
-        m2 = other < m2 ? other : m2;
-      }
-      if (lane == 0) {
-        S.nnk[q] = m2;
-        atomicAdd(&nfall, 1ULL);
-        if ((unsigned)m2 != (unsigned)first) atomicAdd(&nnear, 1ULL);
+      if (lane == k) {
+        rv = w;
+        rid = my;
       }
     }
+  }
+  // The 8 smallest value(p), p < mt, as extract8 gives them (ids: original
+  // indices).  The 8th smallest of the lanes' minima bounds the 8th smallest
+  // of all; a second pass collects what does not exceed it (a few more than 8
+  // values; where the buffer would overflow the 8 best so far stay).
+  template <class C, class Value>
+  NNS_DEV void scan8(const C& S, int mt, unsigned long long* buf, unsigned& rv, int& rid, Value value) const {
+    const int lane = threadIdx.x & 31;
+    const unsigned lt = (1u << lane) - 1u;
+    unsigned mn = 0xffffffffu;
+#pragma unroll 4
+    for (int p = lane; p < mt; p += 32) mn = min(mn, value(p));
+    unsigned v[4] = {mn, 0xffffffffu, 0xffffffffu, 0xffffffffu};
+    int id[4] = {0, 0, 0, 0};
+    extract8(v, id, rv, rid);
+    const unsigned thr = __shfl_sync(0xffffffffu, rv, 7);
+    int cnt = 0;
+    auto take = [&]() {  // the best 8 of the collected ones
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        const unsigned long long w = 32 * u + lane < cnt ? buf[32 * u + lane] : ~0ULL;
+        v[u] = (unsigned)(w >> 32);
+        id[u] = (int)(unsigned)w;
+      }
+      extract8(v, id, rv, rid);
+      __syncwarp();
+    };
+#pragma unroll 1
+    for (int p0 = 0; p0 < mt; p0 += 96) {  // three loads a lane in flight
+      unsigned w[3], bal[3];
+#pragma unroll
+      for (int u = 0; u < 3; ++u) {
+        const int p = p0 + 32 * u + lane;
+        w[u] = p < mt ? value(p) : 0xffffffffu;
+      }
+#pragma unroll
+      for (int u = 0; u < 3; ++u) bal[u] = __ballot_sync(0xffffffffu, p0 + 32 * u + lane < mt && w[u] <= thr);
+      const int add = __popc(bal[0]) + __popc(bal[1]) + __popc(bal[2]);
+      if (!add) continue;
+      if (cnt + add > SEL_BUF) {
+        take();
+        cnt = 8;
+        if (lane < 8) buf[lane] = ((unsigned long long)rv << 32) | (unsigned)rid;
+        __syncwarp();
+      }
+#pragma unroll
+      for (int u = 0; u < 3; ++u) {
+        if ((bal[u] >> lane) & 1u)
+          buf[cnt + __popc(bal[u] & lt)] = ((unsigned long long)w[u] << 32) | (unsigned)S.iidx[p0 + 32 * u + lane];
+        cnt += __popc(bal[u]);
+      }
+      __syncwarp();
+    }
+    take();
+  }
+  // The same for v' while every original supplier is active: each of the 8
+  // smallest lies in one of the 8 groups of 16 with the smallest minima.
+  NNS_DEV void groups8(int j, unsigned& rv, int& rid) const {
+    const int lane = threadIdx.x & 31;
+    const int nb = (kc_ld + 15) >> 4;  // at most 128
+    const float* mrow = scr.vmin + (size_t)(j >> 5) * nb * 32 + (j & 31);
+    unsigned v[4];
+    int id[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const int b = 32 * u + lane;
+      v[u] = b < nb ? ordered_bits(mrow[(size_t)b * 32]) : 0xffffffffu;
+      id[u] = b;
+    }
+    extract8(v, id, rv, rid);
+    // four lanes a group, four values a lane
+    const int b = __shfl_sync(0xffffffffu, rid, lane >> 2);
+    const bool on = __shfl_sync(0xffffffffu, rv, lane >> 2) != 0xffffffffu;
+    const int i0 = 16 * b + 4 * (lane & 3);
+    float4 f = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (on && i0 < kc_ld) f = *reinterpret_cast<const float4*>(scr.vcache + v_at(j, i0));
+    const float e[4] = {f.x, f.y, f.z, f.w};
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      id[u] = i0 + u;
+      v[u] = on && i0 + u < kc_m ? ordered_bits(e[u]) : 0xffffffffu;
+    }
+    extract8(v, id, rv, rid);
+  }
+  // Key of original supplier i against consumer row yrow (16 bytes at a time
+  // where the rows allow it: the same chain).
+  NNS_DEV float exact_key(int i, const float* yrow, bool vec) const {
+    return vec ? key32_sql2_v4(x + (size_t)i * d, yrow, d) : key32<METRIC_SQL2>(x + (size_t)i * d, yrow, d);
+  }
+  // New lists for up to four consumers (one warp; cnt of them, positions
+  // qs(0..cnt)): eight lanes a consumer.  Stores their packed keys in S.nnk.
+  template <int C, class Qs>
+  NNS_DEV void make_lists(CtaCore<C>& S, int mt, int cnt, Qs qs) {
+    const int lane = threadIdx.x & 31, g = lane >> 3, sub = lane & 7;
+    unsigned long long* buf = U.sel + (threadIdx.x >> 5) * SEL_BUF;
+    const bool vec = (d & 3) == 0 && ((reinterpret_cast<uintptr_t>(x) | reinterpret_cast<uintptr_t>(y)) & 15) == 0;
+    const int len = min(rk, mt);
+    // 1.
+    unsigned cv = 0xffffffffu;  // this lane's candidate: v' and original index
+    int i = 0;
+#pragma unroll 1
+    for (int h = 0; h < cnt; ++h) {
+      const int jj = S.jidx[qs(h)];
+      unsigned rv;
+      int rid;
+      if (mt == kc_m) groups8(jj, rv, rid);
+      else scan8(S, mt, buf, rv, rid, [&](int p) { return ordered_bits(scr.vcache[v_at(jj, S.iidx[p])]); });
+      rv = __shfl_sync(0xffffffffu, rv, sub);
+      rid = __shfl_sync(0xffffffffu, rid, sub);
+      if (g == h) {
+        cv = rv;
+        i = rid;
+      }
+    }
+    const int q = qs(min(g, cnt - 1)), j = S.jidx[q];
+    const float* yrow = y + (size_t)j * d;
+    const bool on = g < cnt && sub < len;
+    if (!on) i = 0;
+    const unsigned long long e = on ? pack_key(exact_key(i, yrow, vec), (unsigned)i) : ~0ULL;
+    const int first = __shfl_sync(0xffffffffu, i, lane & 24);  // the approximate choice
+    int rank = 0;
+    unsigned long long best = ~0ULL;
+#pragma unroll
+    for (int u = 0; u < 8; ++u) {
+      const unsigned long long o = __shfl_sync(0xffffffffu, e, (lane & 24) + u);
+      rank += o < e;
+      best = o < best ? o : best;
+    }
+    // 2.
+    const unsigned tb = __shfl_sync(0xffffffffu, cv, (lane & 24) + len - 1);
+    double fl = CUDART_INF;
+    bool bad = false;
+    if (g < cnt && mt > len) {
+      const float tau = __uint_as_float((tb & 0x80000000u) ? (tb & 0x7fffffffu) : ~tb);
+      fl = certify_floor_from_E(scr.ny_o[j], tau, scr.e_o[j], kc_gam);
+      bad = !((double)__uint_as_float((unsigned)(best >> 32)) < fl);
+    }
+    if (on && !bad) scr.list[(size_t)j * BTC_K + rank] = e;
+    if (g < cnt && sub == 0 && !bad) {
+      scr.lnext[j] = len << 8;
+      scr.lfloor[j] = fl;
+      S.nnk[q] = (best & 0xffffffff00000000ULL) | (unsigned)S.off[(int)(unsigned)best];
+      atomicAdd(&ncert, 1ULL);
+      if ((int)(unsigned)best != first) atomicAdd(&nnear, 1ULL);
+    }
+    // 3. left to the FP32 tiles (their keys are not kept)
+    if (g < cnt && sub == 0 && bad) {
+      scr.lnext[j] = 0;
+      const int k = atomicAdd(&nscan, 1);
+      scan_list(S)[k] = q;
+      scan_first(S)[k] = first;
+    }
+    __syncwarp();
+  }
+  // Consumers for the FP32 tiles and their approximate choices (S.mem and
+  // S.mem2 are free during the NNS step).
+  template <int C>
+  NNS_DEV int* scan_list(CtaCore<C>& S) const { return reinterpret_cast<int*>(S.mem); }
+  template <int C>
+  NNS_DEV int* scan_first(CtaCore<C>& S) const { return reinterpret_cast<int*>(S.mem2); }
+  // The FP32 tiles over every active supplier for n consumers of a list.
+  template <int C>
+  NNS_DEV void scan_exact(CtaCore<C>& S, int mt, const int* list, int n) {
+    const int g = threadIdx.x / TG_THREADS, gt = threadIdx.x % TG_THREADS;
+    const int ngroups = kThreads / TG_THREADS;
+    for (int c0 = g * TG_M; c0 < n; c0 += ngroups * TG_M) {
+      unsigned long long out[4];
+      group_nns_tile<false>(x, S.iidx, 0, mt, y, S.jidx, list, c0, min(TG_M, n - c0), d, U.tiles[g], gt, 1 + g, out);
+      const int tx = gt & 15, ty = gt >> 4;
+      if (tx == 0)
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          const int lq = c0 + ty * 4 + i;
+          if (lq < n) S.nnk[list[lq]] = out[i];
+        }
+    }
+  }
+  template <int C>
+  NNS_DEV const unsigned long long* nns_lists(CtaCore<C>& S, int mt, int nt) {
+    const int tid = threadIdx.x;
+    map_positions(S, mt, tid, kThreads);
+    if (tid == 0) nfb = nscan = 0;
     __syncthreads();
+    int cert = 0;
+    for (int q = tid; q < nt; q += kThreads) {
+      unsigned long long key;
+      if (serve(S, mt, S.jidx[q], key)) {
+        S.nnk[q] = key;
+        ++cert;
+      } else {
+        fb[atomicAdd(&nfb, 1)] = q;
+      }
+    }
+    __syncwarp();
+    cert = __reduce_add_sync(0xffffffffu, cert);
+    if ((tid & 31) == 0 && cert) atomicAdd(&ncert, (unsigned long long)cert);
+    __syncthreads();
+    const int n = nfb;
+#pragma unroll 1
+    for (int k = 4 * (tid >> 5); k < n; k += 4 * (kThreads / 32))
+      make_lists(S, mt, min(4, n - k), [&](int h) { return fb[k + h]; });
+    __syncthreads();
+    const int ns = nscan;
+    if (ns > 0) {
+      scan_exact(S, mt, scan_list(S), ns);
+      __syncthreads();
+      for (int k = tid; k < ns; k += kThreads)
+        if (S.iidx[(int)(unsigned)S.nnk[scan_list(S)[k]]] != scan_first(S)[k]) atomicAdd(&nnear, 1ULL);
+      if (tid == 0) nfall += ns;
+      __syncthreads();
+    }
     return S.nnk;
   }
-
   template <int C>
   NNS_DEV const unsigned long long* nns(CtaCore<C>& S, int mt, int nt, long long = 0) {
-    if (kc_on && kc_ready) return nns_cached(S, mt, nt);
+    if (kc_on && kc_ready) return nns_lists(S, mt, nt);
     // with the cache on, this is the pair's first round: the tensor-core
     // pass fills the cache (every v' of the pair) instead of keeping top-K
     const bool fill = kc_on != 0;
     const int tid = threadIdx.x, T = blockDim.x;
     const int warp = tid >> 5, lane = tid & 31;
-    const int qtiles = (nt + TC_BM - 1) / TC_BM;
-    const int stiles = (mt + bn - 1) / bn;
+    // rows of the tiles: the active points, or, to fill the cache, every
+    // original point (the cache's rows and columns are original indices)
+    const int ms = fill ? kc_m : mt, ns = fill ? kc_n : nt;
+    const int qtiles = (ns + TC_BM - 1) / TC_BM;
+    const int stiles = (ms + bn - 1) / bn;
     const int nblk = kb / 16;
     // ---- 1. pack both sides
     if (tid == 0) {
       stat_rx = stat_rx1 = stat_sx = 0u;
       nfb = 0;
     }
-    if (fill) {
-      // no exact key of the pair is known yet
-      const long long total = (long long)kc_m * (long long)kc_n;
-      for (long long e = tid; e < total; e += T) scr.kcache[e] = CUDART_NAN_F;
-    }
+    if (fill)
+      for (int j = tid; j < kc_n; j += T) scr.lnext[j] = 0;  // no lists yet
     __syncthreads();
     {
       // one warp per row: the lanes take the row's coordinates and 16-byte
@@ -309,68 +500,81 @@ struct GeoTC {
       // squared norm within gamma_d |v|^2, the bound the certificate uses.
       const int srows = stiles * bn, qrows = qtiles * TC_BM;
       const int total = srows + qrows;
-      for (int row_id = warp; row_id < total; row_id += T / 32) {
-        const bool sup = row_id < srows;
-        const int p = sup ? row_id : row_id - srows;
-        const int cnt = sup ? mt : nt;
-        const float* row = p < cnt ? (sup ? x + (size_t)S.iidx[p] * d : y + (size_t)S.jidx[p] * d) : nullptr;
-        float mx = 0.f, a2f = 0.f, a1f = 0.f;
-        double a2 = 0.0, a1 = 0.0;
-        const bool want64 = row && !sup && fill;
-        if (row)
-          for (int k = lane; k < d; k += 32) {
-            const float v = row[k];
-            mx = fmaxf(mx, fabsf(v));
-            a2f = __fmaf_rn(v, v, a2f);
-            a1f = __fadd_rn(a1f, fabsf(v));
-            if (want64) {
-              a2 += (double)v * v;
-              a1 += fabs((double)v);
-            }
+      // two rows of a warp at once (their loads overlap)
+#pragma unroll 1
+      for (int row0 = 2 * warp; row0 < total; row0 += 2 * (T / 32)) {
+        const float* rows2[2];
+        float mx[2] = {0.f, 0.f}, a2f[2] = {0.f, 0.f}, a1f[2] = {0.f, 0.f};
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+          const int row_id = row0 + h;
+          const bool sup = row_id < srows;
+          const int p = sup ? row_id : row_id - srows;
+          rows2[h] = nullptr;
+          if (row_id < total && p < (sup ? ms : ns))
+            rows2[h] = (sup ? x : y) + (size_t)(fill ? p : (sup ? S.iidx[p] : S.jidx[p])) * d;
+        }
+        for (int k = lane; k < d; k += 32) {
+          float v[2];
+#pragma unroll
+          for (int h = 0; h < 2; ++h) v[h] = rows2[h] ? rows2[h][k] : 0.f;
+#pragma unroll
+          for (int h = 0; h < 2; ++h) {
+            mx[h] = fmaxf(mx[h], fabsf(v[h]));
+            a2f[h] = __fmaf_rn(v[h], v[h], a2f[h]);
+            a1f[h] = __fadd_rn(a1f[h], fabsf(v[h]));
+          }
+        }
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1)
+#pragma unroll
+          for (int h = 0; h < 2; ++h) {
+            mx[h] = fmaxf(mx[h], __shfl_xor_sync(0xffffffffu, mx[h], o));
+            a2f[h] = __fadd_rn(a2f[h], __shfl_xor_sync(0xffffffffu, a2f[h], o));
+            a1f[h] = __fadd_rn(a1f[h], __shfl_xor_sync(0xffffffffu, a1f[h], o));
           }
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-          mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-          a2f = __fadd_rn(a2f, __shfl_xor_sync(0xffffffffu, a2f, o));
-          a1f = __fadd_rn(a1f, __shfl_xor_sync(0xffffffffu, a1f, o));
-          if (want64) {
-            a2 += __shfl_xor_sync(0xffffffffu, a2, o);
-            a1 += __shfl_xor_sync(0xffffffffu, a1, o);
+        for (int h = 0; h < 2; ++h) {
+          const int row_id = row0 + h;
+          if (row_id >= total) break;
+          const bool sup = row_id < srows;
+          const int p = sup ? row_id : row_id - srows;
+          const float* row = rows2[h];
+          float s = 1.f;  // the row scale of FP16 / FP8 (as row_scale), from the warp's maximum
+          if (row && !fmt_is_bf16(fmt) && mx[h] > 0.f) {
+            int e;
+            frexpf(mx[h], &e);
+            s = ldexpf(1.f, e - 8);
           }
-        }
-        float s = 1.f;  // the row scale of FP16 / FP8 (as row_scale), from the warp's maximum
-        if (row && !fmt_is_bf16(fmt) && mx > 0.f) {
-          int e;
-          frexpf(mx, &e);
-          s = ldexpf(1.f, e - 8);
-        }
-        const int rows = sup ? bn : TC_BM;
-        uint8_t* tile = (sup ? scr.B : scr.A) + (size_t)(p / rows) * rows * kb;
-        for (int c = lane; c < nblk; c += 32) pack_block(row, d, c, s, fmt, tile, rows, p % rows, sup);
-        if (lane == 0) {
-          float* nrm = sup ? scr.nrm_x : scr.nrm_y;
-          float* scl = sup ? scr.scale_x : scr.scale_y;
-          if (row) {
-            const float l2sq = a2f, l1 = a1f;
-            nrm[p] = l2sq;
-            scl[p] = s;
-            if (sup) {
-              scr.nrm_sx[p] = norm_up(l2sq);
-              atomicMax(&stat_rx, __float_as_uint(norm_up(l2sq)));
-              atomicMax(&stat_rx1, __float_as_uint(l1 * (1.f + 1e-4f)));
-              atomicMax(&stat_sx, __float_as_uint(s));
-            } else if (fill) {
-              // what the certificate needs of this consumer in every round
-              const int j = S.jidx[p];
-              scr.ny_o[j] = l2sq;
-              scr.sy_o[j] = s;
-              scr.yl2_o[j] = sqrt(a2) * (1 + 1e-12);
-              scr.yl1_o[j] = a1;
+          const int rows = sup ? bn : TC_BM;
+          uint8_t* tile = (sup ? scr.B : scr.A) + (size_t)(p / rows) * rows * kb;
+          for (int c = lane; c < nblk; c += 32) pack_block(row, d, c, s, fmt, tile, rows, p % rows, sup);
+          if (lane == 0) {
+            float* nrm = sup ? scr.nrm_x : scr.nrm_y;
+            float* scl = sup ? scr.scale_x : scr.scale_y;
+            if (row) {
+              const float l2sq = a2f[h], l1 = a1f[h];
+              nrm[p] = l2sq;
+              scl[p] = s;
+              if (sup) {
+                scr.nrm_sx[p] = norm_up(l2sq);
+                atomicMax(&stat_rx, __float_as_uint(norm_up(l2sq)));
+                atomicMax(&stat_rx1, __float_as_uint(l1 * (1.f + 1e-4f)));
+                atomicMax(&stat_sx, __float_as_uint(s));
+              } else if (fill) {
+                // what the certificate needs of this consumer in every round
+                // (the norms rounded up: the FP64 sums of the other pass take
+                // 256 FP64 operations a row of 128, here half of the packing)
+                scr.ny_o[p] = l2sq;
+                scr.sy_o[p] = s;
+                scr.yl2_o[p] = norm_up(l2sq);
+                scr.yl1_o[p] = l1 * (1.f + 1e-4f);
+              }
+            } else {
+              nrm[p] = CUDART_INF_F;
+              scl[p] = 1.f;
+              if (sup) scr.nrm_sx[p] = 0.f;
             }
-          } else {
-            nrm[p] = CUDART_INF_F;
-            scl[p] = 1.f;
-            if (sup) scr.nrm_sx[p] = 0.f;
           }
         }
       }
@@ -411,9 +615,10 @@ struct GeoTC {
           if (!ok) break;
           for (int st = 0; st < stiles && ok; ++st) {
             const unsigned s = mma_b % nstage, u = mma_b / nstage;
-            const unsigned b = mma_acc & 1, v = mma_acc >> 1;
+            unsigned& na = fill ? mma_accf : mma_acc;
+            const unsigned b = na & 1, v = na >> 1;
             ok = mbar_wait_bounded(&bar_full[s], u & 1);
-            if (ok) ok = mbar_wait_bounded(&bar_acc_empty[b], (v & 1) ^ 1);
+            if (ok) ok = mbar_wait_bounded(fill ? &bar_accf_empty[b] : &bar_acc_empty[b], (v & 1) ^ 1);
             if (!ok) break;
             tc_fence_after();
             const uint32_t b0 = smem_u32(sB + (size_t)s * b_bytes);
@@ -424,12 +629,66 @@ struct GeoTC {
               mma_issue<KIND8 ? FMT_E4M3 : FMT_BF16>(tmem_d, ad, bd, idesc, k > 0 ? 1u : 0u);
             }
             mma_commit(&bar_empty[s]);
-            mma_commit(&bar_acc_full[b]);
+            mma_commit(fill ? &bar_accf_full[b] : &bar_acc_full[b]);
             ++mma_b;
-            ++mma_acc;
+            ++na;
           }
           mma_commit(&bar_a_empty);  // A may be overwritten once these MMAs are done
           ++mma_a;
+        }
+      }
+    } else if (fill) {
+      // Cache fill: four warps per TMEM lane quarter, each a share of the
+      // tile's columns; a thread holds one consumer's 16 columns and writes
+      // them as four 16-byte stores, contiguous over the warp, and their
+      // minimum.  (Four warps, each value stored by itself: 39,000 cycles a
+      // tile of 128 x 128.)
+      if (warp >= 4 && warp < 4 + BTC_FILL_WARPS) {
+        const int quarter = warp & 3, part = (warp - 4) >> 2;
+        const int row = quarter * 32 + lane;
+        unsigned ea = epi_accf;
+        for (int qt = 0; qt < qtiles; ++qt) {
+          const int q = qt * TC_BM + row;
+          const float sy = q < ns ? scr.scale_y[q] : 1.f;
+          const float cy = quant_coeff(fmt, q < ns ? scr.nrm_y[q] : 0.f);
+          float4* vrow = reinterpret_cast<float4*>(scr.vcache + v_at(q, 0));  // column group c at vrow[32 c]
+          float* mrow = scr.vmin + (size_t)(q >> 5) * ((kc_ld + 15) >> 4) * 32 + (q & 31);
+          const bool live = (q & ~31) < ns;  // (a warp's 32 rows are written whole)
+          for (int st = 0; st < stiles; ++st, ++ea) {
+            const unsigned b = ea & 1, v = ea >> 1;
+            if (ok) ok = mbar_wait_bounded(&bar_accf_full[b], v & 1);
+            ok = __all_sync(0xffffffffu, ok);  // warp-uniform: the loads below are warp-wide
+            tc_fence_after();
+            if (ok)
+              for (int c0 = 16 * part; c0 < bn; c0 += 64) {
+                uint32_t r[16];
+                tmem_ld16(tmem_base + ((uint32_t)(quarter * 32) << 16) + b * (uint32_t)bn + (uint32_t)c0, r);
+                const size_t at = (size_t)st * bn + c0;
+                float mn = CUDART_INF_F;
+#pragma unroll
+                for (int e = 0; e < 16; e += 4) {
+                  const float4 nx = *reinterpret_cast<const float4*>(scr.nrm_x + at + e);
+                  const float4 nsx = *reinterpret_cast<const float4*>(scr.nrm_sx + at + e);
+                  float4 w = make_float4(-2.f, -2.f, -2.f, -2.f);
+                  if (!fmt_is_bf16(fmt)) {
+                    const float4 sx = *reinterpret_cast<const float4*>(scr.scale_x + at + e);
+                    w = make_float4(-2.f * sy * sx.x, -2.f * sy * sx.y, -2.f * sy * sx.z, -2.f * sy * sx.w);
+                  }
+                  float4 o;
+                  o.x = __fmaf_rn(-cy, nsx.x, __fmaf_rn(w.x, __uint_as_float(r[e]), nx.x));
+                  o.y = __fmaf_rn(-cy, nsx.y, __fmaf_rn(w.y, __uint_as_float(r[e + 1]), nx.y));
+                  o.z = __fmaf_rn(-cy, nsx.z, __fmaf_rn(w.z, __uint_as_float(r[e + 2]), nx.z));
+                  o.w = __fmaf_rn(-cy, nsx.w, __fmaf_rn(w.w, __uint_as_float(r[e + 3]), nx.w));
+                  // (kc_ld is a multiple of 4: the last vector of a row stays inside it)
+                  if (live && (int)at + e < kc_ld) vrow[(at + e) * 8] = o;
+                  mn = fminf(fminf(mn, o.x), fminf(fminf(o.y, o.z), o.w));
+                }
+                if (live && (int)at < kc_ld) mrow[(at >> 4) * 32] = mn;
+              }
+            tc_fence_before();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&bar_accf_empty[b]);
+          }
         }
       }
     } else if (warp < 6) {
@@ -447,60 +706,27 @@ struct GeoTC {
         for (int st = 0; st < stiles; ++st, ++ea) {
           const unsigned b = ea & 1, v = ea >> 1;
           if (ok) ok = mbar_wait_bounded(&bar_acc_full[b], v & 1);
-          ok = __all_sync(0xffffffffu, ok);  // warp-uniform: the fill below synchronises the warp
+          ok = __all_sync(0xffffffffu, ok);  // warp-uniform: the loads below are warp-wide
           tc_fence_after();
           if (ok) {
             const float* nx = scr.nrm_x + (size_t)st * bn;
-            const float* ns = scr.nrm_sx + (size_t)st * bn;
+            const float* nsx = scr.nrm_sx + (size_t)st * bn;
             const float* sx = scr.scale_x + (size_t)st * bn;
-            // fill: this consumer's row of the cache, by original supplier index
-            float* vrow = (fill && q < nt) ? scr.vcache + (size_t)S.jidx[q] * kc_m : nullptr;
             for (int c0 = 0; c0 < bn; c0 += 16) {
               uint32_t r[16];
               tmem_ld16(tmem_base + ((uint32_t)(quarter * 32) << 16) + b * (uint32_t)bn + (uint32_t)c0, r);
-              float val[16];
 #pragma unroll
               for (int e = 0; e < 16; ++e) {
-                const float acc = __uint_as_float(r[e]);
                 const float w = fmt_is_bf16(fmt) ? -2.f : -2.f * sy * sx[c0 + e];
-                val[e] = __fmaf_rn(-cy, ns[c0 + e], __fmaf_rn(w, acc, nx[c0 + e]));
-              }
-              if (!fill) {
-#pragma unroll
-                for (int e = 0; e < 16; ++e) topk_insert(tv, tp, val[e], st * bn + c0 + e);
-              } else if constexpr (CAP >= 2048) {
-                // transpose the warp's 32 rows x 16 columns through the
-                // fallback list's buffer (unused while the cache fills), so
-                // that each store instruction writes 16 consecutive columns of
-                // two rows instead of one column of 32 rows (XOR-swizzled:
-                // no bank conflicts either way)
-                float* tb = reinterpret_cast<float*>(fb) + (warp - 2) * 512;
-#pragma unroll
-                for (int e = 0; e < 16; ++e) tb[e * 32 + (lane ^ e)] = val[e];
-                __syncwarp();
-                const int e = lane & 15;
-                const int col = st * bn + c0 + e;
-                const int icol = col < mt ? S.iidx[col] : 0;
-#pragma unroll 4
-                for (int it = 0; it < 16; ++it) {
-                  const int rr = 2 * it + (lane >> 4);
-                  const int qq = qt * TC_BM + quarter * 32 + rr;
-                  if (qq < nt && col < mt) scr.vcache[(size_t)S.jidx[qq] * kc_m + icol] = tb[e * 32 + (rr ^ e)];
-                }
-                __syncwarp();
-              } else {
-#pragma unroll
-                for (int e = 0; e < 16; ++e) {
-                  const int col = st * bn + c0 + e;
-                  if (vrow && col < mt) vrow[S.iidx[col]] = val[e];
-                }
+                const float val = __fmaf_rn(-cy, nsx[c0 + e], __fmaf_rn(w, __uint_as_float(r[e]), nx[c0 + e]));
+                topk_insert(tv, tp, val, st * bn + c0 + e);
               }
             }
           }
           tc_fence_before();
           mbar_arrive(&bar_acc_empty[b]);
         }
-        if (q < nt && !fill) {
+        if (q < nt) {
 #pragma unroll
           for (int k = 0; k < BTC_K; ++k) {
             scr.cand_v[(size_t)q * BTC_K + k] = tv[k];
@@ -513,15 +739,14 @@ struct GeoTC {
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
-    if (tid == 64) epi_acc += (unsigned)(qtiles * stiles);
+    if (tid == 64) (fill ? epi_accf : epi_acc) += (unsigned)(qtiles * stiles);
     if (fill) {
       // the cache holds every v' of the pair; this and every later round
       // are answered from it.  The certificate's E of every consumer, once:
       // the supplier maxima of this first round bound every later round's.
       const double rx = __uint_as_float(stat_rx), rx1 = __uint_as_float(stat_rx1);
       const double sxm = __uint_as_float(stat_sx);
-      for (int q = tid; q < nt; q += T) {
-        const int j = S.jidx[q];
+      for (int j = tid; j < ns; j += T) {
         scr.e_o[j] = certify_E(fmt, d, scr.ny_o[j], scr.yl2_o[j], scr.yl1_o[j], scr.sy_o[j], rx, rx1, sxm);
       }
       if (tid == 0) {
@@ -529,7 +754,7 @@ struct GeoTC {
         kc_ready = 1;
       }
       __syncthreads();
-      return nns_cached(S, mt, nt);
+      return nns_lists(S, mt, nt);
     }
     // ---- 3. exact re-rank + certificate (a warp per consumer)
     const double rx = __uint_as_float(stat_rx), rx1 = __uint_as_float(stat_rx1), sxm = __uint_as_float(stat_sx);
@@ -570,23 +795,7 @@ struct GeoTC {
     }
     __syncthreads();
     // ---- 4. FP32 rescan of the consumers that were not certified
-    const int nf = nfb;
-    if (nf > 0) {
-      const int g = tid / TG_THREADS, gt = tid % TG_THREADS;
-      const int ngroups = T / TG_THREADS;
-      for (int c0 = g * TG_M; c0 < nf; c0 += ngroups * TG_M) {
-        unsigned long long out[4];
-        group_nns_tile<false>(x, S.iidx, 0, mt, y, S.jidx, fb, c0, min(TG_M, nf - c0), d, U.tiles[g], gt, 1 + g,
-                              out);
-        const int tx = gt & 15, ty = gt >> 4;
-        if (tx == 0)
-#pragma unroll
-          for (int i = 0; i < 4; ++i) {
-            const int lq = c0 + ty * 4 + i;
-            if (lq < nf) S.nnk[fb[lq]] = out[i];
-          }
-      }
-    }
+    if (nfb > 0) scan_exact(S, mt, fb, nfb);
     __syncthreads();
     return S.nnk;
   }
@@ -624,11 +833,13 @@ __global__ void __launch_bounds__(FIN_THREADS, 1) k_batched_tc(BtcArgs A) {
     for (int b = 0; b < 2; ++b) {
       mbar_init(&G.bar_acc_full[b], 1);
       mbar_init(&G.bar_acc_empty[b], 4 * 32);
+      mbar_init(&G.bar_accf_full[b], 1);
+      mbar_init(&G.bar_accf_empty[b], BTC_FILL_WARPS);
     }
     mbar_init(&G.bar_a_full, 1);
     mbar_init(&G.bar_a_empty, 1);
     mbar_fence_init();
-    G.prod_a = G.prod_b = G.mma_a = G.mma_b = G.mma_acc = G.epi_acc = 0u;
+    G.prod_a = G.prod_b = G.mma_a = G.mma_b = G.mma_acc = G.epi_acc = G.mma_accf = G.epi_accf = 0u;
     G.ncert = G.nfall = G.nnear = 0ULL;
     G.rk = A.rk;
     G.kb = A.kb;
@@ -658,7 +869,8 @@ __global__ void __launch_bounds__(FIN_THREADS, 1) k_batched_tc(BtcArgs A) {
       G.x = B.x + xo * B.d;
       G.y = B.y + yo * B.d;
       G.d = B.d;
-      G.kc_on = (long long)m * n <= A.kc_cap ? 1 : 0;
+      G.kc_ld = m < 16 ? 16 : (int)kmat_ld(m);
+      G.kc_on = btc_cache_values(m, n) <= A.kc_cap ? 1 : 0;
       G.kc_ready = 0;
       G.kc_m = m;
       G.kc_n = n;
@@ -703,8 +915,10 @@ static int batched_tc_t(const BtcArgs& A, int grid, cudaStream_t st) {
 int batched_tc_max_stages(int cap, int kb, int bn, int precision) {
   for (int ns = 4; ns >= 1; --ns) {
     size_t b;
-    if (precision == 3) b = cap <= 512 ? btc_smem_bytes<true, 512>(kb, bn, ns) : btc_smem_bytes<true, 2048>(kb, bn, ns);
-    else b = cap <= 512 ? btc_smem_bytes<false, 512>(kb, bn, ns) : btc_smem_bytes<false, 2048>(kb, bn, ns);
+    if (precision == 3)
+      b = cap <= HD_SMALL_CAP ? btc_smem_bytes<true, HD_SMALL_CAP>(kb, bn, ns) : btc_smem_bytes<true, FIN_MAX_HD>(kb, bn, ns);
+    else
+      b = cap <= HD_SMALL_CAP ? btc_smem_bytes<false, HD_SMALL_CAP>(kb, bn, ns) : btc_smem_bytes<false, FIN_MAX_HD>(kb, bn, ns);
     if (b <= 227 * 1024) return ns;
   }
   return 0;
@@ -716,9 +930,8 @@ int launch_batched_tc(const BatchArgs& base, int precision, int cap, int kb, int
   const int rk = rerank_k >= 1 && rerank_k <= BTC_K ? rerank_k : BTC_K;
   BtcArgs A{base, scratch, slot_bytes, kb, bn, nstage, fmt_of_precision(precision), certified, fallbacks,
             near_ties, rk, kc_cap};
-  const bool k8 = precision == 3;
-  if (cap <= 512) return k8 ? batched_tc_t<true, 512>(A, grid, st) : batched_tc_t<false, 512>(A, grid, st);
-  return k8 ? batched_tc_t<true, 2048>(A, grid, st) : batched_tc_t<false, 2048>(A, grid, st);
+  if (cap != FIN_MAX_HD) return -2;
+  return precision == 3 ? batched_tc_t<true, FIN_MAX_HD>(A, grid, st) : batched_tc_t<false, FIN_MAX_HD>(A, grid, st);
 }
 
 }  // namespace nnsemd

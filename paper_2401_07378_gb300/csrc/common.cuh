@@ -80,19 +80,11 @@ NNS_DEV float key32(const float* x, const float* y, int d) {
 NNS_DEV float key32_sql2_v4(const float* __restrict__ x, const float* y, int d) {
   const float4* x4 = reinterpret_cast<const float4*>(x);
   const float4* y4 = reinterpret_cast<const float4*>(y);
-  float4 a = __ldg(x4), b = y4[0];
-  float t = __fsub_rn(a.x, b.x);
-  float acc = __fmul_rn(t, t);
-  t = __fsub_rn(a.y, b.y);
-  acc = __fmaf_rn(t, t, acc);
-  t = __fsub_rn(a.z, b.z);
-  acc = __fmaf_rn(t, t, acc);
-  t = __fsub_rn(a.w, b.w);
-  acc = __fmaf_rn(t, t, acc);
-  for (int i = 1; i < (d >> 2); ++i) {
-    a = __ldg(x4 + i);
-    b = y4[i];
-    t = __fsub_rn(a.x, b.x);
+  float acc = 0.f;  // (fma from +0 rounds t_0 * t_0 alone)
+#pragma unroll 4
+  for (int i = 0; i < (d >> 2); ++i) {
+    const float4 a = __ldg(x4 + i), b = y4[i];
+    float t = __fsub_rn(a.x, b.x);
     acc = __fmaf_rn(t, t, acc);
     t = __fsub_rn(a.y, b.y);
     acc = __fmaf_rn(t, t, acc);
@@ -140,6 +132,27 @@ NNS_DEV unsigned rp_key32(unsigned long long seed, long long t, int j) {
   z = (z ^ (z >> 27)) * 0x94D049BB133111EBULL;
   z ^= z >> 31;
   return (unsigned)(z >> 32);
+}
+
+// Warp-wide ascending sort of one 64-bit key per lane (bitonic network in
+// which every comparator puts the smaller key on the lower lane).
+NNS_DEV unsigned long long warp_sort_u64(unsigned long long key) {
+  const int lane = threadIdx.x & 31;
+#pragma unroll
+  for (int k = 2; k <= 32; k <<= 1) {
+    {
+      const int partner = lane ^ (k - 1);
+      const unsigned long long o = __shfl_sync(0xffffffffu, key, partner);
+      key = lane < partner ? (o < key ? o : key) : (o > key ? o : key);
+    }
+#pragma unroll
+    for (int j = k >> 2; j > 0; j >>= 1) {
+      const int partner = lane ^ j;
+      const unsigned long long o = __shfl_sync(0xffffffffu, key, partner);
+      key = lane < partner ? (o < key ? o : key) : (o > key ? o : key);
+    }
+  }
+  return key;
 }
 
 // One step of the greedy protocol (Alg. 1): f = min(s, c); s -= f; c -= f.

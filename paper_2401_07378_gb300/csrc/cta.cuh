@@ -71,14 +71,20 @@ struct CtaCore {
   unsigned long long mem2[CAP];
   int cnt[CAP + 1];
   int off[CAP + 1];
-  unsigned long long acc[2][XS_LIMBS];  // exact sums (acc[0]: R; both: the sides' totals)
+  unsigned long long acc[XS_LIMBS];
   int wt[33];
   int mt, nt;
   unsigned nflow;
-  double total[2];
-  // running totals handed back by the one-warp rounds (warp_rounds)
-  unsigned long long w_nnz;
-  long long w_rounds, w_pe;
+  union {
+    double total[2];  // the sides' weight totals (while a pair loads)
+    struct {          // running totals handed back by the one-warp rounds (warp_rounds)
+      unsigned long long w_nnz;
+      long long w_rounds, w_pe;
+    };
+  };
+  // a second exact sum beside acc, while no round runs
+  static_assert(CAP >= XS_LIMBS, "the second accumulator lies in mem2");
+  NNS_DEV unsigned long long* acc2() { return mem2; }
 };
 
 struct CtaOut {
@@ -507,6 +513,7 @@ struct GeoGlobal {
   // 11.7 -> 3.09 ms).
   float* kmat;
   int kld, km, kn, kready;
+  unsigned long long searches;  // consumer searches of all rounds so far
   TileSmem tiles[NT / TG_THREADS];
   struct PX {};
   NNS_DEV void load_x(int, PX&) const {}
@@ -528,6 +535,7 @@ struct GeoGlobal {
     kn = n;
     kmat = km_ && (long long)m * kld <= kcap ? km_ : nullptr;
     kready = 0;
+    searches = 0;
   }
   // The whole key matrix, one 64 x 64 tile per group at a time.
   NNS_DEV void fill() {
@@ -591,8 +599,9 @@ struct GeoGlobal {
   static constexpr bool kWarpRounds = true;
   NNS_DEV bool warp_ready() const { return kmat != nullptr && kready; }
   template <int C>
-  NNS_DEV void warp_nns(CtaCore<C>& S, int mt, int nt) const {
+  NNS_DEV void warp_nns(CtaCore<C>& S, int mt, int nt) {
     const int qa = threadIdx.x & 31, qb = qa + 32;
+    if (threadIdx.x == 0) searches += nt;
     const float* ca = kmat + S.jidx[qa < nt ? qa : 0];
     const float* cb = kmat + S.jidx[qb < nt ? qb : 0];
     unsigned ba = 0xffffffffu, bb = 0xffffffffu;
@@ -616,6 +625,7 @@ struct GeoGlobal {
   }
   template <int C>
   NNS_DEV const unsigned long long* nns(CtaCore<C>& S, int mt, int nt, long long = 0) {
+    if (threadIdx.x == 0) searches += nt;
     if (kmat) {
       if (!kready) {
         fill();
@@ -1103,12 +1113,12 @@ NNS_DEV void cta_rounds(CtaCore<CAP>& S, Geo& G, int metric, const CtaOut& O, un
 // them, and normalise each side's weights by their correctly rounded total.
 // With DP > 0 the coordinates are copied (zero-padded to DP) into xs / ys.
 // The sides go through every step together (one after the other they took
-// twice the latency: 7 us of a 256-point solve).  Clears acc[0].
+// twice the latency: 7 us of a 256-point solve).  Clears acc.
 template <int DP, int CAP>
 NNS_DEV bool cta_load_sides(const float* x, const double* a, int m, const float* y, const double* b, int n, int d,
                             float* xs, float* ys, CtaCore<CAP>& S, unsigned* err) {
   const int tid = threadIdx.x;
-  for (int i = tid; i < 2 * XS_LIMBS; i += blockDim.x) (&S.acc[0][0])[i] = 0ULL;
+  for (int i = tid; i < XS_LIMBS; i += blockDim.x) S.acc[i] = S.acc2()[i] = 0ULL;
   __syncthreads();
   unsigned bad = 0;  // bits 0, 1: a value of x / y not finite; bits 2, 3: a weight of a / b negative
 #pragma unroll 1
@@ -1135,16 +1145,33 @@ NNS_DEV bool cta_load_sides(const float* x, const double* a, int m, const float*
         add[sd] = isfinite(wv) && wv > 0.0 ? wv : 0.0;
       }
     }
-    xs_add_warp(S.acc[0], add[0]);
-    xs_add_warp(S.acc[1], add[1]);
+    xs_add_warp(S.acc, add[0]);
+    xs_add_warp(S.acc2(), add[1]);
   }
   if (DP == 0) {
     // rows checked by the whole CTA, consecutive lanes on consecutive values
 #pragma unroll 1
     for (int sd = 0; sd < 2; ++sd) {
       const float* pts = sd ? y : x;
-      const int64_t cnt = (int64_t)(sd ? n : m) * d;
-      for (int64_t i = tid; i < cnt; i += blockDim.x)
+      const int cnt = (sd ? n : m) * d;  // (at most 2,048 rows of 65,536)
+      int i0 = 0;
+      if ((reinterpret_cast<uintptr_t>(pts) & 15) == 0) {
+        // 16 bytes a load, four in flight
+        const float4* p4 = reinterpret_cast<const float4*>(pts);
+        const int c4 = cnt >> 2;
+        bool nf = false;
+        for (int i = tid; i < c4; i += 4 * blockDim.x) {
+          float4 v[4];
+#pragma unroll
+          for (int u = 0; u < 4; ++u) v[u] = p4[min(i + u * (int)blockDim.x, c4 - 1)];
+#pragma unroll
+          for (int u = 0; u < 4; ++u)
+            nf |= !(isfinite(v[u].x) && isfinite(v[u].y) && isfinite(v[u].z) && isfinite(v[u].w));
+        }
+        if (nf) bad |= 1u << sd;
+        i0 = c4 << 2;
+      }
+      for (int i = i0 + tid; i < cnt; i += blockDim.x)
         if (!isfinite(pts[i])) bad |= 1u << sd;
     }
   }
@@ -1152,7 +1179,7 @@ NNS_DEV bool cta_load_sides(const float* x, const double* a, int m, const float*
 #pragma unroll
   for (int k = 0; k < 4; ++k) all |= __syncthreads_or((bad >> k) & 1u) ? 1u << k : 0u;
   if (tid < 64) {
-    const double t = xs_round_warp(S.acc[tid >> 5]);
+    const double t = xs_round_warp(tid < 32 ? S.acc : S.acc2());
     if ((tid & 31) == 0) S.total[tid >> 5] = t;
   }
   __syncthreads();
@@ -1167,7 +1194,7 @@ NNS_DEV bool cta_load_sides(const float* x, const double* a, int m, const float*
   }
   for (int p = tid; p < m; p += blockDim.x) S.sres[p] = __ddiv_rn(S.sres[p], ta);
   for (int p = tid; p < n; p += blockDim.x) S.cres[p] = __ddiv_rn(S.cres[p], tb);
-  for (int i = tid; i < XS_LIMBS; i += blockDim.x) S.acc[0][i] = 0ULL;
+  for (int i = tid; i < XS_LIMBS; i += blockDim.x) S.acc[i] = 0ULL;
   __syncthreads();
   return true;
 }
@@ -1194,7 +1221,7 @@ NNS_DEV bool cta_solve_pair(CtaCore<CAP>& S, Geo& G, float* xs, float* ys, const
   }
   __syncthreads();
   cta_compact(S, G);  // drop zero weights
-  CtaOut O{S.acc[0], nullptr, nullptr, nullptr, 0, nullptr, nullptr, err};
+  CtaOut O{S.acc, nullptr, nullptr, nullptr, 0, nullptr, nullptr, err};
   O.protocol = protocol;
   O.seed = seed;
   if (fl_i) {
@@ -1214,7 +1241,7 @@ NNS_DEV bool cta_solve_pair(CtaCore<CAP>& S, Geo& G, float* xs, float* ys, const
   pe = 0;
   cta_rounds(S, G, metric, O, nnz, rounds, pe, (long long)m + n);
   __syncthreads();
-  if (threadIdx.x < 32) cost = xs_round_warp(S.acc[0]);  // (thread 0 has it)
+  if (threadIdx.x < 32) cost = xs_round_warp(S.acc);  // (thread 0 has it)
   return true;
 }
 

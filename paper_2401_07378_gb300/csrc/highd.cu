@@ -155,6 +155,7 @@ __global__ void __launch_bounds__(FIN_THREADS, 1) k_batched_hd(BatchArgs A) {
       A.costs[pr] = ok ? cost : CUDART_NAN;
       if (A.rounds) A.rounds[pr] = rounds;
       if (A.pair_evals) A.pair_evals[pr] = pe;
+      if (A.searches) atomicAdd(A.searches, H.G.searches);
     }
     __syncthreads();
   }
@@ -216,6 +217,7 @@ __global__ void __launch_bounds__(HD_SMALL_THREADS, 4) k_batched_hd_small(BatchA
       A.costs[pr] = ok ? cost : CUDART_NAN;
       if (A.rounds) A.rounds[pr] = rounds;
       if (A.pair_evals) A.pair_evals[pr] = pe;
+      if (A.searches) atomicAdd(A.searches, H.G.searches);
     }
     __syncthreads();
   }

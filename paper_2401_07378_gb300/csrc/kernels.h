@@ -149,6 +149,7 @@ struct BatchArgs {
   // 4, used by the pairs whose matrix (m rows of kmat_ld(n) floats) fits
   float* kmat;
   long long kcap;
+  unsigned long long* searches;  // nullable: the consumer searches of all rounds are added here (d > 8, FP32)
 };
 int launch_batched_lowd(const BatchArgs& A, int grid, cudaStream_t st);
 // The same two for pairs of at most LOWD_SMALL_CAP points per side
@@ -222,10 +223,13 @@ int cell_bounds_tc(const float* y, int rows, int d, uint8_t* packed_y, float* y_
 int launch_nns_tc(const SolveBufs& B, const TcBufs& T, int mt, int nt, int precision, cudaStream_t st,
                   const int* sel = nullptr, const int* nsel_dev = nullptr);
 
-// batched_tc.cu: batches of pairs with up to `cap` (512 or 2048) points per
-// side, reduced-precision NNS inside each pair's CTA.
-// kc_cap: entries of each CTA's distance cache (pairs with m * n <= kc_cap
-// are answered from it after their first round; 0 turns it off).
+// batched_tc.cu: batches of pairs with up to `cap` points per side (FIN_MAX_HD;
+// batched_tc_max_stages also answers for HD_SMALL_CAP, 0: rows too long),
+// reduced-precision NNS inside each pair's CTA.
+// kc_cap: values of each CTA's distance cache (pairs whose
+// batched_tc_cache_values fit are answered from it after their first round; 0
+// turns it off).
+long long batched_tc_cache_values(long long m, long long n);
 size_t batched_tc_slot_bytes(int cap, int kb, int bn, long long kc_cap);
 int batched_tc_max_stages(int cap, int kb, int bn, int precision);
 // rerank_k: candidates re-ranked per consumer (1..8; other values: 8);

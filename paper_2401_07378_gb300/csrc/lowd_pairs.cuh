@@ -32,25 +32,25 @@ __global__ void __launch_bounds__(NT, 1) k_solve_small(SolveBufs B, const double
   }
   __syncthreads();
   cta_compact(S, L.G);  // drop zero weights
-  CtaOut O{S.acc[0], B.plan_i, B.plan_j, B.plan_f, (long long)B.plan_cap, nullptr, nullptr, &B.st->err,
+  CtaOut O{S.acc, B.plan_i, B.plan_j, B.plan_f, (long long)B.plan_cap, nullptr, nullptr, &B.st->err,
            B.fl_i, B.fl_j, B.fl_f, B.x, B.y, B.d, B.protocol, B.seed, 0};
   unsigned long long nnz = 0;
   long long rounds = 0, pe = 0;
   cta_rounds(S, L.G, B.metric, O, nnz, rounds, pe, (long long)m + n);
   __syncthreads();
   // the leftover mass; then warp 0 rounds it and warp 1 rounds R
-  for (int i = tid; i < XS_LIMBS; i += blockDim.x) S.acc[1][i] = 0ULL;
+  for (int i = tid; i < XS_LIMBS; i += blockDim.x) S.acc2()[i] = 0ULL;
   __syncthreads();
   for (int base = 0; base < S.mt; base += blockDim.x)  // whole warps (xs_add_warp)
-    xs_add_warp(S.acc[1], base + tid < S.mt ? S.sres[base + tid] : 0.0);
+    xs_add_warp(S.acc2(), base + tid < S.mt ? S.sres[base + tid] : 0.0);
   for (int base = 0; base < S.nt; base += blockDim.x)
-    xs_add_warp(S.acc[1], base + tid < S.nt ? S.cres[base + tid] : 0.0);
+    xs_add_warp(S.acc2(), base + tid < S.nt ? S.cres[base + tid] : 0.0);
   __syncthreads();
   if (tid >= 32 && tid < 64) {
-    const double c = xs_round_warp(S.acc[0]);
+    const double c = xs_round_warp(S.acc);
     if (tid == 32) B.st->cost = c;
   }
-  const double left = tid < 32 ? xs_round_warp(S.acc[1]) : 0.0;
+  const double left = tid < 32 ? xs_round_warp(S.acc2()) : 0.0;
   if (tid == 0) {
     B.st->leftover = left;
     B.st->nnz = nnz;

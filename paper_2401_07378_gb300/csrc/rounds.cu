@@ -549,27 +549,6 @@ struct FlowArgs {
   DevState* st;
 };
 
-// Warp-wide ascending sort of one 64-bit key per lane (bitonic network in
-// which every comparator puts the smaller key on the lower lane).
-NNS_DEV unsigned long long warp_sort_u64(unsigned long long key) {
-  const int lane = threadIdx.x & 31;
-#pragma unroll
-  for (int k = 2; k <= 32; k <<= 1) {
-    {
-      const int partner = lane ^ (k - 1);
-      const unsigned long long o = __shfl_sync(0xffffffffu, key, partner);
-      key = lane < partner ? (o < key ? o : key) : (o > key ? o : key);
-    }
-#pragma unroll
-    for (int j = k >> 2; j > 0; j >>= 1) {
-      const int partner = lane ^ j;
-      const unsigned long long o = __shfl_sync(0xffffffffu, key, partner);
-      key = lane < partner ? (o < key ? o : key) : (o > key ? o : key);
-    }
-  }
-  return key;
-}
-
 // Serve up to 32 sorted members (one per lane, `cnt` valid) from supplier i
 // whose residual is `s` (uniform).  Returns how many were served.
 NNS_DEV int warp_serve(const FlowArgs& A, int i, double& s, unsigned long long key, int cnt) {

@@ -74,11 +74,17 @@ NNS_DEV float bf16x3_part(const float* row, int d, int k, bool supplier) {
   return low ? v - h : h;
 }
 
+// v / s for a power of two s with inverse inv (0 where the inverse is not a
+// normal number): the same value by a multiplication.
+NNS_DEV float unscale(float v, float s, float inv) { return inv != 0.f ? __fmul_rn(v, inv) : __fdiv_rn(v, s); }
+NNS_DEV float scale_inverse(float s) { return s >= 0x1p-126f && s <= 0x1p126f ? __fdiv_rn(1.f, s) : 0.f; }
+
 // Pack 16 bytes (block c) of one row into out (row r of tile t).  row == null
 // writes zeros (padding).  `supplier` picks the BF16X3 segment order.
 NNS_DEV void pack_block(const float* row, int d, int c, float s, int fmt, uint8_t* tile_base, int tile_rows, int r,
                         bool supplier = false) {
   alignas(16) uint8_t bytes[16];
+  const float inv = fmt_is_bf16(fmt) ? 1.f : scale_inverse(s);
   if (fmt == FMT_BF16X3) {
 #pragma unroll
     for (int e = 0; e < 8; ++e) {
@@ -91,13 +97,13 @@ NNS_DEV void pack_block(const float* row, int d, int c, float s, int fmt, uint8_
 #pragma unroll
     for (int e = 0; e < 16; ++e) {
       const int k = c * 16 + e;
-      bytes[e] = to_e4m3((row && k < d) ? row[k] / s : 0.f);
+      bytes[e] = to_e4m3((row && k < d) ? unscale(row[k], s, inv) : 0.f);
     }
   } else {
 #pragma unroll
     for (int e = 0; e < 8; ++e) {
       const int k = c * 8 + e;
-      const uint16_t b = to_bits16((row && k < d) ? row[k] / s : 0.f, fmt);
+      const uint16_t b = to_bits16((row && k < d) ? unscale(row[k], s, inv) : 0.f, fmt);
       bytes[2 * e] = (uint8_t)(b & 0xff);
       bytes[2 * e + 1] = (uint8_t)(b >> 8);
     }
