@@ -540,12 +540,7 @@ struct GeoTC {
           const bool sup = row_id < srows;
           const int p = sup ? row_id : row_id - srows;
           const float* row = rows2[h];
-          float s = 1.f;  // the row scale of FP16 / FP8 (as row_scale), from the warp's maximum
-          if (row && !fmt_is_bf16(fmt) && mx[h] > 0.f) {
-            int e;
-            frexpf(mx[h], &e);
-            s = ldexpf(1.f, e - 8);
-          }
+          const float s = row ? scale_of_max(mx[h], fmt) : 1.f;
           const int rows = sup ? bn : TC_BM;
           uint8_t* tile = (sup ? scr.B : scr.A) + (size_t)(p / rows) * rows * kb;
           for (int c = lane; c < nblk; c += 32) pack_block(row, d, c, s, fmt, tile, rows, p % rows, sup);

@@ -45,41 +45,88 @@ constexpr int TC_SMEM_MAX = 227 * 1024;  // per block, static + dynamic
 constexpr int TC_NACC = 4;                  // FP32 accumulators in tensor memory (a ring of tiles in flight)
 constexpr int TC_NNRM = 4;                  // column-norm slots (a ring of its own, loaded ahead)
 
-// One thread per point (consecutive threads write consecutive 16-byte rows
-// of each column block).  Also writes, per point, the FP32 squared norm, the
-// per-row scale and, in `stats`, the maxima of |v|_2, |v|_1 and the scale
-// over the points (as float bits; all values >= 0).  Row p holds the point
-// idx[sel ? sel[p] : p] for p < cnt (cnt read from cnt_dev when given; the
-// rest is padding).
-__global__ void k_pack_tc(const float* __restrict__ pts, const int* __restrict__ idx, const int* __restrict__ sel,
-                          const int* __restrict__ cnt_dev, int cnt, int rows_pad, int d, int kb, int fmt,
-                          int tile_rows, uint8_t* __restrict__ out, float* __restrict__ nrm, float* __restrict__ nrm_s,
-                          float* __restrict__ scale, unsigned* __restrict__ stats) {
-  const int nblk = kb / 16;
+// Packs rows in groups of PACK_ROWS: a warp reads its rows (coalesced) into
+// shared memory and sums their norms on the way, then each lane takes one row
+// of the group and each warp a share of its 16-byte blocks, so that a warp
+// writes 512 contiguous bytes of a block column.  (One thread per row, walking
+// its own row three times 4 bytes at a time, took 137 us for 131,072 rows of
+// d = 64; the bytes read and written take 13.)  Also writes, per point, the
+// FP32 squared norm (any order of summation keeps it within gamma_d |v|^2, the
+// bound the certificate uses), the per-row scale and, in `stats`, the maxima
+// of |v|_2, |v|_1 and the scale over the points (as float bits; all values >=
+// 0).  Row p holds the point idx[sel ? sel[p] : p] for p < cnt (cnt read from
+// cnt_dev when given; the rest is padding).
+constexpr int PACK_ROWS = 32;
+constexpr int PACK_THREADS = 256;
+
+__global__ void __launch_bounds__(PACK_THREADS)
+    k_pack_tc(const float* __restrict__ pts, const int* __restrict__ idx, const int* __restrict__ sel,
+              const int* __restrict__ cnt_dev, int cnt, int rows_pad, int d, int kb, int fmt, int tile_rows,
+              uint8_t* __restrict__ out, float* __restrict__ nrm, float* __restrict__ nrm_s,
+              float* __restrict__ scale, unsigned* __restrict__ stats) {
+  extern __shared__ float prow[];  // [PACK_ROWS][d rounded up to odd]
+  __shared__ float s_scale[PACK_ROWS];
+  const int nblk = kb / 16, ld = d | 1;
   const int count = cnt_dev ? min(*cnt_dev, cnt) : cnt;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  constexpr int NW = PACK_THREADS / 32, PER = PACK_ROWS / NW;
   unsigned m0 = 0u, m1 = 0u, m2 = 0u;  // this thread's maxima (float bits of values >= 0)
-  for (int p = blockIdx.x * blockDim.x + threadIdx.x; p < rows_pad; p += gridDim.x * blockDim.x) {
-    const float* row = p < count ? pts + (size_t)idx[sel ? sel[p] : p] * d : nullptr;
-    const float s = row_scale(row, d, fmt);
-    const int t = p / tile_rows, r = p % tile_rows;
-    for (int c = 0; c < nblk; ++c)
-      pack_block(row, d, c, s, fmt, out + (size_t)t * tile_rows * kb, tile_rows, r, nrm_s != nullptr);
-    {
-      if (row) {
-        float l2sq, l1;
-        row_norms(row, d, l2sq, l1);
-        nrm[p] = l2sq;
-        if (nrm_s) nrm_s[p] = norm_up(l2sq);
-        scale[p] = s;
-        m0 = max(m0, __float_as_uint(norm_up(l2sq)));
-        m1 = max(m1, __float_as_uint(l1 * (1.f + 1e-4f)));
-        m2 = max(m2, __float_as_uint(s));
-      } else {
-        nrm[p] = CUDART_INF_F;
-        if (nrm_s) nrm_s[p] = 0.f;
-        scale[p] = 1.f;
+  for (int p0 = blockIdx.x * PACK_ROWS; p0 < rows_pad; p0 += gridDim.x * PACK_ROWS) {
+    const float* row[PER];
+    float mx[PER], a2[PER], a1[PER];
+#pragma unroll
+    for (int h = 0; h < PER; ++h) {
+      const int p = p0 + warp * PER + h;
+      row[h] = p < count ? pts + (size_t)idx[sel ? sel[p] : p] * d : nullptr;
+      mx[h] = a2[h] = a1[h] = 0.f;
+    }
+    for (int k = lane; k < d; k += 32) {
+      float v[PER];
+#pragma unroll
+      for (int h = 0; h < PER; ++h) v[h] = row[h] ? row[h][k] : 0.f;
+#pragma unroll
+      for (int h = 0; h < PER; ++h) {
+        prow[(warp * PER + h) * ld + k] = v[h];
+        mx[h] = fmaxf(mx[h], fabsf(v[h]));
+        a2[h] = __fmaf_rn(v[h], v[h], a2[h]);
+        a1[h] = __fadd_rn(a1[h], fabsf(v[h]));
       }
     }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1)
+#pragma unroll
+      for (int h = 0; h < PER; ++h) {
+        mx[h] = fmaxf(mx[h], __shfl_xor_sync(0xffffffffu, mx[h], o));
+        a2[h] = __fadd_rn(a2[h], __shfl_xor_sync(0xffffffffu, a2[h], o));
+        a1[h] = __fadd_rn(a1[h], __shfl_xor_sync(0xffffffffu, a1[h], o));
+      }
+    if (lane == 0) {
+#pragma unroll
+      for (int h = 0; h < PER; ++h) {
+        const int p = p0 + warp * PER + h;
+        const float s = row[h] ? scale_of_max(mx[h], fmt) : 1.f;
+        s_scale[warp * PER + h] = s;
+        if (p < rows_pad) {
+          nrm[p] = row[h] ? a2[h] : CUDART_INF_F;
+          if (nrm_s) nrm_s[p] = row[h] ? norm_up(a2[h]) : 0.f;
+          scale[p] = s;
+        }
+        if (row[h]) {
+          m0 = max(m0, __float_as_uint(norm_up(a2[h])));
+          m1 = max(m1, __float_as_uint(a1[h] * (1.f + 1e-4f)));
+          m2 = max(m2, __float_as_uint(s));
+        }
+      }
+    }
+    __syncthreads();
+    const int p = p0 + lane;
+    if (p < rows_pad) {
+      const int t = p / tile_rows, r = p % tile_rows;
+      const float* mine = p < count ? prow + lane * ld : nullptr;
+      for (int c = warp; c < nblk; c += NW)
+        pack_block(mine, d, c, s_scale[lane], fmt, out + (size_t)t * tile_rows * kb, tile_rows, r, nrm_s != nullptr);
+    }
+    __syncthreads();
   }
   // the maxima: over the warp first, then one atomic per warp (every
   // thread of the block reaches this point: the loop above has no exit)
@@ -410,69 +457,103 @@ struct RerankArgs {
   int kl;               // list length of each chunk (the stride of cand_v / cand_p)
 };
 
-// One warp per packed consumer row.  The first rk candidates of every chunk
-// are re-ranked; tau is the smallest rk-th approximate value over the chunks
-// (every supplier outside them lies at or above it).  A consumer whose exact
-// best differs from the candidate the approximate values ranked first (over
-// all chunks, lowest position on ties) is counted as a near-tie of the
+// RR_ROWS packed consumer rows per block, G lanes a row (8 where the rows'
+// candidates are that few, else a warp).  The first rk candidates of every
+// chunk are re-ranked; tau is the smallest rk-th approximate value over the
+// chunks (every supplier outside them lies at or above it).  A consumer whose
+// exact best differs from the candidate the approximate values ranked first
+// (over all chunks, lowest position on ties) is counted as a near-tie of the
 // operand precision.
-__global__ void k_rerank_certify(RerankArgs R) {
-  const int lane = threadIdx.x & 31;
-  const int r = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-  if (r >= (R.nq_dev ? min(*R.nq_dev, R.nt) : R.nt)) return;
-  const int q = R.sel ? R.sel[r] : r;
-  const float* yrow = R.y + (size_t)R.ja[q] * R.d;
+//
+// The certificate is about fifty FP64 operations a row, and an FP64
+// instruction holds its pipe as long for one active lane as for 32: the last
+// step takes one row per lane of a warp.  (One warp per row, its certificate
+// in one lane, its norms summed in FP64 and its counters updated one by one
+// took 725 us for 131,072 rows, against 100 of candidate rows read.)
+constexpr int RR_ROWS = 32;
+constexpr int RR_THREADS = 256;
+
+template <int G>
+__global__ void __launch_bounds__(RR_THREADS) k_rerank_certify(RerankArgs R) {
+  __shared__ unsigned long long s_best[RR_ROWS], s_abest[RR_ROWS];
+  __shared__ float s_tau[RR_ROWS];
+  const int nq = R.nq_dev ? min(*R.nq_dev, R.nt) : R.nt;
+  const int r0 = blockIdx.x * RR_ROWS;
+  if (r0 >= nq) return;
+  const int sub = threadIdx.x % G;
   const int rk = R.rk;
   const int ncand = R.chunks * rk;
   // rows read 16 bytes at a time where d and both bases allow it
   const bool vec = (R.d & 3) == 0 && ((reinterpret_cast<uintptr_t>(R.x) | reinterpret_cast<uintptr_t>(R.y)) & 15) == 0;
-  unsigned long long best = ~0ULL, abest = ~0ULL;
-  float tau = CUDART_INF_F;  // smallest chunk threshold (rk-th value of each chunk)
-  for (int c = lane; c < ncand; c += 32) {
-    const int chunk = c / rk, k = c % rk;
-    const size_t o = ((size_t)chunk * R.nt_pad + r) * R.kl + k;
-    const int p = R.cand_p[o];
-    if (k == rk - 1) tau = fminf(tau, R.cand_v[o]);
-    if (p < 0) continue;
-    if (k == 0) {
-      const unsigned long long ak = ((unsigned long long)ordered_bits(R.cand_v[o]) << 32) | (unsigned)p;
-      abest = ak < abest ? ak : abest;
+  for (int k0 = threadIdx.x / G; k0 < RR_ROWS; k0 += RR_THREADS / G) {  // (whole warps: RR_ROWS is a multiple)
+    const int r = r0 + k0;
+    unsigned long long best = ~0ULL, abest = ~0ULL;
+    float tau = CUDART_INF_F;  // smallest chunk threshold (rk-th value of each chunk)
+    if (r < nq) {
+      const int q = R.sel ? R.sel[r] : r;
+      const float* yrow = R.y + (size_t)R.ja[q] * R.d;
+      for (int c = sub; c < ncand; c += G) {
+        const int chunk = c / rk, k = c % rk;
+        const size_t o = ((size_t)chunk * R.nt_pad + r) * R.kl + k;
+        const int p = R.cand_p[o];
+        if (k == rk - 1) tau = fminf(tau, R.cand_v[o]);
+        if (p < 0) continue;
+        if (k == 0) {
+          const unsigned long long ak = ((unsigned long long)ordered_bits(R.cand_v[o]) << 32) | (unsigned)p;
+          abest = ak < abest ? ak : abest;
+        }
+        // squared-Euclidean FP32 key (the contraction has no L1 form)
+        const float* xr = R.x + (size_t)R.ia[p] * R.d;
+        const float acc = vec ? key32_sql2_v4(xr, yrow, R.d) : key32<METRIC_SQL2>(xr, yrow, R.d);
+        const unsigned long long key = pack_key(acc, (unsigned)p);
+        best = key < best ? key : best;
+      }
     }
-    // squared-Euclidean FP32 key (the contraction has no L1 form)
-    const float* xr = R.x + (size_t)R.ia[p] * R.d;
-    const float acc = vec ? key32_sql2_v4(xr, yrow, R.d) : key32<METRIC_SQL2>(xr, yrow, R.d);
-    const unsigned long long key = pack_key(acc, (unsigned)p);
-    best = key < best ? key : best;
+#pragma unroll
+    for (int o = G / 2; o > 0; o >>= 1) {
+      const unsigned long long ob = __shfl_xor_sync(0xffffffffu, best, o);
+      best = ob < best ? ob : best;
+      const unsigned long long oa = __shfl_xor_sync(0xffffffffu, abest, o);
+      abest = oa < abest ? oa : abest;
+      tau = fminf(tau, __shfl_xor_sync(0xffffffffu, tau, o));
+    }
+    if (sub == 0) {
+      s_best[k0] = best;
+      s_abest[k0] = abest;
+      s_tau[k0] = tau;
+    }
   }
-  // |y|_2^2 and |y|_1 in FP64, split over the lanes
-  double yl2 = 0.0, yl1 = 0.0;
-  for (int k = lane; k < R.d; k += 32) {
-    yl2 += (double)yrow[k] * yrow[k];
-    yl1 += fabs((double)yrow[k]);
+  __syncthreads();
+  if (threadIdx.x >= 32) return;
+  const int lane = threadIdx.x, r = r0 + lane;
+  const bool live = r < nq;
+  const int q = live ? (R.sel ? R.sel[r] : r) : 0;
+  const unsigned long long best = s_best[lane];
+  bool certified = false;
+  if (live && best != ~0ULL) {
+    // |y|_2 from the FP32 squared norm, rounded up; |y|_1 <= sqrt(d) |y|_2
+    // (it only scales the formats' absolute rounding floors)
+    const float ny = R.nrm_y[r];
+    const double yl2 = norm_up(ny);
+    certified = certify(R.fmt, R.d, ny, yl2, yl2 * sqrt((double)R.d) * (1 + 1e-12), R.scale_y[r],
+                        __uint_as_float(R.stats_x[0]), __uint_as_float(R.stats_x[1]), __uint_as_float(R.stats_x[2]),
+                        s_tau[lane], __uint_as_float((unsigned)(best >> 32)));
   }
-  for (int o = 16; o > 0; o >>= 1) {
-    const unsigned long long ob = __shfl_xor_sync(0xffffffffu, best, o);
-    best = ob < best ? ob : best;
-    const unsigned long long oa = __shfl_xor_sync(0xffffffffu, abest, o);
-    abest = oa < abest ? oa : abest;
-    tau = fminf(tau, __shfl_xor_sync(0xffffffffu, tau, o));
-    yl2 += __shfl_xor_sync(0xffffffffu, yl2, o);
-    yl1 += __shfl_xor_sync(0xffffffffu, yl1, o);
+  if (certified) R.nnkey[q] = best;
+  const unsigned ok = __ballot_sync(0xffffffffu, certified), bad = __ballot_sync(0xffffffffu, live && !certified);
+  const unsigned near =
+      __ballot_sync(0xffffffffu, live && best != ~0ULL && (unsigned)best != (unsigned)s_abest[lane]);
+  int base = 0;
+  if (lane == 0) {
+    if (near) atomicAdd(R.nnear, (unsigned long long)__popc(near));
+    if (ok) atomicAdd(R.ncertified, (unsigned long long)__popc(ok));
+    if (bad) {
+      atomicAdd(R.nfallback_total, (unsigned long long)__popc(bad));
+      base = atomicAdd(R.nfallback, __popc(bad));
+    }
   }
-  if (lane != 0) return;
-  if (best != ~0ULL && (unsigned)best != (unsigned)abest) atomicAdd(R.nnear, 1ULL);
-  yl2 = sqrt(yl2) * (1 + 1e-12);
-  const bool certified =
-      best != ~0ULL && certify(R.fmt, R.d, R.nrm_y[r], yl2, yl1, R.scale_y[r], __uint_as_float(R.stats_x[0]),
-                               __uint_as_float(R.stats_x[1]), __uint_as_float(R.stats_x[2]), tau,
-                               __uint_as_float((unsigned)(best >> 32)));
-  if (certified) {
-    R.nnkey[q] = best;
-    atomicAdd(R.ncertified, 1ULL);
-  } else {
-    R.fallback[atomicAdd(R.nfallback, 1)] = q;
-    atomicAdd(R.nfallback_total, 1ULL);
-  }
+  base = __shfl_sync(0xffffffffu, base, 0);
+  if ((bad >> lane) & 1u) R.fallback[base + __popc(bad & ((1u << lane) - 1u))] = q;
 }
 
 // --------------------------------------------------------------------------
@@ -533,16 +614,17 @@ int launch_nns_tc(const SolveBufs& B, const TcBufs& T, int mt, int nt, int preci
   // pack both sides
   if (cudaMemsetAsync(T.stats, 0, 8 * sizeof(unsigned), st) != cudaSuccess) return -1;
   {
-    const int64_t work = (int64_t)qtiles * TC_BM;
-    int g = (int)std::min<int64_t>((work + 255) / 256, num_sms() * 16);
-    k_pack_tc<<<g, 256, 0, st>>>(B.y, B.ja[B.cur], sel, nsel_dev, nt, qtiles * TC_BM, B.d, kb, fmt, TC_BM, T.A,
-                                 T.nrm_y, nullptr, T.scale_y, T.stats + 4);
-  }
-  {
-    const int64_t work = (int64_t)stiles * bn;
-    int g = (int)std::min<int64_t>((work + 255) / 256, num_sms() * 16);
-    k_pack_tc<<<g, 256, 0, st>>>(B.x, B.ia[B.cur], nullptr, nullptr, mt, stiles * bn, B.d, kb, fmt, bn, T.B,
-                                 T.nrm_x, T.nrm_sx, T.scale_x, T.stats);
+    const size_t smem = (size_t)PACK_ROWS * (B.d | 1) * sizeof(float);
+    if (smem > 48 * 1024 &&
+        cudaFuncSetAttribute(k_pack_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
+      return -1;
+    auto grid = [](int64_t rows) { return (int)std::min<int64_t>((rows + PACK_ROWS - 1) / PACK_ROWS, num_sms() * 16); };
+    k_pack_tc<<<grid((int64_t)qtiles * TC_BM), PACK_THREADS, smem, st>>>(
+        B.y, B.ja[B.cur], sel, nsel_dev, nt, qtiles * TC_BM, B.d, kb, fmt, TC_BM, T.A, T.nrm_y, nullptr, T.scale_y,
+        T.stats + 4);
+    k_pack_tc<<<grid((int64_t)stiles * bn), PACK_THREADS, smem, st>>>(B.x, B.ia[B.cur], nullptr, nullptr, mt, stiles * bn,
+                                                                  B.d, kb, fmt, bn, T.B, T.nrm_x, T.nrm_sx, T.scale_x,
+                                                                  T.stats);
   }
   // chunks of supplier tiles so that the grid covers the GPU several times
   int chunks = (tc_target_ctas() + qtiles - 1) / qtiles;
@@ -577,7 +659,9 @@ int launch_nns_tc(const SolveBufs& B, const TcBufs& T, int mt, int nt, int preci
                chunks,   fmt,        T.cand_v,    T.cand_p,    T.nrm_y,   T.scale_y,   T.stats,
                B.nnkey,  T.fallback, T.nfallback, &B.st->certified, &B.st->fallbacks, &B.st->near_ties,
                sel,      nsel_dev,   rk,          kl};
-  k_rerank_certify<<<(nt + 7) / 8, 256, 0, st>>>(R);
+  const int rblocks = (nt + RR_ROWS - 1) / RR_ROWS;
+  if (chunks * rk <= 8) k_rerank_certify<8><<<rblocks, RR_THREADS, 0, st>>>(R);
+  else k_rerank_certify<32><<<rblocks, RR_THREADS, 0, st>>>(R);
   // FP32 scan of the consumers that were not certified
   launch_nns_f32(B, mt, nt, T.fallback, T.nfallback, st);
   return 0;

@@ -54,11 +54,8 @@ NNS_DEV uint8_t to_e4m3(float v) { return (uint8_t)__nv_cvt_float_to_fp8(v, __NV
 
 // Per-row scale (a power of two) for FP16 / FP8: the largest |v| of the row
 // maps into [2^7, 2^8).  BF16 has FP32's exponent range and uses 1.
-NNS_DEV float row_scale(const float* row, int d, int fmt) {
-  if (!row || fmt_is_bf16(fmt)) return 1.f;
-  float mx = 0.f;
-  for (int k = 0; k < d; ++k) mx = fmaxf(mx, fabsf(row[k]));
-  if (!(mx > 0.f)) return 1.f;
+NNS_DEV float scale_of_max(float mx, int fmt) {
+  if (fmt_is_bf16(fmt) || !(mx > 0.f)) return 1.f;
   int e;
   frexpf(mx, &e);  // mx in [2^(e-1), 2^e)
   return ldexpf(1.f, e - 8);
@@ -110,17 +107,6 @@ NNS_DEV void pack_block(const float* row, int d, int c, float s, int fmt, uint8_
   }
   *reinterpret_cast<uint4*>(tile_base + (size_t)c * tile_rows * 16 + (size_t)r * 16) =
       *reinterpret_cast<const uint4*>(bytes);
-}
-
-// FP32 squared norm (sequential fma) and L1 norm of a row.
-NNS_DEV void row_norms(const float* row, int d, float& l2sq, float& l1) {
-  float acc = 0.f, a1 = 0.f;
-  for (int k = 0; k < d; ++k) {
-    acc = __fmaf_rn(row[k], row[k], acc);
-    a1 = __fadd_rn(a1, fabsf(row[k]));
-  }
-  l2sq = acc;
-  l1 = a1;
 }
 
 // --------------------------------------------------------------------------
