@@ -9,8 +9,8 @@
 //            multi-CTA round (K1 NNS, grouping, greedy flow, compaction);
 //   tail     once they fit, every remaining round in one launch: for d <= 8
 //            on a thread-block cluster (k_finish_cl, up to 2048 points per
-//            side) where the device can co-schedule one, else in one CTA
-//            (k_finish, k_finish_hd);
+//            side; d > 8: k_finish_hd_cl on a key matrix) where the device
+//            can co-schedule one, else in one CTA (k_finish, k_finish_hd);
 //   final    R and the leftover mass as correctly rounded sums.
 // The host reads the two active counts of each multi-CTA round to size the
 // next round's grids: the compaction's count kernel writes them into mapped
@@ -140,8 +140,8 @@ int ensure_ws(nnsemd_ctx* ctx, size_t bytes) {
 }
 
 // Lay out the buffers of a single-pair solve; with base == nullptr only the
-// size is computed.
-size_t layout_solve(void* base, int64_t m, int64_t n, int d, SolveBufs& B, int precision = 0,
+// size is computed.  `tail`: with the key matrix of the d > 8 cluster tail.
+size_t layout_solve(void* base, int64_t m, int64_t n, int d, SolveBufs& B, bool tail, int precision = 0,
                     const nnsemd_proposal* P = nullptr, LearnedBufs* L = nullptr) {
   Carve C(base);
   const int dp = d <= 8 ? padded_dim(d) : 0;
@@ -241,6 +241,9 @@ size_t layout_solve(void* base, int64_t m, int64_t n, int d, SolveBufs& B, int p
   B.fl_j = C.take<int32_t>(m + n);
   B.fl_f = C.take<double>(m + n);
   B.blockcounts = C.take<int>((m + n) / 1024 + 8);
+  B.kmat = nullptr;
+  if (tail && d > 8)
+    B.kmat = C.take<float>((size_t)(std::min<int64_t>(m, FIN_MAX_HD) * kmat_ld(std::min<int64_t>(n, FIN_MAX_HD))));
   return C.off + 256;
 }
 
@@ -398,19 +401,26 @@ int run_solve(nnsemd_ctx* ctx, SolveBufs& B, const double* a, const double* b, d
          (tcb ? 2 : 0) + (5 + (tcb ? 2 : 0) + 2 * sel) * ((B.n + learned->chunk - 1) / learned->chunk);
   }
   while (mt > 0 && nt > 0) {
+    // d > 8: the cluster tail takes over once both active sets fit it (with a
+    // reduced precision or a proposal from the second round on: the first is
+    // theirs), the one-CTA tail at a bounded amount of work per round
+    const bool fits_hd = !lowd && mt <= FIN_MAX_HD && nt <= FIN_MAX_HD;
+    const bool hdcl = fits_hd && finish_hd_cluster_ready(B);
+    const bool own_first = learned || B.precision != NNSEMD_FP32;
     const bool tail = clcap ? (mt <= clcap && nt <= clcap)
                       : lowd ? (mt <= FIN_MAX && nt <= FIN_MAX && (int64_t)mt * nt <= FIN_PAIRS)
-                             : (mt <= FIN_MAX_HD && nt <= FIN_MAX_HD && (int64_t)mt * nt * B.d <= FIN_HD_WORK);
+                             : fits_hd && ((hdcl && !(own_first && rounds == 0)) || (int64_t)mt * nt * B.d <= FIN_HD_WORK);
     if (tail) {
       if (timed) CKD(cudaEventRecord(ctx->ev[2], st));
       B.round0 = rounds;
       const int lrc = clcap  ? launch_finish_cluster(B, round_limit - rounds, st)
                       : lowd ? launch_finish(B, round_limit - rounds, st)
+                      : hdcl ? launch_finish_hd_cluster(B, mt, nt, round_limit - rounds, st)
                              : launch_finish_hd(B, round_limit - rounds, st);
       if (lrc) return drained(fail(ctx, NNSEMD_ERR_CUDA, "finisher launch"));
       if (timed) CKD(cudaEventRecord(ctx->ev[3], st));
       tail_ran = true;
-      L += 1;
+      L += hdcl ? 2 : 1;
       break;
     }
     if (rounds >= round_limit) return drained(fail(ctx, NNSEMD_ERR_ITER_LIMIT, "round limit m + n exceeded"));
@@ -600,9 +610,15 @@ int nnsemd_solve(nnsemd_ctx* ctx, const float* x, const double* a, int64_t m, co
   CK(cudaSetDevice(ctx->device));
   SolveBufs B{};
   LearnedBufs Lb{};
-  size_t bytes = layout_solve(nullptr, m, n, d, B, precision, P, P ? &Lb : nullptr);
-  if ((rc = ensure_ws(ctx, bytes))) return rc;
-  layout_solve(ctx->ws, m, n, d, B, precision, P, P ? &Lb : nullptr);
+  bool tail = true;  // (without its key matrix where the memory is short)
+  rc = ensure_ws(ctx, layout_solve(nullptr, m, n, d, B, tail, precision, P, P ? &Lb : nullptr));
+  if (rc == NNSEMD_ERR_OOM && d > 8) {
+    tail = false;
+    ctx->err.clear();
+    rc = ensure_ws(ctx, layout_solve(nullptr, m, n, d, B, tail, precision, P, P ? &Lb : nullptr));
+  }
+  if (rc) return rc;
+  layout_solve(ctx->ws, m, n, d, B, tail, precision, P, P ? &Lb : nullptr);
   B.x = x;
   B.y = y;
   B.m = m;
@@ -641,7 +657,8 @@ int nnsemd_solve_host(nnsemd_ctx* ctx, const float* x, const double* a, int64_t 
   // device staging for the inputs and the plan, placed after the solve buffers
   SolveBufs B{};
   LearnedBufs Lb{};
-  size_t solve_bytes = layout_solve(nullptr, m, n, d, B, precision, P, P ? &Lb : nullptr);
+  bool tail = true;
+  size_t solve_bytes = layout_solve(nullptr, m, n, d, B, tail, precision, P, P ? &Lb : nullptr);
   const int64_t cap = plan ? std::min<int64_t>(plan->capacity, m + n) : 0;
   auto stage_layout = [&](void* base, float** xd, double** ad, float** yd, double** bd, int32_t** pi, int32_t** pj,
                           double** pf) {
@@ -659,9 +676,15 @@ int nnsemd_solve_host(nnsemd_ctx* ctx, const float* x, const double* a, int64_t 
   float *xd, *yd;
   double *ad, *bd, *pf;
   int32_t *pi, *pj;
-  size_t bytes = stage_layout(nullptr, &xd, &ad, &yd, &bd, &pi, &pj, &pf);
-  if ((rc = ensure_ws(ctx, bytes))) return rc;
-  layout_solve(ctx->ws, m, n, d, B, precision, P, P ? &Lb : nullptr);
+  rc = ensure_ws(ctx, stage_layout(nullptr, &xd, &ad, &yd, &bd, &pi, &pj, &pf));
+  if (rc == NNSEMD_ERR_OOM && d > 8) {  // without the tail's key matrix
+    tail = false;
+    solve_bytes = layout_solve(nullptr, m, n, d, B, tail, precision, P, P ? &Lb : nullptr);
+    ctx->err.clear();
+    rc = ensure_ws(ctx, stage_layout(nullptr, &xd, &ad, &yd, &bd, &pi, &pj, &pf));
+  }
+  if (rc) return rc;
+  layout_solve(ctx->ws, m, n, d, B, tail, precision, P, P ? &Lb : nullptr);
   stage_layout(ctx->ws, &xd, &ad, &yd, &bd, &pi, &pj, &pf);
   cudaStream_t st = ctx->stream;
   CK(cudaMemcpyAsync(xd, x, (size_t)m * d * sizeof(float), cudaMemcpyHostToDevice, st));
@@ -828,12 +851,14 @@ static int solve_batched_impl(nnsemd_ctx* ctx, int32_t num_pairs, const float* x
     maxn = std::max(maxn, y_len(p));
   }
   SolveBufs B{};
-  const size_t large_bytes = large.empty() ? 0 : layout_solve(nullptr, maxm, maxn, d, B, precision);
-  rc = ensure_ws(ctx, layout_head(nullptr) + large_bytes);
-  if (rc == NNSEMD_ERR_OOM && (kc_big || kc_tiny)) {
+  bool tail = true;
+  auto large_bytes = [&] { return large.empty() ? 0 : layout_solve(nullptr, maxm, maxn, d, B, tail, precision); };
+  rc = ensure_ws(ctx, layout_head(nullptr) + large_bytes());
+  if (rc == NNSEMD_ERR_OOM && d > 8) {  // without any key matrix
     kc_big = kc_tiny = 0;
+    tail = false;
     ctx->err.clear();
-    rc = ensure_ws(ctx, layout_head(nullptr) + large_bytes);
+    rc = ensure_ws(ctx, layout_head(nullptr) + large_bytes());
   }
   if (rc) return rc;
   const size_t head = layout_head(ctx->ws);
@@ -965,7 +990,7 @@ static int solve_batched_impl(nnsemd_ctx* ctx, int32_t num_pairs, const float* x
   long long extra_rounds = 0, extra_pe = 0;
   long long extra_cert = 0, extra_fall = 0, extra_near = 0;
   for (int p : large) {
-    layout_solve((char*)ctx->ws + head, maxm, maxn, d, B, precision);
+    layout_solve((char*)ctx->ws + head, maxm, maxn, d, B, tail, precision);
     B.x = x_packed + x_off[p] * d;
     B.y = y_packed + y_begin(p) * d;
     B.m = x_off[p + 1] - x_off[p];

@@ -654,6 +654,92 @@ struct GeoGlobal {
   }
 };
 
+// The tail of a large d > 8 solve on a thread-block cluster: the key matrix of
+// its first round's active points (positions at that time; filled before the
+// launch) stays in global memory, every CTA holds the whole per-point state
+// with each point's row or column, and the NNS step is split over the CTAs
+// and exchanged like GeoSmemCluster's.  A warp takes 32 consumers of the slice
+// and a chunk of the active suppliers, 16 rows in flight.
+template <int CAP, int NT>
+struct GeoMatCluster {
+  static constexpr int kDP = 0;
+  static constexpr int kThreads = NT;
+  static constexpr bool kWarpRounds = true;
+  static constexpr int kSlice = CAP / 8;  // consumers per CTA at most (R >= 8)
+  const float* kmat;
+  int kld;
+  int row[CAP];
+  int col[CAP];
+  unsigned long long xk[2][CAP];   // receive buffers (round parity)
+  unsigned long long red[kSlice];  // the slice's keys merged over chunks; all ones between rounds
+  struct PX { int v; };
+  NNS_DEV void load_x(int p, PX& r) const { r.v = row[p]; }
+  NNS_DEV void store_x(int p, const PX& r) { row[p] = r.v; }
+  NNS_DEV void load_y(int q, PX& r) const { r.v = col[q]; }
+  NNS_DEV void store_y(int q, const PX& r) { col[q] = r.v; }
+  template <int C>
+  NNS_DEV double dist64(const CtaCore<C>&, int, int, int) const { return 0.0; }  // (flows are costed after the tail)
+
+  // The first minimum of column c (this lane's) over the active suppliers
+  // [s0, s1): keys order like their bit patterns (none is negative or NaN).
+  NNS_DEV unsigned long long scan_col(int c, int s0, int s1) const {
+    constexpr int F = 16;
+    unsigned best = 0xffffffffu;
+    int bp = s0;
+    for (int p = s0; p < s1; p += F) {
+      unsigned v[F];
+#pragma unroll
+      for (int e = 0; e < F; ++e) v[e] = __float_as_uint(kmat[(size_t)row[min(p + e, s1 - 1)] * kld + c]);
+#pragma unroll
+      for (int e = 0; e < F; ++e)  // (repeats of the last supplier never win)
+        if (v[e] < best) { best = v[e]; bp = p + e; }
+    }
+    return ((unsigned long long)best << 32) | (unsigned)bp;
+  }
+  NNS_DEV void init() {
+    for (int i = threadIdx.x; i < kSlice; i += NT) red[i] = ~0ULL;
+  }
+  template <int C>
+  NNS_DEV const unsigned long long* nns(CtaCore<C>&, int mt, int nt, long long round) {
+    namespace cg = cooperative_groups;
+    cg::cluster_group cl = cg::this_cluster();
+    const unsigned rank = cl.block_rank(), ncl = cl.num_blocks();
+    const int h = (int)(round & 1);
+    const int q0 = (int)((unsigned)nt * rank / ncl), q1 = (int)((unsigned)nt * (rank + 1) / ncl);
+    const int ns = q1 - q0;
+    constexpr int NW = NT / 32;
+    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int cgroups = (ns + 31) >> 5;
+    if (cgroups > 0 && w < NW / cgroups * cgroups) {  // (at most NW groups: kSlice / 32)
+      const int chunks = NW / cgroups, ch = w / cgroups;
+      const int qa = 32 * (w % cgroups) + lane;
+      const int s0 = (int)((unsigned)(mt * ch) / (unsigned)chunks);
+      const int s1 = (int)((unsigned)(mt * (ch + 1)) / (unsigned)chunks);
+      if (s0 < s1) {
+        const unsigned long long k = scan_col(col[q0 + min(qa, ns - 1)], s0, s1);
+        if (qa < ns) atomicMin(&red[qa], k);
+      }
+    }
+    __syncthreads();
+    for (int i = threadIdx.x; i < ns * (int)ncl; i += NT) {
+      const int r = i / ns, q = i - r * ns;
+      cl.map_shared_rank(&xk[h][0], r)[q0 + q] = red[q];
+    }
+    cl.sync();
+    for (int i = threadIdx.x; i < ns; i += NT) red[i] = ~0ULL;
+    return xk[h];
+  }
+  NNS_DEV bool warp_ready() const { return true; }
+  template <int C>
+  NNS_DEV void warp_nns(CtaCore<C>& S, int mt, int nt) const {
+#pragma unroll 1
+    for (int q = threadIdx.x & 31; q < 64; q += 32) {
+      const unsigned long long k = scan_col(col[min(q, nt - 1)], 0, mt);
+      if (q < nt) S.nnk[q] = k;
+    }
+  }
+};
+
 // Note: GeoGlobal passes the CTA's own index arrays (iidx, jidx) as the
 // "position -> original index" maps, so positions are CTA-local.
 

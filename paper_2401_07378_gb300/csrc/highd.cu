@@ -15,6 +15,8 @@
 //                    pair per CTA, all rounds on chip (Sec. III-D batching).
 #include <math_constants.h>
 
+#include <atomic>
+
 #include "common.cuh"
 #include "cta.cuh"
 #include "kernels.h"
@@ -124,6 +126,157 @@ static int finish_hd_t(const SolveBufs& B, long long round_limit, cudaStream_t s
 
 int launch_finish_hd(const SolveBufs& B, int64_t round_limit, cudaStream_t st) {
   return B.metric == METRIC_L1 ? finish_hd_t<true>(B, round_limit, st) : finish_hd_t<false>(B, round_limit, st);
+}
+
+// --------------------------------------------------------------------------
+// the tail on a thread-block cluster, from a key matrix
+// --------------------------------------------------------------------------
+
+// The FP32 keys of every active supplier (row) and consumer, one 64 x 64 tile
+// per CTA.
+template <bool L1>
+__global__ void __launch_bounds__(TG_THREADS, 3)
+    k_tail_keys(const float* __restrict__ x, const int* __restrict__ ia, int mt, const float* __restrict__ y,
+                const int* __restrict__ ja, int nt, int d, float* __restrict__ kmat, int ld) {
+  __shared__ TileSmem T;
+  const int c0 = blockIdx.x * TG_M, p0 = blockIdx.y * TG_N;
+  const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
+  group_tiles<L1, true>(x, ia, p0, min(p0 + TG_N, mt), y, ja, nullptr, c0, min(TG_M, nt - c0), d, T, threadIdx.x, 0,
+                        [&](int pt, const unsigned long long (&acc)[2][4]) {
+                          const int q = c0 + ty * 4;  // four consecutive consumers: one 16-byte store
+                          if (q >= nt) return;
+#pragma unroll
+                          for (int j = 0; j < 4; ++j) {
+                            const int p = pt + tx * 4 + j;
+                            if (p < mt)
+                              *reinterpret_cast<ulonglong2*>(kmat + (size_t)p * ld + q) =
+                                  make_ulonglong2(acc[0][j], acc[1][j]);
+                          }
+                        });
+}
+
+constexpr int FIN_HD_CL_THREADS = 512;
+constexpr int FIN_HD_CL = 16;  // preferred cluster size (8 where 16 cannot be co-scheduled)
+
+struct MatClusterSmem {
+  CtaCore<FIN_MAX_HD> S;
+  GeoMatCluster<FIN_MAX_HD, FIN_HD_CL_THREADS> G;
+};
+
+// Every remaining round of a d > 8 solve, both active sets at most FIN_MAX_HD
+// points: the scheme of k_finish_cl on the key matrix of k_tail_keys.  One CTA
+// recomputing the distances of its rounds took 335 us for a 300 x 700 pair at
+// d = 128 and could only take over below 2^23 coordinate products a round;
+// the multi-CTA rounds before that cost 40 us and more each.
+__global__ void __launch_bounds__(FIN_HD_CL_THREADS, 1) k_finish_hd_cl(SolveBufs B, int ld, long long round_limit) {
+  namespace cg = cooperative_groups;
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  MatClusterSmem& M = *reinterpret_cast<MatClusterSmem*>(smem_raw);
+  CtaCore<FIN_MAX_HD>& S = M.S;
+  cg::cluster_group cl = cg::this_cluster();
+  const bool leader = cl.block_rank() == 0;
+  const int tid = threadIdx.x;
+  const int mt = B.st->mt, nt = B.st->nt;
+  if (mt > FIN_MAX_HD || nt > FIN_MAX_HD || cl.num_blocks() < 8) {  // the same decision in every CTA
+    if (tid == 0 && leader) atomicOr(&B.st->err, EF_INTERNAL);
+    return;
+  }
+  for (int p = tid; p < mt; p += FIN_HD_CL_THREADS) {
+    M.G.row[p] = p;
+    S.iidx[p] = B.ia[B.cur][p];
+    S.sres[p] = B.s[S.iidx[p]];
+  }
+  for (int q = tid; q < nt; q += FIN_HD_CL_THREADS) {
+    M.G.col[q] = q;
+    S.jidx[q] = B.ja[B.cur][q];
+    S.cres[q] = B.c[S.jidx[q]];
+  }
+  if (tid == 0) {
+    M.G.kmat = B.kmat;
+    M.G.kld = ld;
+    S.mt = mt;
+    S.nt = nt;
+  }
+  M.G.init();
+  // every CTA of the cluster is running before any writes a peer's memory
+  cl.sync();
+  CtaOut O{nullptr, nullptr, nullptr, nullptr, 0, nullptr, nullptr, &B.st->err,
+           nullptr, nullptr, nullptr, B.x, B.y, B.d, B.protocol, B.seed, B.round0, 1};
+  if (leader)
+    O = CtaOut{nullptr, nullptr, nullptr, nullptr, 0, B.s, B.c, &B.st->err,
+               B.fl_i, B.fl_j, B.fl_f, B.x, B.y, B.d, B.protocol, B.seed, B.round0, 0};
+  unsigned long long nnz = B.st->nnz;
+  long long rounds = B.st->rounds, pe = B.st->pair_evals;
+  cta_rounds(S, M.G, B.metric, O, nnz, rounds, pe, round_limit);
+  if (tid == 0 && leader) {
+    B.st->nnz = nnz;
+    B.st->rounds = rounds;
+    B.st->pair_evals = pe;
+    B.st->mt = S.mt;
+    B.st->nt = S.nt;
+  }
+  // no CTA leaves while a peer may still address its shared memory
+  cl.sync();
+}
+
+static_assert(sizeof(MatClusterSmem) <= 227 * 1024, "cluster tail state exceeds shared memory");
+
+static void finish_hd_cl_config(cudaLaunchConfig_t& cfg, cudaLaunchAttribute* at, int cs) {
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = cs;
+  at[0].val.clusterDim.y = 1;
+  at[0].val.clusterDim.z = 1;
+  cfg.gridDim = dim3(cs);
+  cfg.blockDim = dim3(FIN_HD_CL_THREADS);
+  cfg.dynamicSmemBytes = sizeof(MatClusterSmem);
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+}
+
+// Cluster size usable for k_finish_hd_cl on the current device (looked up
+// once per device): the preferred size, 8, or 0.
+static int finish_hd_cl_size() {
+  static std::atomic<int> cache[64];
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 0;
+  const int c = cache[dev].load();
+  if (c) return c > 0 ? c : 0;
+  int found = -1;
+  if (cudaFuncSetAttribute(k_finish_hd_cl, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(MatClusterSmem)) ==
+          cudaSuccess &&
+      cudaFuncSetAttribute(k_finish_hd_cl, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess) {
+    for (int cs : {FIN_HD_CL, 8}) {
+      cudaLaunchConfig_t cfg = {};
+      cudaLaunchAttribute at[1];
+      finish_hd_cl_config(cfg, at, cs);
+      int n = 0;
+      if (cudaOccupancyMaxActiveClusters(&n, k_finish_hd_cl, &cfg) == cudaSuccess && n > 0) {
+        found = cs;
+        break;
+      }
+    }
+  }
+  cudaGetLastError();  // a refused size is an answer, not an error of the solve
+  cache[dev].store(found);
+  return found > 0 ? found : 0;
+}
+
+bool finish_hd_cluster_ready(const SolveBufs& B) { return B.kmat != nullptr && finish_hd_cl_size() > 0; }
+
+int launch_finish_hd_cluster(const SolveBufs& B, int mt, int nt, int64_t round_limit, cudaStream_t st) {
+  const int cs = finish_hd_cl_size();
+  if (!cs || !B.kmat) return -1;
+  const int ld = (int)kmat_ld(nt), cur = B.cur;
+  const dim3 grid((nt + TG_M - 1) / TG_M, (mt + TG_N - 1) / TG_N);
+  if (B.metric == METRIC_L1)
+    k_tail_keys<true><<<grid, TG_THREADS, 0, st>>>(B.x, B.ia[cur], mt, B.y, B.ja[cur], nt, B.d, B.kmat, ld);
+  else
+    k_tail_keys<false><<<grid, TG_THREADS, 0, st>>>(B.x, B.ia[cur], mt, B.y, B.ja[cur], nt, B.d, B.kmat, ld);
+  cudaLaunchConfig_t cfg = {};
+  cudaLaunchAttribute at[1];
+  finish_hd_cl_config(cfg, at, cs);
+  cfg.stream = st;
+  return cudaLaunchKernelEx(&cfg, k_finish_hd_cl, B, ld, (long long)round_limit) == cudaSuccess ? 0 : -1;
 }
 
 template <bool L1>

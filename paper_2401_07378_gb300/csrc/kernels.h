@@ -82,6 +82,7 @@ struct SolveBufs {
   int32_t* fl_i;   // [m+n] flow record of the one-CTA rounds (deferred costing)
   int32_t* fl_j;
   double* fl_f;
+  float* kmat;     // d > 8 (nullable): key matrix of the cluster tail
   int* blockcounts;            // compaction scratch
   unsigned long long* xs_acc;  // 4 exact-sum accumulators of XS_LIMBS limbs
   // Early notification of the active counts (nullable): the compaction's
@@ -171,6 +172,11 @@ int launch_batched_lowd_small(const BatchArgs& A, int grid, cudaStream_t st);
 // ncons_dev when given, else ncons).  Merges into B.nnkey with atomicMin.
 int launch_nns_f32(const SolveBufs& B, int mt, int ncons, const int* cons, const int* ncons_dev, cudaStream_t st);
 int launch_finish_hd(const SolveBufs& B, int64_t round_limit, cudaStream_t st);
+// All remaining rounds on a thread-block cluster (two launches), for active
+// sets of at most FIN_MAX_HD points per side, where finish_hd_cluster_ready
+// (the key matrix is laid out and the device co-schedules the cluster).
+bool finish_hd_cluster_ready(const SolveBufs& B);
+int launch_finish_hd_cluster(const SolveBufs& B, int mt, int nt, int64_t round_limit, cudaStream_t st);
 int launch_batched_hd(const BatchArgs& A, int grid, cudaStream_t st);
 // Batched FP32 solver for pairs of at most HD_SMALL_CAP points per side
 // (d > 8), HD_SMALL_THREADS threads per pair, several pairs per SM.

@@ -1,0 +1,56 @@
+"""The cluster tail of d > 8 solves (key matrix, keys exchanged through
+distributed shared memory) at its capacity, at the one-warp edge and with the
+reduced-precision re-rank and packing before it, against the oracle."""
+import numpy as np
+import pytest
+
+import oracle
+from paper_2401_07378_gb300 import workloads as wl
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def ctx():
+    from paper_2401_07378_gb300 import nnsemd
+    c = nnsemd.Context(0)
+    yield c
+    c.close()
+
+
+def dev(a, dt):
+    return torch.from_numpy(np.ascontiguousarray(a)).to(device="cuda", dtype=dt)
+
+
+def check(ctx, p, metric="l2", **kw):
+    r = oracle.solve_pair(p, metric, threads=0, protocol=kw.get("protocol", "greedy"), seed=kw.get("seed", 0))
+    got = ctx.solve(dev(p.x, torch.float32), dev(p.a, torch.float64), dev(p.y, torch.float32),
+                    dev(p.b, torch.float64), metric=metric, plan=True, **kw)
+    assert got.cost == r.cost and got.stats["rounds"] == r.rounds and got.stats["pair_evals"] == r.pair_evals
+    assert sorted(zip(got.plan_i.tolist(), got.plan_j.tolist(), got.plan_f.tolist())) == sorted(
+        zip(r.plan_i.tolist(), r.plan_j.tolist(), r.plan_f.tolist()))
+    return got
+
+
+@pytest.mark.parametrize("m,n,d", [(1, 1, 9), (1, 2048, 9), (2048, 1, 33), (64, 65, 16), (17, 9, 300), (2048, 2048, 12),
+                                   (2049, 700, 20), (1000, 2047, 10)])
+@pytest.mark.parametrize("metric", ["l2", "l1"])
+def test_tail_equals_oracle(ctx, m, n, d, metric):
+    p = wl.uniform_pair(m, n, d, m + 3 * n + d, "dirichlet")
+    if m > 2:
+        p.a[::7] = 0.0
+        p.x[: m // 2] = np.round(p.x[: m // 2] * 2) / 2
+    if n > 2:
+        p.y[: n // 2] = np.round(p.y[: n // 2] * 2) / 2
+    check(ctx, p, metric)
+    check(ctx, p, metric, protocol="random", seed=5)
+
+
+@pytest.mark.parametrize("precision,d,rk", [("bf16x3", 64, 8), ("bf16x3", 50, 0), ("fp16", 33, 3), ("bf16", 20, 1),
+                                            ("fp8", 9, 16)])
+def test_reduced_precision_before_the_tail(ctx, precision, d, rk):
+    p = wl.gmm_pair(3, n=2600, d=d, components=40)
+    p.a[::9] = 0.0
+    st = check(ctx, p, precision=precision, rerank_k=rk).stats
+    assert st["certified"] + st["fallbacks"] > 0
