@@ -140,8 +140,10 @@ int ensure_ws(nnsemd_ctx* ctx, size_t bytes) {
 }
 
 // Lay out the buffers of a single-pair solve; with base == nullptr only the
-// size is computed.  `tail`: with the key matrix of the d > 8 cluster tail.
-size_t layout_solve(void* base, int64_t m, int64_t n, int d, SolveBufs& B, bool tail, int precision = 0,
+// size is computed.  `extras`: with the buffers of the faster steps that have a
+// plainer form behind them (the d > 8 cluster tail's key matrix, the d <= 3
+// grid), left out where the memory is short.
+size_t layout_solve(void* base, int64_t m, int64_t n, int d, SolveBufs& B, bool extras, int precision = 0,
                     const nnsemd_proposal* P = nullptr, LearnedBufs* L = nullptr) {
   Carve C(base);
   const int dp = d <= 8 ? padded_dim(d) : 0;
@@ -241,8 +243,18 @@ size_t layout_solve(void* base, int64_t m, int64_t n, int d, SolveBufs& B, bool 
   B.fl_j = C.take<int32_t>(m + n);
   B.fl_f = C.take<double>(m + n);
   B.blockcounts = C.take<int>((m + n) / 1024 + 8);
+  B.grid = GridBufs{};
+  if (extras && d <= 3 && m * n >= GRID_MIN_PAIRS) {
+    B.grid.box = C.take<unsigned>(6);
+    B.grid.hist = reinterpret_cast<int*>(C.take<uint8_t>(4 * grid_cells_bytes()));
+    B.grid.start = reinterpret_cast<int*>(C.take<uint8_t>(grid_cells_bytes()));
+    B.grid.xs = C.take<float>((size_t)m * 4);
+    B.grid.ys = C.take<float>((size_t)n * 4);
+    B.grid.boxes = C.take<float>(grid_box_floats(m));
+    B.grid.work = C.take<unsigned long long>(1);
+  }
   B.kmat = nullptr;
-  if (tail && d > 8)
+  if (extras && d > 8)
     B.kmat = C.take<float>((size_t)(std::min<int64_t>(m, FIN_MAX_HD) * kmat_ld(std::min<int64_t>(n, FIN_MAX_HD))));
   return C.off + 256;
 }
@@ -400,6 +412,7 @@ int run_solve(nnsemd_ctx* ctx, SolveBufs& B, const double* a, const double* b, d
     L += (linear_tc_supported(B.d) ? 3 + 3 * passes : 8) + (tch ? 1 : 0) + (tch && linear_tc_supported(B.d) ? 2 : 0) +
          (tcb ? 2 : 0) + (5 + (tcb ? 2 : 0) + 2 * sel) * ((B.n + learned->chunk - 1) / learned->chunk);
   }
+  bool boxed = false;  // the grid's bounding box is there
   while (mt > 0 && nt > 0) {
     // d > 8: the cluster tail takes over once both active sets fit it (with a
     // reduced precision or a proposal from the second round on: the first is
@@ -440,8 +453,18 @@ int run_solve(nnsemd_ctx* ctx, SolveBufs& B, const double* a, const double* b, d
       nrc = launch_nns_tc(B, B.tc, mt, nt, B.precision, st);
       L += 5;
     } else {
+      const bool grid = lowd && grid_nns_wanted(B, mt, nt);
       if (timed) CKD(cudaEventRecord(ctx->ev[0], st));
-      nrc = lowd ? launch_nns_lowd(B, mt, nt, st) : launch_nns_f32(B, mt, nt, nullptr, nullptr, st);
+      nrc = 0;
+      if (grid) {
+        if (!boxed) nrc = launch_grid_bounds(B, mt, nt, st);
+        if (!nrc) nrc = launch_nns_grid(B, mt, nt, st);
+        L += 5 + !boxed;
+        boxed = true;
+      }
+      if (!nrc)
+        nrc = lowd ? launch_nns_lowd(B, mt, nt, st, grid ? B.grid.work : nullptr)
+                   : launch_nns_f32(B, mt, nt, nullptr, nullptr, st);
       if (timed) CKD(cudaEventRecord(ctx->ev[1], st));
       L += 1;
     }
@@ -610,15 +633,15 @@ int nnsemd_solve(nnsemd_ctx* ctx, const float* x, const double* a, int64_t m, co
   CK(cudaSetDevice(ctx->device));
   SolveBufs B{};
   LearnedBufs Lb{};
-  bool tail = true;  // (without its key matrix where the memory is short)
-  rc = ensure_ws(ctx, layout_solve(nullptr, m, n, d, B, tail, precision, P, P ? &Lb : nullptr));
-  if (rc == NNSEMD_ERR_OOM && d > 8) {
-    tail = false;
+  bool extras = true;
+  rc = ensure_ws(ctx, layout_solve(nullptr, m, n, d, B, extras, precision, P, P ? &Lb : nullptr));
+  if (rc == NNSEMD_ERR_OOM) {
+    extras = false;
     ctx->err.clear();
-    rc = ensure_ws(ctx, layout_solve(nullptr, m, n, d, B, tail, precision, P, P ? &Lb : nullptr));
+    rc = ensure_ws(ctx, layout_solve(nullptr, m, n, d, B, extras, precision, P, P ? &Lb : nullptr));
   }
   if (rc) return rc;
-  layout_solve(ctx->ws, m, n, d, B, tail, precision, P, P ? &Lb : nullptr);
+  layout_solve(ctx->ws, m, n, d, B, extras, precision, P, P ? &Lb : nullptr);
   B.x = x;
   B.y = y;
   B.m = m;
@@ -657,8 +680,8 @@ int nnsemd_solve_host(nnsemd_ctx* ctx, const float* x, const double* a, int64_t 
   // device staging for the inputs and the plan, placed after the solve buffers
   SolveBufs B{};
   LearnedBufs Lb{};
-  bool tail = true;
-  size_t solve_bytes = layout_solve(nullptr, m, n, d, B, tail, precision, P, P ? &Lb : nullptr);
+  bool extras = true;
+  size_t solve_bytes = layout_solve(nullptr, m, n, d, B, extras, precision, P, P ? &Lb : nullptr);
   const int64_t cap = plan ? std::min<int64_t>(plan->capacity, m + n) : 0;
   auto stage_layout = [&](void* base, float** xd, double** ad, float** yd, double** bd, int32_t** pi, int32_t** pj,
                           double** pf) {
@@ -677,14 +700,14 @@ int nnsemd_solve_host(nnsemd_ctx* ctx, const float* x, const double* a, int64_t 
   double *ad, *bd, *pf;
   int32_t *pi, *pj;
   rc = ensure_ws(ctx, stage_layout(nullptr, &xd, &ad, &yd, &bd, &pi, &pj, &pf));
-  if (rc == NNSEMD_ERR_OOM && d > 8) {  // without the tail's key matrix
-    tail = false;
-    solve_bytes = layout_solve(nullptr, m, n, d, B, tail, precision, P, P ? &Lb : nullptr);
+  if (rc == NNSEMD_ERR_OOM) {
+    extras = false;
+    solve_bytes = layout_solve(nullptr, m, n, d, B, extras, precision, P, P ? &Lb : nullptr);
     ctx->err.clear();
     rc = ensure_ws(ctx, stage_layout(nullptr, &xd, &ad, &yd, &bd, &pi, &pj, &pf));
   }
   if (rc) return rc;
-  layout_solve(ctx->ws, m, n, d, B, tail, precision, P, P ? &Lb : nullptr);
+  layout_solve(ctx->ws, m, n, d, B, extras, precision, P, P ? &Lb : nullptr);
   stage_layout(ctx->ws, &xd, &ad, &yd, &bd, &pi, &pj, &pf);
   cudaStream_t st = ctx->stream;
   CK(cudaMemcpyAsync(xd, x, (size_t)m * d * sizeof(float), cudaMemcpyHostToDevice, st));
@@ -851,12 +874,12 @@ static int solve_batched_impl(nnsemd_ctx* ctx, int32_t num_pairs, const float* x
     maxn = std::max(maxn, y_len(p));
   }
   SolveBufs B{};
-  bool tail = true;
-  auto large_bytes = [&] { return large.empty() ? 0 : layout_solve(nullptr, maxm, maxn, d, B, tail, precision); };
+  bool extras = true;
+  auto large_bytes = [&] { return large.empty() ? 0 : layout_solve(nullptr, maxm, maxn, d, B, extras, precision); };
   rc = ensure_ws(ctx, layout_head(nullptr) + large_bytes());
-  if (rc == NNSEMD_ERR_OOM && d > 8) {  // without any key matrix
+  if (rc == NNSEMD_ERR_OOM) {  // without key matrices either
     kc_big = kc_tiny = 0;
-    tail = false;
+    extras = false;
     ctx->err.clear();
     rc = ensure_ws(ctx, layout_head(nullptr) + large_bytes());
   }
@@ -990,7 +1013,7 @@ static int solve_batched_impl(nnsemd_ctx* ctx, int32_t num_pairs, const float* x
   long long extra_rounds = 0, extra_pe = 0;
   long long extra_cert = 0, extra_fall = 0, extra_near = 0;
   for (int p : large) {
-    layout_solve((char*)ctx->ws + head, maxm, maxn, d, B, tail, precision);
+    layout_solve((char*)ctx->ws + head, maxm, maxn, d, B, extras, precision);
     B.x = x_packed + x_off[p] * d;
     B.y = y_packed + y_begin(p) * d;
     B.m = x_off[p + 1] - x_off[p];

@@ -54,6 +54,17 @@ struct TcBufs {
   cudaEvent_t ev0, ev1;        // optional: recorded around the tensor-core kernel
 };
 
+// Buffers of the spatially ordered NNS step (lowd_grid.cu, d <= 3).
+struct GridBufs {
+  unsigned* box;             // [6] bounding box of both sets (ordered bits); null: not laid out
+  int* hist;
+  int* start;
+  float* xs;                 // sorted suppliers / consumers, 4 floats a point
+  float* ys;
+  float* boxes;
+  unsigned long long* work;  // what the round's cells hold in common: the kernels' own choice of path
+};
+
 // Buffers of one single-pair solve (device pointers inside the workspace).
 struct SolveBufs {
   int precision;   // nnsemd_precision of the NNS step (0 = FP32)
@@ -61,6 +72,7 @@ struct SolveBufs {
   unsigned long long seed;  // random protocol seed
   long long round0;         // rounds run before the one-CTA tail (random-protocol keys)
   TcBufs tc;       // used when precision != 0
+  GridBufs grid;   // d <= 3
   const float* x;  // original coordinates [m][d]
   const float* y;  // [n][d]
   int64_t m, n;
@@ -112,7 +124,28 @@ int launch_initial_pack(SolveBufs& B, cudaStream_t st);
 int launch_big_round(SolveBufs& B, int mt, int nt, long long round, cudaStream_t st);
 
 // lowd.cu ------------------------------------------------------------------
-int launch_nns_lowd(const SolveBufs& B, int mt, int nt, cudaStream_t st);
+// `grid_work` (nullable): skip the scan where the grid step before it served
+// the round (its own rule on that value).
+int launch_nns_lowd(const SolveBufs& B, int mt, int nt, cudaStream_t st, const unsigned long long* grid_work = nullptr);
+
+// lowd_grid.cu -------------------------------------------------------------
+constexpr int64_t GRID_MIN_PAIRS = 1LL << 26;  // m_t * n_t from which a round takes the grid
+size_t grid_cells_bytes();
+size_t grid_box_floats(int64_t m);
+// The box of the initial active sets (once per solve, before the first grid
+// step).
+int launch_grid_bounds(const SolveBufs& B, int mt, int nt, cudaStream_t st);
+bool grid_nns_wanted(const SolveBufs& B, int mt, int nt);
+// Nearest active supplier of every active consumer into B.nnkey, or nothing
+// where the points share too few cells (launch_nns_lowd with B.grid.work then
+// scans).
+int launch_nns_grid(const SolveBufs& B, int mt, int nt, cudaStream_t st);
+// The rule, on the device (the cells' work is only known there): points that
+// share few cells leave every warp with a large part of the suppliers, and K1
+// scans those at about 1.7 times the rate.
+NNS_DEV bool grid_served(const unsigned long long* work, int mt, int nt) {
+  return *work <= (unsigned long long)mt * (unsigned)nt / 32;
+}
 // Run all remaining rounds of the current active lists in one CTA.
 int launch_finish(const SolveBufs& B, int64_t round_limit, cudaStream_t st);
 // The same on a thread-block cluster (k_finish_cl), for active sets of at
