@@ -145,12 +145,12 @@ typedef struct {
   int64_t kernel_launches;      /* CUDA kernels this call launched */
   double nns_kernel_ms;         /* NNSEMD_FLAG_TIME_KERNELS: summed duration of the multi-CTA NNS launches */
   int64_t nns_kernel_launches;  /* number of those launches */
-  int64_t nns_kernel_pairs;     /* sum of m_t * n_t they evaluated */
+  int64_t nns_kernel_pairs;     /* sum of m_t * n_t they evaluated (n_t: the consumers left to them) */
   double tail_kernel_ms;        /* NNSEMD_FLAG_TIME_KERNELS: duration of the one-CTA tail kernel */
   int64_t near_ties;            /* reduced precision: consumer searches whose exact FP32 re-rank picked
                                    another supplier than the one the operand-precision distances ranked
-                                   first (ties at that precision); in a batch, of the searches that made
-                                   a candidate list.  0 on the FP32 paths: their decisions
+                                   first (ties at that precision), of the searches that made a candidate
+                                   list.  0 on the FP32 paths: their decisions
                                    are the FP32 decisions themselves (the FP32 / FP64 near-ties of the
                                    method are the oracle's to count). */
   int64_t widened;              /* learned proposal: consumer searches certified by the second tier (the

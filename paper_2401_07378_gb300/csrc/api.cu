@@ -243,6 +243,15 @@ size_t layout_solve(void* base, int64_t m, int64_t n, int d, SolveBufs& B, bool 
   B.fl_j = C.take<int32_t>(m + n);
   B.fl_f = C.take<double>(m + n);
   B.blockcounts = C.take<int>((m + n) / 1024 + 8);
+  B.lists = TcLists{};
+  if (extras && precision != NNSEMD_FP32 && !P) {
+    B.lists.list = C.take<unsigned long long>((size_t)n * TCL);
+    B.lists.next = C.take<int>(n);
+    B.lists.floor = C.take<double>(n);
+    B.lists.pos = C.take<int>(m);
+    B.lists.sel = C.take<int>(n);
+    B.lists.nsel = C.take<int>(1);
+  }
   B.grid = GridBufs{};
   if (extras && d <= 3 && m * n >= GRID_MIN_PAIRS) {
     B.grid.box = C.take<unsigned>(6);
@@ -440,6 +449,8 @@ int run_solve(nnsemd_ctx* ctx, SolveBufs& B, const double* a, const double* b, d
     // B.nnkey[0 .. nt) is all ones here: the compaction that produced the
     // active lists reset the key of every surviving consumer
     int nrc;
+    bool nns_timed = timed;
+    long long evals = (long long)mt * nt;  // pairs the NNS kernels evaluate
     if (learned) {
       if (timed) CKD(cudaEventRecord(ctx->ev[0], st));
       nrc = launch_nns_learned(B, *learned, mt, nt, st);
@@ -447,11 +458,35 @@ int run_solve(nnsemd_ctx* ctx, SolveBufs& B, const double* a, const double* b, d
       L += learned_cell_scan(B.d, B.x, B.y) ? 11 : 6;
     } else if (B.precision != NNSEMD_FP32) {
       // tensor-core candidates + exact re-rank + certificate + FP32 rescan;
-      // the timing events bracket the tensor-core kernel alone
+      // the timing events bracket the tensor-core kernel alone.  After the
+      // first round for the consumers that their candidate lists leave open.
       B.tc.ev0 = timed ? ctx->ev[0] : nullptr;
       B.tc.ev1 = timed ? ctx->ev[1] : nullptr;
-      nrc = launch_nns_tc(B, B.tc, mt, nt, B.precision, st);
-      L += 5;
+      if (B.lists.list && rounds > 0) {
+        volatile int* left = ctx->hmap + 9;  // pinned
+        if (launch_serve_lists(B, mt, nt, st))
+          return drained(fail(ctx, NNSEMD_ERR_CUDA, "candidate lists"));
+        CKD(cudaMemcpyAsync((void*)left, B.lists.nsel, sizeof(int), cudaMemcpyDeviceToHost, st));
+        CKD(cudaStreamSynchronize(st));
+        const int nf = *left;
+        L += 2;
+        nrc = 0;
+        evals = (long long)mt * nf;
+        if (nf > TC_SCAN_MIN) {
+          nrc = launch_nns_tc(B, B.tc, mt, nf, B.precision, st, B.lists.sel, nullptr);
+          L += 5;
+        } else {
+          nns_timed = false;
+          if (nf > 0) {
+            launch_add_count(&B.st->fallbacks, (unsigned long long)nf, st);
+            nrc = launch_nns_f32(B, mt, nf, B.lists.sel, nullptr, st);
+            L += 2;
+          }
+        }
+      } else {
+        nrc = launch_nns_tc(B, B.tc, mt, nt, B.precision, st);
+        L += 5;
+      }
     } else {
       const bool grid = lowd && grid_nns_wanted(B, mt, nt);
       if (timed) CKD(cudaEventRecord(ctx->ev[0], st));
@@ -481,11 +516,11 @@ int run_solve(nnsemd_ctx* ctx, SolveBufs& B, const double* a, const double* b, d
     rounds += 1;
     pair_evals += (long long)mt * nt;
     nns_launches += 1;
-    nns_pairs += (long long)mt * nt;
+    nns_pairs += evals;
     unsigned err_bits = 0;
     rc = wait_counts(ctx, st, B.notify_seq, mt, nt, err_bits);
     if (rc) return drained(rc);
-    if (timed) {
+    if (nns_timed) {
       float ms = 0.f;
       CKD(cudaEventSynchronize(ctx->ev[1]));
       CKD(cudaEventElapsedTime(&ms, ctx->ev[0], ctx->ev[1]));

@@ -54,6 +54,20 @@ struct TcBufs {
   cudaEvent_t ev0, ev1;        // optional: recorded around the tensor-core kernel
 };
 
+// Candidate lists kept over the rounds of a reduced-precision solve (tc.cu), by
+// original consumer: up to TCL exact keys (key32 bits << 32 | original
+// supplier) ascending, the next entry to look at | length << 8, and the value a
+// key must stay below to be the nearest active supplier's.
+constexpr int TCL = 8;
+struct TcLists {
+  unsigned long long* list;  // [n][TCL]; null: no lists
+  int* next;                 // [n]
+  double* floor;             // [n]
+  int* pos;                  // [m] position of each active supplier by original index (others: stale)
+  int* sel;                  // [n] consumer positions the lists do not answer
+  int* nsel;
+};
+
 // Buffers of the spatially ordered NNS step (lowd_grid.cu, d <= 3).
 struct GridBufs {
   unsigned* box;             // [6] bounding box of both sets (ordered bits); null: not laid out
@@ -72,6 +86,7 @@ struct SolveBufs {
   unsigned long long seed;  // random protocol seed
   long long round0;         // rounds run before the one-CTA tail (random-protocol keys)
   TcBufs tc;       // used when precision != 0
+  TcLists lists;   // used when precision != 0 and no proposal
   GridBufs grid;   // d <= 3
   const float* x;  // original coordinates [m][d]
   const float* y;  // [n][d]
@@ -261,6 +276,13 @@ int cell_bounds_tc(const float* y, int rows, int d, uint8_t* packed_y, float* y_
 // certificate, FP32 rescan of the rest.  Writes B.nnkey (must be all ones).
 int launch_nns_tc(const SolveBufs& B, const TcBufs& T, int mt, int nt, int precision, cudaStream_t st,
                   const int* sel = nullptr, const int* nsel_dev = nullptr);
+// Answers what it can of a round from B.lists (two launches); the other
+// consumers' positions go to B.lists.sel, their number to *B.lists.nsel.
+int launch_serve_lists(const SolveBufs& B, int mt, int nt, cudaStream_t st);
+// Consumers at or below which a full scan runs in FP32 rather than on the
+// tensor cores (packing every active supplier costs more).
+constexpr int TC_SCAN_MIN = 256;
+void launch_add_count(unsigned long long* ctr, unsigned long long v, cudaStream_t st);
 
 // batched_tc.cu: batches of pairs with up to `cap` points per side (FIN_MAX_HD;
 // batched_tc_max_stages also answers for HD_SMALL_CAP, 0: rows too long),

@@ -288,7 +288,6 @@ int assign_cells(const nnsemd_proposal* P, const float* pts, int64_t N, int* out
 // iota / key scratch for the nearest-centroid search live at the end of the
 // k-means scratch: assign_buf holds N ints, then N 64-bit keys follow the
 // sums array (sized by the caller: cells*d floats + cells ints + N keys).
-static int* g_dummy = nullptr;
 
 int kmeans_fit(nnsemd_proposal* P, const float* pts, int64_t N, int iters, uint64_t seed, int* assign_buf,
                float* sums, int* counts, cudaStream_t st) {
@@ -314,7 +313,6 @@ int kmeans_fit(nnsemd_proposal* P, const float* pts, int64_t N, int iters, uint6
     k_km_accum<<<num_sms() * 8, 256, 0, st>>>(pts, N, d, assign_buf, sums, counts);
     k_km_divide<<<(K * d + 255) / 256, 256, 0, st>>>(P->centroids, sums, counts, K, d);
   }
-  (void)g_dummy;
   return 0;
 }
 
@@ -1186,12 +1184,6 @@ __global__ void __launch_bounds__(256) k_learned_widen(LcArgs A, const int* __re
   }
 }
 
-// Consumers left after the second tier at or below which the full scan
-// runs in FP32 rather than on the tensor cores.
-constexpr int LC_TC_MIN = 256;
-
-__global__ void k_add_count(unsigned long long* ctr, unsigned long long v) { *ctr += v; }
-
 bool learned_cell_scan(int d, const float* x, const float* y) {
   return (d == 32 || d == 64 || d == 128) && ((reinterpret_cast<uintptr_t>(x) | reinterpret_cast<uintptr_t>(y)) & 15) == 0;
 }
@@ -1240,12 +1232,12 @@ int launch_nns_learned(const SolveBufs& B, const LearnedBufs& L, int mt, int nt,
       if (nf > 0 && (cudaMemcpyAsync(&nf2, L.nfallback2, sizeof(int), cudaMemcpyDeviceToHost, st) != cudaSuccess ||
                      cudaStreamSynchronize(st) != cudaSuccess))
         return -1;
-      if (nf2 > LC_TC_MIN) {
+      if (nf2 > TC_SCAN_MIN) {
         if (launch_nns_tc(B, B.tc, mt, nf2, B.precision, st, L.fallback2, nullptr)) return -1;
       } else if (nf2 > 0) {
         // a few consumers: the FP32 scan costs less than packing every
         // active supplier for the tensor cores (counted as fallbacks)
-        k_add_count<<<1, 1, 0, st>>>(&B.st->fallbacks, (unsigned long long)nf2);
+        launch_add_count(&B.st->fallbacks, (unsigned long long)nf2, st);
         launch_nns_f32(B, mt, nt, L.fallback2, L.nfallback2, st);
       }
     }

@@ -54,3 +54,19 @@ def test_reduced_precision_before_the_tail(ctx, precision, d, rk):
     p.a[::9] = 0.0
     st = check(ctx, p, precision=precision, rerank_k=rk).stats
     assert st["certified"] + st["fallbacks"] > 0
+
+
+@pytest.mark.parametrize("m,n,d,precision,rk", [(7000, 6500, 64, "bf16x3", 8), (7000, 7000, 33, "fp16", 0),
+                                                (1000, 5000, 32, "bf16x3", 1), (900, 6000, 50, "bf16", 1),
+                                                (5000, 3000, 20, "fp8", 2)])
+def test_candidate_lists_over_the_rounds(ctx, m, n, d, precision, rk):
+    big = wl.gmm_pair(7, n=max(m, n), d=d, components=60)
+    p = wl.Pair(big.x[:m].copy(), big.a[:m], big.y[:n].copy(), big.b[:n])
+    p.x[::3] = np.round(p.x[::3])  # equal points and keys
+    p.y[::3] = np.round(p.y[::3])
+    r = oracle.solve_pair(p, "l2", threads=0)
+    st = check(ctx, p, precision=precision, rerank_k=rk).stats
+    # every search of the rounds before the tail is counted once
+    rounds = st["nns_kernel_launches"]
+    assert rounds >= 2
+    assert st["certified"] + st["fallbacks"] == int(r.n_t[:rounds].sum())
