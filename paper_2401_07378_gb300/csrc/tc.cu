@@ -760,17 +760,33 @@ int launch_nns_tc(const SolveBufs& B, const TcBufs& T, int mt, int nt, int preci
                                                                   B.d, kb, fmt, bn, T.B, T.nrm_x, T.nrm_sx, T.scale_x,
                                                                   T.stats);
   }
-  // chunks of supplier tiles so that the grid covers the GPU several times
-  int chunks = (tc_target_ctas() + qtiles - 1) / qtiles;
-  if (chunks > stiles) chunks = stiles;
-  if (chunks > T.max_chunks) chunks = T.max_chunks;
+  // candidates re-ranked per chunk; the scan keeps half the lists when that suffices
+  const int rk = T.rerank_k >= 1 && T.rerank_k <= TC_K ? T.rerank_k : TC_K;
+  const int kl = rk <= TC_K / 2 ? TC_K / 2 : TC_K;
+  // Chunks of supplier tiles: waves of CTAs (one per SM) x (tiles of a CTA +
+  // what a CTA costs beside its tiles, about six of them), smallest first.
+  // Aiming at four CTAs per SM alone left a fifth, nearly empty wave (49
+  // consumer tiles x 13 chunks = 637 CTAs).  More chunks also mean more
+  // candidates to re-rank: another count has to save 3 %.
+  int chunks = 1;
+  {
+    // (what the candidate buffers hold: layout_solve)
+    const int most = std::min(std::min(stiles, T.max_chunks), (tc_target_ctas() + qtiles) * TC_K / kl / qtiles);
+    double best = 1e30;
+    for (int c = 1; c <= most; ++c) {
+      const int tiles = (stiles + c - 1) / c;
+      const int64_t ctas = (int64_t)qtiles * ((stiles + tiles - 1) / tiles);
+      const double t = (double)((ctas + num_sms() - 1) / num_sms()) * (tiles + 6);
+      if (t < 0.97 * best) {
+        best = t;
+        chunks = c;
+      }
+    }
+  }
   const int per = (stiles + chunks - 1) / chunks;
   chunks = (stiles + per - 1) / per;
   const size_t a_bytes = (size_t)TC_BM * kb, b_bytes = (size_t)bn * kb;
   const int nt_pad = qtiles * TC_BM;
-  // candidates re-ranked per chunk; the scan keeps half the lists when that suffices
-  const int rk = T.rerank_k >= 1 && T.rerank_k <= TC_K ? T.rerank_k : TC_K;
-  const int kl = rk <= TC_K / 2 ? TC_K / 2 : TC_K;
   TcArgs P{T.A,      T.B,      T.nrm_x,    T.nrm_sx, T.nrm_y,  T.scale_x,  T.scale_y, nt, mt,
            kb,       bn,       0,          per,      stiles,   nt_pad,     T.cand_v,  T.cand_p, &B.st->err,
            nsel_dev};
