@@ -188,6 +188,7 @@ __global__ void __launch_bounds__(tc_threads(FMT, KL), 1) k_nns_tc(TcArgs P) {
   // parts 1.. of each row, merged into part 0's)
   __shared__ __align__(16) float stage[16][EW * 32];
   __shared__ int tag_pos[TagList<KL>::NTAG][EW * 32];  // per epilogue thread: tag -> position
+  __shared__ float seen[PARTS][TC_BM];  // per row and part: its KL / PARTS-th smallest value so far (rounded up)
   static_assert(2 * (PARTS - 1) * KL * TC_BM <= 16 * EW * 32, "the merge lists fit in the staging area");
   float* const merge_v = &stage[0][0];                                              // [PARTS-1][KL][TC_BM]
   int* const merge_p = reinterpret_cast<int*>(&stage[0][0]) + (PARTS - 1) * KL * TC_BM;  // same shape
@@ -303,6 +304,15 @@ __global__ void __launch_bounds__(tc_threads(FMT, KL), 1) k_nns_tc(TcArgs P) {
     unsigned used = 0u;  // tags held by entries of the list
 #pragma unroll
     for (int k = 0; k < KL; ++k) tv[k] = CUDART_INF_F;
+    // The row's parts hold KL / PARTS values each at or below the largest of
+    // their `seen`, so nothing above that can be among the row's KL smallest:
+    // it filters with a row's own list of all columns, not of a part's (about
+    // a third of the insertions).  A stale value of another part is larger.
+    constexpr int SEEN = KL / PARTS - 1;
+    volatile float* const mine = &seen[part][row];
+    *mine = CUDART_INF_F;
+    asm volatile("bar.sync 1, %0;" ::"r"(EW * 32) : "memory");
+    float lim = CUDART_INF_F;
     int* const table = &tag_pos[0][etid];
     constexpr int TSTRIDE = EW * 32;
     for (int t = 0; t < ntiles; ++t) {
@@ -357,11 +367,11 @@ __global__ void __launch_bounds__(tc_threads(FMT, KL), 1) k_nns_tc(TcArgs P) {
           const float mn =
               fminf(fmin3(fmin3(val[0], val[1], val[2]), fmin3(val[3], val[4], val[5]), fmin3(val[6], val[7], val[8])),
                     fmin3(fmin3(val[9], val[10], val[11]), fmin3(val[12], val[13], val[14]), val[15]));
-          if (mn < tv[KL - 1]) {
+          if (mn < lim) {
             // the few columns that beat the current K-th entry: park the
             // block's values, then one (rolled) insertion per such column
             // that still beats it
-            const float thr = tv[KL - 1];
+            const float thr = lim;
             unsigned msk = 0;
 #pragma unroll
             for (int k = 0; k < 16; ++k) {
@@ -373,11 +383,19 @@ __global__ void __launch_bounds__(tc_threads(FMT, KL), 1) k_nns_tc(TcArgs P) {
               const int k = __ffs(msk) - 1;
               msk &= msk - 1;
               const float vk = stage[k][etid];
-              if (vk < tv[KL - 1]) tag_insert<KL>(tv, used, table, TSTRIDE, vk, tile * BN + c0 + k);
+              if (vk < lim) {
+                tag_insert<KL>(tv, used, table, TSTRIDE, vk, tile * BN + c0 + k);
+                lim = fminf(lim, tv[KL - 1]);
+              }
             }
+            if (tv[SEEN] < CUDART_INF_F) *mine = tag_ceil(tv[SEEN], TagList<KL>::MASK);
           }
         }
       }
+      float m = *const_cast<volatile float*>(&seen[0][row]);
+#pragma unroll
+      for (int u = 1; u < PARTS; ++u) m = fmaxf(m, *const_cast<volatile float*>(&seen[u][row]));
+      lim = fminf(tv[KL - 1], m);
       tc_fence_before();
       __syncwarp();
       if (lane == 0) {

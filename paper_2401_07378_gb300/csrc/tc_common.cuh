@@ -295,6 +295,12 @@ __host__ __device__ inline float tag_floor(float v, unsigned mask) {
   return f32_of_bits((u & 0x80000000u) ? (u | mask) : (u & ~mask));
 }
 
+// The largest value that shares the entry's other bits: at least its exact one.
+__host__ __device__ inline float tag_ceil(float v, unsigned mask) {
+  const unsigned u = f32_bits(v);
+  return f32_of_bits((u & 0x80000000u) ? (u & ~mask) : (u | mask));
+}
+
 // Insert value v (finite) of supplier position pos: a free tag takes the
 // position, the tagged value c enters the ascending list, and the entry
 // pushed out (+inf while the list is not full, or c itself when it is above
