@@ -42,7 +42,15 @@ __host__ __device__ constexpr int tc_threads(int fmt, int kl) { return 32 * (3 +
 // what the instantiation actually has left.
 constexpr int TC_SMEM_BUDGET = 150 * 1024;
 constexpr int TC_SMEM_MAX = 227 * 1024;  // per block, static + dynamic
-constexpr int TC_NACC = 4;                  // FP32 accumulators in tensor memory (a ring of tiles in flight)
+// The consumer tile (A) of the 16-bit formats lies in tensor memory: a 128 x
+// 128 x 16 step reads as many bytes of A as of B from shared memory otherwise,
+// and shared-memory bandwidth is what bounds K2 (at 32,768 points a tile of K =
+// 192 took 3,046 cycles: 768 of operand reads, 384 of copies and some 1,450
+// of epilogue accesses).
+__host__ __device__ constexpr bool tc_a_in_tmem(int fmt) { return fmt != FMT_E4M3; }
+// FP32 accumulators in tensor memory (a ring of tiles in flight); beside three
+// of 128 columns A has 128 columns, 512 bytes a row.
+__host__ __device__ constexpr int tc_nacc(int fmt, int bn) { return tc_a_in_tmem(fmt) && bn == 128 ? 3 : 4; }
 constexpr int TC_NNRM = 4;                  // column-norm slots (a ring of its own, loaded ahead)
 
 // Packs rows in groups of PACK_ROWS: a warp reads its rows (coalesced) into
@@ -171,6 +179,8 @@ struct TcArgs {
 template <int FMT, int BN, int KL>
 __global__ void __launch_bounds__(tc_threads(FMT, KL), 1) k_nns_tc(TcArgs P) {
   constexpr int EW = tc_epi_warps(FMT, KL);
+  constexpr bool ATM = tc_a_in_tmem(FMT);
+  constexpr int TC_NACC = tc_nacc(FMT, BN);
   constexpr int PARTS = EW / 4;      // epilogue warps per TMEM lane quarter
   constexpr int CPART = BN / PARTS;  // columns of a tile per epilogue warp
   static_assert(CPART % 16 == 0, "whole 16-column blocks per epilogue warp");
@@ -204,11 +214,11 @@ __global__ void __launch_bounds__(tc_threads(FMT, KL), 1) k_nns_tc(TcArgs P) {
   const uint32_t a_bytes = TC_BM * kb;
   const uint32_t b_bytes = BN * kb;
   uint8_t* sA = smem;
-  uint8_t* sB = smem + a_bytes;
+  uint8_t* sB = ATM ? smem : smem + a_bytes;
   const int NST = P.nstage;
   constexpr uint32_t NCOLS = TC_NACC * BN;  // the accumulator ring
-  constexpr uint32_t TMEM_ALLOC = NCOLS < 32 ? 32 : NCOLS;
-  static_assert(NCOLS <= 512 && (NCOLS & (NCOLS - 1)) == 0, "tensor memory holds 512 columns");
+  constexpr uint32_t TMEM_ALLOC = ATM ? 512 : NCOLS;  // (A from column NCOLS on: kb / 4 columns)
+  static_assert(NCOLS <= 512 && (ATM || (NCOLS & (NCOLS - 1)) == 0), "tensor memory holds 512 columns");
   constexpr uint32_t NRM_BYTES = 3 * BN * sizeof(float);
 
   if (threadIdx.x == 0) {
@@ -233,12 +243,31 @@ __global__ void __launch_bounds__(tc_threads(FMT, KL), 1) k_nns_tc(TcArgs P) {
   tc_fence_after();
   const uint32_t tmem_base = tmem_slot;
   bool ok = true;
+  if (ATM) {
+    // four warps bring A into tensor memory, a quarter of its rows each
+    if (warp >= 4 && warp < 8) {
+      const int quarter = warp & 3;
+      const uint4* src = reinterpret_cast<const uint4*>(P.A + (size_t)qtile * a_bytes) + quarter * 32 + lane;
+      const uint32_t dst = tmem_base + ((uint32_t)(quarter * 32) << 16) + NCOLS;
+      for (int c = 0; c < kb / 16; c += 2) {  // (kb is a multiple of 32)
+        const uint4 u = src[(size_t)c * TC_BM], v = src[(size_t)(c + 1) * TC_BM];
+        tmem_st4(dst + 4 * c, u);
+        tmem_st4(dst + 4 * c + 4, v);
+      }
+      tmem_st_wait();
+    }
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+  }
 
   if (warp == 0) {
     // ---------------- producer: TMA bulk copies of the operand tiles ----------------
     if (lane == 0) {
-      mbar_expect_tx(&bar_a, a_bytes);
-      tma_load_1d(sA, P.A + (size_t)qtile * a_bytes, a_bytes, &bar_a);
+      if (!ATM) {
+        mbar_expect_tx(&bar_a, a_bytes);
+        tma_load_1d(sA, P.A + (size_t)qtile * a_bytes, a_bytes, &bar_a);
+      }
       for (int t = 0; t < ntiles && ok; ++t) {
         const int s = t % NST, u = t / NST;
         ok = mbar_wait_sleep(&bar_empty[s], (u & 1) ^ 1);
@@ -253,7 +282,7 @@ __global__ void __launch_bounds__(tc_threads(FMT, KL), 1) k_nns_tc(TcArgs P) {
       constexpr int AB = fmt_is_bf16(FMT) ? 1 : 0;
       const uint32_t idesc = make_idesc(AB, TC_BM, BN);
       const int ksteps = kb / 32;
-      ok = mbar_wait_bounded(&bar_a, 0);
+      if (!ATM) ok = mbar_wait_bounded(&bar_a, 0);
       const uint32_t a0 = smem_u32(sA);
       for (int t = 0; t < ntiles && ok; ++t) {
         const int s = t % NST, u = t / NST;
@@ -265,9 +294,13 @@ __global__ void __launch_bounds__(tc_threads(FMT, KL), 1) k_nns_tc(TcArgs P) {
         const uint32_t b0 = smem_u32(sB + (size_t)s * b_bytes);
         const uint32_t tmem_d = tmem_base + (uint32_t)(b * BN);
         for (int k = 0; k < ksteps; ++k) {
-          const uint64_t ad = make_desc(a0 + k * 2 * TC_BM * 16, TC_BM * 16, 128);
           const uint64_t bd = make_desc(b0 + k * 2 * BN * 16, BN * 16, 128);
-          mma_issue<FMT>(tmem_d, ad, bd, idesc, k > 0 ? 1u : 0u);
+          if constexpr (ATM) {
+            mma_issue_atm(tmem_d, tmem_base + NCOLS + 8 * k, bd, idesc, k > 0 ? 1u : 0u);
+          } else {
+            const uint64_t ad = make_desc(a0 + k * 2 * TC_BM * 16, TC_BM * 16, 128);
+            mma_issue<FMT>(tmem_d, ad, bd, idesc, k > 0 ? 1u : 0u);
+          }
         }
         mma_commit(&bar_empty[s]);
         mma_commit(&bar_acc_full[b]);
@@ -679,6 +712,10 @@ static int launch_tc_t(TcArgs P, dim3 grid, size_t a_bytes, size_t b_bytes, cuda
   }();
   if (static_smem < 0) return -1;
   const size_t avail = (size_t)(TC_SMEM_MAX - 1024 - static_smem);
+  if (tc_a_in_tmem(FMT)) {
+    if (tc_nacc(FMT, BN) * BN + a_bytes / TC_BM / 4 > 512) return -2;  // (tc_supported keeps rows below 1,024 bytes)
+    a_bytes = 0;
+  }
   if (a_bytes + b_bytes > avail) return -2;
   P.nstage = (int)std::min<size_t>(4, (avail - a_bytes) / b_bytes);
   const size_t smem = a_bytes + (size_t)P.nstage * b_bytes;
