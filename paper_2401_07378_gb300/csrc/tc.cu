@@ -42,6 +42,11 @@ __host__ __device__ constexpr int tc_threads(int fmt, int kl) { return 32 * (3 +
 // what the instantiation actually has left.
 constexpr int TC_SMEM_BUDGET = 150 * 1024;
 constexpr int TC_SMEM_MAX = 227 * 1024;  // per block, static + dynamic
+// The epilogue warps work in groups on alternate tiles: a warp's visit to a tile
+// is a chain of waits and loads, and with every warp on every tile that chain
+// (1,830 cycles), not the MMAs (768 at K = 192) or the shared memory, set the
+// pace.
+constexpr int TC_GROUPS = 2;
 // The consumer tile (A) of the 16-bit formats lies in tensor memory: a 128 x
 // 128 x 16 step reads as many bytes of A as of B from shared memory otherwise,
 // and shared-memory bandwidth is what bounds K2 (at 32,768 points a tile of K =
@@ -181,14 +186,18 @@ __global__ void __launch_bounds__(tc_threads(FMT, KL), 1) k_nns_tc(TcArgs P) {
   constexpr int EW = tc_epi_warps(FMT, KL);
   constexpr bool ATM = tc_a_in_tmem(FMT);
   constexpr int TC_NACC = tc_nacc(FMT, BN);
-  constexpr int PARTS = EW / 4;      // epilogue warps per TMEM lane quarter
-  constexpr int CPART = BN / PARTS;  // columns of a tile per epilogue warp
-  static_assert(CPART % 16 == 0, "whole 16-column blocks per epilogue warp");
+  constexpr int PARTS = EW / 4;               // epilogue warps per TMEM lane quarter, lists per row
+  constexpr int GW = EW / TC_GROUPS;          // epilogue warps that take a tile
+  constexpr int CPART = BN * TC_GROUPS / PARTS;  // columns of a tile per epilogue warp
+  static_assert(CPART % 32 == 0, "whole pairs of 16-column blocks per epilogue warp");
   extern __shared__ __align__(1024) uint8_t smem[];
   __shared__ __align__(8) uint64_t bar_full[8];
   __shared__ __align__(8) uint64_t bar_empty[8];
-  __shared__ __align__(8) uint64_t bar_acc_full[TC_NACC];
-  __shared__ __align__(8) uint64_t bar_acc_empty[TC_NACC];
+  // an accumulator's barriers alternate between two sets, so that a barrier
+  // belongs to tiles of one group and its phases are waited for one by one
+  constexpr int NABAR = TC_GROUPS * TC_NACC;
+  __shared__ __align__(8) uint64_t bar_acc_full[NABAR];
+  __shared__ __align__(8) uint64_t bar_acc_empty[NABAR];
   __shared__ __align__(8) uint64_t bar_nrm_full[TC_NNRM];
   __shared__ __align__(8) uint64_t bar_nrm_empty[TC_NNRM];
   __shared__ __align__(8) uint64_t bar_a;
@@ -226,13 +235,13 @@ __global__ void __launch_bounds__(tc_threads(FMT, KL), 1) k_nns_tc(TcArgs P) {
       mbar_init(&bar_full[s], 1);
       mbar_init(&bar_empty[s], 1);
     }
-    for (int b = 0; b < TC_NACC; ++b) {
+    for (int b = 0; b < NABAR; ++b) {
       mbar_init(&bar_acc_full[b], 1);
-      mbar_init(&bar_acc_empty[b], EW);  // one arrival per epilogue warp
+      mbar_init(&bar_acc_empty[b], GW);  // one arrival per epilogue warp of the group
     }
     for (int n = 0; n < TC_NNRM; ++n) {
       mbar_init(&bar_nrm_full[n], 1);
-      mbar_init(&bar_nrm_empty[n], EW);
+      mbar_init(&bar_nrm_empty[n], GW);
     }
     mbar_init(&bar_a, 1);
     mbar_fence_init();
@@ -286,9 +295,9 @@ __global__ void __launch_bounds__(tc_threads(FMT, KL), 1) k_nns_tc(TcArgs P) {
       const uint32_t a0 = smem_u32(sA);
       for (int t = 0; t < ntiles && ok; ++t) {
         const int s = t % NST, u = t / NST;
-        const int b = t % TC_NACC, v = t / TC_NACC;
+        const int b = t % TC_NACC, f = t - TC_NACC;  // f: the tile that had this accumulator
         ok = mbar_wait_sleep(&bar_full[s], u & 1);
-        if (ok) ok = mbar_wait_sleep(&bar_acc_empty[b], (v & 1) ^ 1);
+        if (ok && f >= 0) ok = mbar_wait_sleep(&bar_acc_empty[f % NABAR], (f / NABAR) & 1);
         if (!ok) break;
         tc_fence_after();
         const uint32_t b0 = smem_u32(sB + (size_t)s * b_bytes);
@@ -303,7 +312,7 @@ __global__ void __launch_bounds__(tc_threads(FMT, KL), 1) k_nns_tc(TcArgs P) {
           }
         }
         mma_commit(&bar_empty[s]);
-        mma_commit(&bar_acc_full[b]);
+        mma_commit(&bar_acc_full[t % NABAR]);
       }
     }
   } else if (warp == 2) {
@@ -327,7 +336,8 @@ __global__ void __launch_bounds__(tc_threads(FMT, KL), 1) k_nns_tc(TcArgs P) {
     const int e = warp - 3;
     const int etid = e * 32 + lane;
     const int quarter = warp & 3;  // TMEM lanes 32*quarter .. +31
-    const int part = e >> 2;
+    const int part = e >> 2;                              // this warp's list of its rows
+    const int group = part / (PARTS / TC_GROUPS), cpart = part % (PARTS / TC_GROUPS);
     const int row = quarter * 32 + lane;
     const int q = qtile * TC_BM + row;
     const float sy = (q < P.nt) ? P.scale_y[q] : 1.f;
@@ -348,10 +358,11 @@ __global__ void __launch_bounds__(tc_threads(FMT, KL), 1) k_nns_tc(TcArgs P) {
     float lim = CUDART_INF_F;
     int* const table = &tag_pos[0][etid];
     constexpr int TSTRIDE = EW * 32;
-    for (int t = 0; t < ntiles; ++t) {
-      const int b = t % TC_NACC, v = t / TC_NACC;
+    static_assert(TC_NNRM % TC_GROUPS == 0, "a norm slot belongs to tiles of one group");
+    for (int t = group; t < ntiles; t += TC_GROUPS) {
+      const int b = t % TC_NACC, a = t % NABAR, v = t / NABAR;
       const int n = t % TC_NNRM, w = t / TC_NNRM;
-      if (ok) ok = mbar_wait_sleep(&bar_acc_full[b], v & 1, 200u);
+      if (ok) ok = mbar_wait_sleep(&bar_acc_full[a], v & 1, 200u);
       if (ok) ok = mbar_wait_sleep(&bar_nrm_full[n], w & 1, 200u);
       tc_fence_after();
       if (ok) {
@@ -359,69 +370,71 @@ __global__ void __launch_bounds__(tc_threads(FMT, KL), 1) k_nns_tc(TcArgs P) {
         const float* nx = nrm_buf[n][0];
         const float* ns = nrm_buf[n][1];
         const float* sx = nrm_buf[n][2];
-        // all of this warp's columns of the accumulator at once (one wait
-        // for NB loads in flight), then two columns per packed FP32x2 step
-        constexpr int NB = CPART / 16;
-        uint32_t rr[NB][16];
-#pragma unroll
-        for (int bb = 0; bb < NB; ++bb)
-          tmem_ld16_async(tmem_base + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(b * BN + part * CPART + 16 * bb),
-                          rr[bb]);
-        tmem_ld_wait(rr);
+        // 32 of this warp's columns of the accumulator at once (one wait for
+        // two loads in flight), then two columns per packed FP32x2 step
+        constexpr int NB = 2;
         const unsigned long long mcy2 = f2_pack(-cy, -cy);
         const unsigned long long w2c = f2_pack(-2.f, -2.f);
         const unsigned long long wsy2 = f2_pack(-2.f * sy, -2.f * sy);
-#pragma unroll
-        for (int bb = 0; bb < NB; ++bb) {
-          const int c0 = part * CPART + 16 * bb;
-          const uint32_t(&r)[16] = rr[bb];
-          float val[16];
-#pragma unroll
-          for (int k = 0; k < 16; k += 4) {
-            const float4 vx = *reinterpret_cast<const float4*>(nx + c0 + k);
-            const float4 vs = *reinterpret_cast<const float4*>(ns + c0 + k);
-            unsigned long long w01 = w2c, w23 = w2c;
-            if (!fmt_is_bf16(FMT)) {
-              // w = (-2 sy) sx: both powers of two, so the product is exact
-              const float4 vc = *reinterpret_cast<const float4*>(sx + c0 + k);
-              w01 = f2_mul(wsy2, f2_pack(vc.x, vc.y));
-              w23 = f2_mul(wsy2, f2_pack(vc.z, vc.w));
-            }
-            const unsigned long long a01 = f2_pack(__uint_as_float(r[k]), __uint_as_float(r[k + 1]));
-            const unsigned long long a23 = f2_pack(__uint_as_float(r[k + 2]), __uint_as_float(r[k + 3]));
-            const unsigned long long v01 = f2_fma(mcy2, f2_pack(vs.x, vs.y), f2_fma(w01, a01, f2_pack(vx.x, vx.y)));
-            const unsigned long long v23 = f2_fma(mcy2, f2_pack(vs.z, vs.w), f2_fma(w23, a23, f2_pack(vx.z, vx.w)));
-            val[k] = f2_lo(v01);
-            val[k + 1] = f2_hi(v01);
-            val[k + 2] = f2_lo(v23);
-            val[k + 3] = f2_hi(v23);
-          }
-          // the block's minimum as a tree of three-input minima (8 for 16)
-          const float mn =
-              fminf(fmin3(fmin3(val[0], val[1], val[2]), fmin3(val[3], val[4], val[5]), fmin3(val[6], val[7], val[8])),
-                    fmin3(fmin3(val[9], val[10], val[11]), fmin3(val[12], val[13], val[14]), val[15]));
-          if (mn < lim) {
-            // the few columns that beat the current K-th entry: park the
-            // block's values, then one (rolled) insertion per such column
-            // that still beats it
-            const float thr = lim;
-            unsigned msk = 0;
-#pragma unroll
-            for (int k = 0; k < 16; ++k) {
-              msk |= (val[k] < thr ? 1u : 0u) << k;
-              stage[k][etid] = val[k];
-            }
 #pragma unroll 1
-            while (msk) {
-              const int k = __ffs(msk) - 1;
-              msk &= msk - 1;
-              const float vk = stage[k][etid];
-              if (vk < lim) {
-                tag_insert<KL>(tv, used, table, TSTRIDE, vk, tile * BN + c0 + k);
-                lim = fminf(lim, tv[KL - 1]);
+        for (int cc = cpart * CPART; cc < (cpart + 1) * CPART; cc += 16 * NB) {
+          uint32_t rr[NB][16];
+#pragma unroll
+          for (int bb = 0; bb < NB; ++bb)
+            tmem_ld16_async(tmem_base + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(b * BN + cc + 16 * bb), rr[bb]);
+          tmem_ld_wait(rr);
+#pragma unroll
+          for (int bb = 0; bb < NB; ++bb) {
+            const int c0 = cc + 16 * bb;
+            const uint32_t(&r)[16] = rr[bb];
+            float val[16];
+#pragma unroll
+            for (int k = 0; k < 16; k += 4) {
+              const float4 vx = *reinterpret_cast<const float4*>(nx + c0 + k);
+              const float4 vs = *reinterpret_cast<const float4*>(ns + c0 + k);
+              unsigned long long w01 = w2c, w23 = w2c;
+              if (!fmt_is_bf16(FMT)) {
+                // w = (-2 sy) sx: both powers of two, so the product is exact
+                const float4 vc = *reinterpret_cast<const float4*>(sx + c0 + k);
+                w01 = f2_mul(wsy2, f2_pack(vc.x, vc.y));
+                w23 = f2_mul(wsy2, f2_pack(vc.z, vc.w));
               }
+              const unsigned long long a01 = f2_pack(__uint_as_float(r[k]), __uint_as_float(r[k + 1]));
+              const unsigned long long a23 = f2_pack(__uint_as_float(r[k + 2]), __uint_as_float(r[k + 3]));
+              const unsigned long long v01 = f2_fma(mcy2, f2_pack(vs.x, vs.y), f2_fma(w01, a01, f2_pack(vx.x, vx.y)));
+              const unsigned long long v23 = f2_fma(mcy2, f2_pack(vs.z, vs.w), f2_fma(w23, a23, f2_pack(vx.z, vx.w)));
+              val[k] = f2_lo(v01);
+              val[k + 1] = f2_hi(v01);
+              val[k + 2] = f2_lo(v23);
+              val[k + 3] = f2_hi(v23);
             }
-            if (tv[SEEN] < CUDART_INF_F) *mine = tag_ceil(tv[SEEN], TagList<KL>::MASK);
+            // the block's minimum as a tree of three-input minima (8 for 16)
+            const float mn =
+                fminf(fmin3(fmin3(val[0], val[1], val[2]), fmin3(val[3], val[4], val[5]), fmin3(val[6], val[7], val[8])),
+                      fmin3(fmin3(val[9], val[10], val[11]), fmin3(val[12], val[13], val[14]), val[15]));
+            if (mn < lim) {
+              // the few columns that beat the current K-th entry: park the
+              // block's values, then one (rolled) insertion per such column
+              // that still beats it
+              const float thr = lim;
+              unsigned msk = 0;
+#pragma unroll
+              for (int k = 0; k < 16; ++k) {
+                msk |= (val[k] < thr ? 1u : 0u) << k;
+                stage[k][etid] = val[k];
+              }
+#pragma unroll 1
+              while (msk) {
+                const int k = __ffs(msk) - 1;
+                msk &= msk - 1;
+                const float vk = stage[k][etid];
+                if (vk < lim) {
+                  tag_insert<KL>(tv, used, table, TSTRIDE, vk, tile * BN + c0 + k);
+                  lim = fminf(lim, tv[KL - 1]);
+                }
+              }
+              if (tv[SEEN] < CUDART_INF_F) *mine = tag_ceil(tv[SEEN], TagList<KL>::MASK);
+            }
           }
         }
       }
@@ -432,7 +445,7 @@ __global__ void __launch_bounds__(tc_threads(FMT, KL), 1) k_nns_tc(TcArgs P) {
       tc_fence_before();
       __syncwarp();
       if (lane == 0) {
-        mbar_arrive(&bar_acc_empty[b]);
+        mbar_arrive(&bar_acc_empty[a]);
         mbar_arrive(&bar_nrm_empty[n]);
       }
     }
