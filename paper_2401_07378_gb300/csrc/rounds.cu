@@ -328,10 +328,11 @@ __global__ void __launch_bounds__(CP_THREADS) k_compact_scatter(CompactArgs A) {
   const int first = sd == 0 ? 0 : A.side[0].nblocks;
   __shared__ int s_off;
   __shared__ int wsum[CP_THREADS / 32 + 1];
-  if (threadIdx.x == 0) {
+  if (threadIdx.x < 32) {  // survivors of the blocks before this one
     int o = 0;
-    for (int b = first; b < first + lb; ++b) o += A.blockcounts[b];
-    s_off = o;
+    for (int b = first + threadIdx.x; b < first + lb; b += 32) o += A.blockcounts[b];
+    o = __reduce_add_sync(0xffffffffu, o);
+    if (threadIdx.x == 0) s_off = o;
   }
   // flags of this thread's items
   int flags[CP_ITEMS];

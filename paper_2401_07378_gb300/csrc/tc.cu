@@ -522,7 +522,7 @@ struct RerankArgs {
   int kl;               // list length of each chunk (the stride of cand_v / cand_p)
 };
 
-// RR_ROWS packed consumer rows per block, G lanes a row (8 where the rows'
+// RR_ROWS (8 or 32) packed consumer rows per block, G lanes a row (8 where the rows'
 // candidates are that few, else a warp).  The first rk candidates of every
 // chunk are re-ranked; tau is the smallest rk-th approximate value over the
 // chunks (every supplier outside them lies at or above it).  A consumer whose
@@ -535,10 +535,12 @@ struct RerankArgs {
 // step takes one row per lane of a warp.  (One warp per row, its certificate
 // in one lane, its norms summed in FP64 and its counters updated one by one
 // took 725 us for 131,072 rows, against 100 of candidate rows read.)
-constexpr int RR_ROWS = 32;
+// Where a block of 32 rows would leave SMs idle (few consumers, many chunks of
+// candidates: a few thousand consumers of a learned round took 300 us), RR_ROWS
+// is 8, one row a warp.
 constexpr int RR_THREADS = 256;
 
-template <int G>
+template <int G, int RR_ROWS>
 __global__ void __launch_bounds__(RR_THREADS) k_rerank_certify(RerankArgs R) {
   __shared__ unsigned long long s_best[RR_ROWS], s_abest[RR_ROWS];
   __shared__ float s_tau[RR_ROWS];
@@ -649,9 +651,9 @@ __global__ void __launch_bounds__(RR_THREADS) k_rerank_certify(RerankArgs R) {
   __syncthreads();
   if (threadIdx.x >= 32) return;
   const int lane = threadIdx.x, r = r0 + lane;
-  const bool live = r < nq;
+  const bool live = lane < RR_ROWS && r < nq;
   const int q = live ? (R.sel ? R.sel[r] : r) : 0;
-  const unsigned long long best = s_best[lane];
+  const unsigned long long best = live ? s_best[lane] : ~0ULL;
   bool certified = false;
   if (live && best != ~0ULL) {
     // |y|_2 from the FP32 squared norm, rounded up; |y|_1 <= sqrt(d) |y|_2
@@ -877,9 +879,10 @@ int launch_nns_tc(const SolveBufs& B, const TcBufs& T, int mt, int nt, int preci
                chunks,   fmt,        T.cand_v,    T.cand_p,    T.nrm_y,   T.scale_y,   T.stats,
                B.nnkey,  T.fallback, T.nfallback, &B.st->certified, &B.st->fallbacks, &B.st->near_ties,
                sel,      nsel_dev,   B.lists,     rk,          kl};
-  const int rblocks = (nt + RR_ROWS - 1) / RR_ROWS;
-  if (chunks * rk <= 8) k_rerank_certify<8><<<rblocks, RR_THREADS, 0, st>>>(R);
-  else k_rerank_certify<32><<<rblocks, RR_THREADS, 0, st>>>(R);
+  const bool wide = chunks * rk > 8, few = nt < 32 * 4 * num_sms();
+  if (!wide) k_rerank_certify<8, 32><<<(nt + 31) / 32, RR_THREADS, 0, st>>>(R);
+  else if (few) k_rerank_certify<32, 8><<<(nt + 7) / 8, RR_THREADS, 0, st>>>(R);
+  else k_rerank_certify<32, 32><<<(nt + 31) / 32, RR_THREADS, 0, st>>>(R);
   // FP32 scan of the consumers that were not certified
   launch_nns_f32(B, mt, nt, T.fallback, T.nfallback, st);
   return 0;
@@ -1095,14 +1098,18 @@ __global__ void k_argmax_parts(const unsigned long long* __restrict__ part, int 
   out[r] = (int)(0xffffffffu - (unsigned)(best & 0xffffffffu));
 }
 
-// Per point: |p|^2 (sequential fma, relative error <= gamma_d) rounded down
-// and |p| rounded up.
+// Per point: |p|^2 (relative error <= gamma_d in any order of summation)
+// rounded down and |p| rounded up.  Eight lanes a point: one lane walking a row
+// left the GPU idle at 4,096 rows (12.4 us).
 __global__ void k_point_norms(const float* __restrict__ pts, int n, int d, float* __restrict__ sq_lo,
                               float* __restrict__ nrm_up) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= n) return;
+  const int i = (blockIdx.x * blockDim.x + threadIdx.x) >> 3, sub = threadIdx.x & 7;
   float s = 0.f;
-  for (int k = 0; k < d; ++k) s = __fmaf_rn(pts[(size_t)i * d + k], pts[(size_t)i * d + k], s);
+  if (i < n)
+    for (int k = sub; k < d; k += 8) s = __fmaf_rn(pts[(size_t)i * d + k], pts[(size_t)i * d + k], s);
+#pragma unroll
+  for (int o = 4; o > 0; o >>= 1) s = __fadd_rn(s, __shfl_xor_sync(0xffffffffu, s, o));
+  if (i >= n || sub != 0) return;
   const double g = certify_gamma(d);
   sq_lo[i] = __fmul_rd(s, __double2float_rd(1.0 - g));
   nrm_up[i] = __fsqrt_ru(__fmul_ru(s, __double2float_ru(1.0 + g / (1.0 - g))));
@@ -1167,14 +1174,14 @@ bool cell_bounds_tc_supported(int d) { return d % 16 == 0 && linear_tc_supported
 
 int cell_bounds_tc_cells(const float* mu, int cells, int d, uint8_t* packed, float* sq_lo, float* nrm_up,
                          cudaStream_t st) {
-  k_point_norms<<<(cells + 255) / 256, 256, 0, st>>>(mu, cells, d, sq_lo, nrm_up);
+  k_point_norms<<<(cells + 31) / 32, 256, 0, st>>>(mu, cells, d, sq_lo, nrm_up);
   return pack_rows(mu, cells, d, FMT_BF16X3, true, packed, st);
 }
 
 int cell_bounds_tc(const float* y, int rows, int d, uint8_t* packed_y, float* y_sq_lo, float* y_nrm_up,
                    const uint8_t* packed_mu, const float* mu_sq_lo, const float* mu_nrm_up, const float* radius,
                    int cells, float* out, unsigned* err, cudaStream_t st) {
-  k_point_norms<<<(rows + 255) / 256, 256, 0, st>>>(y, rows, d, y_sq_lo, y_nrm_up);
+  k_point_norms<<<(rows + 31) / 32, 256, 0, st>>>(y, rows, d, y_sq_lo, y_nrm_up);
   if (pack_rows(y, rows, d, FMT_BF16X3, false, packed_y, st)) return -1;
   // |<y~, mu~> - <y, mu>| <= (Q + K 2^-22 nf^2) |y| |mu| for the BF16X3
   // copies (the certificate's quantisation and accumulation terms, K = 3d
