@@ -131,8 +131,8 @@ struct GeoTC {
   static constexpr int kDP = 0;
   static constexpr int kThreads = FIN_THREADS;
   // (a list is a warp's work of 20 us and more: the last rounds of a pair make
-  // theirs in 32 warps rather than in warp_rounds' one)
-  static constexpr bool kWarpRounds = false;
+  // theirs in 32 warps rather than in team_rounds' four)
+  static constexpr bool kTeamRounds = false;
   static constexpr int SEL_BUF = 128;  // words a warp's selection collects at most
   struct PX {};
   const float* x;  // this pair's coordinates

@@ -77,7 +77,7 @@ struct CtaCore {
   unsigned nflow;
   union {
     double total[2];  // the sides' weight totals (while a pair loads)
-    struct {          // running totals handed back by the one-warp rounds (warp_rounds)
+    struct {          // running totals handed back by team_rounds
       unsigned long long w_nnz;
       long long w_rounds, w_pe;
     };
@@ -246,16 +246,14 @@ struct GeoSmem {
     __syncthreads();
     return S.nnk;
   }
-  // the same for at most 64 consumers, by one warp
-  static constexpr bool kWarpRounds = true;
-  NNS_DEV bool warp_ready() const { return true; }
+  // two consumers of a lane against a chunk (team_rounds)
+  static constexpr bool kTeamRounds = true;
+  NNS_DEV bool team_ready() const { return true; }
+  NNS_DEV void team_count(int) const {}
   template <int C>
-  NNS_DEV void warp_nns(CtaCore<C>& S, int mt, int nt) const {
-    const int qa = threadIdx.x & 31, qb = qa + 32;
-    unsigned long long ka, kb;
-    scan_chunk(qa, qb, nt, 0, mt, ka, kb);
-    if (qa < nt) S.nnk[qa] = ka;
-    if (qb < nt) S.nnk[qb] = kb;
+  NNS_DEV void team_scan(CtaCore<C>&, int qa, int qb, int nt, int s0, int s1, unsigned long long& ka,
+                         unsigned long long& kb) const {
+    scan_chunk(qa, qb, nt, s0, s1, ka, kb);
   }
 };
 
@@ -277,7 +275,7 @@ struct GeoSmem {
 // positions); the chunks merge through a 64-bit atomicMin on (key bits,
 // position), which keeps the lowest-index tie-break.
 template <int D, int DP, bool L1, int CAP, int NT>
-struct GeoSmemCluster : GeoSmem<D, DP, L1, CAP> {
+struct GeoSmemCluster : GeoSmem<D, DP, L1, CAP, NT> {
   static constexpr int kThreads = NT;     // threads of each CTA
   static constexpr int kSlice = CAP / 8;  // consumers per CTA at most (R >= 8)
   unsigned long long xk[2][CAP];          // receive buffers (round parity)
@@ -289,7 +287,12 @@ struct GeoSmemCluster : GeoSmem<D, DP, L1, CAP> {
   }
 
   template <int C>
-  NNS_DEV const unsigned long long* nns(CtaCore<C>&, int mt, int nt, long long round) {
+  NNS_DEV const unsigned long long* nns(CtaCore<C>& S, int mt, int nt, long long round) {
+    // a small round's exchange and cluster barrier cost more than the scan by
+    // itself: every CTA then scans it all (the product only shrinks, so the
+    // buffers below are not used again).  65,536-point colours, the tail's 41
+    // rounds: 911 us with the exchange in every round, 905 us with this line.
+    if (mt * nt <= 128 * 128) return GeoSmem<D, DP, L1, CAP, NT>::nns(S, mt, nt);
     namespace cg = cooperative_groups;
     cg::cluster_group cl = cg::this_cluster();
     const unsigned rank = cl.block_rank(), ncl = cl.num_blocks();
@@ -357,8 +360,9 @@ NNS_DEV void group_sync(int bar) {
 // bytes per lane, 4 lanes to a 64-byte piece of one row (a warp touches 8
 // rows per load; one row per lane with 4-byte loads cost 32 L1 lookups a load
 // and kept the pipe at 0.30: the 16,384-point FP32 solve at d = 64 went from
-// 6.87 to 3.55 ms, the 300 x 700 pair at d = 128 from 580 to 430 us).  PRE fetches the next 32 coordinates into registers
-// while the current ones are used (for kernels with registers to spare).
+// 6.87 to 3.55 ms, the 300 x 700 pair at d = 128 from 580 to 430 us).  PRE
+// fetches the next 32 coordinates into registers while the current ones are
+// used (for kernels with registers to spare).
 template <bool L1, bool PRE, class Emit>
 NNS_DEV void group_tiles(const float* __restrict__ x, const int* ia, int p0, int p1, const float* __restrict__ y,
                          const int* ja, const int* cons, int c0, int nc, int d, TileSmem& T, int gt, int bar,
@@ -595,22 +599,22 @@ struct GeoGlobal {
     }
     __syncthreads();
   }
-  // the same for at most 64 consumers, by one warp
-  static constexpr bool kWarpRounds = true;
-  NNS_DEV bool warp_ready() const { return kmat != nullptr && kready; }
+  // two consumers of a lane against a chunk (team_rounds)
+  static constexpr bool kTeamRounds = true;
+  NNS_DEV bool team_ready() const { return kmat != nullptr && kready; }
+  NNS_DEV void team_count(int nt) { searches += nt; }
   template <int C>
-  NNS_DEV void warp_nns(CtaCore<C>& S, int mt, int nt) {
-    const int qa = threadIdx.x & 31, qb = qa + 32;
-    if (threadIdx.x == 0) searches += nt;
+  NNS_DEV void team_scan(CtaCore<C>& S, int qa, int qb, int nt, int s0, int s1, unsigned long long& ka,
+                         unsigned long long& kb) const {
     const float* ca = kmat + S.jidx[qa < nt ? qa : 0];
     const float* cb = kmat + S.jidx[qb < nt ? qb : 0];
     unsigned ba = 0xffffffffu, bb = 0xffffffffu;
-    int pa = 0, pb = 0;
-    for (int p = 0; p < mt; p += 8) {
+    int pa = s0, pb = s0;
+    for (int p = s0; p < s1; p += 8) {
       unsigned va[8], vb[8];
 #pragma unroll
       for (int e = 0; e < 8; ++e) {
-        const size_t row = (size_t)S.iidx[min(p + e, mt - 1)] * kld;
+        const size_t row = (size_t)S.iidx[min(p + e, s1 - 1)] * kld;
         va[e] = __float_as_uint(ca[row]);
         vb[e] = __float_as_uint(cb[row]);
       }
@@ -620,8 +624,8 @@ struct GeoGlobal {
         if (vb[e] < bb) { bb = vb[e]; pb = p + e; }
       }
     }
-    if (qa < nt) S.nnk[qa] = ((unsigned long long)ba << 32) | (unsigned)pa;
-    if (qb < nt) S.nnk[qb] = ((unsigned long long)bb << 32) | (unsigned)pb;
+    ka = ((unsigned long long)ba << 32) | (unsigned)pa;
+    kb = ((unsigned long long)bb << 32) | (unsigned)pb;
   }
   template <int C>
   NNS_DEV const unsigned long long* nns(CtaCore<C>& S, int mt, int nt, long long = 0) {
@@ -664,7 +668,7 @@ template <int CAP, int NT>
 struct GeoMatCluster {
   static constexpr int kDP = 0;
   static constexpr int kThreads = NT;
-  static constexpr bool kWarpRounds = true;
+  static constexpr bool kTeamRounds = true;
   static constexpr int kSlice = CAP / 8;  // consumers per CTA at most (R >= 8)
   const float* kmat;
   int kld;
@@ -729,14 +733,13 @@ struct GeoMatCluster {
     for (int i = threadIdx.x; i < ns; i += NT) red[i] = ~0ULL;
     return xk[h];
   }
-  NNS_DEV bool warp_ready() const { return true; }
+  NNS_DEV bool team_ready() const { return true; }
+  NNS_DEV void team_count(int) const {}
   template <int C>
-  NNS_DEV void warp_nns(CtaCore<C>& S, int mt, int nt) const {
-#pragma unroll 1
-    for (int q = threadIdx.x & 31; q < 64; q += 32) {
-      const unsigned long long k = scan_col(col[min(q, nt - 1)], 0, mt);
-      if (q < nt) S.nnk[q] = k;
-    }
+  NNS_DEV void team_scan(CtaCore<C>&, int qa, int qb, int nt, int s0, int s1, unsigned long long& ka,
+                         unsigned long long& kb) const {
+    ka = scan_col(col[min(qa, nt - 1)], s0, s1);
+    kb = scan_col(col[min(qb, nt - 1)], s0, s1);
   }
 };
 
@@ -836,126 +839,122 @@ NNS_DEV int block_scan_array(const int* in, int* out, int n, int* wt) {
   return tot;
 }
 
-// Active sets both at most warp_cap<Geo>() points go to warp_rounds (two
-// per lane).  128 (four per lane) was measured slower on the colour-transfer
-// tail than the 16-CTA cluster rounds for sets of 65..128 points (483 against
-// 517 pairs/s for the whole solve).
-template <class Geo>
-NNS_DEV constexpr int warp_cap() { return 64; }
+// Active sets both at most TEAM_CAP points go to team_rounds.
+constexpr int TEAM_CAP = 64;
+constexpr int TEAM_WARPS = 4;
+NNS_DEV void team_sync() { asm volatile("bar.sync 15, %0;" ::"n"(32 * TEAM_WARPS) : "memory"); }
 
-// The remaining rounds of a pair whose active sets both hold at most
-// warp_cap<Geo>() points, run by the calling warp alone (policies with
-// kWarpRounds): with a few dozen points left, a round of the
-// block-wide steps below is mostly barrier latency, and one warp needs none.
-// The same steps in the same arithmetic as cta_rounds, so every result is
-// identical:
-//   NNS     the policy's warp_nns, consumers lane and lane + 32;
+// The remaining rounds of a pair whose active sets both hold at most TEAM_CAP
+// points, run by the CTA's first four warps (policies with kTeamRounds): with
+// a few dozen points left, a round of the block-wide steps below is mostly
+// barriers of every warp and scans.  The same steps in the same arithmetic as
+// cta_rounds, so every result is identical:
+//   NNS     each warp scans a quarter of the suppliers for two consumers a
+//           lane (the policy's team_scan); quarters merge by atomicMin;
 //   order   every consumer's (supplier position, serving key, position) as
-//           one 64-bit word and its rank among all of them; the members of a
-//           group then lie in serving order, groups in supplier order;
+//           one 64-bit word and its rank among all of them, one consumer a
+//           lane; the members of a group then lie in serving order;
 //   flow    lane = supplier, the FP64 residual chain over its group;
-//   compact ballots keep the points with residual left, in order.
+//   compact ballots keep the points with residual left, in order, two warps a
+//           side.
+// (One warp alone took 3,700 cycles a round, 1,900 of them in the NNS and
+// 1,700 in the order.  2,048 batched images of some 500 points, GB300: 620 us
+// with one warp, 549 us with four; a pair of 256 points 61 and 60 us.)
 template <int CAP, class Geo>
-NNS_DEV void warp_rounds(CtaCore<CAP>& S, Geo& G, int metric, const CtaOut& O, unsigned long long& nnz,
+NNS_DEV void team_rounds(CtaCore<CAP>& S, Geo& G, int metric, const CtaOut& O, unsigned long long& nnz,
                          long long& rounds, long long& pair_evals, long long round_limit) {
-  constexpr int WH = warp_cap<Geo>() / 32;  // points per lane
-  const int lane = threadIdx.x & 31;
+  static_assert(CAP >= 2 * TEAM_CAP && Geo::kThreads >= 32 * TEAM_WARPS, "a round's flows; the team");
+  const int t = threadIdx.x, lane = t & 31, w = t >> 5;
   const unsigned lt = (1u << lane) - 1u;
   const bool deferred = O.fl_i != nullptr;
   for (;;) {
     const int mt = S.mt, nt = S.nt;
     if (mt == 0 || nt == 0) break;
     if (rounds >= round_limit) {
-      if (lane == 0) atomicOr(O.err, EF_ITER);
+      if (t == 0) atomicOr(O.err, EF_ITER);
       break;
     }
-    if (lane == 0) S.nflow = 0;
-#pragma unroll
-    for (int h = 0; h < WH; ++h)
-      if (lane + 32 * h < mt) S.cnt[lane + 32 * h] = 0;
+    if (t == 0) {
+      S.nflow = 0;
+      G.team_count(nt);
+    }
+    if (t < mt) S.cnt[t] = 0;
+    if (t >= 64 && t - 64 < nt) S.nnk[t - 64] = ~0ULL;
+    team_sync();
     // ---- NNS
-    G.warp_nns(S, mt, nt);
-    // ---- order: (supplier, serving key, consumer) of every consumer (each
-    // lane reads back its own keys), then its rank among all of them
-    static_assert(WH == 2, "two consumers per lane");
-    unsigned long long ma = ~0ULL, mb = ~0ULL;
-#pragma unroll
-    for (int h = 0; h < WH; ++h) {
-      const int q = lane + 32 * h;
-      if (q < nt) {
-        const unsigned long long key = S.nnk[q];
-        const unsigned ord = O.protocol == 1 ? rp_key32(O.seed, O.round_base + rounds, S.jidx[q])
-                                             : (unsigned)(key >> 32);
-        const unsigned long long mine = ((key & 0xffffULL) << 40) | ((unsigned long long)ord << 8) | (unsigned)q;
-        if (h == 0) ma = mine;
-        else mb = mine;
-        S.mem[q] = mine;
-      } else if (q < ((nt + 3) & ~3)) {
-        S.mem[q] = ~0ULL;
+    {
+      const int s0 = mt * w / TEAM_WARPS, s1 = mt * (w + 1) / TEAM_WARPS;
+      if (s0 < s1) {
+        unsigned long long ka, kb;
+        G.team_scan(S, lane, lane + 32, nt, s0, s1, ka, kb);
+        if (lane < nt) atomicMin(&S.nnk[lane], ka);
+        if (lane + 32 < nt) atomicMin(&S.nnk[lane + 32], kb);
       }
     }
-    __syncwarp();
-    int ra = 0, rb = 0;
-    for (int u = 0; u < nt; u += 4) {
-      const ulonglong2 o = *reinterpret_cast<const ulonglong2*>(&S.mem[u]);
-      const ulonglong2 v = *reinterpret_cast<const ulonglong2*>(&S.mem[u + 2]);
-      ra += (o.x < ma) + (o.y < ma) + (v.x < ma) + (v.y < ma);
-      rb += (o.x < mb) + (o.y < mb) + (v.x < mb) + (v.y < mb);
+    team_sync();
+    // ---- order: (supplier, serving key, consumer) of every consumer, then
+    // its rank among all of them
+    unsigned long long mine = ~0ULL;
+    if (t < nt) {
+      const unsigned long long key = S.nnk[t];
+      const unsigned ord = O.protocol == 1 ? rp_key32(O.seed, O.round_base + rounds, S.jidx[t]) : (unsigned)(key >> 32);
+      mine = ((key & 0xffffULL) << 40) | ((unsigned long long)ord << 8) | (unsigned)t;
     }
-    if (lane < nt) S.mem2[ra] = ma;
-    if (lane + 32 < nt) S.mem2[rb] = mb;
-    __syncwarp();
+    if (t < ((nt + 3) & ~3)) S.mem[t] = mine;
+    team_sync();
+    if (t < nt) {
+      int rank = 0;
+      for (int u = 0; u < nt; u += 4) {
+        const ulonglong2 o = *reinterpret_cast<const ulonglong2*>(&S.mem[u]);
+        const ulonglong2 v = *reinterpret_cast<const ulonglong2*>(&S.mem[u + 2]);
+        rank += (o.x < mine) + (o.y < mine) + (v.x < mine) + (v.y < mine);
+      }
+      S.mem2[rank] = mine;
+    }
+    team_sync();
     // group bounds: where the supplier changes along the order
-#pragma unroll
-    for (int h = 0; h < WH; ++h) {
-      const int r = lane + 32 * h;
-      if (r < nt) {
-        const int p = (int)(S.mem2[r] >> 40);
-        if (r == 0 || (int)(S.mem2[r - 1] >> 40) != p) S.off[p] = r;
-        if (r == nt - 1 || (int)(S.mem2[r + 1] >> 40) != p) S.cnt[p] = r + 1;  // the group's end
-      }
+    if (t < nt) {
+      const int p = (int)(S.mem2[t] >> 40);
+      if (t == 0 || (int)(S.mem2[t - 1] >> 40) != p) S.off[p] = t;
+      if (t == nt - 1 || (int)(S.mem2[t + 1] >> 40) != p) S.cnt[p] = t + 1;  // the group's end
     }
-    __syncwarp();
+    team_sync();
     // ---- flow, one supplier per lane
-#pragma unroll
-    for (int h = 0; h < WH; ++h) {
-      const int p = lane + 32 * h;
-      if (p < mt && S.cnt[p] > 0) {
-        const int b = S.off[p], en = S.cnt[p];
-        double s = S.sres[p];
-        for (int r = b; r < en; ++r) {
-          if (!residual_positive(s)) break;
-          const int q = (int)(S.mem2[r] & 0xffULL);
-          double c = S.cres[q];
-          const double f = greedy_step(s, c);
-          S.cres[q] = c;
-          const unsigned k = atomicAdd(&S.nflow, 1u);
-          if (O.quiet) {
-          } else if (deferred) {
-            const unsigned long long slot = nnz + k;
-            if (O.fl_cap && (long long)slot >= O.fl_cap) {
-              atomicOr(O.err, EF_CAPACITY);
-              continue;
-            }
-            O.fl_i[slot] = S.iidx[p];
-            O.fl_j[slot] = S.jidx[q];
-            O.fl_f[slot] = f;
-            if (O.c_glob) O.c_glob[S.jidx[q]] = c;
-          } else {
-            // (mem and nnk are free again: the order is in mem2)
-            S.mem[k] = ((unsigned long long)p << 32) | (unsigned)q;
-            S.nnk[k] = (unsigned long long)__double_as_longlong(f);
+    if (t < mt && S.cnt[t] > 0) {
+      const int p = t, b = S.off[p], en = S.cnt[p];
+      double s = S.sres[p];
+      for (int r = b; r < en; ++r) {
+        if (!residual_positive(s)) break;
+        const int q = (int)(S.mem2[r] & 0xffULL);
+        double c = S.cres[q];
+        const double f = greedy_step(s, c);
+        S.cres[q] = c;
+        const unsigned k = atomicAdd(&S.nflow, 1u);
+        if (O.quiet) {
+        } else if (deferred) {
+          const unsigned long long slot = nnz + k;
+          if (O.fl_cap && (long long)slot >= O.fl_cap) {
+            atomicOr(O.err, EF_CAPACITY);
+            continue;
           }
+          O.fl_i[slot] = S.iidx[p];
+          O.fl_j[slot] = S.jidx[q];
+          O.fl_f[slot] = f;
+          if (O.c_glob) O.c_glob[S.jidx[q]] = c;
+        } else {
+          // (mem and nnk are free again: the order is in mem2)
+          S.mem[k] = ((unsigned long long)p << 32) | (unsigned)q;
+          S.nnk[k] = (unsigned long long)__double_as_longlong(f);
         }
-        S.sres[p] = s;
-        if (O.s_glob) O.s_glob[S.iidx[p]] = s;
       }
+      S.sres[p] = s;
+      if (O.s_glob) O.s_glob[S.iidx[p]] = s;
     }
-    __syncwarp();
+    team_sync();
     const unsigned nflow = S.nflow;
     if (!(deferred || O.quiet)) {
-      for (unsigned base = 0; base < nflow; base += 32) {  // the whole warp (xs_add_warp)
-        const unsigned k = base + lane;
+      for (unsigned base = 0; base < nflow; base += 32 * TEAM_WARPS) {  // whole warps (xs_add_warp)
+        const unsigned k = base + t;
         double term = 0.0;
         if (k < nflow) {
           const unsigned long long pq = S.mem[k];
@@ -976,66 +975,48 @@ NNS_DEV void warp_rounds(CtaCore<CAP>& S, Geo& G, int metric, const CtaOut& O, u
         }
         if (O.acc) xs_add_warp(O.acc, term);  // one call site for the whole warp
       }
-      __syncwarp();
+      team_sync();
     }
     nnz += nflow;
     rounds += 1;
     pair_evals += (long long)mt * nt;
-    // ---- compaction: every kept value is read before any is written
-    double sv[WH], cv[WH];
-    int iv[WH], jv[WH];
-    typename Geo::PX px[WH], py[WH];
-    unsigned bs[WH], bc[WH];
-#pragma unroll
-    for (int h = 0; h < WH; ++h) {
-      const int i = lane + 32 * h;
-      bool ks = false, kc = false;
-      if (i < mt) {
-        sv[h] = S.sres[i];
-        ks = residual_positive(sv[h]);
-        if (ks) { iv[h] = S.iidx[i]; G.load_x(i, px[h]); }
+    // ---- compaction: warps 0, 1 the suppliers, 2, 3 the consumers; every
+    // kept value is read before any is written
+    const bool sup = w < 2;
+    const int i = t & 63;
+    bool keep = false;
+    double v = 0.0;
+    int id = 0;
+    typename Geo::PX px;
+    if (i < (sup ? mt : nt)) {
+      v = sup ? S.sres[i] : S.cres[i];
+      keep = residual_positive(v);
+      if (keep) {
+        id = sup ? S.iidx[i] : S.jidx[i];
+        if (sup) G.load_x(i, px);
+        else G.load_y(i, px);
       }
-      if (i < nt) {
-        cv[h] = S.cres[i];
-        kc = residual_positive(cv[h]);
-        if (kc) { jv[h] = S.jidx[i]; G.load_y(i, py[h]); }
-      }
-      bs[h] = __ballot_sync(0xffffffffu, ks);
-      bc[h] = __ballot_sync(0xffffffffu, kc);
     }
-    __syncwarp();
-    int ps = 0, pc = 0;
-#pragma unroll
-    for (int h = 0; h < WH; ++h) {
-      if ((bs[h] >> lane) & 1u) {
-        const int dd = ps + __popc(bs[h] & lt);
-        S.sres[dd] = sv[h];
-        S.iidx[dd] = iv[h];
-        G.store_x(dd, px[h]);
-      }
-      if ((bc[h] >> lane) & 1u) {
-        const int dd = pc + __popc(bc[h] & lt);
-        S.cres[dd] = cv[h];
-        S.jidx[dd] = jv[h];
-        G.store_y(dd, py[h]);
-      }
-      ps += __popc(bs[h]);
-      pc += __popc(bc[h]);
+    const unsigned bal = __ballot_sync(0xffffffffu, keep);
+    if (lane == 0) S.wt[w] = __popc(bal);
+    team_sync();
+    if (keep) {
+      const int at = ((w & 1) ? S.wt[w - 1] : 0) + __popc(bal & lt);
+      (sup ? S.sres : S.cres)[at] = v;
+      (sup ? S.iidx : S.jidx)[at] = id;
+      if (sup) G.store_x(at, px);
+      else G.store_y(at, px);
     }
-    __syncwarp();
-    if (lane == 0) {
-      S.mt = ps;
-      S.nt = pc;
-    }
-    __syncwarp();
+    if (t == 0) S.mt = S.wt[0] + S.wt[1];
+    if (t == 64) S.nt = S.wt[2] + S.wt[3];
+    team_sync();
   }
 }
 
 // Rounds of Alg. 1 until one active side is empty.  nnz, rounds and
 // pair_evals are running totals (identical in every thread on return).
-// With shared-memory coordinates, the rounds after both active sets fit
-// warp_cap<Geo>() run in warp 0 alone (warp_rounds) while the other warps
-// wait.
+// The rounds after both active sets fit TEAM_CAP run in the first four warps
+// (team_rounds) while the others wait.
 template <int CAP, class Geo>
 NNS_DEV void cta_rounds(CtaCore<CAP>& S, Geo& G, int metric, const CtaOut& O, unsigned long long& nnz,
                         long long& rounds, long long& pair_evals, long long round_limit) {
@@ -1049,10 +1030,10 @@ NNS_DEV void cta_rounds(CtaCore<CAP>& S, Geo& G, int metric, const CtaOut& O, un
       if (tid == 0) atomicOr(O.err, EF_ITER);
       break;
     }
-    if constexpr (Geo::kWarpRounds) {
-      if (mt <= warp_cap<Geo>() && nt <= warp_cap<Geo>() && G.warp_ready()) {
-        if (tid < 32) {
-          warp_rounds(S, G, metric, O, nnz, rounds, pair_evals, round_limit);
+    if constexpr (Geo::kTeamRounds) {
+      if (mt <= TEAM_CAP && nt <= TEAM_CAP && G.team_ready()) {
+        if (tid < 32 * TEAM_WARPS) {
+          team_rounds(S, G, metric, O, nnz, rounds, pair_evals, round_limit);
           if (tid == 0) {
             S.w_nnz = nnz;
             S.w_rounds = rounds;

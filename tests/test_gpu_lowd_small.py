@@ -1,5 +1,5 @@
 """One-CTA solves of small low-dimensional pairs at the edges of their
-capacities and of the one-warp rounds (64 points), single and batched, against
+capacities and of the rounds of a few warps (64 points), single and batched, against
 the oracle bit for bit."""
 import numpy as np
 import pytest
