@@ -192,7 +192,7 @@ size_t layout_solve(void* base, int64_t m, int64_t n, int d, SolveBufs& B, bool 
     L->mup = C.take<uint8_t>(tca ? linear_tc_packed_bytes(K, d) : 0);
     L->mu_bias = C.take<float>(tca ? K : 0);
     L->xp = C.take<uint8_t>(tca ? linear_tc_packed_bytes(L->assign_chunk, d) : 0);
-    L->apart = C.take<unsigned long long>(tca ? (size_t)L->assign_chunk * ((K + 127) / 128) : 0);
+    L->apart = C.take<unsigned long long>(tca ? L->assign_chunk : 0);
     const bool tcb = cell_bounds_tc_supported(d);
     L->mup3 = C.take<uint8_t>(tcb ? linear_tc_packed_bytes(K, 3 * d) : 0);
     L->mu_sq_lo = C.take<float>(tcb ? K : 0);

@@ -85,7 +85,7 @@ struct LearnedBufs {
   uint8_t* mup;         // centroids packed for linear_tc
   float* mu_bias;       // [cells] -|mu_c|^2 / 2
   uint8_t* xp;          // [assign_chunk] supplier rows packed
-  unsigned long long* apart;  // [assign_chunk][cells / 128] partial row maxima
+  unsigned long long* apart;  // [assign_chunk] row maxima
   // the cell bounds on the tensor cores
   uint8_t* mup3;        // centroids packed as BF16X3 splits
   float* mu_sq_lo;      // [cells]

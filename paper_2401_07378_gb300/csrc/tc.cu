@@ -23,6 +23,7 @@
 // warps per row, a share of the columns each) and update its top-K.  Every
 // wait on an mbarrier is bounded and raises EF_TIMEOUT instead of hanging.
 #include <algorithm>
+#include <climits>
 #include <cmath>
 
 #include "common.cuh"
@@ -910,7 +911,7 @@ struct LinArgs {
   const float* bias;         // STORE / ARGMAX: [N]
   float* Z;                  // STORE / LOWER: [rows][N]
   uint8_t* P;                // PACK_RELU: relu(S + b) packed in BF16 as the next layer's X (N values a row)
-  unsigned long long* part;  // ARGMAX: [rows][ceil(N / 128)]
+  unsigned long long* part;  // ARGMAX: [rows], all zero before the launch
   // LOWER: the rows and columns as points; X and W hold BF16X3 copies
   const float* row_sq_lo;    // [rows] |y|^2 rounded down
   const float* row_nrm_up;   // [rows] |y| rounded up
@@ -938,164 +939,245 @@ __global__ void k_pack_rows(const float* __restrict__ src, int rows, int rows_pa
   }
 }
 
-// One CTA per 128 x 128 block of S: both tiles by one bulk copy each, K / 16
-// MMAs into a 128-column accumulator, then every thread takes its row's 128
-// values through the mode's epilogue (columns >= N and rows >= rows are
-// skipped; ARGMAX keeps the largest S + b, lowest column on ties, as a
-// packed key in part[row][column tile]).
+// 128 x 128 blocks of S, a contiguous range of them (columns fastest) per
+// CTA.  One thread loads and multiplies: the W tile of the next block arrives
+// by a bulk copy while this one's K / 16 MMAs run into one of two 128-column
+// accumulators (the X tile stays until the range reaches the next row of
+// blocks), and eight epilogue warps (lane quadrant x column half) take the
+// other accumulator's values through the mode's epilogue: columns >= N and
+// rows >= rows are skipped; ARGMAX keeps each row's largest S + b, lowest
+// column on ties, as a packed key over the CTA's blocks and merges it into
+// part[row].
 //
 // LOWER: with S~ the computed <y~, mu~> of the BF16X3 copies, |S~ - <y, mu>|
 // <= err_coeff |y| |mu| (+ 1e-30 for the subnormal floors), so
 //   |y - mu|^2 >= |y|^2_lo + |mu|^2_lo - 2 (S~ + err_coeff |y|_up |mu|_up),
 // and the bound on the squared distance to any point of cell `col` is
 // max(0, sqrt(that) - r_col)^2, every step rounded toward the bound.
+//
+// Bound by the epilogue: some 14 instructions and a 4-byte store per value.
+// Stores go out through a warp's staging rows as 64 contiguous bytes of eight
+// rows (16 bytes of 32 rows per store cost 32 L1 lookups each).  One block
+// per CTA, load, multiply and epilogue one after the other, took 52.7 us
+// (LOWER) and 40.3 us (STORE) for 4,096 rows x 4,096 columns at 64 and 256
+// coordinates; now 32.7 and 24.3 us.
+constexpr int LIN_EPI = 8;                        // epilogue warps
+constexpr int LIN_THREADS = 32 * (LIN_EPI + 1);
+constexpr int LIN_STAGE = 20;                     // floats per staged row (16 and a pad: no bank conflicts)
+constexpr int LIN_SMEM = 3 * LIN_TILE * 2 * LIN_MAX_K + LIN_EPI * 32 * LIN_STAGE * 4;
+
 template <int MODE>
-__global__ void __launch_bounds__(128, 1) k_linear_tc(LinArgs A) {
+__global__ void __launch_bounds__(LIN_THREADS, 1) k_linear_tc(LinArgs A, int tiles, int ncol) {
   extern __shared__ __align__(1024) uint8_t smem[];
-  __shared__ __align__(8) uint64_t bar_ld;
-  __shared__ __align__(8) uint64_t bar_mma;
+  __shared__ __align__(8) uint64_t bar_full[2], bar_mma[2], bar_free[2];
   __shared__ uint32_t tslot;
-  __shared__ float col_a[LIN_TILE], col_b[LIN_TILE], col_c[LIN_TILE];  // the tile's per-column terms
+  __shared__ __align__(16) float s_col[LIN_EPI][3][64];  // a block's per-column terms, each warp its own copy
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const uint32_t tile_bytes = LIN_TILE * 2 * A.K;
-  {
-    const int n = blockIdx.x * LIN_TILE + threadIdx.x;
-    const bool in = n < A.N;
-    if (MODE == LIN_LOWER) {
-      col_a[threadIdx.x] = in ? A.col_sq_lo[n] : 0.f;
-      col_b[threadIdx.x] = in ? A.col_nrm_up[n] : 0.f;
-      col_c[threadIdx.x] = in ? A.col_radius[n] : 0.f;
-    } else {
-      col_a[threadIdx.x] = in ? A.bias[n] : 0.f;
-    }
-  }
   uint8_t* sX = smem;
-  uint8_t* sW = smem + tile_bytes;
+  uint8_t* sW = smem + tile_bytes;  // two buffers
+  const int t0 = (int)((int64_t)tiles * blockIdx.x / gridDim.x);
+  const int nt = (int)((int64_t)tiles * (blockIdx.x + 1) / gridDim.x) - t0;
   if (threadIdx.x == 0) {
-    mbar_init(&bar_ld, 1);
-    mbar_init(&bar_mma, 1);
+#pragma unroll
+    for (int i = 0; i < 2; ++i) {
+      mbar_init(&bar_full[i], 1);
+      mbar_init(&bar_mma[i], 1);
+      mbar_init(&bar_free[i], LIN_EPI);
+    }
     mbar_fence_init();
   }
-  if (warp == 0) tmem_alloc(&tslot, LIN_TILE);
+  if (warp == LIN_EPI) tmem_alloc(&tslot, 2 * LIN_TILE);
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = tslot;
-  if (threadIdx.x == 0) {
-    mbar_expect_tx(&bar_ld, 2 * tile_bytes);
-    tma_load_1d(sX, A.X + (size_t)blockIdx.y * tile_bytes, tile_bytes, &bar_ld);
-    tma_load_1d(sW, A.W + (size_t)blockIdx.x * tile_bytes, tile_bytes, &bar_ld);
-    if (mbar_wait_bounded(&bar_ld, 0)) {
-      tc_fence_after();
+  if (warp == LIN_EPI) {
+    if (lane == 0) {
+      auto load = [&](int i, bool with_x) {
+        const int t = t0 + i, b = i & 1;
+        mbar_expect_tx(&bar_full[b], (with_x ? 2 : 1) * tile_bytes);
+        if (with_x) tma_load_1d(sX, A.X + (size_t)(t / ncol) * tile_bytes, tile_bytes, &bar_full[b]);
+        tma_load_1d(sW + b * tile_bytes, A.W + (size_t)(t % ncol) * tile_bytes, tile_bytes, &bar_full[b]);
+      };
       const uint32_t idesc = make_idesc(1, LIN_TILE, LIN_TILE);
-      const uint32_t x0 = smem_u32(sX), w0 = smem_u32(sW);
-      for (int k = 0; k < A.K / 16; ++k)
-        mma_issue<FMT_BF16>(tmem, make_desc(x0 + k * 2 * LIN_TILE * 16, LIN_TILE * 16, 128),
-                            make_desc(w0 + k * 2 * LIN_TILE * 16, LIN_TILE * 16, 128), idesc, k > 0 ? 1u : 0u);
-      mma_commit(&bar_mma);
+      const uint32_t x0 = smem_u32(sX);
+      bool ok = true;
+      int loaded = 0, arrived = 0, issued = 0;
+      if (nt > 0) {
+        load(0, true);
+        loaded = 1;
+      }
+      for (int i = 0; i < nt; ++i) {
+        const int b = i & 1;
+        const unsigned ph = (unsigned)(i >> 1) & 1u;
+        const bool next = i + 1 < nt, new_row = next && (t0 + i + 1) % ncol == 0;
+        if (next && !new_row) {  // the buffer of block i - 1
+          if (i > 0 && !(ok = mbar_wait_bounded(&bar_mma[b ^ 1], (unsigned)((i - 1) >> 1) & 1u))) break;
+          load(i + 1, false);
+          loaded = i + 2;
+        }
+        if (!(ok = mbar_wait_bounded(&bar_full[b], ph))) break;
+        arrived = i + 1;
+        if (i > 1 && !(ok = mbar_wait_bounded(&bar_free[b], ph ^ 1u))) break;  // block i - 2 is read
+        tc_fence_after();
+        const uint32_t w0 = smem_u32(sW + b * tile_bytes);
+        for (int k = 0; k < A.K / 16; ++k)
+          mma_issue<FMT_BF16>(tmem + (uint32_t)(b * LIN_TILE),
+                              make_desc(x0 + k * 2 * LIN_TILE * 16, LIN_TILE * 16, 128),
+                              make_desc(w0 + k * 2 * LIN_TILE * 16, LIN_TILE * 16, 128), idesc, k > 0 ? 1u : 0u);
+        mma_commit(&bar_mma[b]);
+        issued = i + 1;
+        if (new_row) {  // X may go once its last MMAs are done
+          if (!(ok = mbar_wait_bounded(&bar_mma[b], ph))) break;
+          load(i + 1, true);
+          loaded = i + 2;
+        }
+      }
+      if (!ok) {  // leave no copy and no MMA in flight
+        for (int i = arrived; i < loaded; ++i) mbar_wait_bounded(&bar_full[i & 1], (unsigned)(i >> 1) & 1u);
+        if (issued > 0) mbar_wait_bounded(&bar_mma[(issued - 1) & 1], (unsigned)((issued - 1) >> 1) & 1u);
+        atomicOr(A.err, EF_TIMEOUT);
+      }
     }
-  }
-  // the accumulator (every lane of a warp agrees before the aligned loads)
-  const bool ok = __all_sync(0xffffffffu, mbar_wait_bounded(&bar_mma, 0));
-  tc_fence_after();
-  if (ok) {
-    const int row = blockIdx.y * LIN_TILE + warp * 32 + lane;
-    const int n0 = blockIdx.x * LIN_TILE;
-    const bool live = row < A.rows;
-    float ysq = 0.f, ynr = 0.f;
-    if (MODE == LIN_LOWER && live) {
-      ysq = A.row_sq_lo[row];
-      ynr = A.row_nrm_up[row];
-    }
+    __syncwarp();
+  } else {
+    const int quad = warp & 3, half = warp >> 2;
+    float* stage = reinterpret_cast<float*>(smem + 3 * tile_bytes) + warp * 32 * LIN_STAGE;
+    float(*col)[64] = s_col[warp];
     unsigned long long best = 0ULL;
-#pragma unroll 1
-    for (int cb = 0; cb < LIN_TILE; cb += 64) {
+    for (int i = 0; i < nt; ++i) {
+      const int t = t0 + i, b = i & 1;
+      const int row = t / ncol * LIN_TILE + quad * 32 + lane;
+      const int n0 = t % ncol * LIN_TILE + half * 64;
+      const bool live = row < A.rows;
+      __syncwarp();  // the previous block's reads of col
+#pragma unroll
+      for (int u = lane; u < 64; u += 32) {
+        const int n = n0 + u;
+        const bool in = n < A.N;
+        if (MODE == LIN_LOWER) {
+          col[0][u] = in ? A.col_sq_lo[n] : 0.f;
+          col[1][u] = in ? A.col_nrm_up[n] : 0.f;
+          col[2][u] = in ? A.col_radius[n] : 0.f;
+        } else {
+          col[0][u] = in ? A.bias[n] : 0.f;
+        }
+      }
+      float ysq = 0.f, ynr = 0.f;
+      if (MODE == LIN_LOWER && live) {
+        ysq = A.row_sq_lo[row];
+        ynr = A.row_nrm_up[row];
+      }
+      // (every lane of a warp agrees before the aligned loads)
+      if (!__all_sync(0xffffffffu, mbar_wait_bounded(&bar_mma[b], (unsigned)(i >> 1) & 1u))) {
+        if (lane == 0) atomicOr(A.err, EF_TIMEOUT);
+        break;
+      }
+      tc_fence_after();
       uint32_t rr[4][16];
 #pragma unroll
-      for (int b = 0; b < 4; ++b) tmem_ld16_async(tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)(cb + 16 * b), rr[b]);
+      for (int g = 0; g < 4; ++g)
+        tmem_ld16_async(tmem + ((uint32_t)(quad * 32) << 16) + (uint32_t)(b * LIN_TILE + half * 64 + 16 * g), rr[g]);
       tmem_ld_wait(rr);
-      if (MODE == LIN_PACK_RELU) {
-        // 16 columns = two 16-byte blocks of the next layer's packed row
-        // (zeros for padding rows, so the next tile holds no garbage)
-        const int kb = 2 * A.N;
-        uint8_t* base = A.P + (size_t)(row / LIN_TILE) * LIN_TILE * kb + (size_t)(row % LIN_TILE) * 16;
+      tc_fence_before();
+      __syncwarp();
+      if (lane == 0) mbar_arrive(&bar_free[b]);
 #pragma unroll
-        for (int b = 0; b < 4; ++b) {
-          const int nb = n0 + cb + 16 * b;
-          if (nb >= A.N) continue;
+      for (int g = 0; g < 4; ++g) {
+        const int nb = n0 + 16 * g;
+        if (nb >= A.N) continue;
+        if constexpr (MODE == LIN_PACK_RELU) {
+          // 16 columns = two 16-byte blocks of the next layer's packed row
+          // (zeros for padding rows, so the next tile holds no garbage)
+          const int kb = 2 * A.N;
+          uint8_t* base = A.P + (size_t)(row / LIN_TILE) * LIN_TILE * kb + (size_t)(row % LIN_TILE) * 16;
           uint32_t w[8];
 #pragma unroll
           for (int e = 0; e < 8; ++e) {
-            const float lo = live ? fmaxf(__uint_as_float(rr[b][2 * e]) + col_a[nb - n0 + 2 * e], 0.f) : 0.f;
-            const float hi = live ? fmaxf(__uint_as_float(rr[b][2 * e + 1]) + col_a[nb - n0 + 2 * e + 1], 0.f) : 0.f;
+            const float lo = live ? fmaxf(__uint_as_float(rr[g][2 * e]) + col[0][16 * g + 2 * e], 0.f) : 0.f;
+            const float hi = live ? fmaxf(__uint_as_float(rr[g][2 * e + 1]) + col[0][16 * g + 2 * e + 1], 0.f) : 0.f;
             w[e] = (uint32_t)__bfloat16_as_ushort(__float2bfloat16_rn(lo)) |
                    ((uint32_t)__bfloat16_as_ushort(__float2bfloat16_rn(hi)) << 16);
           }
           *reinterpret_cast<uint4*>(base + (size_t)(nb / 8) * LIN_TILE * 16) = make_uint4(w[0], w[1], w[2], w[3]);
           *reinterpret_cast<uint4*>(base + (size_t)(nb / 8 + 1) * LIN_TILE * 16) = make_uint4(w[4], w[5], w[6], w[7]);
+        } else if constexpr (MODE == LIN_ARGMAX) {
+#pragma unroll
+          for (int e = 0; e < 16; ++e) {
+            const int n = nb + e;
+            const unsigned long long key =
+                ((unsigned long long)ordered_bits(__uint_as_float(rr[g][e]) + col[0][16 * g + e]) << 32) |
+                (0xffffffffu - (unsigned)n);
+            if (n < A.N && key > best) best = key;
+          }
+        } else {
+#pragma unroll
+          for (int e = 0; e < 16; e += 4) {
+            const float4 c0 = *reinterpret_cast<const float4*>(&col[0][16 * g + e]);
+            const float ca[4] = {c0.x, c0.y, c0.z, c0.w};
+            float out[4];
+            if (MODE == LIN_STORE) {
+#pragma unroll
+              for (int f = 0; f < 4; ++f) out[f] = __uint_as_float(rr[g][e + f]) + ca[f];
+            } else {
+              const float4 c1 = *reinterpret_cast<const float4*>(&col[1][16 * g + e]);
+              const float4 c2 = *reinterpret_cast<const float4*>(&col[2][16 * g + e]);
+              const float cn[4] = {c1.x, c1.y, c1.z, c1.w}, cr[4] = {c2.x, c2.y, c2.z, c2.w};
+#pragma unroll
+              for (int f = 0; f < 4; ++f) {
+                const float sv = __uint_as_float(rr[g][e + f]);
+                const float eb = __fmaf_ru(A.err_coeff, __fmul_ru(ynr, cn[f]), 1e-30f);
+                const float d2 = __fsub_rd(__fadd_rd(ysq, ca[f]), __fmul_ru(2.f, __fadd_ru(sv, eb)));
+                // sqrt from below: x * rsqrtf(x) is within 2^-22 of sqrt(x)
+                // (rsqrtf is documented to 2 ulp), and the factor 1 - 2^-20
+                // takes it under; tiny or non-positive x gives 0
+                const float dist = d2 > 1e-30f ? __fmul_rd(__fmul_rd(d2, rsqrtf(d2)), 0.99999905f) : 0.f;
+                const float gap = __fsub_rd(dist, cr[f]);
+                out[f] = gap > 0.f ? __fmul_rd(gap, gap) : 0.f;
+              }
+            }
+            *reinterpret_cast<float4*>(stage + lane * LIN_STAGE + e) = make_float4(out[0], out[1], out[2], out[3]);
+          }
+          __syncwarp();
+          // eight rows of 64 bytes at a time
+          const int n = nb + 4 * (lane & 3);
+#pragma unroll
+          for (int h = 0; h < 4; ++h) {
+            const int r = 8 * h + (lane >> 2);
+            const int gr = row - lane + r;
+            const float4 v = *reinterpret_cast<const float4*>(stage + r * LIN_STAGE + 4 * (lane & 3));
+            if (gr < A.rows) {
+              float* zr = A.Z + (size_t)gr * A.N;
+              if ((A.N & 3) == 0) {
+                if (n < A.N) *reinterpret_cast<float4*>(zr + n) = v;
+              } else {
+                const float o[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+                for (int f = 0; f < 4; ++f)
+                  if (n + f < A.N) zr[n + f] = o[f];
+              }
+            }
+          }
+          __syncwarp();
         }
-        continue;
       }
-      if (!live) continue;
-#pragma unroll
-      for (int b = 0; b < 4; ++b)
-#pragma unroll
-        for (int e = 0; e < 16; e += 4) {
-          const int nq = n0 + cb + 16 * b + e;
-          float out[4];
-#pragma unroll
-          for (int f = 0; f < 4; ++f) {
-            const int n = nq + f;
-            const float sv = __uint_as_float(rr[b][e + f]);
-            out[f] = 0.f;
-            if (n >= A.N) continue;
-            const int cl = n - n0;
-            if (MODE == LIN_ARGMAX) {
-              const unsigned long long key =
-                  ((unsigned long long)ordered_bits(sv + col_a[cl]) << 32) | (0xffffffffu - (unsigned)n);
-              best = key > best ? key : best;
-            } else if (MODE == LIN_STORE) {
-              out[f] = sv + col_a[cl];
-            } else {
-              const float eb = __fmaf_ru(A.err_coeff, __fmul_ru(ynr, col_b[cl]), 1e-30f);
-              const float d2 = __fsub_rd(__fadd_rd(ysq, col_a[cl]), __fmul_ru(2.f, __fadd_ru(sv, eb)));
-              // sqrt from below: x * rsqrtf(x) is within 2^-22 of sqrt(x)
-              // (rsqrtf is documented to 2 ulp), and the factor 1 - 2^-20
-              // takes it under; tiny or non-positive x gives 0
-              const float dist = d2 > 1e-30f ? __fmul_rd(__fmul_rd(d2, rsqrtf(d2)), 0.99999905f) : 0.f;
-              const float gap = __fsub_rd(dist, col_c[cl]);
-              out[f] = gap > 0.f ? __fmul_rd(gap, gap) : 0.f;
-            }
-          }
-          if (MODE != LIN_ARGMAX) {
-            float* zr = A.Z + (size_t)row * A.N;
-            if ((A.N & 3) == 0 && nq + 3 < A.N) {
-              *reinterpret_cast<float4*>(zr + nq) = make_float4(out[0], out[1], out[2], out[3]);
-            } else {
-#pragma unroll
-              for (int f = 0; f < 4; ++f)
-                if (nq + f < A.N) zr[nq + f] = out[f];
-            }
-          }
-        }
+      if (MODE == LIN_ARGMAX && (i + 1 == nt || (t + 1) % ncol == 0)) {
+        if (live) atomicMax(A.part + row, best);
+        best = 0ULL;
+      }
     }
-    if (MODE == LIN_ARGMAX && live) A.part[(size_t)row * gridDim.x + blockIdx.x] = best;
-  } else if (threadIdx.x == 0) {
-    atomicOr(A.err, EF_TIMEOUT);
   }
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
-  if (warp == 0) tmem_dealloc(tmem, LIN_TILE);
+  if (warp == LIN_EPI) tmem_dealloc(tmem, 2 * LIN_TILE);
 }
 
-// out[row] = the column of the row's largest partial key
-__global__ void k_argmax_parts(const unsigned long long* __restrict__ part, int rows, int tiles, int* __restrict__ out) {
+// out[row] = the column of the row's largest key
+__global__ void k_argmax_parts(const unsigned long long* __restrict__ part, int rows, int* __restrict__ out) {
   const int r = blockIdx.x * blockDim.x + threadIdx.x;
-  if (r >= rows) return;
-  unsigned long long best = 0ULL;
-  for (int t = 0; t < tiles; ++t) best = max(best, part[(size_t)r * tiles + t]);
-  out[r] = (int)(0xffffffffu - (unsigned)(best & 0xffffffffu));
+  if (r < rows) out[r] = (int)(0xffffffffu - (unsigned)(part[r] & 0xffffffffu));
 }
 
 // Per point: |p|^2 (relative error <= gamma_d in any order of summation)
@@ -1136,12 +1218,14 @@ int pack_rows_bf16(const float* src, int rows, int K, uint8_t* out, cudaStream_t
 template <int MODE>
 static int launch_linear_tc(const LinArgs& A, cudaStream_t st) {
   if (!linear_tc_supported(A.K) || A.rows <= 0 || A.N <= 0) return -2;
-  const int smem = 2 * LIN_TILE * 2 * LIN_MAX_K;
   static const bool attr =
-      cudaFuncSetAttribute(k_linear_tc<MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) == cudaSuccess;
+      cudaFuncSetAttribute(k_linear_tc<MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, LIN_SMEM) == cudaSuccess;
   if (!attr) return -1;
-  dim3 grid((A.N + LIN_TILE - 1) / LIN_TILE, (A.rows + LIN_TILE - 1) / LIN_TILE);
-  k_linear_tc<MODE><<<grid, 128, 2 * LIN_TILE * 2 * A.K, st>>>(A);
+  const int ncol = (A.N + LIN_TILE - 1) / LIN_TILE;
+  const int64_t tiles = (int64_t)ncol * ((A.rows + LIN_TILE - 1) / LIN_TILE);
+  if (tiles > INT_MAX) return -2;
+  const int smem = 3 * LIN_TILE * 2 * A.K + LIN_EPI * 32 * LIN_STAGE * 4;
+  k_linear_tc<MODE><<<(int)std::min<int64_t>(tiles, num_sms()), LIN_THREADS, smem, st>>>(A, (int)tiles, ncol);
   return cudaGetLastError() == cudaSuccess ? 0 : -1;
 }
 
@@ -1164,9 +1248,10 @@ int linear_tc_argmax(const uint8_t* X, int rows, int K, const uint8_t* W, const 
                      unsigned long long* part, int* out, unsigned* err, cudaStream_t st) {
   LinArgs A{};
   A.X = X, A.W = W, A.K = K, A.rows = rows, A.N = N, A.bias = bias, A.part = part, A.err = err;
+  if (rows > 0 && cudaMemsetAsync(part, 0, (size_t)rows * sizeof(unsigned long long), st) != cudaSuccess) return -1;
   const int rc = launch_linear_tc<LIN_ARGMAX>(A, st);
   if (rc) return rc;
-  k_argmax_parts<<<(rows + 255) / 256, 256, 0, st>>>(part, rows, (N + LIN_TILE - 1) / LIN_TILE, out);
+  k_argmax_parts<<<(rows + 255) / 256, 256, 0, st>>>(part, rows, out);
   return cudaGetLastError() == cudaSuccess ? 0 : -1;
 }
 
