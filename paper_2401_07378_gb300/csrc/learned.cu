@@ -428,142 +428,169 @@ __global__ void __launch_bounds__(256) k_select_rows(const float* __restrict__ V
   }
 }
 
-constexpr int SEL_WARPS = 8;   // rows per block of the one-warp selection
+constexpr int SEL_WARPS = 4;   // rows per block of the one-warp selection
 constexpr int SEL_CAP = 256;   // candidates a warp keeps in shared memory
 constexpr int SEL_DEPTH = 8;   // 16-byte loads of a lane in flight
 
 // The same selection (the PROP_LIST largest keys, lowest column first among
 // equal keys, written in that order), one warp per row, with no atomics:
-//  1. the row's columns fall into 64 groups (lane x half of the row); the
-//     two largest keys of every group form a set S, and T is the 64th
-//     largest key of S, so at least 64 keys of the row are >= T;
-//  2. the keys > T are gathered; with fewer than 64 of
-//     them, the first keys == T in column order complete the 64 (exactly
-//     the selection's tie rule), else the 64 are among the gathered ones;
+//  1. the row's columns fall into 64 groups (a lane's even and odd cells, a
+//     cell being VPC 16-byte vectors, or one column in rows that do not split
+//     into vectors); the two largest cell maxima of every group form a set S,
+//     and T is the 64th largest of S, so at least 64 keys of the row are >= T;
+//  2. the keys >= T are gathered from the cells whose maximum reaches T (more
+//     than SEL_CAP: the keys > T, completed by the first keys == T in column
+//     order, exactly the selection's tie rule);
 //  3. each gathered key's rank by (key descending, column ascending) places
 //     the 64 first.
 // A row with more than SEL_CAP keys > T is left to k_select_rows through
-// over_rows / n_over.  Needs cols >= 2 * PROP_LIST.
+// over_rows / n_over.  Needs cols >= 2 * PROP_LIST, and with VPC > 0
+// cols <= 4096 VPC, a multiple of 256, and 16-byte aligned rows.
 //
-// Bound by one warp's way through its row (4,096 rows are one wave): the loads
-// go out eight at a time, and a rank loop reads two words for up to four of a
-// lane's own.  4,096 rows x 4,096 columns: 49.9 us with one load at a time, a
-// shared counter per gathered key and a rank loop per own word; now 44.4 us.
-template <bool LARGEST>
-__global__ void __launch_bounds__(32 * SEL_WARPS, 4) k_select_rows_warp(const float* __restrict__ V, int rows, int cols,
-                                                                   int* __restrict__ out_idx, float* __restrict__ out_val,
-                                                                   int out_stride, int* __restrict__ over_rows,
-                                                                   int* __restrict__ n_over) {
+// Bound by one warp's way through its row (4,096 rows are one wave).  The cell
+// maxima stay in registers, so that the row is read once, eight loads in
+// flight, and only some 80 of its cells again.  4,096 rows x 4,096 columns:
+// 49.9 us for the scores when every pass read the row, 44.4 us with eight loads
+// in flight in the first, now 22.2 us.
+template <bool LARGEST, int VPC>
+__global__ void __launch_bounds__(32 * SEL_WARPS, 7)
+    k_select_rows_warp(const float* __restrict__ V, int rows, int cols, int* __restrict__ out_idx,
+                       float* __restrict__ out_val, int out_stride, int* __restrict__ over_rows,
+                       int* __restrict__ n_over) {
   // gathered words: key, then the complement of the column
   __shared__ __align__(16) unsigned long long c_word[SEL_WARPS][SEL_CAP + 2];
+  __shared__ unsigned short c_cell[SEL_WARPS][VPC ? SEL_CAP : 1];
   const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int r = blockIdx.x * SEL_WARPS + w;
   if (r >= rows) return;
   const float* row = V + (size_t)r * cols;
+  const float4* row4 = reinterpret_cast<const float4*>(row);
+  const unsigned lt = (1u << lane) - 1u;
   auto key_of = [](float v) -> unsigned {
     const unsigned o = ordered_bits(v);
     return LARGEST ? o : ~o;
   };
-  // 1. the two largest keys of each group (lane, half); every group holds
-  // at least two columns (cols >= 128), so all 128 entries are real keys
-  // (starting both at 0, the smallest key, gives the two largest of any
-  // group of two or more keys).  Rows whose columns split into whole
-  // 16-byte vectors per lane and half are read 16 bytes at a time (the
-  // group of a lane is then its vectors in that half).
-  const int half = cols / 2;
-  const bool vec = (cols & 255) == 0 && (reinterpret_cast<uintptr_t>(row) & 15) == 0;
-  auto top2 = [](unsigned k, unsigned& a1, unsigned& a2) {
-    a2 = max(a2, min(a1, k));
-    a1 = max(a1, k);
-  };
+  auto max_of = [&](const float4& v) { return max(max(key_of(v.x), key_of(v.y)), max(key_of(v.z), key_of(v.w))); };
   auto word = [](unsigned k, int c) { return ((unsigned long long)k << 32) | (0xffffffffu - (unsigned)c); };
+  // 1. the two largest cell maxima of each group (0, the smallest key, where a
+  // group has fewer than two: at least 64 of S are keys of the row all the
+  // same)
   unsigned a1[2] = {0u, 0u}, a2[2] = {0u, 0u};
+  auto top2 = [&](unsigned k, int h) {
+    a2[h] = max(a2[h], min(a1[h], k));
+    a1[h] = max(a1[h], k);
+  };
+  constexpr int CELLS = VPC ? 32 : 1;
+  unsigned mx[CELLS];  // this lane's cell maxima
+  const int steps = cols / 128;
+  if constexpr (VPC > 0) {
+    constexpr int DEPTH = SEL_DEPTH / VPC;  // cells per batch of loads
 #pragma unroll
-  for (int h = 0; h < 2; ++h) {
-    if (vec) {
-      const float4* r4 = reinterpret_cast<const float4*>(row) + h * (half / 4) + lane;
-      const int steps = half / 128;
-      int f = 0;
-      for (; f + SEL_DEPTH <= steps; f += SEL_DEPTH) {
-        float4 v[SEL_DEPTH];
+    for (int g = 0; g < CELLS; g += DEPTH) {
+      float4 v[DEPTH][VPC];
 #pragma unroll
-        for (int u = 0; u < SEL_DEPTH; ++u) v[u] = r4[32 * (f + u)];
+      for (int u = 0; u < DEPTH; ++u)
 #pragma unroll
-        for (int u = 0; u < SEL_DEPTH; ++u) {
-          top2(key_of(v[u].x), a1[h], a2[h]);
-          top2(key_of(v[u].y), a1[h], a2[h]);
-          top2(key_of(v[u].z), a1[h], a2[h]);
-          top2(key_of(v[u].w), a1[h], a2[h]);
-        }
+        for (int e = 0; e < VPC; ++e)
+          if ((g + u) * VPC + e < steps) v[u][e] = row4[32 * ((g + u) * VPC + e) + lane];
+#pragma unroll
+      for (int u = 0; u < DEPTH; ++u) {
+        unsigned k = 0u;
+#pragma unroll
+        for (int e = 0; e < VPC; ++e)
+          if ((g + u) * VPC + e < steps) k = max(k, max_of(v[u][e]));
+        mx[g + u] = k;
+        top2(k, u & 1);
       }
-      for (; f < steps; ++f) {
-        const float4 v = r4[32 * f];
-        top2(key_of(v.x), a1[h], a2[h]);
-        top2(key_of(v.y), a1[h], a2[h]);
-        top2(key_of(v.z), a1[h], a2[h]);
-        top2(key_of(v.w), a1[h], a2[h]);
-      }
-    } else {
-      for (int c = h * half + lane; c < (h ? cols : half); c += 32) top2(key_of(row[c]), a1[h], a2[h]);
+    }
+  } else {
+    int h = 0;
+    for (int c = lane; c < cols; c += 32, h ^= 1) {
+      const unsigned k = key_of(row[c]);
+      if (h) top2(k, 1);
+      else top2(k, 0);
     }
   }
-  // T: the largest key of S with at least 64 keys of S at or above it,
-  // bit by bit from the top (the count of keys >= t only falls as t grows,
-  // so the largest t that keeps it at 64 is the 64th largest key of S)
+  // T: the largest key with at least 64 members of S at or above it, bit by
+  // bit from the top (the count of keys >= t only falls as t grows, so the
+  // largest t that keeps it at 64 is the 64th largest key of S)
   unsigned T = 0u;
   for (int bit = 31; bit >= 0; --bit) {
     const unsigned t = T | (1u << bit);
     const unsigned ge = (a1[0] >= t) + (a2[0] >= t) + (a1[1] >= t) + (a2[1] >= t);
     if (__reduce_add_sync(0xffffffffu, ge) >= PROP_LIST) T = t;
   }
-  // 2. keys > T (ranked in step 3, so their order here does not matter)
+  // 2. the keys at or above `from` (ranked in step 3, so their order here does
+  // not matter)
   int n = 0;
-  auto gather = [&](unsigned k, int c) {  // the whole warp
-    const unsigned bal = __ballot_sync(0xffffffffu, k > T);
-    if (bal) {
-      const int pos = n + __popc(bal & ((1u << lane) - 1u));
-      if (k > T && pos < SEL_CAP) c_word[w][pos] = word(k, c);
-      n += __popc(bal);
+  auto gather = [&](unsigned k, int c, bool p) {  // the whole warp
+    const unsigned bal = __ballot_sync(0xffffffffu, p);
+    const int pos = n + __popc(bal & lt);
+    if (p && pos < SEL_CAP) c_word[w][pos] = word(k, c);
+    n += __popc(bal);
+  };
+  auto collect = [&](unsigned from) {
+    n = 0;
+    __syncwarp();
+    if constexpr (VPC > 0) {
+      int nc = 0;
+#pragma unroll
+      for (int u = 0; u < CELLS; ++u) {
+        const bool p = u * VPC < steps && mx[u] >= from;
+        const unsigned bal = __ballot_sync(0xffffffffu, p);
+        const int pos = nc + __popc(bal & lt);
+        if (p && pos < SEL_CAP) c_cell[w][pos] = (unsigned short)(32 * u + lane);
+        nc += __popc(bal);
+      }
+      __syncwarp();
+      if (nc > SEL_CAP) {  // as many keys at least
+        n = nc;
+        return;
+      }
+      for (int base = 0; base < nc; base += 32) {
+        const bool in = base + lane < nc;
+        const int cell = c_cell[w][in ? base + lane : base];
+#pragma unroll
+        for (int e = 0; e < VPC; ++e) {
+          const int f = (cell >> 5) * VPC + e;
+          const bool have = in && f < steps;
+          const int f4 = 32 * f + (cell & 31);
+          const float4 v = have ? row4[f4] : make_float4(0.f, 0.f, 0.f, 0.f);
+          const unsigned k[4] = {key_of(v.x), key_of(v.y), key_of(v.z), key_of(v.w)};
+#pragma unroll
+          for (int i = 0; i < 4; ++i) gather(k[i], 4 * f4 + i, have && k[i] >= from);
+        }
+      }
+    } else {
+      for (int base = 0; base < cols; base += 32) {
+        const int c = base + lane;
+        const unsigned k = c < cols ? key_of(row[c]) : 0u;
+        gather(k, c, c < cols && k >= from);
+      }
     }
   };
-  if (vec) {
-    const float4* r4 = reinterpret_cast<const float4*>(row) + lane;
-    const int steps = cols / 128;
-    for (int f = 0; f < steps; f += 2) {  // (cols is a multiple of 256)
-      const float4 v = r4[32 * f], v2 = r4[32 * (f + 1)];
-      const int c = 4 * (32 * f + lane);
-      gather(key_of(v.x), c);
-      gather(key_of(v.y), c + 1);
-      gather(key_of(v.z), c + 2);
-      gather(key_of(v.w), c + 3);
-      gather(key_of(v2.x), c + 128);
-      gather(key_of(v2.y), c + 129);
-      gather(key_of(v2.z), c + 130);
-      gather(key_of(v2.w), c + 131);
-    }
-  } else {
-    for (int base = 0; base < cols; base += 32) {
-      const int c = base + lane;
-      gather(c < cols ? key_of(row[c]) : 0u, c);
-    }
-  }
+  collect(T);
   if (n > SEL_CAP) {
-    if (lane == 0) over_rows[atomicAdd(n_over, 1)] = r;
-    return;
-  }
-  // ... completed by the first keys == T when fewer than 64 exceed it
-  for (int base = 0; base < cols && n < PROP_LIST; base += 32) {
-    const int c = base + lane;
-    const bool p = c < cols && key_of(row[c]) == T;
-    const unsigned bal = __ballot_sync(0xffffffffu, p);
-    const int pos = n + __popc(bal & ((1u << lane) - 1u));
-    if (p && pos < PROP_LIST) c_word[w][pos] = word(T, c);
-    n = min(PROP_LIST, n + __popc(bal));
+    if (T == 0xffffffffu) n = 0;
+    else collect(T + 1u);
+    if (n > SEL_CAP) {
+      if (lane == 0) over_rows[atomicAdd(n_over, 1)] = r;
+      return;
+    }
+    // ... completed by the first keys == T when fewer than 64 exceed it
+    for (int base = 0; base < cols && n < PROP_LIST; base += 32) {
+      const int c = base + lane;
+      const bool p = c < cols && key_of(row[c]) == T;
+      const unsigned bal = __ballot_sync(0xffffffffu, p);
+      const int pos = n + __popc(bal & lt);
+      if (p && pos < PROP_LIST) c_word[w][pos] = word(T, c);
+      n = min(PROP_LIST, n + __popc(bal));
+    }
   }
   if (lane < 2) c_word[w][n + lane] = 0ULL;  // (the scan below takes two words at a time)
   __syncwarp();
-  // 3. ranks (words are distinct), four of a lane's words against each word
-  // read; the first PROP_LIST are written
+  // 3. ranks (words are distinct), up to four of a lane's words against each
+  // word read; the first PROP_LIST are written
   for (int base = 0; base < n; base += 128) {
     unsigned long long mine[4];
     int rank[4] = {0, 0, 0, 0};
@@ -675,8 +702,15 @@ static void select_rows(const float* V, int rows, int cols, int* out_idx, float*
                         cudaStream_t st) {
   if (cols >= 2 * PROP_LIST) {
     cudaMemsetAsync(L.nsel_over, 0, sizeof(int), st);
-    k_select_rows_warp<LARGEST><<<(rows + SEL_WARPS - 1) / SEL_WARPS, 32 * SEL_WARPS, 0, st>>>(
-        V, rows, cols, out_idx, out_val, PROP_LIST, L.sel_over, L.nsel_over);
+    auto warps = [&](auto vpc) {
+      k_select_rows_warp<LARGEST, decltype(vpc)::value><<<(rows + SEL_WARPS - 1) / SEL_WARPS, 32 * SEL_WARPS, 0, st>>>(
+          V, rows, cols, out_idx, out_val, PROP_LIST, L.sel_over, L.nsel_over);
+    };
+    // whole vectors of aligned rows, up to 32 cells a lane; else a column at a time
+    const bool vec = (cols & 255) == 0 && (reinterpret_cast<uintptr_t>(V) & 15) == 0;
+    if (vec && cols <= 4096) warps(std::integral_constant<int, 1>());
+    else if (vec && cols <= 2 * 4096) warps(std::integral_constant<int, 2>());
+    else warps(std::integral_constant<int, 0>());
     k_select_rows<LARGEST><<<rows, 256, cols * sizeof(unsigned), st>>>(V, rows, cols, out_idx, out_val, PROP_LIST,
                                                                        L.sel_over, L.nsel_over);
   } else {

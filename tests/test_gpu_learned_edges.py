@@ -1,7 +1,6 @@
 """Solves with a proposal at the edges of its passes' tiles and selections
-(128 x 128 blocks of rows and cells, 256 columns a vectorised row, 64 cells
-kept), against the oracle bit for bit, and the consumer counts of the search
-adding up."""
+(128 x 128 blocks of rows and cells, rows of 256 and of 4,096 columns, 64 cells
+kept), against the oracle bit for bit."""
 import numpy as np
 import pytest
 
@@ -21,7 +20,8 @@ def ctx():
 
 
 @pytest.mark.parametrize("d,hidden", [(64, 256), (48, 80), (32, 16)])
-@pytest.mark.parametrize("cells,n", [(64, 2100), (129, 2177), (256, 2049), (263, 2500), (512, 2560), (1030, 4097)])
+@pytest.mark.parametrize("cells,n", [(64, 2100), (129, 2177), (256, 2049), (263, 2500), (512, 2560), (1030, 4097),
+                                     (4096, 4500), (6400, 6500)])
 def test_solve_with_proposal_equals_oracle(ctx, d, hidden, cells, n):
     from paper_2401_07378_gb300 import nnsemd
     p = wl.gmm_pair(cells + d, n=n, d=d, components=50)
