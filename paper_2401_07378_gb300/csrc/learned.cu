@@ -1059,8 +1059,15 @@ __global__ void k_lc_group(LcArgs A) {
 // registers; the cell's active suppliers pass through shared memory
 // LC_TILE rows at a time and every thread runs the key32<SQL2> chain of
 // four suppliers at once against its row.
+//
+// Bound by the L1 path beside the FP32 pipe (0.38 of it): with the consumers'
+// rows read one row a lane (32 lookups a load) those cost as many cycles as the
+// arithmetic.  Round 0 of 131,072 points, 32 cells of 32 suppliers a consumer:
+// 1,445 us that way, 1,144 us with the rows read coalesced (five CTAs per SM
+// in both).
 template <int D>
-__global__ void __launch_bounds__(LC_THREADS) k_lc_keys(LcArgs A) {
+__global__ void __launch_bounds__(LC_THREADS, D == 128 ? 3 : 5) k_lc_keys(LcArgs A) {
+  static_assert(LC_TILE * 2 == LC_THREADS && D % 32 == 0, "a warp's half rows fit its part of xs");
   __shared__ __align__(16) float xs[LC_TILE][D];
   __shared__ int ps[LC_TILE];
   __shared__ int s_wi;
@@ -1082,16 +1089,36 @@ __global__ void __launch_bounds__(LC_THREADS) k_lc_keys(LcArgs A) {
     const int qi = (wi - A.work_off[c]) * LC_THREADS + tid;
     const bool has = qi < A.qoff[c + 1] - A.qoff[c];
     const int q = has ? A.qlist[A.qoff[c] + qi] : 0;
+    // the consumers' rows, half at a time through this warp's part of xs (free
+    // here): read coalesced, then one row a lane; 16-byte columns swizzled so
+    // that neither side meets bank conflicts
     float yr[D];
-    if (has) {
-      const float4* y4 = reinterpret_cast<const float4*>(A.y + (size_t)A.ja[q] * D);
+    {
+      constexpr int C4 = D / 8;  // 16-byte columns of half a row
+      const int lane = tid & 31, j = A.ja[q];
+      float4* part = reinterpret_cast<float4*>(&xs[0][0]) + (tid >> 5) * 32 * C4;
+      auto at = [](int r, int k) { return r * C4 + (k ^ (C4 >= 8 ? r & 7 : (r >> 1) & (C4 - 1))); };
 #pragma unroll
-      for (int k = 0; k < D / 4; ++k) {
-        const float4 v = y4[k];
-        yr[4 * k] = v.x;
-        yr[4 * k + 1] = v.y;
-        yr[4 * k + 2] = v.z;
-        yr[4 * k + 3] = v.w;
+      for (int h = 0; h < 2; ++h) {
+        float4 v[C4];
+#pragma unroll
+        for (int i = 0; i < C4; ++i) {
+          const int r = (32 * i + lane) / C4, k = (32 * i + lane) % C4;
+          const int jr = __shfl_sync(0xffffffffu, j, r);
+          v[i] = reinterpret_cast<const float4*>(A.y + (size_t)jr * D)[h * C4 + k];
+        }
+        __syncwarp();
+#pragma unroll
+        for (int i = 0; i < C4; ++i) part[at((32 * i + lane) / C4, (32 * i + lane) % C4)] = v[i];
+        __syncwarp();
+#pragma unroll
+        for (int k = 0; k < C4; ++k) {
+          const float4 u = part[at(lane, k)];
+          yr[4 * (h * C4 + k)] = u.x;
+          yr[4 * (h * C4 + k) + 1] = u.y;
+          yr[4 * (h * C4 + k) + 2] = u.z;
+          yr[4 * (h * C4 + k) + 3] = u.w;
+        }
       }
     }
     unsigned long long best = ~0ULL;

@@ -19,7 +19,7 @@ def ctx():
     c.close()
 
 
-@pytest.mark.parametrize("d,hidden", [(64, 256), (48, 80), (32, 16)])
+@pytest.mark.parametrize("d,hidden", [(64, 256), (48, 80), (32, 16), (128, 32)])
 @pytest.mark.parametrize("cells,n", [(64, 2100), (129, 2177), (256, 2049), (263, 2500), (512, 2560), (1030, 4097),
                                      (4096, 4500), (6400, 6500)])
 def test_solve_with_proposal_equals_oracle(ctx, d, hidden, cells, n):
