@@ -9,14 +9,18 @@
 //                       memory and move with the compaction;
 //   GeoGlobal (d > 8)   coordinates stay in global memory (L2) and are read
 //                       by original index; the NNS step runs 64 x 64 tiles
-//                       staged in shared memory by 256-thread groups;
+//                       staged in shared memory by 256-thread groups,
+//                       or, for batched pairs, read from a matrix of the
+//                       pair's keys computed once;
+//   GeoMatCluster (d > 8) the tail of a large solve on a cluster, from a key
+//                       matrix;
 //   GeoSmemCluster      GeoSmem on every CTA of a thread-block cluster: each
 //                       CTA holds the whole state, finds the nearest
 //                       supplier of its slice of the consumers and sends the
 //                       keys to every CTA through distributed shared memory;
 //                       the rest of the round runs, identically, in every
 //                       CTA (one of them writes the results).
-// Grouping, greedy order, flow and compaction are the same for both.
+// Grouping, greedy order, flow and compaction are the same for all.
 #pragma once
 
 #include <cooperative_groups.h>
