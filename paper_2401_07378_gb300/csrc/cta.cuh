@@ -473,7 +473,9 @@ NNS_DEV void group_tiles(const float* __restrict__ x, const int* ia, int p0, int
 
 // The lowest (key32 bits << 32 | position) over the suppliers [p0, p1) of
 // each consumer of group_tiles; returned, in the threads with tx == 0, for
-// their 4 consumers (others: ~0).
+// their 4 consumers (~0 only where p0 == p1).  A thread starts at +inf and its
+// own first supplier, so a consumer whose keys all overflow to +inf gets the
+// first position, as from a scan in order.
 template <bool L1, bool PRE = false>
 NNS_DEV void group_nns_tile(const float* __restrict__ x, const int* ia, int p0, int p1, const float* __restrict__ y,
                             const int* ja, const int* cons, int c0, int nc, int d, TileSmem& T, int gt, int bar,
@@ -482,7 +484,7 @@ NNS_DEV void group_nns_tile(const float* __restrict__ x, const int* ia, int p0, 
   float best[4];
   int bpos[4];
 #pragma unroll
-  for (int i = 0; i < 4; ++i) { best[i] = CUDART_INF_F; bpos[i] = -1; }
+  for (int i = 0; i < 4; ++i) { best[i] = CUDART_INF_F; bpos[i] = p0 + tx * 4 < p1 ? p0 + tx * 4 : -1; }
   group_tiles<L1, PRE>(x, ia, p0, p1, y, ja, cons, c0, nc, d, T, gt, bar,
                        [&](int pt, const unsigned long long (&acc)[2][4]) {
 #pragma unroll

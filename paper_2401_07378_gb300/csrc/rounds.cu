@@ -513,14 +513,17 @@ __global__ void k_group_alloc(const int* __restrict__ cnt, int mt, int2* __restr
 }
 
 // Member key: the serving order (greedy: the distance key bits; random:
-// the round's SplitMix64 key of the consumer) << 32 | consumer position.
-__global__ void k_group_scatter(const unsigned long long* __restrict__ nnkey, int nt, int* __restrict__ cnt,
+// the round's SplitMix64 key of the consumer) << 32 | consumer position.  A
+// consumer without a supplier (k_group_count has raised EF_INTERNAL) is left
+// out.
+__global__ void k_group_scatter(const unsigned long long* __restrict__ nnkey, int nt, int mt, int* __restrict__ cnt,
                                 const int2* __restrict__ seg, unsigned long long* __restrict__ member,
                                 const int* __restrict__ ja, int protocol, unsigned long long seed, long long round) {
   const int q = blockIdx.x * blockDim.x + threadIdx.x;
   if (q >= nt) return;
   const unsigned long long key = nnkey[q];
-  const int p = (int)(key & 0xffffffffULL);
+  const unsigned p = (unsigned)(key & 0xffffffffULL);
+  if (p >= (unsigned)mt) return;
   const int slot = seg[p].x + atomicSub(cnt + p, 1) - 1;
   const unsigned long long order =
       protocol == 1 ? ((unsigned long long)rp_key32(seed, round, ja[q]) << 32) : (key & 0xffffffff00000000ULL);
@@ -773,7 +776,7 @@ int launch_big_round(SolveBufs& B, int mt, int nt, long long round, cudaStream_t
   const int cur = B.cur;
   k_group_count<<<(nt + 255) / 256, 256, 0, st>>>(B.nnkey, nt, mt, B.cnt, &B.st->err, B.st);
   k_group_alloc<<<(mt + 255) / 256, 256, 0, st>>>(B.cnt, mt, B.seg, B.seglist, B.biglist, B.medlist, B.st);
-  k_group_scatter<<<(nt + 255) / 256, 256, 0, st>>>(B.nnkey, nt, B.cnt, B.seg, B.member, B.ja[cur], B.protocol,
+  k_group_scatter<<<(nt + 255) / 256, 256, 0, st>>>(B.nnkey, nt, mt, B.cnt, B.seg, B.member, B.ja[cur], B.protocol,
                                                     B.seed, round);
   FlowArgs F{B.ia[cur], B.ja[cur], B.seg,  B.seglist, B.biglist, B.medlist, B.member,
              B.s,       B.c,       B.fl_i, B.fl_j,    B.fl_f,    B.st};
