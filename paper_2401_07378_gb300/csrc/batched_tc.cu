@@ -374,7 +374,9 @@ struct GeoTC {
     }
     const int q = qs(min(g, cnt - 1)), j = S.jidx[q];
     const float* yrow = y + (size_t)j * d;
-    const bool on = g < cnt && sub < len;
+    // (a supplier whose norm overflows has v' = NaN, which orders like the word
+    // for none: it may be missing here, so its consumers go to 3.)
+    const bool wanted = g < cnt && sub < len, on = wanted && cv != 0xffffffffu;
     if (!on) i = 0;
     const unsigned long long e = on ? pack_key(exact_key(i, yrow, vec), (unsigned)i) : ~0ULL;
     const int first = __shfl_sync(0xffffffffu, i, lane & 24);  // the approximate choice
@@ -389,11 +391,11 @@ struct GeoTC {
     // 2.
     const unsigned tb = __shfl_sync(0xffffffffu, cv, (lane & 24) + len - 1);
     double fl = CUDART_INF;
-    bool bad = false;
+    bool bad = ((__ballot_sync(0xffffffffu, wanted && !on) >> (lane & 24)) & 0xffu) != 0;
     if (g < cnt && mt > len) {
       const float tau = __uint_as_float((tb & 0x80000000u) ? (tb & 0x7fffffffu) : ~tb);
       fl = certify_floor_from_E(scr.ny_o[j], tau, scr.e_o[j], kc_gam);
-      bad = !((double)__uint_as_float((unsigned)(best >> 32)) < fl);
+      bad |= !((double)__uint_as_float((unsigned)(best >> 32)) < fl);
     }
     if (on && !bad) scr.list[(size_t)j * BTC_K + rank] = e;
     if (g < cnt && sub == 0 && !bad) {

@@ -43,6 +43,19 @@ def far_consumers(m, n, d, seed, every=7):
     return p
 
 
+def far_suppliers(m, n, d, seed):
+    """Every other supplier so far out that its squared norm overflows, some
+    consumers beside those, and little weight on the first supplier."""
+    p = wl.uniform_pair(m, n, d, seed, "dirichlet")
+    p.x[1::2] *= FAR
+    p.x[1::2, 0] = FAR
+    far = p.x[1::2]
+    k = p.y[::3].shape[0]
+    p.y[::3] = far[np.arange(k) % far.shape[0]] * np.float32(1 + 2 ** -12)
+    p.a[0] = 1e-3 * p.a.min()
+    return p
+
+
 @pytest.mark.parametrize("precision", ["fp32", "bf16", "fp16", "fp8", "bf16x3"])
 @pytest.mark.parametrize("d", [9, 64])
 def test_batched_far_consumers(ctx, d, precision):
@@ -52,6 +65,19 @@ def test_batched_far_consumers(ctx, d, precision):
     costs, stats = ctx.solve_batched(*batch_args(pairs), metric="l2", precision=precision)
     assert costs.cpu().numpy().tolist() == [r.cost for r in ref]
     assert stats["rounds"] == sum(r.rounds for r in ref)
+
+
+@pytest.mark.parametrize("rk", [0, 3])
+@pytest.mark.parametrize("precision", ["bf16", "fp16", "fp8", "bf16x3"])
+@pytest.mark.parametrize("d", [9, 64])
+def test_batched_far_suppliers(ctx, d, precision, rk):
+    pairs = [far_suppliers(m, n, d, 3 * d + k)
+             for k, (m, n) in enumerate([(2, 513), (5, 600), (8, 700), (9, 530), (24, 1025), (520, 7), (600, 640)])]
+    ref = [oracle.solve_pair(p, "l2") for p in pairs]
+    costs, stats = ctx.solve_batched(*batch_args(pairs), metric="l2", precision=precision, rerank_k=rk)
+    assert costs.cpu().numpy().tolist() == [r.cost for r in ref]
+    assert stats["rounds"] == sum(r.rounds for r in ref)
+    assert stats["certified"] + stats["fallbacks"] == sum(int(r.n_t.sum()) for r in ref)
 
 
 @pytest.mark.parametrize("metric", ["l2", "sql2"])
