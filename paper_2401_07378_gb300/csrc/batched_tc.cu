@@ -758,10 +758,13 @@ struct GeoTC {
     for (int q = warp; q < nt; q += T / 32) {
       const float* yrow = y + (size_t)S.jidx[q] * d;
       unsigned long long best = ~0ULL;
+      int have = 0;  // candidates: all active suppliers where the list is not full, or some are lost to overflow
       if (lane < rk) {
         const int p = scr.cand_p[(size_t)q * BTC_K + lane];
+        have = p >= 0;
         if (p >= 0) best = pack_key(key32<METRIC_SQL2>(x + (size_t)S.iidx[p] * d, yrow, d), (unsigned)p);
       }
+      have = __reduce_add_sync(0xffffffffu, have);
       double yl2 = 0.0, yl1 = 0.0;
       for (int k = lane; k < d; k += 32) {
         yl2 += (double)yrow[k] * yrow[k];
@@ -778,9 +781,9 @@ struct GeoTC {
         // approximate best, and an exact best elsewhere is a near-tie
         const float tau = scr.cand_v[(size_t)q * BTC_K + rk - 1];
         if (best != ~0ULL && (int)(unsigned)best != scr.cand_p[(size_t)q * BTC_K]) atomicAdd(&nnear, 1ULL);
-        const bool cert = best != ~0ULL && certify(fmt, d, scr.nrm_y[q], sqrt(yl2) * (1 + 1e-12), yl1,
-                                                    scr.scale_y[q], rx, rx1, sxm, tau,
-                                                    __uint_as_float((unsigned)(best >> 32)));
+        const bool cert = best != ~0ULL && (tau <= 3.402823466e38f || have == mt) &&
+                          certify(fmt, d, scr.nrm_y[q], sqrt(yl2) * (1 + 1e-12), yl1, scr.scale_y[q], rx, rx1, sxm, tau,
+                                  __uint_as_float((unsigned)(best >> 32)));
         if (cert) {
           S.nnk[q] = best;
           atomicAdd(&ncert, 1ULL);

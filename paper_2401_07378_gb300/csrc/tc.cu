@@ -519,6 +519,7 @@ struct RerankArgs {
   const int* sel;       // packed row -> consumer position (nullable: identity)
   const int* nq_dev;    // rows in use (nullable: nt)
   TcLists lists;        // candidate lists to make (list == nullptr: none)
+  int mt;               // active suppliers
   int rk;               // candidates of each chunk re-ranked (1 .. kl)
   int kl;               // list length of each chunk (the stride of cand_v / cand_p)
 };
@@ -546,7 +547,7 @@ __global__ void __launch_bounds__(RR_THREADS) k_rerank_certify(RerankArgs R) {
   __shared__ unsigned long long s_best[RR_ROWS], s_abest[RR_ROWS];
   __shared__ float s_tau[RR_ROWS];
   __shared__ unsigned s_drop[RR_ROWS];  // the smallest key (bits) a list leaves out
-  __shared__ int s_len[RR_ROWS];
+  __shared__ int s_len[RR_ROWS], s_have[RR_ROWS];
   const int nq = R.nq_dev ? min(*R.nq_dev, R.nt) : R.nt;
   const int r0 = blockIdx.x * RR_ROWS;
   if (r0 >= nq) return;
@@ -562,7 +563,7 @@ __global__ void __launch_bounds__(RR_THREADS) k_rerank_certify(RerankArgs R) {
     // this lane's two smallest keys by original index, and the smallest other
     unsigned long long e1 = ~0ULL, e2 = ~0ULL;
     unsigned drop = 0xffffffffu;
-    int j = 0;
+    int j = 0, have = 0;
     if (r < nq) {
       const int q = R.sel ? R.sel[r] : r;
       j = R.ja[q];
@@ -573,6 +574,7 @@ __global__ void __launch_bounds__(RR_THREADS) k_rerank_certify(RerankArgs R) {
         const int p = R.cand_p[o];
         if (k == rk - 1) tau = fminf(tau, R.cand_v[o]);
         if (p < 0) continue;
+        ++have;
         if (k == 0) {
           const unsigned long long ak = ((unsigned long long)ordered_bits(R.cand_v[o]) << 32) | (unsigned)p;
           abest = ak < abest ? ak : abest;
@@ -642,8 +644,10 @@ __global__ void __launch_bounds__(RR_THREADS) k_rerank_certify(RerankArgs R) {
       const unsigned long long oa = __shfl_xor_sync(0xffffffffu, abest, o);
       abest = oa < abest ? oa : abest;
       tau = fminf(tau, __shfl_xor_sync(0xffffffffu, tau, o));
+      have += __shfl_xor_sync(0xffffffffu, have, o);
     }
     if (sub == 0) {
+      s_have[k0] = have;
       s_best[k0] = best;
       s_abest[k0] = abest;
       s_tau[k0] = tau;
@@ -662,13 +666,15 @@ __global__ void __launch_bounds__(RR_THREADS) k_rerank_certify(RerankArgs R) {
     const float ny = R.nrm_y[r];
     const double yl2 = norm_up(ny);
     const float tau = s_tau[lane], key = __uint_as_float((unsigned)(best >> 32));
-    // (as certify; the bound itself serves the list too)
+    // (as certify; the bound itself serves the list too.  tau = +inf: no list
+    // is full, so every supplier is a candidate, unless its value was lost to
+    // an overflowing norm)
     double fl = CUDART_INF;
     if (tau <= 3.402823466e38f)
       fl = certify_floor(R.fmt, R.d, ny, yl2, yl2 * sqrt((double)R.d) * (1 + 1e-12), R.scale_y[r],
                          __uint_as_float(R.stats_x[0]), __uint_as_float(R.stats_x[1]), __uint_as_float(R.stats_x[2]),
                          tau);
-    certified = !(tau <= 3.402823466e38f) || (double)key < fl;
+    certified = tau <= 3.402823466e38f ? (double)key < fl : s_have[lane] == R.mt;
     if (R.lists.list) {
       const unsigned drop = s_drop[lane];
       if (drop != 0xffffffffu) fl = fmin(fl, (double)__uint_as_float(drop));
@@ -879,7 +885,7 @@ int launch_nns_tc(const SolveBufs& B, const TcBufs& T, int mt, int nt, int preci
   RerankArgs R{B.x,      B.y,        B.ia[B.cur], B.ja[B.cur], B.d,       nt,          nt_pad,
                chunks,   fmt,        T.cand_v,    T.cand_p,    T.nrm_y,   T.scale_y,   T.stats,
                B.nnkey,  T.fallback, T.nfallback, &B.st->certified, &B.st->fallbacks, &B.st->near_ties,
-               sel,      nsel_dev,   B.lists,     rk,          kl};
+               sel,      nsel_dev,   B.lists,     mt,          rk,          kl};
   const bool wide = chunks * rk > 8, few = nt < 32 * 4 * num_sms();
   if (!wide) k_rerank_certify<8, 32><<<(nt + 31) / 32, RR_THREADS, 0, st>>>(R);
   else if (few) k_rerank_certify<32, 8><<<(nt + 7) / 8, RR_THREADS, 0, st>>>(R);

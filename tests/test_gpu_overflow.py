@@ -83,6 +83,17 @@ def test_batched_far_suppliers(ctx, d, precision, rk):
 @pytest.mark.parametrize("metric", ["l2", "sql2"])
 def test_large_far_consumers_fp32(ctx, metric):
     p = far_consumers(3000, 2500, 40, 3)
-    r = oracle.solve_pair(p, metric)
+    r = oracle.solve_pair(p, metric, threads=0)
     got = ctx.solve(*pair_args(p), metric=metric)
     assert got.cost == r.cost and got.stats["rounds"] == r.rounds
+
+
+@pytest.mark.parametrize("precision", ["bf16", "fp16", "fp8", "bf16x3"])
+@pytest.mark.parametrize("m,n,d", [(3000, 2500, 40), (40, 4000, 64), (17, 9000, 64)])
+def test_large_reduced_precision(ctx, m, n, d, precision):
+    for p in (far_consumers(m, n, d, m), far_suppliers(m, n, d, n)):
+        r = oracle.solve_pair(p, "l2", threads=0)
+        for rk in (0, 8):
+            got = ctx.solve(*pair_args(p), metric="l2", precision=precision, rerank_k=rk)
+            assert got.cost == r.cost and got.stats["rounds"] == r.rounds
+            assert got.stats["certified"] + got.stats["fallbacks"] <= int(r.n_t.sum())
