@@ -198,6 +198,11 @@ __global__ void __launch_bounds__(FIN_HD_CL_THREADS, 1) k_finish_hd_cl(SolveBufs
     S.nt = nt;
   }
   M.G.init();
+  // the running totals are read before the barrier: the leader writes them back
+  // after its rounds, and a solve whose rounds are all local (few points) has
+  // no other barrier between that and a late CTA's read
+  unsigned long long nnz = B.st->nnz;
+  long long rounds = B.st->rounds, pe = B.st->pair_evals;
   // every CTA of the cluster is running before any writes a peer's memory
   cl.sync();
   CtaOut O{nullptr, nullptr, nullptr, nullptr, 0, nullptr, nullptr, &B.st->err,
@@ -205,8 +210,6 @@ __global__ void __launch_bounds__(FIN_HD_CL_THREADS, 1) k_finish_hd_cl(SolveBufs
   if (leader)
     O = CtaOut{nullptr, nullptr, nullptr, nullptr, 0, B.s, B.c, &B.st->err,
                B.fl_i, B.fl_j, B.fl_f, B.x, B.y, B.d, B.protocol, B.seed, B.round0, 0};
-  unsigned long long nnz = B.st->nnz;
-  long long rounds = B.st->rounds, pe = B.st->pair_evals;
   cta_rounds(S, M.G, B.metric, O, nnz, rounds, pe, round_limit);
   if (tid == 0 && leader) {
     B.st->nnz = nnz;
