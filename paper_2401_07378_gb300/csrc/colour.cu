@@ -127,6 +127,8 @@ constexpr int KM_BLOCK_POINTS = 65536;
 constexpr int KM_TILE = 1024;           // centroids staged at a time
 constexpr int KM_MAX_KD = 2048;         // k * d whose limbs fit a block's shared memory
 constexpr int KM_MAX_COUNTS = 4096;     // k whose sizes are counted in shared memory first
+// the most dynamic shared memory a launch takes: a tile, the sizes, the sums
+constexpr int KM_SMEM_MAX = 4 * (KM_TILE * 8 + KM_MAX_COUNTS + KM_MAX_KD * KM_LIMBS);
 
 NNS_DEV void km_add(unsigned* acc, float v) {
   const unsigned bits = __float_as_uint(v) & 0x7fffffffu;
@@ -310,7 +312,10 @@ int km_assign_t(const float* pts, int64_t N, int k, const float* cent, int* labe
   const size_t smem = sizeof(float) * ((tile + 7) & ~7) * DP +
                       (k <= KM_MAX_COUNTS ? sizeof(unsigned) * k : 0) +
                       (acc ? sizeof(unsigned) * k * (size_t)(D * KM_LIMBS) : 0);
-  if (cudaFuncSetAttribute(k_km_assign<D, DP, P>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
+  // (the limit belongs to the kernel on the device, not to this call: set to
+  // less by another thread, a launch in between would be refused)
+  static_assert(KM_SMEM_MAX <= 227 * 1024, "fits a block");
+  if (cudaFuncSetAttribute(k_km_assign<D, DP, P>, cudaFuncAttributeMaxDynamicSharedMemorySize, KM_SMEM_MAX) != cudaSuccess)
     return -1;
   // one pass per block where the blocks then fit two per SM; never more
   // points in a block than its 32-bit limbs can take

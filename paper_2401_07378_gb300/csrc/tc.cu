@@ -72,6 +72,7 @@ constexpr int TC_NNRM = 4;                  // column-norm slots (a ring of its 
 // cnt_dev when given; the rest is padding).
 constexpr int PACK_ROWS = 32;
 constexpr int PACK_THREADS = 256;
+constexpr int PACK_SMEM_MAX = 200 * 1024;  // rows of 1,600 coordinates; tc_supported ends at 800
 
 __global__ void __launch_bounds__(PACK_THREADS)
     k_pack_tc(const float* __restrict__ pts, const int* __restrict__ idx, const int* __restrict__ sel,
@@ -826,8 +827,11 @@ int launch_nns_tc(const SolveBufs& B, const TcBufs& T, int mt, int nt, int preci
   if (cudaMemsetAsync(T.stats, 0, 8 * sizeof(unsigned), st) != cudaSuccess) return -1;
   {
     const size_t smem = (size_t)PACK_ROWS * (B.d | 1) * sizeof(float);
+    // (one limit for every row length: it belongs to the kernel on the device,
+    // and another thread's shorter rows must not lower it under this launch)
+    if (smem > PACK_SMEM_MAX) return -2;
     if (smem > 48 * 1024 &&
-        cudaFuncSetAttribute(k_pack_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
+        cudaFuncSetAttribute(k_pack_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, PACK_SMEM_MAX) != cudaSuccess)
       return -1;
     auto grid = [](int64_t rows) { return (int)std::min<int64_t>((rows + PACK_ROWS - 1) / PACK_ROWS, num_sms() * 16); };
     k_pack_tc<<<grid((int64_t)qtiles * TC_BM), PACK_THREADS, smem, st>>>(
