@@ -905,9 +905,10 @@ template <bool KIND8, int CAP>
 static int batched_tc_t(const BtcArgs& A, int grid, cudaStream_t st) {
   const size_t smem = btc_smem_bytes<KIND8, CAP>(A.kb, A.bn, A.nstage);
   if (smem > 227 * 1024) return -2;
-  // (all a block can have, whatever this launch takes: the limit belongs to the
-  // kernel on the device, and another thread's launch may need more)
-  constexpr size_t all = 227 * 1024 - 16;  // (beside the two static words)
+  // (what nearly every launch stays below, whatever this one takes: the limit
+  // belongs to the kernel on the device, and another thread's launch may need
+  // more)
+  constexpr size_t all = 225 * 1024;  // (the static words are padded to the alignment of the dynamic part)
   cudaError_t e = cudaFuncSetAttribute(k_batched_tc<KIND8, CAP>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        (int)(smem > all ? smem : all));
   if (e != cudaSuccess) return -1;

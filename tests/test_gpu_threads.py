@@ -57,3 +57,15 @@ def test_reduced_precision_rows_of_different_lengths():
         jobs.append(lambda c, v=(x, a, y, b): (torch.tensor(c.solve(*v, precision="fp8").cost),))
     torch.cuda.synchronize()
     run_threads(jobs, 20)
+
+
+def test_batched_reduced_precision_rows_of_different_lengths():
+    g = torch.Generator(device="cuda").manual_seed(7)
+    off = torch.arange(0, 9 * 600, 600).numpy()
+    jobs = []
+    for d, precision in ((16, "fp16"), (150, "fp16"), (90, "fp16"), (200, "bf16")):
+        x, y = (torch.randn(8 * 600, d, generator=g, device="cuda") for _ in range(2))
+        a, b = (torch.rand(8 * 600, generator=g, device="cuda", dtype=torch.float64) + 0.1 for _ in range(2))
+        jobs.append(lambda c, v=(x, a, off, y, b, off), p=precision: (c.solve_batched(*v, precision=p)[0],))
+    torch.cuda.synchronize()
+    run_threads(jobs, 20)
