@@ -253,7 +253,7 @@ size_t layout_solve(void* base, int64_t m, int64_t n, int d, SolveBufs& B, bool 
     B.lists.nsel = C.take<int>(1);
   }
   B.grid = GridBufs{};
-  if (extras && d <= 3 && m * n >= GRID_MIN_PAIRS) {
+  if (extras && d <= 3 && std::min(m, n) >= GRID_MIN_SIDE) {
     B.grid.box = C.take<unsigned>(6);
     B.grid.hist = reinterpret_cast<int*>(C.take<uint8_t>(4 * grid_cells_bytes()));
     B.grid.start = reinterpret_cast<int*>(C.take<uint8_t>(grid_cells_bytes()));

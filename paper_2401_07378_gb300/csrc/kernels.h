@@ -144,7 +144,15 @@ int launch_big_round(SolveBufs& B, int mt, int nt, long long round, cudaStream_t
 int launch_nns_lowd(const SolveBufs& B, int mt, int nt, cudaStream_t st, const unsigned long long* grid_work = nullptr);
 
 // lowd_grid.cu -------------------------------------------------------------
-constexpr int64_t GRID_MIN_PAIRS = 1LL << 26;  // m_t * n_t from which a round takes the grid
+// Points of the smaller side from which a round takes the grid.  Its five small
+// launches and the query's chain of blocks take some 45 us where K1 takes 53 at
+// 16,384 x 16,384 points, and the query's time per warp grows with the larger
+// side alone: few consumers, or few suppliers to sort many consumers for, leave
+// it behind K1 (whole solves with the grid from 2^26 pairs on, without and with
+// it: 8,192 x 8,192 uniform points d = 2 495 and 527 us, 300,000 x 300 101 and
+// 156 ms, 200,000 x 3,000 12.3 and 18.9 ms; 32,768 x 32,768 d = 3 1,170 and 954
+// us).
+constexpr int64_t GRID_MIN_SIDE = 1 << 14;
 size_t grid_cells_bytes();
 size_t grid_box_floats(int64_t m);
 // The box of the initial active sets (once per solve, before the first grid

@@ -30,6 +30,8 @@
 // K1 845).
 #include <math_constants.h>
 
+#include <algorithm>
+
 #include "common.cuh"
 #include "kernels.h"
 
@@ -371,11 +373,9 @@ int launch_grid_bounds(const SolveBufs& B, int mt, int nt, cudaStream_t st) {
   return 0;
 }
 
-// Large rounds in up to three dimensions.  The six small launches and the
-// query take about 40 us whatever the size; K1 takes that long at some 2^27
-// pairs.
+// Large rounds in up to three dimensions, both sides large.
 bool grid_nns_wanted(const SolveBufs& B, int mt, int nt) {
-  return B.grid.box && B.d <= 3 && (int64_t)mt * nt >= GRID_MIN_PAIRS;
+  return B.grid.box && B.d <= 3 && std::min(mt, nt) >= GRID_MIN_SIDE;
 }
 
 int launch_nns_grid(const SolveBufs& B, int mt, int nt, cudaStream_t st) {
