@@ -78,7 +78,7 @@ TOL_FP32 = 1e-5                # relative error bound of the FP32 forms against 
 TOL_REDUCED = 1e-3             # ... of the reduced-precision and learned forms
 WORK_FILE = os.path.join(ROOT, "tests", "golden", "colour_transfer_oracle.json")
 KEY_MATRIX_MAX = 512           # batched pairs (d > 8) up to this size run on FP32 key matrices in any precision
-GRID_MAX_D, GRID_MIN_SIDE = 3, 1 << 14  # rounds the grid search takes from K1
+GRID_MAX_D, GRID_MIN_SIDE = 3, 7 << 11  # rounds the grid search takes from K1
 COUNTERS_FILE = os.path.join(ROOT, "profiles", "k_nns_lowd_colour_transfer.json")
 
 WORKLOADS = {
@@ -611,7 +611,7 @@ def run_ours(args) -> dict | None:
             rl["note"] = "achieved counts the full scan's 2d ops per pair: an effective rate, not pipe utilisation"
         elif d <= GRID_MAX_D and min(int(inp.x.shape[0]), int(inp.y.shape[0])) >= GRID_MIN_SIDE:
             # the large rounds go through the grid search, which visits a small part of the pairs
-            rl["kernel"] = "NNS step: grid search of the rounds of 16,384 points a side and more, k_nns_lowd (K1) of the others"
+            rl["kernel"] = "NNS step: grid search of the rounds of 14,336 points a side and more, k_nns_lowd (K1) of the others"
             rl["note"] = ("achieved counts the full scan's 2d ops per pair: an effective rate of the exact search, "
                           "not pipe utilisation, so no fraction is given; bound by latency")
             rl["frac"], rl["traffic"] = None, None

@@ -260,7 +260,7 @@ size_t layout_solve(void* base, int64_t m, int64_t n, int d, SolveBufs& B, bool 
     B.grid.xs = C.take<float>((size_t)m * 4);
     B.grid.ys = C.take<float>((size_t)n * 4);
     B.grid.boxes = C.take<float>(grid_box_floats(m));
-    B.grid.work = C.take<unsigned long long>(1);
+    B.grid.work = C.take<unsigned long long>(2);
   }
   B.kmat = nullptr;
   if (extras && d > 8)
@@ -422,6 +422,12 @@ int run_solve(nnsemd_ctx* ctx, SolveBufs& B, const double* a, const double* b, d
          (tcb ? 2 : 0) + (5 + (tcb ? 2 : 0) + 2 * sel) * ((B.n + learned->chunk - 1) / learned->chunk);
   }
   bool boxed = false;  // the grid's bounding box is there
+  // a round's points did not suit the grid (set on the device): the next four
+  // rounds go without a try, after another refusal the next eight, and so on
+  // (an attempt costs up to some 100 us; the sets change slowly)
+  volatile int* no_grid = ctx->hmap + 10;
+  *no_grid = 0;
+  int grid_rest = 0, grid_pause = 4;
   while (mt > 0 && nt > 0) {
     // d > 8: the cluster tail takes over once both active sets fit it (with a
     // reduced precision or a proposal from the second round on: the first is
@@ -488,7 +494,7 @@ int run_solve(nnsemd_ctx* ctx, SolveBufs& B, const double* a, const double* b, d
         L += 5;
       }
     } else {
-      const bool grid = lowd && grid_nns_wanted(B, mt, nt);
+      const bool grid = lowd && grid_nns_wanted(B, mt, nt) && --grid_rest < 0;
       if (timed) CKD(cudaEventRecord(ctx->ev[0], st));
       nrc = 0;
       if (grid) {
@@ -498,7 +504,7 @@ int run_solve(nnsemd_ctx* ctx, SolveBufs& B, const double* a, const double* b, d
         boxed = true;
       }
       if (!nrc)
-        nrc = lowd ? launch_nns_lowd(B, mt, nt, st, grid ? B.grid.work : nullptr)
+        nrc = lowd ? launch_nns_lowd(B, mt, nt, st, grid ? B.grid.work : nullptr, ctx->dmap + 10)
                    : launch_nns_f32(B, mt, nt, nullptr, nullptr, st);
       if (timed) CKD(cudaEventRecord(ctx->ev[1], st));
       L += 1;
@@ -520,6 +526,11 @@ int run_solve(nnsemd_ctx* ctx, SolveBufs& B, const double* a, const double* b, d
     unsigned err_bits = 0;
     rc = wait_counts(ctx, st, B.notify_seq, mt, nt, err_bits);
     if (rc) return drained(rc);
+    if (*no_grid) {
+      *no_grid = 0;
+      grid_rest = grid_pause;
+      grid_pause *= 2;
+    }
     if (nns_timed) {
       float ms = 0.f;
       CKD(cudaEventSynchronize(ctx->ev[1]));

@@ -27,7 +27,7 @@ struct nnsemd_ctx {
   void* cws = nullptr;                 // scratch of the colour-transfer entry points (colour.cu)
   size_t cws_bytes = 0;
   nnsemd::DevState* hstate = nullptr;  // pinned mirror of the device state
-  volatile int* hmap = nullptr;        // mapped pinned words: [0..3] a round's active counts, [8] an error word, [9] consumers left by the lists (host view)
+  volatile int* hmap = nullptr;        // mapped pinned words: [0..3] a round's active counts, [8] an error word, [9] consumers left by the lists, [10] the grid is refused (host view)
   int* dmap = nullptr;                 // the same words, device view
   int notify_seq = 0;                  // sequence number of the last requested notification
   std::string err;

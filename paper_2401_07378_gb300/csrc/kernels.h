@@ -76,7 +76,7 @@ struct GridBufs {
   float* xs;                 // sorted suppliers / consumers, 4 floats a point
   float* ys;
   float* boxes;
-  unsigned long long* work;  // what the round's cells hold in common: the kernels' own choice of path
+  unsigned long long* work;  // [2] what the round's cells hold in common and its visits (grid_served)
 };
 
 // Buffers of one single-pair solve (device pointers inside the workspace).
@@ -140,34 +140,42 @@ int launch_big_round(SolveBufs& B, int mt, int nt, long long round, cudaStream_t
 
 // lowd.cu ------------------------------------------------------------------
 // `grid_work` (nullable): skip the scan where the grid step before it served
-// the round (its own rule on that value).
-int launch_nns_lowd(const SolveBufs& B, int mt, int nt, cudaStream_t st, const unsigned long long* grid_work = nullptr);
+// the round (grid_served), else say so in *refused (host memory mapped into the
+// device).
+int launch_nns_lowd(const SolveBufs& B, int mt, int nt, cudaStream_t st, const unsigned long long* grid_work = nullptr,
+                    int* refused = nullptr);
 
 // lowd_grid.cu -------------------------------------------------------------
-// Points of the smaller side from which a round takes the grid.  Its five small
-// launches and the query's chain of blocks take some 45 us where K1 takes 53 at
-// 16,384 x 16,384 points, and the query's time per warp grows with the larger
-// side alone: few consumers, or few suppliers to sort many consumers for, leave
+// Points of the smaller side from which a round takes the grid.  Its four small
+// launches and the query take some 50 us and the gaps between them 10 where K1
+// takes 82 (just below 16,384 x 16,384 points, d = 3) and 48 (some 13,000 a side),
+// and the query's time per warp grows with the larger side alone: few consumers, or few suppliers to sort many consumers for, leave
 // it behind K1 (whole solves with the grid from 2^26 pairs on, without and with
 // it: 8,192 x 8,192 uniform points d = 2 495 and 527 us, 300,000 x 300 101 and
 // 156 ms, 200,000 x 3,000 12.3 and 18.9 ms; 32,768 x 32,768 d = 3 1,170 and 954
 // us).
-constexpr int64_t GRID_MIN_SIDE = 1 << 14;
+constexpr int64_t GRID_MIN_SIDE = 7 << 11;
 size_t grid_cells_bytes();
 size_t grid_box_floats(int64_t m);
 // The box of the initial active sets (once per solve, before the first grid
 // step).
 int launch_grid_bounds(const SolveBufs& B, int mt, int nt, cudaStream_t st);
 bool grid_nns_wanted(const SolveBufs& B, int mt, int nt);
-// Nearest active supplier of every active consumer into B.nnkey, or nothing
-// where the points share too few cells (launch_nns_lowd with B.grid.work then
-// scans).
+// Nearest active supplier of every active consumer into B.nnkey, unless the rule
+// below sends the round to K1 (launch_nns_lowd with B.grid.work, behind it).
 int launch_nns_grid(const SolveBufs& B, int mt, int nt, cudaStream_t st);
-// The rule, on the device (the cells' work is only known there): points that
-// share few cells leave every warp with a large part of the suppliers, and K1
-// scans those at about 1.7 times the rate.
+// The rule, on the device (what it reads is only known there).  work[0]: points
+// that share few cells lie in no order, so every block has to be looked at; known
+// before the sort.  work[1]: the (consumer, block) pairs the query has scanned,
+// which the cells do not tell (suppliers on a circle around the consumers, two
+// sets in different places).  All of them cost about four times K1's scan
+// (65,536 points on a circle, d = 2: 5.4 ms with K1, 20.3 with every block
+// visited), so a query that is past a sixteenth stops; the keys it has stored
+// stay (K1 merges by minima).
+NNS_DEV unsigned long long grid_most_visits(int mt, int nt) { return (unsigned long long)mt * (unsigned)nt / (32 * 16); }
 NNS_DEV bool grid_served(const unsigned long long* work, int mt, int nt) {
-  return *work <= (unsigned long long)mt * (unsigned)nt / 32;
+  const ulonglong2 w = __ldcg(reinterpret_cast<const ulonglong2*>(work));
+  return w.x <= (unsigned long long)mt * (unsigned)nt / 32 && w.y <= grid_most_visits(mt, nt);
 }
 // Run all remaining rounds of the current active lists in one CTA.
 int launch_finish(const SolveBufs& B, int64_t round_limit, cudaStream_t st);

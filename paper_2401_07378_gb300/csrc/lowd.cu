@@ -50,8 +50,11 @@ template <int D, int DP, bool L1, int K1_P>
 __global__ void __launch_bounds__(K1_THREADS, k1_min_blocks(D, K1_P))
     k_nns_lowd(const float* __restrict__ xa, int mt, int chunk, const float* __restrict__ ya, int nt,
                unsigned long long* __restrict__ nnkey, unsigned* __restrict__ err,
-               const unsigned long long* __restrict__ grid_work) {
-  if (grid_work && grid_served(grid_work, mt, nt)) return;  // (the whole grid leaves)
+               const unsigned long long* __restrict__ grid_work, int* __restrict__ refused) {
+  if (grid_work) {
+    if (grid_served(grid_work, mt, nt)) return;  // (the whole grid leaves)
+    if (blockIdx.x + blockIdx.y + threadIdx.x == 0) *refused = 1;
+  }
   static_assert(K1_TS % 8 == 0, "tile must hold whole groups");
   static_assert(K1_P % 2 == 0, "consumers are packed in pairs");
   __shared__ __align__(128) float tile[2][K1_TS * DP];
@@ -256,23 +259,24 @@ static K1Shape k1_shape(int D, int mt, int nt) {
 }
 
 template <int D, int DP, bool L1>
-static void nns_lowd_t(const SolveBufs& B, int mt, int nt, cudaStream_t st, const unsigned long long* gw) {
+static void nns_lowd_t(const SolveBufs& B, int mt, int nt, cudaStream_t st, const unsigned long long* gw, int* rf) {
   const K1Shape sh = k1_shape(D, mt, nt);
   dim3 grid(sh.gx, sh.gy);
   if (sh.P == 2)
     k_nns_lowd<D, DP, L1, 2><<<grid, K1_THREADS, 0, st>>>(B.xa[B.cur], mt, sh.chunk, B.ya[B.cur], nt, B.nnkey,
-                                                          &B.st->err, gw);
+                                                          &B.st->err, gw, rf);
   else
     k_nns_lowd<D, DP, L1, k1_p(D)><<<grid, K1_THREADS, 0, st>>>(B.xa[B.cur], mt, sh.chunk, B.ya[B.cur], nt,
-                                                                B.nnkey, &B.st->err, gw);
+                                                                B.nnkey, &B.st->err, gw, rf);
 }
 
-int launch_nns_lowd(const SolveBufs& B, int mt, int nt, cudaStream_t st, const unsigned long long* grid_work) {
+int launch_nns_lowd(const SolveBufs& B, int mt, int nt, cudaStream_t st, const unsigned long long* grid_work,
+                    int* refused) {
   const bool l1 = B.metric == METRIC_L1;
 #define NNS_CASE(DD, DPP)                                             \
   case DD:                                                            \
-    if (l1) nns_lowd_t<DD, DPP, true>(B, mt, nt, st, grid_work);      \
-    else nns_lowd_t<DD, DPP, false>(B, mt, nt, st, grid_work);        \
+    if (l1) nns_lowd_t<DD, DPP, true>(B, mt, nt, st, grid_work, refused);  \
+    else nns_lowd_t<DD, DPP, false>(B, mt, nt, st, grid_work, refused);    \
     break;
   switch (B.d) {
     NNS_CASE(1, 2) NNS_CASE(2, 2) NNS_CASE(3, 4) NNS_CASE(4, 4)

@@ -44,6 +44,7 @@ constexpr int GS = 1024;          // suppliers per super-block
 constexpr int GRID_CELLS = 65536; // room for the cells of one side
 constexpr int Q_WARPS = 8;        // warps per CTA of the query
 constexpr int Q_CONS = 8;         // consumers per warp
+constexpr int GRID_TELL = 256;    // a warp adds its visits to the round's total in steps of so many
 
 // cells along one axis: 2^16 in one dimension, 2^8 in two, 2^5 in three
 __host__ __device__ constexpr int grid_bits(int D) { return D == 1 ? 16 : (D == 2 ? 8 : 5); }
@@ -66,7 +67,7 @@ struct GridArgs {
   float4* xs;        // sorted suppliers: coordinates, position (bits)
   float4* ys;        // sorted consumers
   float* boxes;      // [blocks][8]: minima (3, pad), maxima (3, pad); then the super-blocks
-  unsigned long long* work;  // sum over the cells of suppliers x consumers
+  unsigned long long* work;  // [0]: sum over the cells of suppliers x consumers; [1]: visits (k_grid_nns)
   unsigned long long* nnkey;
 };
 
@@ -124,13 +125,27 @@ __global__ void __launch_bounds__(256) k_grid_bounds(GridArgs A) {
   }
 }
 
+// The counter of a point's cell before its point.  A warp whose points lie in
+// one cell takes it at once (they would queue up at one address).  Every lane
+// calls it; those without a point pass a negative counter number.
+NNS_DEV int count_cell(int* counters, int c) {
+  int same;
+  __match_all_sync(0xffffffffu, c, &same);
+  if (!same) return c >= 0 ? atomicAdd(counters + c, 1) : 0;
+  const int lane = threadIdx.x & 31;
+  int at = 0;
+  if (c >= 0 && lane == 0) at = atomicAdd(counters + c, 32);
+  return __shfl_sync(0xffffffffu, at, 0) + lane;
+}
+
 template <int D, int DP>
 __global__ void __launch_bounds__(256) k_grid_count(GridArgs A) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= A.mt + A.nt) return;
   const bool sup = i < A.mt;
-  const float* p = sup ? A.xa + (size_t)i * DP : A.ya + (size_t)(i - A.mt) * DP;
-  atomicAdd(A.hist + (sup ? 0 : GRID_CELLS) + morton_cell<D>(p, A.box), 1);
+  int c = -1;
+  if (i < A.mt + A.nt)
+    c = (sup ? 0 : GRID_CELLS) + morton_cell<D>(sup ? A.xa + (size_t)i * DP : A.ya + (size_t)(i - A.mt) * DP, A.box);
+  count_cell(A.hist, c);
 }
 
 // One block per side: exclusive scan of the cell counts (the next place of
@@ -190,19 +205,21 @@ __global__ void __launch_bounds__(1024) k_grid_scan(GridArgs A) {
 
 template <int D, int DP>
 __global__ void __launch_bounds__(256) k_grid_scatter(GridArgs A) {
+  if (!grid_served(A.work, A.mt, A.nt)) return;
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= A.mt + A.nt) return;
-  const bool sup = i < A.mt;
-  const int pos = sup ? i : i - A.mt;
+  const bool sup = i < A.mt, in = i < A.mt + A.nt;
+  const int pos = sup ? i : (in ? i - A.mt : 0);
   const float* p = (sup ? A.xa : A.ya) + (size_t)pos * DP;
-  const int at = atomicAdd(A.next + (sup ? 0 : GRID_CELLS) + morton_cell<D>(p, A.box), 1);
-  (sup ? A.xs : A.ys)[at] = make_float4(p[0], D > 1 ? p[D > 1 ? 1 : 0] : 0.f, D > 2 ? p[D > 2 ? 2 : 0] : 0.f,
-                                        __uint_as_float((unsigned)pos));
+  const int at = count_cell(A.next, in ? (sup ? 0 : GRID_CELLS) + morton_cell<D>(p, A.box) : -1);
+  if (in)
+    (sup ? A.xs : A.ys)[at] = make_float4(p[0], D > 1 ? p[D > 1 ? 1 : 0] : 0.f, D > 2 ? p[D > 2 ? 2 : 0] : 0.f,
+                                          __uint_as_float((unsigned)pos));
 }
 
 // One block of 1,024 threads per super-block, one warp per block.
 template <int D>
 __global__ void __launch_bounds__(GS) k_grid_boxes(GridArgs A) {
+  if (!grid_served(A.work, A.mt, A.nt)) return;
   __shared__ unsigned slo[3][32], shi[3][32];
   const int i = blockIdx.x * GS + threadIdx.x, lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   const int nb = (A.mt + GB - 1) / GB;
@@ -256,7 +273,8 @@ NNS_DEV bool beyond(float lb, float best) { return __fmul_rd(lb, 1.f - 0x1p-20f)
 
 template <int D, bool L1>
 __global__ void __launch_bounds__(32 * Q_WARPS) k_grid_nns(GridArgs A) {
-  if (!grid_served(A.work, A.mt, A.nt)) return;
+  // (the visits grow meanwhile: a warp leaves as one)
+  if (!__all_sync(0xffffffffu, grid_served(A.work, A.mt, A.nt))) return;
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   const int q0 = (blockIdx.x * Q_WARPS + w) * Q_CONS;
   if (q0 >= A.nt) return;
@@ -270,6 +288,16 @@ __global__ void __launch_bounds__(32 * Q_WARPS) k_grid_nns(GridArgs A) {
   unsigned bpos = 0xffffffffu;
   const int nb = (A.mt + GB - 1) / GB, nsup = (A.mt + GS - 1) / GS;
   const float* sboxes = A.boxes + (size_t)nb * 8;
+  // (consumer, block) pairs scanned so far and those added to the round's total;
+  // false once the round has too many: K1 serves it
+  int visits = 0, told = 0;
+  auto go_on = [&]() {
+    if (visits - told < GRID_TELL) return true;
+    unsigned long long sum = 0;
+    if (lane == 0) sum = atomicAdd(A.work + 1, (unsigned long long)(visits - told)) + (unsigned)(visits - told);
+    told = visits;
+    return __shfl_sync(0xffffffffu, sum, 0) <= grid_most_visits(A.mt, A.nt);
+  };
   // supplier of this lane in block b (past the end: a NaN, which no key beats)
   auto fetch = [&](int b) {
     const int i = b * GB + lane;
@@ -279,6 +307,7 @@ __global__ void __launch_bounds__(32 * Q_WARPS) k_grid_nns(GridArgs A) {
   auto scan = [&](const float4& v, unsigned mask) {
     const float x[3] = {v.x, v.y, v.z};
     const unsigned pos = __float_as_uint(v.w);
+    visits += __popc(mask);
     for (; mask; mask &= mask - 1) {
       const int c = __ffs(mask) - 1;
       float yc[3] = {0.f, 0.f, 0.f};
@@ -332,6 +361,7 @@ __global__ void __launch_bounds__(32 * Q_WARPS) k_grid_nns(GridArgs A) {
         if (bm) scan(v1, __shfl_sync(0xffffffffu, need, l1));
         bm &= bm - 1;
       }
+      if (!go_on()) return;
     }
   }
   if (lane < nq) A.nnkey[__float_as_uint(yq.w)] = pack_key(best, bpos);
@@ -343,7 +373,7 @@ int grid_t(const SolveBufs& B, int mt, int nt, cudaStream_t st) {
   GridArgs A{B.xa[B.cur], B.ya[B.cur], mt, nt, G.box, G.hist, G.hist + 2 * GRID_CELLS, G.start, (float4*)G.xs, (float4*)G.ys, G.boxes, G.work,
              B.nnkey};
   if (cudaMemsetAsync(G.hist, 0, 2 * GRID_CELLS * sizeof(int), st) != cudaSuccess) return -1;
-  if (cudaMemsetAsync(G.work, 0, sizeof(unsigned long long), st) != cudaSuccess) return -1;
+  if (cudaMemsetAsync(G.work, 0, 2 * sizeof(unsigned long long), st) != cudaSuccess) return -1;
   const int g = (mt + nt + 255) / 256;
   k_grid_count<D, DP><<<g, 256, 0, st>>>(A);
   k_grid_scan<D><<<2, 1024, 0, st>>>(A);

@@ -10,7 +10,7 @@ from paper_2401_07378_gb300 import workloads as wl
 torch = pytest.importorskip("torch")
 pytestmark = pytest.mark.gpu
 
-SIDE = 1 << 14       # the smaller side from which a round takes the step
+SIDE = 7 << 11       # the smaller side from which a round takes the step
 ROUND, GRID = 7, 5   # launches of a round with K1; what the step adds to it
 
 
@@ -52,3 +52,51 @@ def test_size_rule(ctx, m, n, d, want):
         got = solve(ctx, p, metric)
         assert got.cost == r.cost and got.stats["rounds"] == r.rounds and got.stats["pair_evals"] == r.pair_evals
         assert (grid_rounds(got.stats) > 0) == want, got.stats
+
+
+def points(kind, n, d, rng, consumers):
+    if kind == "uniform":
+        return rng.random((n, d))
+    if kind == "clusters":
+        c = np.random.default_rng(5).random((6, d))
+        return c[rng.integers(0, 6, n)] + rng.normal(0, 0.01, (n, d))
+    if kind == "lattice":  # many equal points and keys
+        return rng.integers(0, 40, (n, d)) - 20.0
+    if kind == "outlier":  # one far point: every other one in a single cell
+        p = rng.random((n, d)) * 1e-3
+        p[0] = 1e6
+        return p
+    if kind == "ring":  # every supplier about as near as any other
+        p = rng.normal(size=(n, d))
+        return 1e-3 * p if consumers else p / np.linalg.norm(p, axis=1, keepdims=True)
+    if kind == "line":  # an axis without extent
+        p = rng.random((n, d))
+        p[:, -1] = 0.25
+        return p
+    if kind == "tiny":  # squares in the subnormal range
+        return rng.random((n, d)) * 1e-20
+    if kind == "huge":  # squares overflow
+        return (rng.random((n, d)) - 0.5) * 1e20
+    raise ValueError(kind)
+
+
+# want: rounds with the step (None: not told); one where it refuses the points
+@pytest.mark.parametrize("kind,d,want", [("uniform", 3, None), ("clusters", 2, None), ("lattice", 3, None),
+                                         ("line", 2, None), ("tiny", 3, None), ("huge", 3, None),
+                                         ("outlier", 1, 1), ("outlier", 3, 1), ("ring", 2, 1),
+                                         ("ring", 3, 1)])
+def test_refused_points_try_the_step_once(ctx, kind, d, want):
+    rng = np.random.default_rng(len(kind) + d)
+    m, n = (34000, 33900) if want else (SIDE + 1, SIDE + 16)  # (more than one round of that size where it matters)
+    p = wl.Pair(points(kind, m, d, rng, False).astype(np.float32), rng.exponential(1.0, m),
+                points(kind, n, d, rng, True).astype(np.float32), rng.exponential(1.0, n))
+    if not want:
+        p.a[::11 * SIDE] = 0.0
+    for metric in ("l2",) if kind in ("tiny", "huge") or want else ("l2", "l1"):
+        r = oracle.solve_pair(p, metric, threads=0)
+        got = solve(ctx, p, metric)
+        assert got.cost == r.cost and got.stats["rounds"] == r.rounds and got.stats["pair_evals"] == r.pair_evals
+        took = grid_rounds(got.stats)
+        assert took >= 1
+        if want:
+            assert took == want and int((np.minimum(r.m_t, r.n_t) >= SIDE).sum()) > want
