@@ -516,9 +516,9 @@ struct GeoGlobal {
   const float* x;  // [m][d] original coordinates (global)
   const float* y;  // [n][d]
   int d;
-  // The pair's key matrix (nullable): the FP32 key of every original
-  // supplier (row, kld floats apart) and consumer, computed once in the first
-  // round's NNS step; every round is then a minimum over rows of active
+  // The pair's key matrix (nullable), by original supplier (row, kld floats
+  // apart) and consumer: the FP32 keys are computed once in the first round's NNS
+  // step; every round is then a minimum over rows of active
   // suppliers instead of m_t n_t d operations (1 x 4,096 documents, d = 300:
   // 11.7 -> 3.09 ms).
   float* kmat;
@@ -564,6 +564,33 @@ struct GeoGlobal {
                                  if (p < km)
                                    *reinterpret_cast<ulonglong2*>(kmat + (size_t)p * kld + q) =
                                        make_ulonglong2(acc[0][j], acc[1][j]);
+                               }
+                             });
+    }
+  }
+  // The same for a pair of which some points have no weight: the keys of the mt
+  // and nt active ones alone (200 pairs of 1,000 points, d = 300, 5 % of the
+  // weights not zero: 7.5 ms with every point's keys, 0.43 with these, 1.7
+  // without a matrix).
+  template <int C>
+  __device__ __noinline__ void fill_active(const CtaCore<C>& S, int mt, int nt) {
+    const int g = threadIdx.x / TG_THREADS, gt = threadIdx.x % TG_THREADS;
+    const int tx = gt & 15, ty = gt >> 4;
+    const int ct = (nt + TG_M - 1) / TG_M, items = ct * ((mt + TG_N - 1) / TG_N);
+    for (int it = g; it < items; it += NT / TG_THREADS) {
+      const int c0 = (it % ct) * TG_M, p0 = (it / ct) * TG_N;
+      group_tiles<L1, false>(x, S.iidx, p0, min(p0 + TG_N, mt), y, S.jidx, nullptr, c0, min(TG_M, nt - c0), d, tiles[g],
+                             gt, 1 + g, [&](int pt, const unsigned long long (&acc)[2][4]) {
+#pragma unroll
+                               for (int j = 0; j < 4; ++j) {
+                                 const int p = pt + tx * 4 + j;
+                                 if (p >= mt) break;
+                                 float* row = kmat + (size_t)S.iidx[p] * kld;
+#pragma unroll
+                                 for (int i = 0; i < 4; ++i) {
+                                   const int q = c0 + ty * 4 + i;
+                                   if (q < nt) row[S.jidx[q]] = (i & 1) ? f2_hi(acc[i >> 1][j]) : f2_lo(acc[i >> 1][j]);
+                                 }
                                }
                              });
     }
@@ -638,7 +665,8 @@ struct GeoGlobal {
     if (threadIdx.x == 0) searches += nt;
     if (kmat) {
       if (!kready) {
-        fill();
+        if (mt == km && nt == kn) fill();  // (positions are the original indices)
+        else fill_active(S, mt, nt);
         __syncthreads();
         if (threadIdx.x == 0) kready = 1;  // (read again after this step's barriers)
       }
