@@ -47,12 +47,15 @@ struct BtcScratch {
   float* cand_v;    // [cap][BTC_K]
   int* cand_p;
   // distance cache of a pair that fits kc_cap values (see GeoTC::nns_lists), by
-  // original consumer j and supplier i: approximate ranking values v' of the
-  // tensor-core pass, [j / 32][i / 4][j % 32][i % 4] (a warp of 32 consumers
-  // writes four columns as 512 contiguous bytes), and the minimum of each 16
-  // suppliers, [j / 32][i / 16][j % 32]
+  // the positions j, i of consumer and supplier in the pair's first round:
+  // approximate ranking values v' of the tensor-core pass, [j / 32][i / 4][j %
+  // 32][i % 4] (a warp of 32 consumers writes four columns as 512 contiguous
+  // bytes), and the minimum of each 16 suppliers, [j / 32][i / 16][j % 32]; and
+  // those positions by original index, the suppliers' and (from cap on) the
+  // consumers' (unset where every point has weight: the original index itself)
   float* vcache;
   float* vmin;
+  int* pos;
   // candidate lists by original consumer: (exact key bits << 32 | original
   // supplier) ascending, the next entry to look at | length << 8, and the
   // value a key must stay below to be the nearest (certify_floor)
@@ -96,6 +99,7 @@ __host__ __device__ inline size_t btc_slot_layout(uint8_t* base, int cap, int kb
   s.cand_p = (int*)take((size_t)cap * BTC_K * sizeof(int));
   s.vcache = (float*)take((size_t)kc_cap * sizeof(float));
   s.vmin = (float*)take((size_t)(kc_cap / 8) * sizeof(float));  // (kc_ld / 16 rounded up is at most kc_ld / 8 from 16 columns on)
+  s.pos = (int*)take(kc_cap ? 2 * (size_t)cap * sizeof(int) : 0);
   s.list = (unsigned long long*)take(kc_cap ? (size_t)cap * BTC_K * sizeof(unsigned long long) : 0);
   s.lnext = (int*)take(kc_cap ? (size_t)cap * sizeof(int) : 0);
   s.lfloor = (double*)take(kc_cap ? (size_t)cap * sizeof(double) : 0);
@@ -160,9 +164,10 @@ struct GeoTC {
   int nfb, nscan;
   unsigned long long ncert, nfall, nnear;
   // distance cache of the current pair: on (m * n fits), filled (after the
-  // pair's first round), the pair's supplier and consumer counts (the row
-  // length and the number of rows)
-  int kc_on, kc_ready, kc_m, kc_n, kc_ld;
+  // pair's first round), the active suppliers of that round and its row length,
+  // whether every point was active then (positions are original indices)
+  int kc_on, kc_ready, kc_m, kc_ld, kc_dense;
+  int pair_m, pair_n;  // the pair's points
   double kc_gam;  // gamma_d of the certificate
   int fb[CAP];
   // staging: tensor-core operand tiles or FP32 fallback tiles (never both at
@@ -227,6 +232,9 @@ struct GeoTC {
     }
     return false;
   }
+  // cache row of an original consumer, column of an original supplier
+  NNS_DEV int row_of(int j) const { return kc_dense ? j : scr.pos[CAP + j]; }
+  NNS_DEV int col_of(int i) const { return kc_dense ? i : scr.pos[i]; }
   NNS_DEV size_t v_at(int j, int i) const {
     return ((((size_t)(j >> 5) * (kc_ld >> 2)) + (i >> 2)) * 32 + (j & 31)) * 4 + (i & 3);
   }
@@ -313,8 +321,9 @@ struct GeoTC {
     }
     take();
   }
-  // The same for v' while every original supplier is active: each of the 8
-  // smallest lies in one of the 8 groups of 16 with the smallest minima.
+  // The same for v' of cache row j while every supplier of the first round is
+  // active (ids: positions): each of the 8 smallest lies in one of the 8 groups of
+  // 16 with the smallest minima.
   NNS_DEV void groups8(int j, unsigned& rv, int& rid) const {
     const int lane = threadIdx.x & 31;
     const int nb = (kc_ld + 15) >> 4;  // at most 128
@@ -360,11 +369,15 @@ struct GeoTC {
     int i = 0;
 #pragma unroll 1
     for (int h = 0; h < cnt; ++h) {
-      const int jj = S.jidx[qs(h)];
+      const int jj = row_of(S.jidx[qs(h)]);
       unsigned rv;
       int rid;
-      if (mt == kc_m) groups8(jj, rv, rid);
-      else scan8(S, mt, buf, rv, rid, [&](int p) { return ordered_bits(scr.vcache[v_at(jj, S.iidx[p])]); });
+      if (mt == kc_m) {
+        groups8(jj, rv, rid);
+        rid = S.iidx[rid];
+      } else {
+        scan8(S, mt, buf, rv, rid, [&](int p) { return ordered_bits(scr.vcache[v_at(jj, col_of(S.iidx[p]))]); });
+      }
       rv = __shfl_sync(0xffffffffu, rv, sub);
       rid = __shfl_sync(0xffffffffu, rid, sub);
       if (g == h) {
@@ -481,19 +494,28 @@ struct GeoTC {
     const bool fill = kc_on != 0;
     const int tid = threadIdx.x, T = blockDim.x;
     const int warp = tid >> 5, lane = tid & 31;
-    // rows of the tiles: the active points, or, to fill the cache, every
-    // original point (the cache's rows and columns are original indices)
-    const int ms = fill ? kc_m : mt, ns = fill ? kc_n : nt;
-    const int qtiles = (ns + TC_BM - 1) / TC_BM;
-    const int stiles = (ms + bn - 1) / bn;
+    const int qtiles = (nt + TC_BM - 1) / TC_BM;
+    const int stiles = (mt + bn - 1) / bn;
     const int nblk = kb / 16;
     // ---- 1. pack both sides
     if (tid == 0) {
       stat_rx = stat_rx1 = stat_sx = 0u;
       nfb = 0;
     }
-    if (fill)
-      for (int j = tid; j < kc_n; j += T) scr.lnext[j] = 0;  // no lists yet
+    if (fill) {
+      // the cache's rows and columns are this round's positions
+      const bool dense = mt == pair_m && nt == pair_n;
+      if (tid == 0) {
+        kc_m = mt;
+        kc_ld = mt < 16 ? 16 : (int)kmat_ld(mt);
+        kc_dense = dense;
+      }
+      for (int q = tid; q < nt; q += T) scr.lnext[S.jidx[q]] = 0;  // no lists yet
+      if (!dense) {
+        for (int p = tid; p < mt; p += T) scr.pos[S.iidx[p]] = p;
+        for (int q = tid; q < nt; q += T) scr.pos[CAP + S.jidx[q]] = q;
+      }
+    }
     __syncthreads();
     {
       // one warp per row: the lanes take the row's coordinates and 16-byte
@@ -513,8 +535,7 @@ struct GeoTC {
           const bool sup = row_id < srows;
           const int p = sup ? row_id : row_id - srows;
           rows2[h] = nullptr;
-          if (row_id < total && p < (sup ? ms : ns))
-            rows2[h] = (sup ? x : y) + (size_t)(fill ? p : (sup ? S.iidx[p] : S.jidx[p])) * d;
+          if (row_id < total && p < (sup ? mt : nt)) rows2[h] = (sup ? x : y) + (size_t)(sup ? S.iidx[p] : S.jidx[p]) * d;
         }
         for (int k = lane; k < d; k += 32) {
           float v[2];
@@ -562,10 +583,11 @@ struct GeoTC {
                 // what the certificate needs of this consumer in every round
                 // (the norms rounded up: the FP64 sums of the other pass take
                 // 256 FP64 operations a row of 128, here half of the packing)
-                scr.ny_o[p] = l2sq;
-                scr.sy_o[p] = s;
-                scr.yl2_o[p] = norm_up(l2sq);
-                scr.yl1_o[p] = l1 * (1.f + 1e-4f);
+                const int j = S.jidx[p];
+                scr.ny_o[j] = l2sq;
+                scr.sy_o[j] = s;
+                scr.yl2_o[j] = norm_up(l2sq);
+                scr.yl1_o[j] = l1 * (1.f + 1e-4f);
               }
             } else {
               nrm[p] = CUDART_INF_F;
@@ -646,11 +668,11 @@ struct GeoTC {
         unsigned ea = epi_accf;
         for (int qt = 0; qt < qtiles; ++qt) {
           const int q = qt * TC_BM + row;
-          const float sy = q < ns ? scr.scale_y[q] : 1.f;
-          const float cy = quant_coeff(fmt, q < ns ? scr.nrm_y[q] : 0.f);
+          const float sy = q < nt ? scr.scale_y[q] : 1.f;
+          const float cy = quant_coeff(fmt, q < nt ? scr.nrm_y[q] : 0.f);
           float4* vrow = reinterpret_cast<float4*>(scr.vcache + v_at(q, 0));  // column group c at vrow[32 c]
           float* mrow = scr.vmin + (size_t)(q >> 5) * ((kc_ld + 15) >> 4) * 32 + (q & 31);
-          const bool live = (q & ~31) < ns;  // (a warp's 32 rows are written whole)
+          const bool live = (q & ~31) < nt;  // (a warp's 32 rows are written whole)
           for (int st = 0; st < stiles; ++st, ++ea) {
             const unsigned b = ea & 1, v = ea >> 1;
             if (ok) ok = mbar_wait_bounded(&bar_accf_full[b], v & 1);
@@ -743,7 +765,8 @@ struct GeoTC {
       // the supplier maxima of this first round bound every later round's.
       const double rx = __uint_as_float(stat_rx), rx1 = __uint_as_float(stat_rx1);
       const double sxm = __uint_as_float(stat_sx);
-      for (int j = tid; j < ns; j += T) {
+      for (int q = tid; q < nt; q += T) {
+        const int j = S.jidx[q];
         scr.e_o[j] = certify_E(fmt, d, scr.ny_o[j], scr.yl2_o[j], scr.yl1_o[j], scr.sy_o[j], rx, rx1, sxm);
       }
       if (tid == 0) {
@@ -869,11 +892,10 @@ __global__ void __launch_bounds__(FIN_THREADS, 1) k_batched_tc(BtcArgs A) {
       G.x = B.x + xo * B.d;
       G.y = B.y + yo * B.d;
       G.d = B.d;
-      G.kc_ld = m < 16 ? 16 : (int)kmat_ld(m);
       G.kc_on = btc_cache_values(m, n) <= A.kc_cap ? 1 : 0;
       G.kc_ready = 0;
-      G.kc_m = m;
-      G.kc_n = n;
+      G.pair_m = m;
+      G.pair_n = n;
     }
     __syncthreads();
     double cost = 0.0;
