@@ -66,7 +66,7 @@ struct BtcScratch {
   float* sy_o;
   float* yl2_o;
   float* yl1_o;
-  double* e_o;      // per original consumer: E of the certificate (certify_E)
+  double* e_o;      // per original consumer: E of the certificate (certify_E); 0: its cache row holds exact keys
 };
 
 // Values of a pair's distance cache (rows padded to whole warps, columns to
@@ -196,7 +196,7 @@ struct GeoTC {
   // certificate bound (every supplier outside the list has v' >= tau, the
   // list's largest).  A consumer whose list runs out, or whose next entry the
   // bound does not certify, makes a new one from the suppliers active now
-  // (a warp makes four at a time):
+  // (a warp makes up to four at a time):
   //   1. the rk smallest v' (ties by position), their exact FP32 keys, one
   //      per lane in the definition's sequential order, ordered by (key,
   //      original index: positions keep that order);
@@ -204,7 +204,9 @@ struct GeoTC {
   //      supplier maxima (a superset of every later round's); with no other
   //      active supplier every entry is the answer in its turn;
   //   3. not certified: the FP32 tiles over every active supplier, for all
-  //      such consumers of the round together.
+  //      such consumers of the round together.  Their exact keys take the place
+  //      of v' in the cache (E = 0 says so), where a later selection by (key,
+  //      position) needs no certificate.
   // A consumer takes about two searches, so 8 entries serve it; 32 cost more
   // in exact keys (each lane walks its own row) than they saved.  1,000
   // retrieval pairs (256..2,048 points, d = 128, FP16): 43.5 ms with the
@@ -240,7 +242,7 @@ struct GeoTC {
   }
   // The 8 smallest of the warp's words v (four a lane, ~0 for none), in order
   // in lanes 0..7 with their ids: eight minima over the warp, each by one
-  // reduction; equal words by lane.
+  // reduction; equal words in the order of v[0] of every lane, v[1], ...
   NNS_DEV void extract8(unsigned (&v)[4], const int (&id)[4], unsigned& rv, int& rid) const {
     const int lane = threadIdx.x & 31;
     rv = 0xffffffffu;
@@ -250,10 +252,9 @@ struct GeoTC {
       const unsigned mine = min(min(v[0], v[1]), min(v[2], v[3]));
       const unsigned w = __reduce_min_sync(0xffffffffu, mine);
       if (w == 0xffffffffu) break;
-      const int src = __ffs(__ballot_sync(0xffffffffu, mine == w)) - 1;
-      int my = id[3];
-      const int u = v[0] == w ? 0 : (v[1] == w ? 1 : (v[2] == w ? 2 : 3));
-      my = u == 0 ? id[0] : (u == 1 ? id[1] : (u == 2 ? id[2] : id[3]));
+      const unsigned u = v[0] == w ? 0u : (v[1] == w ? 1u : (v[2] == w ? 2u : 3u));
+      const int src = (int)(__reduce_min_sync(0xffffffffu, mine == w ? 32 * u + lane : 0xffffffffu) & 31u);
+      int my = u == 0 ? id[0] : (u == 1 ? id[1] : (u == 2 ? id[2] : id[3]));
       my = __shfl_sync(0xffffffffu, my, src);
       if (lane == src) {
         if (u == 0) v[0] = 0xffffffffu;
@@ -372,7 +373,7 @@ struct GeoTC {
       const int jj = row_of(S.jidx[qs(h)]);
       unsigned rv;
       int rid;
-      if (mt == kc_m) {
+      if (mt == kc_m && scr.e_o[S.jidx[qs(h)]] != 0.0) {
         groups8(jj, rv, rid);
         rid = S.iidx[rid];
       } else {
@@ -405,7 +406,7 @@ struct GeoTC {
     const unsigned tb = __shfl_sync(0xffffffffu, cv, (lane & 24) + len - 1);
     double fl = CUDART_INF;
     bool bad = ((__ballot_sync(0xffffffffu, wanted && !on) >> (lane & 24)) & 0xffu) != 0;
-    if (g < cnt && mt > len) {
+    if (g < cnt && mt > len && scr.e_o[j] != 0.0) {
       const float tau = __uint_as_float((tb & 0x80000000u) ? (tb & 0x7fffffffu) : ~tb);
       fl = certify_floor_from_E(scr.ny_o[j], tau, scr.e_o[j], kc_gam);
       bad |= !((double)__uint_as_float((unsigned)(best >> 32)) < fl);
@@ -418,7 +419,7 @@ struct GeoTC {
       atomicAdd(&ncert, 1ULL);
       if ((int)(unsigned)best != first) atomicAdd(&nnear, 1ULL);
     }
-    // 3. left to the FP32 tiles (their keys are not kept)
+    // 3. left to the FP32 tiles
     if (g < cnt && sub == 0 && bad) {
       scr.lnext[j] = 0;
       const int k = atomicAdd(&nscan, 1);
@@ -433,20 +434,44 @@ struct GeoTC {
   NNS_DEV int* scan_list(CtaCore<C>& S) const { return reinterpret_cast<int*>(S.mem); }
   template <int C>
   NNS_DEV int* scan_first(CtaCore<C>& S) const { return reinterpret_cast<int*>(S.mem2); }
-  // The FP32 tiles over every active supplier for n consumers of a list.
-  template <int C>
-  NNS_DEV void scan_exact(CtaCore<C>& S, int mt, const int* list, int n) {
+  // The FP32 tiles over every active supplier for n consumers of a list; KEEP:
+  // their keys replace v' in the cache.  Up to 128 consumers leave groups
+  // without a tile: those share the suppliers, and the parts merge by atomicMin.
+  template <bool KEEP, int C>
+  __device__ __noinline__ void scan_exact(CtaCore<C>& S, int mt, const int* list, int n) {
     const int g = threadIdx.x / TG_THREADS, gt = threadIdx.x % TG_THREADS;
-    const int ngroups = kThreads / TG_THREADS;
-    for (int c0 = g * TG_M; c0 < n; c0 += ngroups * TG_M) {
+    const int tx = gt & 15, ty = gt >> 4;
+    constexpr int ngroups = kThreads / TG_THREADS;
+    const int ct = (n + TG_M - 1) / TG_M, parts = max(1, ngroups / ct);
+    if (parts > 1) {
+      for (int k = threadIdx.x; k < n; k += kThreads) S.nnk[list[k]] = ~0ULL;
+      __syncthreads();
+    }
+    for (int it = g; it < ct * parts; it += ngroups) {
+      const int c0 = (it % ct) * TG_M, part = it / ct;
+      const int p0 = mt * part / parts, p1 = mt * (part + 1) / parts;
       unsigned long long out[4];
-      group_nns_tile<false>(x, S.iidx, 0, mt, y, S.jidx, list, c0, min(TG_M, n - c0), d, U.tiles[g], gt, 1 + g, out);
-      const int tx = gt & 15, ty = gt >> 4;
+      group_nns_tile<false>(x, S.iidx, p0, p1, y, S.jidx, list, c0, min(TG_M, n - c0), d, U.tiles[g], gt, 1 + g, out,
+                            [&](int pt, const unsigned long long (&acc)[2][4]) {
+                              if (!KEEP) return;
+#pragma unroll 1
+                              for (int i = 0; i < 4 && c0 + ty * 4 + i < n; ++i) {
+                                const int r = row_of(S.jidx[list[c0 + ty * 4 + i]]);
+#pragma unroll
+                                for (int j = 0; j < 4; ++j) {
+                                  const unsigned long long a = i < 2 ? acc[0][j] : acc[1][j];
+                                  const int p = pt + tx * 4 + j;
+                                  if (p < p1) scr.vcache[v_at(r, col_of(S.iidx[p]))] = (i & 1) ? f2_hi(a) : f2_lo(a);
+                                }
+                              }
+                            });
       if (tx == 0)
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
           const int lq = c0 + ty * 4 + i;
-          if (lq < n) S.nnk[list[lq]] = out[i];
+          if (lq >= n) break;
+          if (parts > 1) atomicMin(&S.nnk[list[lq]], out[i]);
+          else S.nnk[list[lq]] = out[i];
         }
     }
   }
@@ -471,16 +496,22 @@ struct GeoTC {
     if ((tid & 31) == 0 && cert) atomicAdd(&ncert, (unsigned long long)cert);
     __syncthreads();
     const int n = nfb;
+    // (a warp makes its lists one after the other: as few each as the warps allow)
+    const int per = min(4, (n + kThreads / 32 - 1) / (kThreads / 32));
 #pragma unroll 1
-    for (int k = 4 * (tid >> 5); k < n; k += 4 * (kThreads / 32))
-      make_lists(S, mt, min(4, n - k), [&](int h) { return fb[k + h]; });
+    for (int k = per * (tid >> 5); k < n; k += per * (kThreads / 32))
+      make_lists(S, mt, min(per, n - k), [&](int h) { return fb[k + h]; });
     __syncthreads();
     const int ns = nscan;
     if (ns > 0) {
-      scan_exact(S, mt, scan_list(S), ns);
+      scan_exact<true>(S, mt, scan_list(S), ns);
       __syncthreads();
-      for (int k = tid; k < ns; k += kThreads)
-        if (S.iidx[(int)(unsigned)S.nnk[scan_list(S)[k]]] != scan_first(S)[k]) atomicAdd(&nnear, 1ULL);
+      for (int k = tid; k < ns; k += kThreads) {
+        const int q = scan_list(S)[k], j = S.jidx[q];
+        if (S.iidx[(int)(unsigned)S.nnk[q]] != scan_first(S)[k]) atomicAdd(&nnear, 1ULL);
+        scr.ny_o[j] = 0.f;  // |x - y|^2 itself is in the cache
+        scr.e_o[j] = 0.0;
+      }
       if (tid == 0) nfall += ns;
       __syncthreads();
     }
@@ -818,7 +849,7 @@ struct GeoTC {
     }
     __syncthreads();
     // ---- 4. FP32 rescan of the consumers that were not certified
-    if (nfb > 0) scan_exact(S, mt, fb, nfb);
+    if (nfb > 0) scan_exact<false>(S, mt, fb, nfb);
     __syncthreads();
     return S.nnk;
   }

@@ -475,11 +475,15 @@ NNS_DEV void group_tiles(const float* __restrict__ x, const int* ia, int p0, int
 // each consumer of group_tiles; returned, in the threads with tx == 0, for
 // their 4 consumers (~0 only where p0 == p1).  A thread starts at +inf and its
 // own first supplier, so a consumer whose keys all overflow to +inf gets the
-// first position, as from a scan in order.
-template <bool L1, bool PRE = false>
+// first position, as from a scan in order.  each(pt, acc) sees every tile of
+// keys as group_tiles' emit does.
+struct NoTile {
+  NNS_DEV void operator()(int, const unsigned long long (&)[2][4]) const {}
+};
+template <bool L1, bool PRE = false, class Each = NoTile>
 NNS_DEV void group_nns_tile(const float* __restrict__ x, const int* ia, int p0, int p1, const float* __restrict__ y,
                             const int* ja, const int* cons, int c0, int nc, int d, TileSmem& T, int gt, int bar,
-                            unsigned long long out[4]) {
+                            unsigned long long out[4], Each each = Each()) {
   const int tx = gt & 15;
   float best[4];
   int bpos[4];
@@ -495,6 +499,7 @@ NNS_DEV void group_nns_tile(const float* __restrict__ x, const int* ia, int p0, 
                              if (lo < best[2 * i]) { best[2 * i] = lo; bpos[2 * i] = pt + tx * 4 + j; }
                              if (hi < best[2 * i + 1]) { best[2 * i + 1] = hi; bpos[2 * i + 1] = pt + tx * 4 + j; }
                            }
+                         each(pt, acc);
                        });
   // reduce over the 16 threads sharing each consumer (adjacent lanes)
 #pragma unroll
