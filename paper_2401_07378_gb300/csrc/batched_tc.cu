@@ -62,10 +62,10 @@ struct BtcScratch {
   unsigned long long* list;
   int* lnext;
   double* lfloor;
-  float* ny_o;      // per original consumer: FP32 squared norm, scale, norms rounded up
+  float* ny_o;      // per original consumer: FP32 squared norm, scale, FP64 norms
   float* sy_o;
-  float* yl2_o;
-  float* yl1_o;
+  double* yl2_o;
+  double* yl1_o;
   double* e_o;      // per original consumer: E of the certificate (certify_E); 0: its cache row holds exact keys
 };
 
@@ -105,8 +105,8 @@ __host__ __device__ inline size_t btc_slot_layout(uint8_t* base, int cap, int kb
   s.lfloor = (double*)take(kc_cap ? (size_t)cap * sizeof(double) : 0);
   s.ny_o = (float*)take(kc_cap ? (size_t)cap * sizeof(float) : 0);
   s.sy_o = (float*)take(kc_cap ? (size_t)cap * sizeof(float) : 0);
-  s.yl2_o = (float*)take(kc_cap ? (size_t)cap * sizeof(float) : 0);
-  s.yl1_o = (float*)take(kc_cap ? (size_t)cap * sizeof(float) : 0);
+  s.yl2_o = (double*)take(kc_cap ? (size_t)cap * sizeof(double) : 0);
+  s.yl1_o = (double*)take(kc_cap ? (size_t)cap * sizeof(double) : 0);
   s.e_o = (double*)take(kc_cap ? (size_t)cap * sizeof(double) : 0);
   if (out) *out = s;
   return (off + 255) & ~(size_t)255;
@@ -612,13 +612,9 @@ struct GeoTC {
                 atomicMax(&stat_sx, __float_as_uint(s));
               } else if (fill) {
                 // what the certificate needs of this consumer in every round
-                // (the norms rounded up: the FP64 sums of the other pass take
-                // 256 FP64 operations a row of 128, here half of the packing)
                 const int j = S.jidx[p];
                 scr.ny_o[j] = l2sq;
                 scr.sy_o[j] = s;
-                scr.yl2_o[j] = norm_up(l2sq);
-                scr.yl1_o[j] = l1 * (1.f + 1e-4f);
               }
             } else {
               nrm[p] = CUDART_INF_F;
@@ -692,8 +688,38 @@ struct GeoTC {
       // tile's columns; a thread holds one consumer's 16 columns and writes
       // them as four 16-byte stores, contiguous over the warp, and their
       // minimum.  (Four warps, each value stored by itself: 39,000 cycles a
-      // tile of 128 x 128.)
-      if (warp >= 4 && warp < 4 + BTC_FILL_WARPS) {
+      // tile of 128 x 128.)  The other warps meanwhile sum the consumers' FP64
+      // norms for the certificate (an FP64 instruction takes 16 cycles a warp: beside
+      // the packing's loads they were half of the packing).
+      constexpr int first = 4 + BTC_FILL_WARPS;
+      if (warp >= first) {
+        // two rows at a time; their four sums share the steps over the lanes
+        for (int q = 2 * (warp - first); q < nt; q += 2 * (T / 32 - first)) {
+          const float* yrow[2];
+          double a2[2] = {0.0, 0.0}, a1[2] = {0.0, 0.0};
+#pragma unroll
+          for (int h = 0; h < 2; ++h) yrow[h] = y + (size_t)S.jidx[min(q + h, nt - 1)] * d;
+          for (int k = lane; k < d; k += 32)
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+              const double v = yrow[h][k];
+              a2[h] += v * v;
+              a1[h] += fabs(v);
+            }
+          // lanes 0..15 take the first row's sums, the others the second's; then
+          // the lower eight of each |y|_2^2, the upper |y|_1
+          const bool up = (lane & 16) != 0, l1 = (lane & 8) != 0;
+          const double s2 = (up ? a2[1] : a2[0]) + __shfl_xor_sync(0xffffffffu, up ? a2[0] : a2[1], 16);
+          const double s1 = (up ? a1[1] : a1[0]) + __shfl_xor_sync(0xffffffffu, up ? a1[0] : a1[1], 16);
+          double sum = (l1 ? s1 : s2) + __shfl_xor_sync(0xffffffffu, l1 ? s2 : s1, 8);
+          for (int o = 4; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+          if ((lane & 7) == 0 && q + (lane >> 4) < nt) {
+            const int j = S.jidx[q + (lane >> 4)];
+            if (l1) scr.yl1_o[j] = sum;
+            else scr.yl2_o[j] = sqrt(sum) * (1 + 1e-12);
+          }
+        }
+      } else if (warp >= 4) {
         const int quarter = warp & 3, part = (warp - 4) >> 2;
         const int row = quarter * 32 + lane;
         unsigned ea = epi_accf;

@@ -547,6 +547,7 @@ template <int G, int RR_ROWS>
 __global__ void __launch_bounds__(RR_THREADS) k_rerank_certify(RerankArgs R) {
   __shared__ unsigned long long s_best[RR_ROWS], s_abest[RR_ROWS];
   __shared__ float s_tau[RR_ROWS];
+  __shared__ double s_l2[RR_ROWS], s_l1[RR_ROWS];  // |y|_2^2 and |y|_1
   __shared__ unsigned s_drop[RR_ROWS];  // the smallest key (bits) a list leaves out
   __shared__ int s_len[RR_ROWS], s_have[RR_ROWS];
   const int nq = R.nq_dev ? min(*R.nq_dev, R.nt) : R.nt;
@@ -565,6 +566,7 @@ __global__ void __launch_bounds__(RR_THREADS) k_rerank_certify(RerankArgs R) {
     unsigned long long e1 = ~0ULL, e2 = ~0ULL;
     unsigned drop = 0xffffffffu;
     int j = 0, have = 0;
+    double l2 = 0.0, l1 = 0.0;
     if (r < nq) {
       const int q = R.sel ? R.sel[r] : r;
       j = R.ja[q];
@@ -594,6 +596,11 @@ __global__ void __launch_bounds__(RR_THREADS) k_rerank_certify(RerankArgs R) {
         } else {
           drop = min(drop, (unsigned)(e >> 32));
         }
+      }
+      for (int k = sub; k < R.d; k += G) {
+        const double v = yrow[k];
+        l2 += v * v;
+        l1 += fabs(v);
       }
     }
     if (R.lists.list) {
@@ -646,13 +653,19 @@ __global__ void __launch_bounds__(RR_THREADS) k_rerank_certify(RerankArgs R) {
       abest = oa < abest ? oa : abest;
       tau = fminf(tau, __shfl_xor_sync(0xffffffffu, tau, o));
       have += __shfl_xor_sync(0xffffffffu, have, o);
+      // (FP64: the first step leaves l2 to the lower lanes and l1 to the upper)
+      const bool up = (sub & (G / 2)) != 0;
+      const double send = o == G / 2 ? (up ? l2 : l1) : l2;
+      l2 = (o == G / 2 && up ? l1 : l2) + __shfl_xor_sync(0xffffffffu, send, o);
     }
     if (sub == 0) {
       s_have[k0] = have;
       s_best[k0] = best;
       s_abest[k0] = abest;
       s_tau[k0] = tau;
+      s_l2[k0] = l2;
     }
+    if (sub == G / 2) s_l1[k0] = l2;
   }
   __syncthreads();
   if (threadIdx.x >= 32) return;
@@ -662,17 +675,15 @@ __global__ void __launch_bounds__(RR_THREADS) k_rerank_certify(RerankArgs R) {
   const unsigned long long best = live ? s_best[lane] : ~0ULL;
   bool certified = false;
   if (live && best != ~0ULL) {
-    // |y|_2 from the FP32 squared norm, rounded up; |y|_1 <= sqrt(d) |y|_2
-    // (it only scales the formats' absolute rounding floors)
     const float ny = R.nrm_y[r];
-    const double yl2 = norm_up(ny);
+    const double yl2 = sqrt(s_l2[lane]) * (1 + 1e-12);
     const float tau = s_tau[lane], key = __uint_as_float((unsigned)(best >> 32));
     // (as certify; the bound itself serves the list too.  tau = +inf: no list
     // is full, so every supplier is a candidate, unless its value was lost to
     // an overflowing norm)
     double fl = CUDART_INF;
     if (tau <= 3.402823466e38f)
-      fl = certify_floor(R.fmt, R.d, ny, yl2, yl2 * sqrt((double)R.d) * (1 + 1e-12), R.scale_y[r],
+      fl = certify_floor(R.fmt, R.d, ny, yl2, s_l1[lane], R.scale_y[r],
                          __uint_as_float(R.stats_x[0]), __uint_as_float(R.stats_x[1]), __uint_as_float(R.stats_x[2]),
                          tau);
     certified = tau <= 3.402823466e38f ? (double)key < fl : s_have[lane] == R.mt;
