@@ -143,9 +143,13 @@ typedef struct {
   int64_t certified;            /* reduced precision: consumer searches settled by the re-rank */
   int64_t fallbacks;            /* reduced precision: consumer searches redone by the FP32 scan */
   int64_t kernel_launches;      /* CUDA kernels this call launched */
-  double nns_kernel_ms;         /* NNSEMD_FLAG_TIME_KERNELS: summed duration of the multi-CTA NNS launches */
-  int64_t nns_kernel_launches;  /* number of those launches */
-  int64_t nns_kernel_pairs;     /* sum of m_t * n_t they evaluated (n_t: the consumers left to them) */
+  double nns_kernel_ms;         /* NNSEMD_FLAG_TIME_KERNELS: summed duration of the NNS steps of the
+                                   multi-CTA rounds (reduced precision: of the tensor-core kernel or, where
+                                   candidate lists leave a few consumers, of their FP32 scan) */
+  int64_t nns_kernel_launches;  /* number of those rounds */
+  int64_t nns_kernel_pairs;     /* pairs those durations stand for: the sum of m_t * n_t, n_t the consumers
+                                   that no candidate list answered; with the grid search (d <= 3, large
+                                   rounds) the full m_t * n_t, of which it visits a small part */
   double tail_kernel_ms;        /* NNSEMD_FLAG_TIME_KERNELS: duration of the one-CTA tail kernel */
   int64_t near_ties;            /* reduced precision: consumer searches whose exact FP32 re-rank picked
                                    another supplier than the one the operand-precision distances ranked

@@ -465,7 +465,8 @@ int run_solve(nnsemd_ctx* ctx, SolveBufs& B, const double* a, const double* b, d
     } else if (B.precision != NNSEMD_FP32) {
       // tensor-core candidates + exact re-rank + certificate + FP32 rescan;
       // the timing events bracket the tensor-core kernel alone.  After the
-      // first round for the consumers that their candidate lists leave open.
+      // first round for the consumers that their candidate lists leave open (a
+      // few of them: the FP32 scan alone, timed in its place).
       B.tc.ev0 = timed ? ctx->ev[0] : nullptr;
       B.tc.ev1 = timed ? ctx->ev[1] : nullptr;
       if (B.lists.list && rounds > 0) {
@@ -481,13 +482,14 @@ int run_solve(nnsemd_ctx* ctx, SolveBufs& B, const double* a, const double* b, d
         if (nf > TC_SCAN_MIN) {
           nrc = launch_nns_tc(B, B.tc, mt, nf, B.precision, st, B.lists.sel, nullptr);
           L += 5;
+        } else if (nf > 0) {
+          launch_add_count(&B.st->fallbacks, (unsigned long long)nf, st);
+          if (timed) CKD(cudaEventRecord(ctx->ev[0], st));
+          nrc = launch_nns_f32(B, mt, nf, B.lists.sel, nullptr, st);
+          if (timed) CKD(cudaEventRecord(ctx->ev[1], st));
+          L += 2;
         } else {
-          nns_timed = false;
-          if (nf > 0) {
-            launch_add_count(&B.st->fallbacks, (unsigned long long)nf, st);
-            nrc = launch_nns_f32(B, mt, nf, B.lists.sel, nullptr, st);
-            L += 2;
-          }
+          nns_timed = false;  // the lists answered all: no pair is evaluated
         }
       } else {
         nrc = launch_nns_tc(B, B.tc, mt, nt, B.precision, st);
