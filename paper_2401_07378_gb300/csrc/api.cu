@@ -793,6 +793,9 @@ int nnsemd_solve_host(nnsemd_ctx* ctx, const float* x, const double* a, int64_t 
   return NNSEMD_OK;
 }
 
+// Captured batched launches a context keeps (NNSEMD_FLAG_GRAPH).
+constexpr size_t MAX_GRAPHS = 32;
+
 // The batched solver.  With y_off == nullptr every pair's consumers are the
 // same n_shared rows of y_packed / b_packed (one-to-many).
 static int solve_batched_impl(nnsemd_ctx* ctx, int32_t num_pairs, const float* x_packed, const double* a_packed,
@@ -884,8 +887,13 @@ static int solve_batched_impl(nnsemd_ctx* ctx, int32_t num_pairs, const float* x
   // key matrices of the d > 8 FP32 solvers, one slot per CTA; a solver whose
   // slots exceed the budget, or any if the memory is not there, computes the
   // keys again in every round instead
+  // (slots in steps of a sixteenth of their size, so that batches of nearly the
+  // same pairs replay the same graph)
   auto km_slot = [&](int64_t km, int g) -> long long {
-    return d <= 8 || (double)km * g * sizeof(float) > KC_BUDGET_BYTES ? 0 : (km + 63) & ~63LL;
+    int64_t step = 64;
+    while (step * 16 <= km) step *= 2;
+    km = (km + step - 1) / step * step;
+    return d <= 8 || (double)km * g * sizeof(float) > KC_BUDGET_BYTES ? 0 : km;
   };
   long long kc_big = tc ? 0 : km_slot(km_big, gbig), kc_tiny = km_slot(km_tiny, gtiny);
   // workspace: offsets, pair list, queue/error/counters, per-pair counters,
@@ -1047,6 +1055,11 @@ static int solve_batched_impl(nnsemd_ctx* ctx, int32_t num_pairs, const float* x
         ce = cudaGraphInstantiate(&exec, graph, 0);
         cudaGraphDestroy(graph);
         if (ce != cudaSuccess) return cuda_fail(ctx, ce, "cudaGraphInstantiate");
+        if (ctx->graphs.size() >= MAX_GRAPHS) {  // the oldest makes room (it may still run, on any stream)
+          cudaDeviceSynchronize();
+          cudaGraphExecDestroy(ctx->graphs.front().exec);
+          ctx->graphs.erase(ctx->graphs.begin());
+        }
         ctx->graphs.push_back({key, exec});
         g = &ctx->graphs.back();
       }
