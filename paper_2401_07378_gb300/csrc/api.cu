@@ -120,15 +120,23 @@ struct Carve {
   }
 };
 
-int ensure_ws(nnsemd_ctx* ctx, size_t bytes) {
+// `spare`: a layout that has a smaller one behind it; where the device is too
+// full for it the workspace stays as it is (else every call of a full device
+// would give it back, fail, and allocate the smaller one again).
+int ensure_ws(nnsemd_ctx* ctx, size_t bytes, bool spare = false) {
   if (bytes <= ctx->ws_bytes) return NNSEMD_OK;
+  size_t want = bytes + bytes / 8;
+  if (spare) {
+    size_t free_bytes = 0, total = 0;
+    if (cudaMemGetInfo(&free_bytes, &total) == cudaSuccess && free_bytes + ctx->ws_bytes < want)
+      return fail(ctx, NNSEMD_ERR_OOM, "workspace of %zu bytes: %zu free", want, free_bytes);
+  }
   if (ctx->ws) {
     cudaStreamSynchronize(ctx->stream);
     cudaFree(ctx->ws);
     ctx->ws = nullptr;
     ctx->ws_bytes = 0;
   }
-  size_t want = bytes + bytes / 8;
   cudaError_t e = cudaMalloc(&ctx->ws, want);
   if (e != cudaSuccess) {
     cudaGetLastError();
@@ -682,7 +690,7 @@ int nnsemd_solve(nnsemd_ctx* ctx, const float* x, const double* a, int64_t m, co
   SolveBufs B{};
   LearnedBufs Lb{};
   bool extras = true;
-  rc = ensure_ws(ctx, layout_solve(nullptr, m, n, d, B, extras, precision, P, P ? &Lb : nullptr));
+  rc = ensure_ws(ctx, layout_solve(nullptr, m, n, d, B, extras, precision, P, P ? &Lb : nullptr), true);
   if (rc == NNSEMD_ERR_OOM) {
     extras = false;
     ctx->err.clear();
@@ -747,7 +755,7 @@ int nnsemd_solve_host(nnsemd_ctx* ctx, const float* x, const double* a, int64_t 
   float *xd, *yd;
   double *ad, *bd, *pf;
   int32_t *pi, *pj;
-  rc = ensure_ws(ctx, stage_layout(nullptr, &xd, &ad, &yd, &bd, &pi, &pj, &pf));
+  rc = ensure_ws(ctx, stage_layout(nullptr, &xd, &ad, &yd, &bd, &pi, &pj, &pf), true);
   if (rc == NNSEMD_ERR_OOM) {
     extras = false;
     solve_bytes = layout_solve(nullptr, m, n, d, B, extras, precision, P, P ? &Lb : nullptr);
@@ -932,7 +940,7 @@ static int solve_batched_impl(nnsemd_ctx* ctx, int32_t num_pairs, const float* x
   SolveBufs B{};
   bool extras = true;
   auto large_bytes = [&] { return large.empty() ? 0 : layout_solve(nullptr, maxm, maxn, d, B, extras, precision); };
-  rc = ensure_ws(ctx, layout_head(nullptr) + large_bytes());
+  rc = ensure_ws(ctx, layout_head(nullptr) + large_bytes(), true);
   if (rc == NNSEMD_ERR_OOM) {  // without key matrices either
     kc_big = kc_tiny = 0;
     extras = false;
