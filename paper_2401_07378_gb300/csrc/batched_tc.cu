@@ -62,7 +62,7 @@ struct BtcScratch {
   unsigned long long* list;
   int* lnext;
   double* lfloor;
-  float* ny_o;      // per original consumer: FP32 squared norm, scale, FP64 norms
+  float* ny_o;      // per original consumer: FP32 squared norm, scale, FP64 |y|_2^2 and |y|_1
   float* sy_o;
   double* yl2_o;
   double* yl1_o;
@@ -688,38 +688,11 @@ struct GeoTC {
       // tile's columns; a thread holds one consumer's 16 columns and writes
       // them as four 16-byte stores, contiguous over the warp, and their
       // minimum.  (Four warps, each value stored by itself: 39,000 cycles a
-      // tile of 128 x 128.)  The other warps meanwhile sum the consumers' FP64
-      // norms for the certificate (an FP64 instruction takes 16 cycles a warp: beside
-      // the packing's loads they were half of the packing).
-      constexpr int first = 4 + BTC_FILL_WARPS;
-      if (warp >= first) {
-        // two rows at a time; their four sums share the steps over the lanes
-        for (int q = 2 * (warp - first); q < nt; q += 2 * (T / 32 - first)) {
-          const float* yrow[2];
-          double a2[2] = {0.0, 0.0}, a1[2] = {0.0, 0.0};
-#pragma unroll
-          for (int h = 0; h < 2; ++h) yrow[h] = y + (size_t)S.jidx[min(q + h, nt - 1)] * d;
-          for (int k = lane; k < d; k += 32)
-#pragma unroll
-            for (int h = 0; h < 2; ++h) {
-              const double v = yrow[h][k];
-              a2[h] += v * v;
-              a1[h] += fabs(v);
-            }
-          // lanes 0..15 take the first row's sums, the others the second's; then
-          // the lower eight of each |y|_2^2, the upper |y|_1
-          const bool up = (lane & 16) != 0, l1 = (lane & 8) != 0;
-          const double s2 = (up ? a2[1] : a2[0]) + __shfl_xor_sync(0xffffffffu, up ? a2[0] : a2[1], 16);
-          const double s1 = (up ? a1[1] : a1[0]) + __shfl_xor_sync(0xffffffffu, up ? a1[0] : a1[1], 16);
-          double sum = (l1 ? s1 : s2) + __shfl_xor_sync(0xffffffffu, l1 ? s2 : s1, 8);
-          for (int o = 4; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
-          if ((lane & 7) == 0 && q + (lane >> 4) < nt) {
-            const int j = S.jidx[q + (lane >> 4)];
-            if (l1) scr.yl1_o[j] = sum;
-            else scr.yl2_o[j] = sqrt(sum) * (1 + 1e-12);
-          }
-        }
-      } else if (warp >= 4) {
+      // tile of 128 x 128.)  Meanwhile the other warps, and these when they are
+      // done, sum the consumers' FP64 norms for the certificate (an FP64 instruction
+      // takes 16 cycles a warp: beside the packing's loads they were half of the
+      // packing).
+      if (warp >= 4 && warp < 4 + BTC_FILL_WARPS) {
         const int quarter = warp & 3, part = (warp - 4) >> 2;
         const int row = quarter * 32 + lane;
         unsigned ea = epi_accf;
@@ -765,6 +738,35 @@ struct GeoTC {
             __syncwarp();
             if (lane == 0) mbar_arrive(&bar_accf_empty[b]);
           }
+        }
+      }
+      // two rows at a time; their four sums share the steps over the lanes
+      for (;;) {
+        int q = 0;
+        if (lane == 0) q = atomicAdd(&nfb, 2);  // (its next use starts from 0)
+        q = __shfl_sync(0xffffffffu, q, 0);
+        if (q >= nt) break;
+        const float* yrow[2];
+        double a2[2] = {0.0, 0.0}, a1[2] = {0.0, 0.0};
+#pragma unroll
+        for (int h = 0; h < 2; ++h) yrow[h] = y + (size_t)S.jidx[min(q + h, nt - 1)] * d;
+        for (int k = lane; k < d; k += 32)
+#pragma unroll
+          for (int h = 0; h < 2; ++h) {
+            const double v = yrow[h][k];
+            a2[h] += v * v;
+            a1[h] += fabs(v);
+          }
+        // lanes 0..15 take the first row's sums, the others the second's; then
+        // the lower eight of each |y|_2^2, the upper |y|_1
+        const bool up = (lane & 16) != 0, l1 = (lane & 8) != 0;
+        const double s2 = (up ? a2[1] : a2[0]) + __shfl_xor_sync(0xffffffffu, up ? a2[0] : a2[1], 16);
+        const double s1 = (up ? a1[1] : a1[0]) + __shfl_xor_sync(0xffffffffu, up ? a1[0] : a1[1], 16);
+        double sum = (l1 ? s1 : s2) + __shfl_xor_sync(0xffffffffu, l1 ? s2 : s1, 8);
+        for (int o = 4; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+        if ((lane & 7) == 0 && q + (lane >> 4) < nt) {
+          const int j = S.jidx[q + (lane >> 4)];
+          (l1 ? scr.yl1_o : scr.yl2_o)[j] = sum;
         }
       }
     } else if (warp < 6) {
@@ -824,7 +826,8 @@ struct GeoTC {
       const double sxm = __uint_as_float(stat_sx);
       for (int q = tid; q < nt; q += T) {
         const int j = S.jidx[q];
-        scr.e_o[j] = certify_E(fmt, d, scr.ny_o[j], scr.yl2_o[j], scr.yl1_o[j], scr.sy_o[j], rx, rx1, sxm);
+        scr.e_o[j] = certify_E(fmt, d, scr.ny_o[j], sqrt(scr.yl2_o[j]) * (1 + 1e-12), scr.yl1_o[j], scr.sy_o[j], rx, rx1,
+                                sxm);
       }
       if (tid == 0) {
         kc_gam = certify_gamma(d);
