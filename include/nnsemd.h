@@ -35,7 +35,8 @@
  *
  * Memory: every array argument is caller-owned.  Pointers are DEVICE
  * pointers unless the name or comment says host.  The context owns only its
- * workspace (grown on demand, freed by nnsemd_destroy).  Coordinates are
+ * workspace (grown on demand to the largest call, freed by nnsemd_destroy; a
+ * batch of d > 8 pairs of up to 2,048 points takes up to some 3 GB).  Coordinates are
  * float32 row-major [points][d] (4-byte aligned); weights are float64
  * (8-byte aligned).
  *
@@ -98,7 +99,8 @@ typedef struct {
                                        batch the first time a (d, precision, size) class is seen; the winner
                                        is kept in the context for later calls */
 #define NNSEMD_FLAG_GRAPH 4         /* nnsemd_solve_batched: capture the device work of the call in a CUDA
-                                       graph and replay it while the buffers and sizes repeat */
+                                       graph and replay it while the buffers and sizes repeat (a
+                                       context keeps the last 32 captures) */
 
 /* How a supplier serves the consumers that picked it (Sec. III-A):
  * GREEDY (the paper's default, Alg. 1) in ascending distance, equal

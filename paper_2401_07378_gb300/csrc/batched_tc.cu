@@ -210,7 +210,7 @@ struct GeoTC {
   // A consumer takes about two searches, so 8 entries serve it; 32 cost more
   // in exact keys (each lane walks its own row) than they saved.  1,000
   // retrieval pairs (256..2,048 points, d = 128, FP16): 43.5 ms with the
-  // candidates selected anew in every round, 16.3 ms so.
+  // candidates selected anew in every round, 16.1 ms so.
   //
   // S.off holds, by original index, the position of each active supplier
   // (free until the round's grouping); a stale entry fails its check.

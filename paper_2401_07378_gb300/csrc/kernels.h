@@ -16,7 +16,8 @@ constexpr int K1_TS = 256;
 // cudaDevAttrMultiProcessorCount, looked up once per device); grids are
 // sized in multiples of it.
 int num_sms();
-// K2 grid target (consumer tiles x supplier chunks): four CTAs per SM.
+// K2's candidate buffers hold this many (consumer tile, supplier chunk) pairs:
+// four CTAs per SM (launch_nns_tc chooses the chunks).
 inline int tc_target_ctas() { return 4 * num_sms(); }
 constexpr int PAD_POINTS = K1_TS;
 // Largest active set the single-CTA solver keeps in shared memory (d <= 8:
@@ -223,7 +224,9 @@ int launch_batched_lowd(const BatchArgs& A, int grid, cudaStream_t st);
 // pairs hide and more threads lengthen: 2,048 image pairs of 80..400 points
 // took 2.01 ms with one 1,024-thread CTA per SM, 881 us with two of 512
 // threads, 610 us with four of 256 and 607 us with six of 128; a single
-// 256-point pair 84 us at 1,024 threads, 58 at 512, 62 at 256 and at 128.
+// 256-point pair 84 us at 1,024 threads, 58 at 512, 62 at 256 and at 128.  (The
+// single pair takes the batches' 256 threads too: a class of 512 would be sixteen
+// instantiations more for 4 us.)
 constexpr int LOWD_SMALL_CAP = 512;
 constexpr int LOWD_SMALL_THREADS = 256;
 constexpr int LOWD_SMALL_PER_SM = 4;

@@ -535,9 +535,10 @@ struct RerankArgs {
 //
 // The certificate is about fifty FP64 operations a row, and an FP64
 // instruction holds its pipe as long for one active lane as for 32: the last
-// step takes one row per lane of a warp.  (One warp per row, its certificate
-// in one lane, its norms summed in FP64 and its counters updated one by one
-// took 725 us for 131,072 rows, against 100 of candidate rows read.)
+// step takes one row per lane of a warp; the FP64 norms before it are sums over
+// a row's lanes.  (One warp per row, its certificate in one lane and its counters
+// updated one by one took 725 us for 131,072 rows, against 100 of candidate rows
+// read.)
 // Where a block of 32 rows would leave SMs idle (few consumers, many chunks of
 // candidates: a few thousand consumers of a learned round took 300 us), RR_ROWS
 // is 8, one row a warp.
